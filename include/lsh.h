@@ -62,7 +62,10 @@ enum { LSH_GREEN_TRUNCATED = 0, LSH_GREEN_FILTERED = 1, LSH_GREEN_FD = 2 };
  * products and CG scalars in double, wrapped in iterative refinement whose
  * residual b - K x is computed to double-precision accuracy: in double-float
  * arithmetic (see LSH_F64_DF) where the grid allows it, else with the FP64
- * operator.  The environment variable LSH_NO_DF=1 at lsh_setup forces the
+ * operator.  Where K is definite the FP32 CG is preconditioned by a diagonal
+ * (1 / (|M_beta| + g), g the diagonal of the filtered Green operator, 0 for the
+ * others), and so is FP64 CG on handles with a per-voxel field; FP64 CG on
+ * phase maps is not.  The stopping rule is on the residual itself either way.  The environment variable LSH_NO_DF=1 at lsh_setup forces the
  * FP64 operator. */
 enum { LSH_FP64 = 0, LSH_MIXED = 1 };
 /* element type of fields passed to lsh_apply.  LSH_F64_DF: FP64 fields, the

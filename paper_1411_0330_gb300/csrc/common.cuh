@@ -40,6 +40,7 @@ template <typename T> __device__ __forceinline__ C2<T> cscale(C2<T> a, T s) { re
 // Device-resident state of one Krylov solve.  Scalars are always FP64.
 struct SolverState {
   double rr;        // (r_k, r_k)
+  double rz;        // (r_k, D r_k), D the preconditioner (rr where there is none)
   double bb;        // (b, b) of the system being solved
   double tol2;      // stop when rr <= tol2 (= tol^2 bb)
   double alpha;     // alpha of the last completed iteration (0 after breakdown)
@@ -194,6 +195,13 @@ __device__ __forceinline__ double gather_partials_sys(const double* partials, un
   s = block_sum(s);
   if (threadIdx.x == 0) *counter = 0u;
   return s;
+}
+
+// The same for two sums of one block: the second one's partials sit `off` further on.
+__device__ __forceinline__ bool publish_partial_sys2(double* partials, long long off, unsigned int b, unsigned int nb,
+                                                     double v, double w, unsigned int* counter) {
+  if (threadIdx.x == 0) partials[off + b] = w;  // ordered before the ticket by publish_partial_sys's fence
+  return publish_partial_sys(partials, b, nb, v, counter);
 }
 
 // Scalars of one system's MINRES recurrence (Lanczos + Givens, Paige-Saunders),

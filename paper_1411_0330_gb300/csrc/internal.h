@@ -46,6 +46,12 @@ template <typename T> struct OpArgs {
   const T* mtab;               // per phase * c: diagonal of M (no scale field)
   const T* modtab;             // per phase * c: diagonal of A_phase (scale field)
   T ref[6];                    // diagonal of A0 (internal basis)
+  // diagonal preconditioner of the CG iterations, D = 1 / (|M_beta| + gpre): 0 none,
+  // 1 per phase, 2 per voxel (scale or fraction field).  The residual buffer then
+  // holds z = D r, so that p = z + beta p needs no phase map.
+  int pre;
+  const T* dtab;               // per phase * c: D (1 outside I0)
+  T gpre[6];                   // share of the diagonal of the Green operator, per component
   const T* loads;              // [S][6] macroscopic load per system (internal basis)
   // Green operator computed in the z pass instead of read from gtab (truncated
   // operator, FP32): physics, grid lengths, signed-frequency tables, constants
@@ -107,11 +113,12 @@ template <typename T>
 void launch_xinv(const OpArgs<T>& a, const LaunchCfg& L, int mode, const T* xin, T* out, SolverState* st,
                  double* partials, cudaStream_t s);
 template <typename T>
-void launch_cg_update(T* r, const T* q, long long n, int S, SolverState* st, double* partials, int G, cudaStream_t s);
+void launch_cg_update(const OpArgs<T>& a, T* r, const T* q, SolverState* st, double* partials, long long off2, int G,
+                      cudaStream_t s);
 template <typename T>
 void launch_cg_finalize(T* x, const T* p, long long n, int S, const SolverState* st, int G, cudaStream_t s);
 template <typename T>
-void launch_cg_begin(const T* r, long long n, int S, SolverState* st, double* partials, double tol,
+void launch_cg_begin(const OpArgs<T>& a, T* r, SolverState* st, double* partials, long long off2, double tol,
                      const double* bb_given, int G, cudaStream_t s);
 template <typename T>
 void launch_fill_rhs(const OpArgs<T>& a, T* r, T* x, int G, cudaStream_t s);
@@ -126,8 +133,10 @@ void launch_gamma_table(const OpArgs<T>& a, int dim, int physics, int green, con
 template <typename T>
 void launch_rotate_scalar(const T* in, T* out, long long V, int nsys, int d, const double* R, int to_internal,
                           cudaStream_t s);
-void launch_d2f_begin(const double* r64, bool df_pairs, float* r32, float* x32, long long n, int S, SolverState* st,
-                      double* partials, double tol, const unsigned char* active, int G, cudaStream_t s);
+void launch_gamma_diag(const OpArgs<double>& a, double* partials, int nblk, double* out, cudaStream_t s);
+void launch_d2f_begin(const OpArgs<float>& a, const double* r64, bool df_pairs, float* r32, float* x32, SolverState* st,
+                      double* partials, long long off2, double tol, const unsigned char* active, int G,
+                      cudaStream_t s);
 void launch_f2d_axpy(double* x64, const float* x32, long long n, cudaStream_t s);
 void launch_scan_phase(const unsigned char* phase, long long V, int B, const unsigned char* act, int nphase,
                        SolverState* st, double* partials, int G, cudaStream_t s);

@@ -17,6 +17,7 @@
 // Every pass handles S independent systems at once (batched loads and
 // microstructures); each system has its own CG state and reductions.
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "fft.cuh"
@@ -402,7 +403,7 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_xinv(OpArgs<T
             sst->alpha = 0.0;
             sst->done = 1;
           } else {
-            sst->alpha = sst->rr / sum;
+            sst->alpha = sst->rz / sum;
           }
         } else if (MODE == 3) {
           sst->pq = sum;  // (v, K v) for MINRES: any sign, no breakdown test
@@ -434,7 +435,7 @@ __global__ void __launch_bounds__(kThreads) k_dot_finalize(SolverState* __restri
       sst->alpha = 0.0;
       sst->done = 1;
     } else {
-      sst->alpha = sst->rr / sum;
+      sst->alpha = sst->rz / sum;
     }
   }
 }
@@ -714,43 +715,114 @@ __global__ void k_mr_begin(SolverState* __restrict__ st, MinresScalars* __restri
 
 // ------------------------------------------------------------------ CG vector kernels
 // Grid (G, S): blockIdx.y is the system, n the elements per system.
-template <typename T>
-__global__ void __launch_bounds__(kThreads) k_cg_update(T* __restrict__ r, const T* __restrict__ q, long long n,
-                                                        SolverState* __restrict__ st, double* __restrict__ partials) {
+//
+// The elements of a system one component plane after the other, so that the
+// component is uniform in each sweep and the voxel index needs no division;
+// 16-byte pieces where every plane starts on a 16-byte boundary.
+template <typename T, typename F> __device__ __forceinline__ void sweep_planes(int c, long long V, F f) {
+  constexpr int VEC = 16 / sizeof(T);
+  const long long nv = (V % VEC == 0) ? V / VEC : 0;
+  const long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x, di = (long long)gridDim.x * blockDim.x;
+  for (int comp = 0; comp < c; ++comp) {
+    for (long long i = i0; i < nv; i += di) f(comp, i * VEC, std::integral_constant<int, VEC>());
+    for (long long i = nv * VEC + i0; i < V; i += di) f(comp, i, std::integral_constant<int, 1>());
+  }
+}
+
+// Diagonal preconditioner D = 1 / (|M_beta| + gpre) of one voxel (PRE of OpArgs).
+// Why: K = M + P Gamma P has the condition number of M's spread times Gamma's.  For
+// the truncated and the finite-difference operator Gamma is A0^{-1/2} times a
+// projector times A0^{-1/2}; with D = |M|^{-1} (gpre = 0) the preconditioned
+// operator is the identity plus a compression of (A - A0), whose condition number
+// is the contrast itself instead of the contrast times that of Gamma.  The
+// filtered operator has no kernel of that size, there D is the diagonal of K.
+// FP32 iterations to 5e-6 (and 1e-10), 32^3 spheres at f = 0.3: contrast 10
+// truncated 46 (88) -> 22 (39), filtered 38 (75) -> 24 (46); contrast 1000
+// truncated 415 (850) -> 223 (400), filtered 116 (232) -> 72 (144).
+template <typename T, int PRE>
+__device__ __forceinline__ T precond(const OpArgs<T>& a, const T* __restrict__ dloc, int comp, int ph, long long pv) {
+  if constexpr (PRE == 1) return dloc[ph * a.c + comp];
+  const T f = (T)a.scale[pv];
+  if (a.frac) {
+    const T m = f * a.mtab[a.c + comp] + ((T)1 - f) * a.mtab[comp];  // Eq. (def_ah)
+    return (T)1 / (fabs(m) + a.gpre[comp]);
+  }
+  const T d = fabs(f * a.modtab[ph * a.c + comp] - a.ref[comp]);
+  return a.gpre[comp] == (T)0 ? d : d / ((T)1 + a.gpre[comp] * d);
+}
+
+template <int VEC> __device__ __forceinline__ void phase_load(const unsigned char* __restrict__ p, int* ph) {
+  if constexpr (VEC == 4) {
+    const uchar4 q = *reinterpret_cast<const uchar4*>(p);
+    ph[0] = q.x; ph[1] = q.y; ph[2] = q.z; ph[3] = q.w;
+  } else if constexpr (VEC == 2) {
+    const uchar2 q = *reinterpret_cast<const uchar2*>(p);
+    ph[0] = q.x; ph[1] = q.y;
+  } else {
+    ph[0] = p[0];
+  }
+}
+
+// r -= alpha q (PRE: z -= alpha D q on the stored z = D r) and the sums (r, r),
+// (r, z) -> beta, convergence.
+template <typename T, int PRE>
+__global__ void __launch_bounds__(kThreads) k_cg_update(OpArgs<T> a, T* __restrict__ r, const T* __restrict__ q,
+                                                        SolverState* __restrict__ st, double* __restrict__ partials,
+                                                        long long off2) {
   const int s = blockIdx.y;
   SolverState* sst = st + s;
   if (sst->done) return;
+  __shared__ T dloc[PRE == 1 ? 256 * 6 : 1];
+  if (PRE == 1) {
+    for (int i = threadIdx.x; i < a.nphase * a.c; i += blockDim.x) dloc[i] = a.dtab[i];
+    __syncthreads();
+  }
   const T al = (T)sst->alpha;
+  const long long n = (long long)a.c * a.V;
   T* rs = r + s * n;
   const T* qs = q + s * n;
-  Acc<T> acc;
-  constexpr int VEC = 16 / sizeof(T);
-  // 16-byte accesses only when every system's range starts on a 16-byte boundary
-  const long long nv = (n % VEC == 0) ? n / VEC : 0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nv; i += (long long)gridDim.x * blockDim.x) {
+  const long long pbase = (long long)((a.sys0 + s) / a.sys_per_ms) * a.V;
+  Acc<T> acc, accz;
+  // without the preconditioner nothing depends on the component: one flat sweep
+  sweep_planes<T>(PRE ? a.c : 1, PRE ? a.V : n, [&](int comp, long long i, auto vec) {
+    constexpr int VEC = decltype(vec)::value;
+    const long long g = comp * a.V + i;
     T rv[VEC], qv[VEC];
-    vload<T, VEC>(rs + i * VEC, rv);
-    vload<T, VEC>(qs + i * VEC, qv);
+    int ph[VEC];
+    if (PRE) phase_load<VEC>(a.phase + pbase + i, ph);
+    vload<T, VEC>(rs + g, rv);
+    vload<T, VEC>(qs + g, qv);
 #pragma unroll
     for (int u = 0; u < VEC; ++u) {
-      rv[u] -= al * qv[u];
-      acc.add(rv[u] * rv[u]);
+      if constexpr (PRE == 0) {
+        rv[u] -= al * qv[u];
+        acc.add(rv[u] * rv[u]);
+      } else {
+        const T d = precond<T, PRE>(a, dloc, comp, ph[u], pbase + i + u);
+        rv[u] -= al * (d * qv[u]);
+        const T ru = rv[u] / d;
+        acc.add(ru * ru);
+        accz.add(ru * rv[u]);
+      }
     }
-    vstore<T, VEC>(rs + i * VEC, rv);
-  }
-  for (long long i = nv * VEC + blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    const T rv = rs[i] - al * qs[i];
-    rs[i] = rv;
-    acc.add(rv * rv);
-  }
+    vstore<T, VEC>(rs + g, rv);
+  });
   const double tot = block_reduce(acc);
+  double totz = 0.0;
+  if (PRE) {
+    __syncthreads();
+    totz = block_reduce(accz);
+  }
   double* part = partials + (long long)s * gridDim.x;
-  if (publish_partial_sys(part, blockIdx.x, gridDim.x, tot, &sst->counter[1])) {
+  const bool last = PRE ? publish_partial_sys2(part, off2, blockIdx.x, gridDim.x, tot, totz, &sst->counter[1])
+                        : publish_partial_sys(part, blockIdx.x, gridDim.x, tot, &sst->counter[1]);
+  if (last) {
     const double rrn = gather_partials_sys(part, gridDim.x, &sst->counter[1]);
+    const double rzn = PRE ? gather_partials_sys(part + off2, gridDim.x, &sst->counter[1]) : rrn;
     if (threadIdx.x == 0) {
-      sst->beta = rrn / sst->rr;
+      sst->beta = rzn / sst->rz;
       sst->rr = rrn;
+      sst->rz = rzn;
       sst->iter += 1;
       if (!isfinite(rrn)) {
         sst->status = 5;
@@ -775,23 +847,46 @@ __global__ void k_cg_finalize(T* __restrict__ x, const T* __restrict__ p, long l
     xs[i] += a * ps[i];
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kThreads) k_cg_begin(const T* __restrict__ r, long long n,
-                                                       SolverState* __restrict__ st, double* __restrict__ partials,
-                                                       double tol, const double* __restrict__ bb_given) {
+// Start of a CG solve on the right-hand side in r: (r, r), and with PRE r <- z = D r
+// and (r, z).
+template <typename T, int PRE>
+__global__ void __launch_bounds__(kThreads) k_cg_begin(OpArgs<T> a, T* __restrict__ r, SolverState* __restrict__ st,
+                                                       double* __restrict__ partials, long long off2, double tol,
+                                                       const double* __restrict__ bb_given) {
   const int s = blockIdx.y;
-  const T* rs = r + s * n;
-  Acc<T> acc;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    acc.add(rs[i] * rs[i]);
+  const long long n = (long long)a.c * a.V;
+  T* rs = r + s * n;
+  const long long pbase = (long long)((a.sys0 + s) / a.sys_per_ms) * a.V;
+  Acc<T> acc, accz;
+  sweep_planes<T>(a.c, a.V, [&](int comp, long long i, auto vec) {
+    constexpr int VEC = decltype(vec)::value;
+    T rv[VEC];
+    int ph[VEC];
+    if (PRE) phase_load<VEC>(a.phase + pbase + i, ph);
+    vload<T, VEC>(rs + comp * a.V + i, rv);
+#pragma unroll
+    for (int u = 0; u < VEC; ++u) {
+      acc.add(rv[u] * rv[u]);
+      if constexpr (PRE != 0) {
+        const T z = precond<T, PRE>(a, a.dtab, comp, ph[u], pbase + i + u) * rv[u];
+        accz.add(z * rv[u]);
+        rv[u] = z;
+      }
+    }
+    if (PRE) vstore<T, VEC>(rs + comp * a.V + i, rv);
+  });
   const double tot = block_reduce(acc);
+  __syncthreads();
+  const double totz = PRE ? block_reduce(accz) : 0.0;
   double* part = partials + (long long)s * gridDim.x;
   SolverState* sst = st + s;
-  if (publish_partial_sys(part, blockIdx.x, gridDim.x, tot, &sst->counter[2])) {
+  if (publish_partial_sys2(part, off2, blockIdx.x, gridDim.x, tot, totz, &sst->counter[2])) {
     const double rr = gather_partials_sys(part, gridDim.x, &sst->counter[2]);
+    const double rz = gather_partials_sys(part + off2, gridDim.x, &sst->counter[2]);
     if (threadIdx.x == 0) {
       const double bb = bb_given != nullptr ? bb_given[s] : rr;
       sst->rr = rr;
+      sst->rz = PRE ? rz : rr;
       sst->bb = bb;
       sst->tol2 = tol * tol * bb;
       sst->alpha = 0.0;
@@ -1051,32 +1146,60 @@ __global__ void k_gamma_table(OpArgs<T> a, GammaCtx g, const int* __restrict__ k
 }
 
 // ------------------------------------------------------------------ mixed precision helpers
-// r32 = (float) r64, x32 = 0, inner CG state begun with tolerance tol relative
-// to the new right-hand side; systems with active[s] == 0 start done.
+// r32 = (float) r64 (PRE: z32 = D r32), x32 = 0, inner CG state begun with tolerance
+// tol relative to the new right-hand side; systems with active[s] == 0 start done.
 // DFIN: r64's elements hold double-float pairs (h, l); the FP32 residual is h
-template <bool DFIN>
-__global__ void __launch_bounds__(kThreads) k_d2f_begin(const double* __restrict__ r64, float* __restrict__ r32,
-                                                        float* __restrict__ x32, long long n,
+template <bool DFIN, int PRE>
+__global__ void __launch_bounds__(kThreads) k_d2f_begin(OpArgs<float> a, const double* __restrict__ r64,
+                                                        float* __restrict__ r32, float* __restrict__ x32,
                                                         SolverState* __restrict__ st, double* __restrict__ partials,
-                                                        double tol, const unsigned char* __restrict__ active) {
+                                                        long long off2, double tol,
+                                                        const unsigned char* __restrict__ active) {
   const int s = blockIdx.y;
+  const long long n = (long long)a.c * a.V;
   const double* r64s = r64 + s * n;
   float* r32s = r32 + s * n;
   float* x32s = x32 + s * n;
-  Acc<float> acc;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const float v = DFIN ? reinterpret_cast<const float2*>(r64s)[i].x : (float)r64s[i];
-    r32s[i] = v;
-    x32s[i] = 0.0f;
-    acc.add(v * v);
-  }
+  const long long pbase = (long long)((a.sys0 + s) / a.sys_per_ms) * a.V;
+  Acc<float> acc, accz;
+  sweep_planes<float>(a.c, a.V, [&](int comp, long long i, auto vec) {
+    constexpr int VEC = decltype(vec)::value;
+    const long long g = comp * a.V + i;
+    float v[VEC], zero[VEC];
+    int ph[VEC];
+    if (PRE) phase_load<VEC>(a.phase + pbase + i, ph);
+    if constexpr (VEC == 4) {
+      const double2 d0 = *reinterpret_cast<const double2*>(r64s + g), d1 = *reinterpret_cast<const double2*>(r64s + g + 2);
+      const double d[4] = {d0.x, d0.y, d1.x, d1.y};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) v[u] = DFIN ? __int_as_float(__double2loint(d[u])) : (float)d[u];
+    } else {
+      v[0] = DFIN ? reinterpret_cast<const float2*>(r64s)[g].x : (float)r64s[g];
+    }
+#pragma unroll
+    for (int u = 0; u < VEC; ++u) {
+      zero[u] = 0.0f;
+      acc.add(v[u] * v[u]);
+      if constexpr (PRE != 0) {
+        const float z = precond<float, PRE>(a, a.dtab, comp, ph[u], pbase + i + u) * v[u];
+        accz.add(z * v[u]);
+        v[u] = z;
+      }
+    }
+    vstore<float, VEC>(r32s + g, v);
+    vstore<float, VEC>(x32s + g, zero);
+  });
   const double tot = block_reduce(acc);
+  __syncthreads();
+  const double totz = PRE ? block_reduce(accz) : 0.0;
   double* part = partials + (long long)s * gridDim.x;
   SolverState* sst = st + s;
-  if (publish_partial_sys(part, blockIdx.x, gridDim.x, tot, &sst->counter[2])) {
+  if (publish_partial_sys2(part, off2, blockIdx.x, gridDim.x, tot, totz, &sst->counter[2])) {
     const double rr = gather_partials_sys(part, gridDim.x, &sst->counter[2]);
+    const double rz = gather_partials_sys(part + off2, gridDim.x, &sst->counter[2]);
     if (threadIdx.x == 0) {
       sst->rr = rr;
+      sst->rz = PRE ? rz : rr;
       sst->bb = rr;
       sst->tol2 = tol * tol * rr;
       sst->alpha = sst->beta = sst->pq = 0.0;
@@ -1085,6 +1208,25 @@ __global__ void __launch_bounds__(kThreads) k_d2f_begin(const double* __restrict
       sst->done = (!active[s] || rr <= sst->tol2) ? 1 : 0;
     }
   }
+}
+
+// Diagonal of the Green operator in space, per component: sum over the full spectrum
+// of the tabulated Gamma_ii (the table carries 1/V); half-spectrum columns other than
+// kx = 0 and nx/2 count twice.  Partial sums per block, summed by k_comp_final.
+__global__ void __launch_bounds__(kThreads) k_gamma_diag(OpArgs<double> a, double* __restrict__ partials) {
+  const int comp = blockIdx.y, c = a.c;
+  const int ncop = ((c * (c + 1) / 2) + 3) & ~3;
+  int coef = 0;
+  for (int i = 0; i < comp; ++i) coef += c - i;
+  const long long nf = (long long)a.nz * a.ny * a.nxh;
+  double acc = 0.0;
+  for (long long f = blockIdx.x * (long long)blockDim.x + threadIdx.x; f < nf; f += (long long)gridDim.x * blockDim.x) {
+    const int kx = (int)(f % a.nxh);
+    const double w = (kx == 0 || 2 * kx == a.nx) ? 1.0 : 2.0;
+    acc += w * a.gtab[gamma_elem<double>((f / a.nxh) * a.ts + kx, coef, ncop)];
+  }
+  acc = block_sum(acc);
+  if (threadIdx.x == 0) partials[(long long)comp * gridDim.x + blockIdx.x] = acc;
 }
 
 __global__ void k_f2d_axpy(double* __restrict__ x64, const float* __restrict__ x32, long long n) {
@@ -1307,17 +1449,24 @@ void launch_rotate_scalar(const T* in, T* out, long long V, int nsys, int d, con
 }
 
 template <typename T>
-void launch_cg_update(T* r, const T* q, long long n, int S, SolverState* st, double* partials, int G, cudaStream_t s) {
-  k_cg_update<T><<<dim3(G, S), kThreads, 0, s>>>(r, q, n, st, partials);
+void launch_cg_update(const OpArgs<T>& a, T* r, const T* q, SolverState* st, double* partials, long long off2, int G,
+                      cudaStream_t s) {
+  const dim3 g(G, a.S);
+  if (a.pre == 0) k_cg_update<T, 0><<<g, kThreads, 0, s>>>(a, r, q, st, partials, off2);
+  else if (a.pre == 1) k_cg_update<T, 1><<<g, kThreads, 0, s>>>(a, r, q, st, partials, off2);
+  else k_cg_update<T, 2><<<g, kThreads, 0, s>>>(a, r, q, st, partials, off2);
 }
 template <typename T>
 void launch_cg_finalize(T* x, const T* p, long long n, int S, const SolverState* st, int G, cudaStream_t s) {
   k_cg_finalize<T><<<dim3(G, S), kThreads, 0, s>>>(x, p, n, st);
 }
 template <typename T>
-void launch_cg_begin(const T* r, long long n, int S, SolverState* st, double* partials, double tol,
+void launch_cg_begin(const OpArgs<T>& a, T* r, SolverState* st, double* partials, long long off2, double tol,
                      const double* bb_given, int G, cudaStream_t s) {
-  k_cg_begin<T><<<dim3(G, S), kThreads, 0, s>>>(r, n, st, partials, tol, bb_given);
+  const dim3 g(G, a.S);
+  if (a.pre == 0) k_cg_begin<T, 0><<<g, kThreads, 0, s>>>(a, r, st, partials, off2, tol, bb_given);
+  else if (a.pre == 1) k_cg_begin<T, 1><<<g, kThreads, 0, s>>>(a, r, st, partials, off2, tol, bb_given);
+  else k_cg_begin<T, 2><<<g, kThreads, 0, s>>>(a, r, st, partials, off2, tol, bb_given);
 }
 template <typename T> void launch_fill_rhs(const OpArgs<T>& a, T* r, T* x, int G, cudaStream_t s) {
   k_fill_rhs<T><<<dim3(G, a.S), kThreads, 0, s>>>(a, r, x);
@@ -1353,10 +1502,20 @@ void launch_gamma_table(const OpArgs<T>& a, int dim, int physics, int green, con
   const int grid = (int)std::min<long long>((nf + 127) / 128, 152LL * 16);
   k_gamma_table<T><<<grid, 128, 0, s>>>(a, g, kofy, kofz);
 }
-void launch_d2f_begin(const double* r64, bool df_pairs, float* r32, float* x32, long long n, int S, SolverState* st,
-                      double* partials, double tol, const unsigned char* active, int G, cudaStream_t s) {
-  if (df_pairs) k_d2f_begin<true><<<dim3(G, S), kThreads, 0, s>>>(r64, r32, x32, n, st, partials, tol, active);
-  else k_d2f_begin<false><<<dim3(G, S), kThreads, 0, s>>>(r64, r32, x32, n, st, partials, tol, active);
+void launch_d2f_begin(const OpArgs<float>& a, const double* r64, bool df_pairs, float* r32, float* x32, SolverState* st,
+                      double* partials, long long off2, double tol, const unsigned char* active, int G,
+                      cudaStream_t s) {
+  const dim3 g(G, a.S);
+#define LSH_D2F(DFIN, PRE) \
+  k_d2f_begin<DFIN, PRE><<<g, kThreads, 0, s>>>(a, r64, r32, x32, st, partials, off2, tol, active)
+  if (a.pre == 0) { if (df_pairs) LSH_D2F(true, 0); else LSH_D2F(false, 0); }
+  else if (a.pre == 1) { if (df_pairs) LSH_D2F(true, 1); else LSH_D2F(false, 1); }
+  else { if (df_pairs) LSH_D2F(true, 2); else LSH_D2F(false, 2); }
+#undef LSH_D2F
+}
+void launch_gamma_diag(const OpArgs<double>& a, double* partials, int nblk, double* out, cudaStream_t s) {
+  k_gamma_diag<<<dim3(nblk, a.c), kThreads, 0, s>>>(a, partials);
+  k_comp_final<<<a.c, kThreads, 0, s>>>(partials, nblk, out);
 }
 void launch_f2d_axpy(double* x64, const float* x32, long long n, cudaStream_t s) {
   const int grid = (int)std::max(1LL, std::min((n + kThreads - 1) / kThreads, 152LL * 16));
@@ -1381,10 +1540,11 @@ void launch_scale_grad(const double* tau_all, const double* W, const unsigned ch
   template void launch_zgamma<T>(const OpArgs<T>&, const LaunchCfg&, const SolverState*, cudaStream_t);            \
   template void launch_xinv<T>(const OpArgs<T>&, const LaunchCfg&, int, const T*, T*, SolverState*, double*,       \
                                cudaStream_t);                                                                      \
-  template void launch_cg_update<T>(T*, const T*, long long, int, SolverState*, double*, int, cudaStream_t);       \
+  template void launch_cg_update<T>(const OpArgs<T>&, T*, const T*, SolverState*, double*, long long, int,         \
+                                    cudaStream_t);                                                                 \
   template void launch_cg_finalize<T>(T*, const T*, long long, int, const SolverState*, int, cudaStream_t);        \
-  template void launch_cg_begin<T>(const T*, long long, int, SolverState*, double*, double, const double*, int,    \
-                                   cudaStream_t);                                                                  \
+  template void launch_cg_begin<T>(const OpArgs<T>&, T*, SolverState*, double*, long long, double, const double*,  \
+                                   int, cudaStream_t);                                                             \
   template void launch_fill_rhs<T>(const OpArgs<T>&, T*, T*, int, cudaStream_t);                                   \
   template void launch_rotate<T>(const T*, T*, long long, int, int, cudaStream_t);                                 \
   template void launch_comp_sums<T>(const T*, int, long long, int, double*, int, double*, cudaStream_t);           \

@@ -164,7 +164,7 @@ __device__ __forceinline__ bool xinv_rows(const OpArgs<float>& a, const float* _
             sst->alpha = 0.0;
             sst->done = 1;
           } else {
-            sst->alpha = sst->rr / sum;
+            sst->alpha = sst->rz / sum;
           }
         } else {
           sst->aux[0] = sum;
@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(TH, TH == 256 ? 2 : 4) k_xinv_reg(OpArgs<float
             sst->alpha = 0.0;
             sst->done = 1;
           } else {
-            sst->alpha = sst->rr / sum;
+            sst->alpha = sst->rz / sum;
           }
         } else {
           sst->aux[0] = sum;

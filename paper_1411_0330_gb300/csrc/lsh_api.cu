@@ -427,7 +427,7 @@ Layout make_layout(const Derived& d) {
                                       (long long)S * d.c * d.nz});
   l.nparts = np;
   l.off_state = take(sizeof(SolverState) * (size_t)(3 * S + d.B));
-  l.off_partials = take(sizeof(double) * (size_t)np);
+  l.off_partials = take(sizeof(double) * 2 * (size_t)np);  // two sums per block where a kernel forms two
   l.off_phase = take((size_t)(d.B * d.V));
   l.off_scale = take(d.has_scale ? sizeof(float) * (size_t)(d.B * d.V) : 0);
   l.off_act = take(256);
@@ -438,8 +438,8 @@ Layout make_layout(const Derived& d) {
   l.off_kofz32 = take(sizeof(int) * d.nz);
   l.off_sums = take(sizeof(double) * (size_t)S * d.c);
   l.off_W = take(sizeof(double) * 64);
-  l.off_tabd = take(sizeof(double) * 2 * 256 * 6);
-  l.off_tabf = take(sizeof(float) * 2 * 256 * 6);
+  l.off_tabd = take(sizeof(double) * 3 * 256 * 6);
+  l.off_tabf = take(sizeof(float) * 3 * 256 * 6);
   l.off_loads_d = take(sizeof(double) * 6 * (size_t)S);
   l.off_loads_f = take(sizeof(float) * 6 * (size_t)S);
   l.off_bb = take(sizeof(double) * (size_t)S);
@@ -630,6 +630,12 @@ void init_prec(lsh_handle* h, PrecBufs<T>& P, const size_t* off_f, size_t off_H,
   a.nphase = d.nphase;
   a.mtab = P.mtab;
   a.modtab = P.modtab;
+  // preconditioner of the CG iterations: the FP32 ones of the mixed solver wherever K is
+  // definite, and FP64 CG with a per-voxel field.  FP64 CG on phase maps is the plain
+  // method the mixed solver is measured against.
+  a.dtab = P.modtab + 256 * 6;
+  a.pre = (d.definite == 0 || (sizeof(T) == 8 && !d.has_scale)) ? 0 : (d.has_scale ? 2 : 1);
+  for (int i = 0; i < 6; ++i) a.gpre[i] = (T)0;
   for (int i = 0; i < 6; ++i) a.ref[i] = (T)(i < d.c ? d.ref_in[i] : 0.0);
   a.loads = P.loads;
   // FP32 truncated operator: computed on the fly in the z pass (no table read)
@@ -874,7 +880,7 @@ template <typename T> void enqueue_cg_iteration(lsh_handle* h, PrecBufs<T>& P, c
   if (timed) cudaEventRecordWithFlags(e[4], s, rf);
   launch_xinv<T>(a, P.L, 1, P.p, P.q, P.st, h->partials, s);
   if (timed) cudaEventRecordWithFlags(e[5], s, rf);
-  launch_cg_update<T>(P.r, P.q, (long long)a.c * a.V, a.S, P.st, h->partials, P.L.ew_per_sys, s);
+  launch_cg_update<T>(a, P.r, P.q, P.st, h->partials, h->lay.nparts, P.L.ew_per_sys, s);
   if (timed) {
     cudaEventRecordWithFlags(e[6], s, rf);
     h->ev_used += 7;
@@ -1194,12 +1200,12 @@ lsh_status solve_wave(lsh_handle* h, const Wave& w, bool warm, const lsh_solve_o
   } else if (d.precision == LSH_FP64) {
     if (!warm) {
       launch_fill_rhs<double>(ad, Pd.r, Pd.x, G, h->stream);
-      launch_cg_begin<double>(Pd.r, n, S, Pd.st, h->partials, tol, h->bbdev, G, h->stream);
+      launch_cg_begin<double>(ad, Pd.r, Pd.st, h->partials, h->lay.nparts, tol, h->bbdev, G, h->stream);
       h->launches += 2;
     } else {
       if ((stt = residual64(h, ad, Pd.x, Pd.r))) return stt;
       for (int s = 0; s < S; ++s) infos[s].applies64 += 1;
-      launch_cg_begin<double>(Pd.r, n, S, Pd.st, h->partials, tol, h->bbdev, G, h->stream);
+      launch_cg_begin<double>(ad, Pd.r, Pd.st, h->partials, h->lay.nparts, tol, h->bbdev, G, h->stream);
       h->launches += 1;
     }
     if ((stt = last_launch())) return stt;
@@ -1263,8 +1269,8 @@ lsh_status solve_wave(lsh_handle* h, const Wave& w, bool warm, const lsh_solve_o
           if (active[s] && bb[s] > 0) worst = std::max(worst, std::sqrt(rr[s] / bb[s]));
         if (worst > 0.0) itol_k = std::min(1e-3, std::max(itol, 0.5 * tol / worst));
       }
-      launch_d2f_begin(Pd.r, rdf, Pf.r, Pf.x, n, S, Pf.st, h->partials, itol_k, h->flags, Pf.L.ew_per_sys,
-                       h->stream);
+      launch_d2f_begin(af, Pd.r, rdf, Pf.r, Pf.x, Pf.st, h->partials, h->lay.nparts, itol_k, h->flags,
+                       Pf.L.ew_per_sys, h->stream);
       h->launches += 1;
       if ((stt = cg_run<float>(h, Pf, af, maxit - total_max, check, graphs, st))) return stt;
       launch_f2d_axpy(Pd.x, Pf.x, n * S, h->stream);
@@ -1449,8 +1455,8 @@ lsh_status lsh_setup(const lsh_problem* prob, void* workspace, size_t bytes, voi
   twiddles<double>(d.nz, tmpd); twd.insert(twd.end(), tmpd.begin(), tmpd.end());
   std::vector<float> twf(twd.size());
   for (size_t i = 0; i < twd.size(); ++i) twf[i] = (float)twd[i];
-  std::vector<double> tabd(2 * 256 * 6, 0.0);
-  std::vector<float> tabf(2 * 256 * 6, 0.0f);
+  std::vector<double> tabd(3 * 256 * 6, 0.0);
+  std::vector<float> tabf(3 * 256 * 6, 0.0f);
   for (int ph = 0; ph < d.nphase; ++ph)
     for (int i = 0; i < d.c; ++i) {
       tabd[ph * d.c + i] = d.m_in[ph * d.c + i];
@@ -1493,6 +1499,32 @@ lsh_status lsh_setup(const lsh_problem* prob, void* workspace, size_t bytes, voi
   if (d.precision == LSH_MIXED)
     launch_gamma_table<float>(h->pf.a, d.dim, d.physics, d.green, d.ref_user, h->kofy32, h->kofz32, st,
                               d.rotated ? d.A0full : nullptr, d.rotated ? d.R : nullptr);
+  if (h->pd.a.pre || (d.precision == LSH_MIXED && h->pf.a.pre)) {
+    // diagonal preconditioner 1 / (|M| + g): g = 0 where Gamma is a projector up to A0
+    // (truncated, finite differences), else the Green operator's diagonal in space
+    double g[6] = {0, 0, 0, 0, 0, 0};
+    if (d.green == LSH_GREEN_FILTERED) {
+      launch_gamma_diag(h->pd.a, h->partials, 152, h->sums, st);
+      SETUP_CK(cudaMemcpyAsync(g, h->sums, sizeof(double) * d.c, cudaMemcpyDeviceToHost, st));
+      SETUP_CK(cudaStreamSynchronize(st));
+    }
+    std::vector<double> dd(256 * 6, 1.0);
+    std::vector<float> df(256 * 6, 1.0f);
+    for (int ph = 0; ph < d.nphase; ++ph)
+      for (int i = 0; i < d.c; ++i)
+        if (d.act[ph] && !d.has_scale) dd[ph * d.c + i] = 1.0 / (std::fabs(d.m_in[ph * d.c + i]) + g[i]);
+    for (size_t i = 0; i < dd.size(); ++i) df[i] = (float)dd[i];
+    for (int i = 0; i < 6; ++i) {
+      h->pd.a.gpre[i] = g[i];
+      h->pf.a.gpre[i] = (float)g[i];
+    }
+    SETUP_CK(cudaMemcpyAsync(const_cast<double*>(h->pd.a.dtab), dd.data(), sizeof(double) * dd.size(),
+                             cudaMemcpyHostToDevice, st));
+    if (d.precision == LSH_MIXED)
+      SETUP_CK(cudaMemcpyAsync(const_cast<float*>(h->pf.a.dtab), df.data(), sizeof(float) * df.size(),
+                               cudaMemcpyHostToDevice, st));
+    SETUP_CK(cudaStreamSynchronize(st));
+  }
   if (l.df) {
     const long long nf = (long long)d.nz * d.ny * d.ts, ncop = (d.ncoef + 3) & ~3;
     if (d.plane && !(reg_len(d.ny) && reg_len(d.nz))) {
@@ -1763,7 +1795,7 @@ lsh_status lsh_autotune(lsh_handle* h, lsh_tune_report* rep) {
     for (auto& f : fake) {
       f = SolverState{};
       f.iter = 1;
-      f.rr = 1.0;
+      f.rr = f.rz = 1.0;
     }
     LSH_CK(cudaMemcpyAsync(P.st, fake.data(), sizeof(SolverState) * d.Smax, cudaMemcpyHostToDevice, s));
     // the separate x and y passes need natural y order for the FP32 table on

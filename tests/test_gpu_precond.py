@@ -1,0 +1,72 @@
+"""The diagonal preconditioner of the CG iterations (GPU) against the oracle's solutions, over the forms
+that reach it: every Green operator, phase tables with voxels outside I0, operators of either sign, per-voxel
+scale and fraction fields, plane and separate passes, lengths whose planes are no whole number of vectors."""
+import numpy as np
+import pytest
+
+import oracle
+from helpers import k_mu
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+if torch.cuda.is_available():
+    from paper_1411_0330_gb300 import lsh
+
+KM, MUM = k_mu(1.0, 0.3)
+KI, MUI = k_mu(10.0, 0.2)
+
+
+def rel(a, b):
+    return np.abs(np.asarray(a) - np.asarray(b)).max() / np.abs(np.asarray(b)).max()
+
+
+# C* tolerances: 1e-8 mixed, 1e-10 FP64 (the accuracy the solvers are held to), solves at 1e-11
+@pytest.mark.parametrize("shape", [(5, 7, 9), (6, 10, 14), (16, 16, 16), (4, 32, 32)])
+@pytest.mark.parametrize("green", [0, 1])
+def test_elastic_phases_with_voxels_outside_I0(shape, green):
+    rng = np.random.default_rng(sum(shape) + green)
+    ph = rng.integers(0, 3, shape).astype(np.uint8)
+    ref = np.array([0.5 * KM, 0.5 * MUM])
+    mods = np.array([[KM, MUM], list(ref), [KI, MUI]])  # the middle phase is the reference: outside I0
+    h = lsh.Handle(torch.from_numpy(ph).cuda(), mods, physics=lsh.ELASTIC, green=green, precision=lsh.MIXED, ref=ref)
+    A, infos = h.effective(tol=1e-11)
+    Ao, _ = oracle.effective(oracle.Problem(ph, mods, physics=1, green=green, ref=ref), tol=1e-13)
+    assert rel(A, Ao) < 1e-8, rel(A, Ao)
+    assert all(i["status"] == 0 and i["relres"] <= 1e-11 for i in infos)
+
+
+@pytest.mark.parametrize("shape", [(15, 9), (32, 20), (7, 9, 5), (16, 16, 16)])
+@pytest.mark.parametrize("green", [0, 1, 2])
+@pytest.mark.parametrize("above", [False, True])
+def test_scalar_either_sign(shape, green, above):
+    """Reference below or above every phase (K positive or negative definite)."""
+    d = len(shape)
+    rng = np.random.default_rng(sum(shape) + green)
+    ph = rng.integers(0, 3, shape).astype(np.uint8)
+    mods = np.array([np.diag(rng.uniform(1.0, 6.0, d)) for _ in range(3)])
+    ref = (9.0 if above else 0.5) * np.eye(d)
+    h = lsh.Handle(torch.from_numpy(ph).cuda(), mods, green=green, precision=lsh.MIXED, ref=ref)
+    A, infos = h.effective(tol=1e-11)
+    Ao, _ = oracle.effective(oracle.Problem(ph, mods, green=green, ref=ref), tol=1e-13)
+    assert rel(A, Ao) < 1e-8, rel(A, Ao)
+    assert all(i["status"] == 0 and i["relres"] <= 1e-11 for i in infos)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("kind", ["scale", "fraction"])
+@pytest.mark.parametrize("shape,green", [((5, 7, 9), 0), ((6, 10, 12), 1), ((16, 16, 16), 1)])
+def test_elastic_voxel_fields(shape, green, kind, precision):
+    rng = np.random.default_rng(sum(shape) + green)
+    ph = (rng.random(shape) < 0.3).astype(np.uint8) if kind == "scale" else np.zeros(shape, np.uint8)
+    f = rng.uniform(0.5, 2.0, shape) if kind == "scale" else rng.uniform(0.0, 1.0, shape)
+    f = f.astype(np.float32)
+    mods = np.array([[KM, MUM], [KI, MUI]])
+    ref = np.array([0.25 * KM, 0.25 * MUM])
+    kw = {kind: torch.from_numpy(f).cuda()}
+    h = lsh.Handle(torch.from_numpy(ph).cuda(), mods, physics=lsh.ELASTIC, green=green, precision=precision, ref=ref,
+                   **kw)
+    A, infos = h.effective(tol=1e-11)
+    ok = {"scale" if kind == "scale" else "frac": f.astype(np.float64)}
+    Ao, _ = oracle.effective(oracle.Problem(ph, mods, physics=1, green=green, ref=ref, **ok), tol=1e-13)
+    assert rel(A, Ao) < (1e-8 if precision else 1e-10), rel(A, Ao)
+    assert all(i["status"] == 0 and i["relres"] <= 1e-11 for i in infos)
