@@ -131,6 +131,8 @@ def pass_traffic(kind, V, c, nx, nxh, ncoef, b):
         return cV * (2 * b * half + 2 * b + 1)
     if kind == "cg_update":      # r, q in; r out
         return cV * 3 * b
+    if kind == "x_inverse_update":  # the inverse pass that updates z itself: spectrum, p, z in; z out; phase byte
+        return cV * (2 * b * half + 3 * b + 1)
     raise KeyError(kind)
 
 
@@ -368,6 +370,13 @@ def batch_config(meta):
                   "(> 129 MB), no flush needed"}
 
 
+def pass_kind(prof, k):
+    """The byte count that applies to pass k of a profile: where the CG update did not run as a
+    kernel of its own, the inverse pass did it."""
+    fused = k == "x_inverse_local" and not prof["pass_launches"]["cg_update"]
+    return "x_inverse_update" if fused else k
+
+
 def batch_pass_bytes(k, n, filtered=True):
     """Algorithmic FP32 bytes of pass k per live system-iteration on an n^3 grid (6
     components), and the Gamma-table bytes read once per launch (filtered operator)."""
@@ -448,7 +457,7 @@ def run_batch(args, rank, world, local):
         pass did not run: the plane passes do the y transforms inside the x passes)."""
         if not p["pass_launches"][k]:
             return 0.0
-        per_sys, table = batch_pass_bytes(k, n)
+        per_sys, table = batch_pass_bytes(pass_kind(p, k), n)
         return per_sys * p["timed_sys_iters"] + table * p["pass_launches"][k]
 
     tot_b = {k: sum(bytes_of(p, n, k) for p, n in zip(prof_mx, grid_of)) for k in lsh.PASS_NAMES}
@@ -582,7 +591,7 @@ def run_contrast256(args):
                 for k in lsh.PASS_NAMES:
                     if not pf["pass_launches"][k]:
                         continue
-                    per_sys, table = batch_pass_bytes(k, n)
+                    per_sys, table = batch_pass_bytes(pass_kind(pf, k), n)
                     byts = per_sys * pf["timed_sys_iters"] + table * pf["pass_launches"][k]
                     gbs = byts / (pf["pass_ms"][k] / 1e3) / 1e9
                     passes[k] = {"ms_per_launch": pf["pass_ms"][k] / pf["pass_launches"][k], "gbs": gbs,
@@ -963,7 +972,7 @@ def run_spheres128(args, rank, world, local):
     def pass_bytes(k, filtered):
         """Algorithmic bytes of one launch over the 6 load systems; the Gamma table
         (filtered operator only; the truncated one is computed in the kernel) counts once."""
-        b = 6 * pass_traffic(k, V, 6, N, nxh, 21 if filtered else 0, 4)
+        b = 6 * pass_traffic(pass_kind(prof_mx[0], k), V, 6, N, nxh, 21 if filtered else 0, 4)
         if k == "z_gamma" and filtered:
             b -= 5 * V * 21 * 4 * nxh / N
         return b

@@ -171,12 +171,14 @@ typedef struct lsh_tune_report {
                      brought in and written back by TMA, double-buffered, with the
                      FFT and Gamma exchanges in the tile's buffer; 11 the same on
                      the plan N = R1 x 4 with the 4-point FFT level and Gamma in one
-                     register phase (z lengths up to 128)                           */
+                     register phase (z lengths up to 128), which also leaves
+                     (p, Gamma p): the CG update then runs in the inverse pass       */
   float xf_ms[2]; /* measured time of one launch per candidate (-1: not available)   */
   float x_ms[4];
   float y_ms[2];
   float z_ms[10];
-  float xy_ms[2]; /* one CG iteration's passes summed: separate x/y passes, plane passes */
+  float xy_ms[2]; /* one CG iteration's passes without the CG update summed: separate
+                     x/y passes, plane passes (less the update they fuse)            */
   float zp_ms[7]; /* z pass on the ky-major spectrum, variants 0, 6, 8, 9, 7, 10, 11  */
 } lsh_tune_report;
 
@@ -296,7 +298,9 @@ lsh_status lsh_apply_noalloc(const lsh_problem *prob, const double *x, double *y
  * iteration measured with CUDA events recorded on the handle's stream
  * between consecutive launches.  Pass kinds: 0 x-forward (with the CG
  * prologue), 1 y-forward, 2 z-forward + Gamma^h product + z-inverse,
- * 3 y-inverse, 4 x-inverse (with local term and (p, Kp)), 5 CG update. */
+ * 3 y-inverse, 4 x-inverse (with local term and (p, Kp)), 5 CG update.  The
+ * plane passes with z variant 11 update the residual in the inverse pass: kind
+ * 4 then covers that (with the scalars of the iteration) and kind 5 does not run. */
 typedef struct lsh_profile {
   long long launches;          /* kernels launched since the last reset            */
   long long timed_iters;       /* CG iterations covered by pass_ms                 */

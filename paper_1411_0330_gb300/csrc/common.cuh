@@ -46,7 +46,8 @@ struct SolverState {
   double alpha;     // alpha of the last completed iteration (0 after breakdown)
   double beta;      // beta_{k-1}
   double pq;        // (p_k, K p_k)
-  double aux[4];    // extra reduction results (component sums, ...)
+  double aux[4];    // extra reduction results: residual norm; in a CG solve of the fused plane
+                    // schedule (p, M p), (z, M z), (z, M p) (kernels_plane.cu)
   int iter;         // completed CG iterations
   int done;         // nonzero: converged or failed, later kernels return at once
   int status;       // lsh_status-compatible code set on device (0, breakdown)

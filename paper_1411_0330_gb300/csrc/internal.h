@@ -89,6 +89,7 @@ template <typename T> struct OpArgs {
   int plane;
   int tlay;
   C2<T>* nq;
+  int fuse;  // plane passes with z variant 11: the CG update runs in the inverse pass
   int l2pf;  // plane passes, input planes requested into L2 at a block's start: bit 0 the
              // forward pass's x, r, p; bit 1 the inverse pass's p and phase planes
 };
@@ -165,7 +166,9 @@ bool encode_y_map(CUtensorMap* out, void* H, int hs, int ny, long long planes);
 bool launch_zgamma_tma(const OpArgs<float>& a, int var, const SolverState* st, cudaStream_t s);
 bool tma_z_variant_fits(const OpArgs<float>& a, int var);
 bool launch_zgamma_regp(const OpArgs<float>& a, const SolverState* st, cudaStream_t s);
-bool launch_zgamma_pipe(const OpArgs<float>& a, bool fused, const SolverState* st, cudaStream_t s);
+bool launch_zgamma_pipe(const OpArgs<float>& a, bool fused, const SolverState* st, cudaStream_t s,
+                        double* partials = nullptr);
+int zdot_count(const OpArgs<float>& a);
 bool encode_zpipe_maps(CUtensorMap* th, CUtensorMap* tq, void* H, void* NQ, int hs, int ny, int nz, int c,
                        long long nsys);
 void zpipe_prepare();
@@ -195,6 +198,10 @@ bool launch_xyfwd(const OpArgs<float>& a, int mode, const float* in, float* x, c
                   const SolverState* st, cudaStream_t s);
 bool launch_xyinv(const OpArgs<float>& a, int mode, const float* xin, float* out, SolverState* st, double* partials,
                   cudaStream_t s);
+// CG iteration with the update of z fused into the inverse pass (kernels_plane.cu)
+void launch_cg_alpha(SolverState* st, const double* partials, int nb, int S, cudaStream_t s);
+bool launch_xyinv_update(const OpArgs<float>& a, const float* p, float* z, SolverState* st, double* partials,
+                         long long off, cudaStream_t s);
 void plane_prepare();
 
 }  // namespace lsh

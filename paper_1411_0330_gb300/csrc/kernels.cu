@@ -1161,13 +1161,14 @@ __global__ void __launch_bounds__(kThreads) k_d2f_begin(OpArgs<float> a, const d
   float* r32s = r32 + s * n;
   float* x32s = x32 + s * n;
   const long long pbase = (long long)((a.sys0 + s) / a.sys_per_ms) * a.V;
-  Acc<float> acc, accz;
+  Acc<float> acc, accz, accm;
+  const bool zmz = a.plane && a.fuse;  // (z, M z) for the fused plane schedule
   sweep_planes<float>(a.c, a.V, [&](int comp, long long i, auto vec) {
     constexpr int VEC = decltype(vec)::value;
     const long long g = comp * a.V + i;
     float v[VEC], zero[VEC];
     int ph[VEC];
-    if (PRE) phase_load<VEC>(a.phase + pbase + i, ph);
+    phase_load<VEC>(a.phase + pbase + i, ph);
     if constexpr (VEC == 4) {
       const double2 d0 = *reinterpret_cast<const double2*>(r64s + g), d1 = *reinterpret_cast<const double2*>(r64s + g + 2);
       const double d[4] = {d0.x, d0.y, d1.x, d1.y};
@@ -1185,6 +1186,15 @@ __global__ void __launch_bounds__(kThreads) k_d2f_begin(OpArgs<float> a, const d
         accz.add(z * v[u]);
         v[u] = z;
       }
+      if (zmz) {
+        int active;
+        float m = local_coef<float>(a, pbase + i + u, comp, &active);
+        if (a.frac) {
+          const float f = a.scale[pbase + i + u];
+          m = f * a.mtab[a.c + comp] + (1.f - f) * a.mtab[comp];
+        }
+        accm.add(m * v[u] * v[u]);
+      }
     }
     vstore<float, VEC>(r32s + g, v);
     vstore<float, VEC>(x32s + g, zero);
@@ -1192,14 +1202,20 @@ __global__ void __launch_bounds__(kThreads) k_d2f_begin(OpArgs<float> a, const d
   const double tot = block_reduce(acc);
   __syncthreads();
   const double totz = PRE ? block_reduce(accz) : 0.0;
+  __syncthreads();
+  const double totm = zmz ? block_reduce(accm) : 0.0;
   double* part = partials + (long long)s * gridDim.x;
   SolverState* sst = st + s;
+  if (threadIdx.x == 0) part[2 * off2 + blockIdx.x] = totm;
   if (publish_partial_sys2(part, off2, blockIdx.x, gridDim.x, tot, totz, &sst->counter[2])) {
     const double rr = gather_partials_sys(part, gridDim.x, &sst->counter[2]);
     const double rz = gather_partials_sys(part + off2, gridDim.x, &sst->counter[2]);
+    const double zm = gather_partials_sys(part + 2 * off2, gridDim.x, &sst->counter[2]);
     if (threadIdx.x == 0) {
       sst->rr = rr;
       sst->rz = PRE ? rz : rr;
+      sst->aux[0] = sst->aux[2] = 0.0;
+      sst->aux[1] = zm;
       sst->bb = rr;
       sst->tol2 = tol * tol * rr;
       sst->alpha = sst->beta = sst->pq = 0.0;

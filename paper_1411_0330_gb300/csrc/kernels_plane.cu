@@ -370,24 +370,32 @@ __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyfwd(Op
 
 // MODE 0: out = P (M xin + g).  MODE 4 (CG): q = P (M p + g) and this block's
 // part of (p, q) in partials[s * c nz + block of the system].
+// MODE 5 (CG, alpha known before this pass): q is not stored, z -= alpha D q is formed
+// here (z = D r in `out`, D the preconditioner, 1 without one) and this block's parts of
+// (r, r), (r, z), (z, M z), (z, M p) go to partials + {0, 1, 2, 3} off; k_cg_beta sums
+// them.  Against MODE 4 and the CG update kernel the q field is neither written nor read
+// and r is read where p and the phases already are: 12.5 instead of 14.25 field passes
+// per iteration.
 template <int N, int MODE>
 __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyinv(OpArgs<float> a, const float* __restrict__ xin,
                                                            float* __restrict__ out, const SolverState* __restrict__ st,
-                                                           double* __restrict__ partials) {
+                                                           double* __restrict__ partials, long long off) {
   typedef PlaneCfg<N> PC;
   constexpr int RS = PC::RS, TH = PC::TH, NV = PC::NV;
   const int cnz = a.c * a.nz;
   const int s = blockIdx.x / cnz;
   const int blk = blockIdx.x - s * cnz;
   const int comp = blk / a.nz, z = blk - comp * a.nz;
-  if (MODE == 4 && st[s].done) return;
+  if (MODE >= 4 && st[s].done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* PL = reinterpret_cast<float2*>(smem_raw);
   float2* tw = PL + N * RS;
   float* PR = reinterpret_cast<float*>(PL);
-  // per-phase tables after the plane (sized by the launch: nphase * (4 c + 1) bytes)
+  // this component's per-phase values after the plane (sized by the launch): M (or the
+  // modulus with a scale field), D, activity
   float* mloc = reinterpret_cast<float*>(tw + N);
-  unsigned char* aloc = reinterpret_cast<unsigned char*>(mloc + a.nphase * a.c);
+  float* dloc = mloc + a.nphase;
+  unsigned char* aloc = reinterpret_cast<unsigned char*>(dloc + a.nphase);
   __shared__ __align__(8) uint64_t bar;
   const long long slab = (long long)(s * a.c + comp) * N;
   if (threadIdx.x == 0) {
@@ -399,15 +407,18 @@ __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyinv(Op
   for (int ky = threadIdx.x; ky < N; ky += TH)
     bulk_load_1d(PL + ky * RS, a.H + ((slab + ky) * a.nz + z) * a.hs, (uint32_t)(sizeof(float2) * RS), &bar);
   for (int u = threadIdx.x; u < N; u += TH) tw[u] = a.twx[u];
-  const int ntab = a.nphase * a.c;
-  for (int u = threadIdx.x; u < ntab; u += TH) mloc[u] = (a.scale && !a.frac) ? a.modtab[u] : a.mtab[u];
-  for (int u = threadIdx.x; u < a.nphase; u += TH) aloc[u] = a.act[u];
+  for (int u = threadIdx.x; u < a.nphase; u += TH) {
+    mloc[u] = (a.scale && !a.frac) ? a.modtab[u * a.c + comp] : a.mtab[u * a.c + comp];
+    dloc[u] = MODE == 5 && a.pre == 1 ? a.dtab[u * a.c + comp] : 1.f;
+    aloc[u] = a.act[u];
+  }
   // the epilogue's p plane and phase plane go to L2 while the transforms run
   const long long plane = (long long)blockIdx.x * N * N;
   const long long pbase = (long long)((a.sys0 + s) / a.sys_per_ms) * a.V + (long long)z * N * N;
-  if ((a.l2pf & 2) && threadIdx.x < 9) {
+  if ((a.l2pf & 2) && threadIdx.x < (MODE == 5 ? 17 : 9)) {
     constexpr uint32_t PB = (uint32_t)(sizeof(float) * N * N);
     if (threadIdx.x < 8) bulk_prefetch_l2(reinterpret_cast<const char*>(xin + plane) + threadIdx.x * (PB / 8), PB / 8);
+    else if (threadIdx.x > 8) bulk_prefetch_l2(reinterpret_cast<const char*>(out + plane) + (threadIdx.x - 9) * (PB / 8), PB / 8);
     else if ((pbase & 15) == 0) bulk_prefetch_l2(a.phase + pbase, (uint32_t)(N * N));
   }
   float2 nqv = make_float2(0.f, 0.f);
@@ -426,30 +437,35 @@ __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyinv(Op
   // the epilogue's p and phase loads go out in batches of B groups of four
   // voxels, each batch in flight while the previous one is worked on; two
   // register sets take the batches in turn (no copies between them)
-  constexpr int B = PC::IT % 2 == 0 ? 2 : 1;
-  float4 xb0[B], xb1[B];
+  constexpr int B = PC::IT % 2 == 0 && MODE != 5 ? 2 : 1;
+  constexpr int ZB = MODE == 5 ? B : 1;
+  float4 xb0[B], xb1[B], zb0[ZB], zb1[ZB];
   uchar4 hb0[B], hb1[B];
-  auto load_batch = [&](int it0, float4* xb, uchar4* hb) {
+  auto load_batch = [&](int it0, float4* xb, uchar4* hb, float4* zb) {
 #pragma unroll
     for (int b = 0; b < B; ++b) {
       const int idx = threadIdx.x + (it0 + b) * TH;
       const int row = idx / NV, xx = (idx - row * NV) * 4;
       xb[b] = *reinterpret_cast<const float4*>(xin + plane + (long long)row * N + xx);
       hb[b] = *reinterpret_cast<const uchar4*>(a.phase + pbase + (long long)row * N + xx);
+      if (MODE == 5) zb[b] = *reinterpret_cast<const float4*>(out + plane + (long long)row * N + xx);
     }
   };
   plane_x_inv<N>(PL, tw);
-  load_batch(0, xb0, hb0);
+  load_batch(0, xb0, hb0, zb0);
   __syncthreads();
-  Acc<float> acc;
+  Acc<float> acc, accz, accm, accp;
+  const float al = MODE == 5 ? (float)st[s].alpha : 0.f;
   // two phases without a voxel field (the common case): both phases' M and
   // activity in registers, selected per voxel instead of read from the tables;
   // both active (A0 differs from both phases): no projection to apply
   const bool two = a.nphase <= 2 && !a.scale;
-  const float m0 = mloc[comp], m1 = a.nphase > 1 ? mloc[a.c + comp] : m0;
+  const float m0 = mloc[0], m1 = a.nphase > 1 ? mloc[1] : m0;
+  const float d0 = dloc[0], d1 = a.nphase > 1 ? dloc[1] : d0;
+  const float e0 = 1.f / d0, e1 = 1.f / d1;
   const bool act0 = aloc[0] != 0, act1 = a.nphase > 1 ? aloc[1] != 0 : act0;
   const bool both = two && act0 && act1;
-  auto work = [&](int it0, const float4* xc, const uchar4* hc) {
+  auto work = [&](int it0, const float4* xc, const uchar4* hc, const float4* zc) {
 #pragma unroll
     for (int b = 0; b < B; ++b) {
       const int idx = threadIdx.x + (it0 + b) * TH;
@@ -461,6 +477,49 @@ __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyinv(Op
       const unsigned char ph[4] = {hc[b].x, hc[b].y, hc[b].z, hc[b].w};
       const float gv[4] = {g4.x, g4.y, g4.z, g4.w};
       float ov[4];
+      if constexpr (MODE == 5) {
+        float z[4] = {zc[b].x, zc[b].y, zc[b].z, zc[b].w};
+        float srr = 0.f, srz = 0.f, szm = 0.f, spm = 0.f;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          float m, d, e;
+          bool active = true;
+          if (two) {
+            const bool p1 = ph[u] != 0;
+            m = p1 ? m1 : m0;
+            d = p1 ? d1 : d0;
+            e = p1 ? e1 : e0;
+            if (!both) active = p1 ? act1 : act0;
+          } else {
+            active = aloc[ph[u]] != 0;
+            m = mloc[ph[u]];
+            d = dloc[ph[u]];
+            if (a.scale) {
+              const float f = a.scale[vox + u];
+              if (a.frac) {
+                m = f * mloc[1] + (1.f - f) * mloc[0];  // Eq. (def_ah)
+              } else {
+                m = 1.f / (f * m - a.ref[comp]);
+              }
+              if (a.pre) d = 1.f / (fabsf(m) + a.gpre[comp]);
+            }
+            e = 1.f / d;
+          }
+          const float q = active ? fmaf(m, xq[u], gv[u]) : 0.f;
+          z[u] = fmaf(-al, d * q, z[u]);
+          const float r = z[u] * e, zm = z[u] * m;
+          srr = fmaf(r, r, srr);
+          srz = fmaf(r, z[u], srz);
+          szm = fmaf(zm, z[u], szm);
+          spm = fmaf(zm, xq[u], spm);
+        }
+        acc.add(srr);
+        accz.add(srz);
+        accm.add(szm);
+        accp.add(spm);
+        *reinterpret_cast<float4*>(out + g) = make_float4(z[0], z[1], z[2], z[3]);
+        continue;
+      }
       if (both) {
 #pragma unroll
         for (int u = 0; u < 4; ++u) ov[u] = fmaf(ph[u] != 0 ? m1 : m0, xq[u], gv[u]);
@@ -475,10 +534,10 @@ __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyinv(Op
         for (int u = 0; u < 4; ++u) {
           const int pp = ph[u];
           const bool active = aloc[pp] != 0;
-          float m = mloc[pp * a.c + comp];
+          float m = mloc[pp];
           if (a.scale) {
             const float f = a.scale[vox + u];
-            m = a.frac ? f * mloc[a.c + comp] + (1.f - f) * mloc[comp]  // Eq. (def_ah)
+            m = a.frac ? f * mloc[1] + (1.f - f) * mloc[0]  // Eq. (def_ah)
                        : 1.f / (f * m - a.ref[comp]);
           }
           ov[u] = active ? m * xq[u] + gv[u] : 0.f;
@@ -491,11 +550,23 @@ __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyinv(Op
   };
 #pragma unroll 1
   for (int it0 = 0; it0 < PC::IT; it0 += 2 * B) {
-    if (it0 + B < PC::IT) load_batch(it0 + B, xb1, hb1);
-    work(it0, xb0, hb0);
+    if (it0 + B < PC::IT) load_batch(it0 + B, xb1, hb1, zb1);
+    work(it0, xb0, hb0, zb0);
     if (it0 + B >= PC::IT) break;
-    if (it0 + 2 * B < PC::IT) load_batch(it0 + 2 * B, xb0, hb0);
-    work(it0 + B, xb1, hb1);
+    if (it0 + 2 * B < PC::IT) load_batch(it0 + 2 * B, xb0, hb0, zb0);
+    work(it0 + B, xb1, hb1, zb1);
+  }
+  if constexpr (MODE == 5) {
+    double* part = partials + (long long)s * cnz + blk;
+    auto store = [&](const Acc<float>& v, long long at) {
+      const double tot = block_reduce(v);
+      if (threadIdx.x == 0) part[at] = tot;
+      __syncthreads();
+    };
+    store(acc, 0);
+    store(accz, off);
+    store(accm, 2 * off);
+    store(accp, 3 * off);
   }
   if (MODE == 4) {
     const double tot = block_reduce(acc);
@@ -503,20 +574,84 @@ __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyinv(Op
   }
 }
 
+// Scalars of a CG iteration whose inverse pass updates z (MODE 5).  One block per
+// system; partials summed in block order.
+//
+// alpha = (r, z) / (p, K p) before the inverse pass: (p, Gamma p) from the z pass's
+// tiles, (p, M p) from its recurrence under p = z + beta p_old,
+//   (p, M p) = (z, M z) + 2 beta (z, M p_old) + beta^2 (p_old, M p_old),
+// whose sums the previous inverse pass (at the start, the start kernel) left in aux.
+__global__ void __launch_bounds__(256) k_cg_alpha(SolverState* __restrict__ st, const double* __restrict__ partials,
+                                                  int nb) {
+  const int s = blockIdx.x;
+  SolverState* sst = st + s;
+  if (sst->done) return;
+  const double* part = partials + (long long)s * nb;
+  double v = 0.0;
+  for (int i = threadIdx.x; i < nb; i += blockDim.x) v += part[i];
+  const double sum = block_sum(v);
+  if (threadIdx.x == 0) {
+    const double b = sst->beta;
+    const double pmp = sst->iter == 0 ? sst->aux[1] : sst->aux[1] + 2.0 * b * sst->aux[2] + b * b * sst->aux[0];
+    const double pq = pmp + sum;
+    sst->aux[0] = pmp;
+    sst->pq = pq;
+    if (!(fabs(pq) > 0.0) || !isfinite(pq) || !isfinite(sst->rr)) {
+      sst->status = 5;  // LSH_ERR_BREAKDOWN
+      sst->alpha = 0.0;
+      sst->done = 1;
+    } else {
+      sst->alpha = sst->rz / pq;
+    }
+  }
+}
+
+// beta, (r, r), the sums of the next (p, M p), convergence.
+__global__ void __launch_bounds__(256) k_cg_beta(SolverState* __restrict__ st, const double* __restrict__ partials,
+                                                 long long off, int nb) {
+  const int s = blockIdx.x;
+  SolverState* sst = st + s;
+  if (sst->done) return;
+  double v[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int i = threadIdx.x; i < nb; i += blockDim.x)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] += partials[k * off + (long long)s * nb + i];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    v[k] = block_sum(v[k]);
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    sst->beta = v[1] / sst->rz;
+    sst->rr = v[0];
+    sst->rz = v[1];
+    sst->aux[1] = v[2];
+    sst->aux[2] = v[3];
+    sst->iter += 1;
+    if (!isfinite(v[0])) {
+      sst->status = 5;
+      sst->done = 1;
+    } else if (v[0] <= sst->tol2) {
+      sst->done = 1;
+    }
+  }
+}
+
 namespace {
 
 // dynamic shared memory of the inverse kernel: the plane, the twiddles and the phase tables
 template <int N> size_t plane_inv_smem(const OpArgs<float>& a) {
-  return PlaneCfg<N>::SMEM + (((size_t)a.nphase * (4 * a.c + 1) + 15) & ~(size_t)15);
+  return PlaneCfg<N>::SMEM + (((size_t)a.nphase * 9 + 15) & ~(size_t)15);
 }
 
 template <int N> void plane_attrs() {
   const int sm = (int)PlaneCfg<N>::SMEM;
-  const int smi = (int)(PlaneCfg<N>::SMEM + 256 * 25);  // up to 256 phases of 6 components
+  const int smi = (int)(PlaneCfg<N>::SMEM + 256 * 9);  // up to 256 phases
   cudaFuncSetAttribute(k_xyfwd<N, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
   cudaFuncSetAttribute(k_xyfwd<N, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
   cudaFuncSetAttribute(k_xyinv<N, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, smi);
   cudaFuncSetAttribute(k_xyinv<N, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smi);
+  cudaFuncSetAttribute(k_xyinv<N, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize, smi);
 }
 
 template <int N> bool plane_fwd_n(const OpArgs<float>& a, int mode, const float* in, float* x, const float* r,
@@ -530,16 +665,19 @@ template <int N> bool plane_fwd_n(const OpArgs<float>& a, int mode, const float*
 }
 
 template <int N> bool plane_inv_n(const OpArgs<float>& a, int mode, const float* xin, float* out, SolverState* st,
-                                  double* partials, cudaStream_t s) {
+                                  double* partials, long long off, cudaStream_t s) {
   typedef PlaneCfg<N> PC;
   if (a.hs < PC::RS || (a.hs & 1) != 0) return false;
   const unsigned grid = (unsigned)((long long)a.S * a.c * a.nz);
   const size_t smem = plane_inv_smem<N>(a);
   if (mode == 0) {
-    k_xyinv<N, 0><<<grid, PC::TH, smem, s>>>(a, xin, out, st, partials);
-  } else {
-    k_xyinv<N, 4><<<grid, PC::TH, smem, s>>>(a, xin, out, st, partials);
+    k_xyinv<N, 0><<<grid, PC::TH, smem, s>>>(a, xin, out, st, partials, 0);
+  } else if (mode == 1) {
+    k_xyinv<N, 4><<<grid, PC::TH, smem, s>>>(a, xin, out, st, partials, 0);
     launch_dot_finalize(st, partials, a.c * a.nz, a.S, s);
+  } else {
+    k_xyinv<N, 5><<<grid, PC::TH, smem, s>>>(a, xin, out, st, partials, off);
+    k_cg_beta<<<a.S, 256, 0, s>>>(st, partials, off, a.c * a.nz);
   }
   return true;
 }
@@ -562,18 +700,34 @@ bool launch_xyfwd(const OpArgs<float>& a, int mode, const float* in, float* x, c
   }
 }
 
-bool launch_xyinv(const OpArgs<float>& a, int mode, const float* xin, float* out, SolverState* st, double* partials,
-                  cudaStream_t s) {
-  if (a.nx != a.ny || mode < 0 || mode > 1) return false;
+namespace {
+bool xyinv_n(const OpArgs<float>& a, int mode, const float* xin, float* out, SolverState* st, double* partials,
+             long long off, cudaStream_t s) {
+  if (a.nx != a.ny) return false;
   switch (a.nx) {
-    case 16: return plane_inv_n<16>(a, mode, xin, out, st, partials, s);
-    case 32: return plane_inv_n<32>(a, mode, xin, out, st, partials, s);
-    case 48: return plane_inv_n<48>(a, mode, xin, out, st, partials, s);
-    case 64: return plane_inv_n<64>(a, mode, xin, out, st, partials, s);
-    case 96: return plane_inv_n<96>(a, mode, xin, out, st, partials, s);
-    case 128: return plane_inv_n<128>(a, mode, xin, out, st, partials, s);
+    case 16: return plane_inv_n<16>(a, mode, xin, out, st, partials, off, s);
+    case 32: return plane_inv_n<32>(a, mode, xin, out, st, partials, off, s);
+    case 48: return plane_inv_n<48>(a, mode, xin, out, st, partials, off, s);
+    case 64: return plane_inv_n<64>(a, mode, xin, out, st, partials, off, s);
+    case 96: return plane_inv_n<96>(a, mode, xin, out, st, partials, off, s);
+    case 128: return plane_inv_n<128>(a, mode, xin, out, st, partials, off, s);
     default: return false;
   }
+}
+}  // namespace
+
+bool launch_xyinv(const OpArgs<float>& a, int mode, const float* xin, float* out, SolverState* st, double* partials,
+                  cudaStream_t s) {
+  return mode >= 0 && mode <= 1 && xyinv_n(a, mode, xin, out, st, partials, 0, s);
+}
+
+bool launch_xyinv_update(const OpArgs<float>& a, const float* p, float* z, SolverState* st, double* partials,
+                         long long off, cudaStream_t s) {
+  return xyinv_n(a, 2, p, z, st, partials, off, s);
+}
+
+void launch_cg_alpha(SolverState* st, const double* partials, int nb, int S, cudaStream_t s) {
+  k_cg_alpha<<<S, 256, 0, s>>>(st, partials, nb);
 }
 
 void plane_prepare() {

@@ -79,9 +79,12 @@ template <int Q> __device__ __forceinline__ int zp_grow(int kz) {
 // transforms over u, applies Gamma^h_k at kz = k1 + R1 k2 to the NC components
 // of each k2, transforms back and writes the same rows.  The coefficients of
 // the next k2 load while the current ones are applied.
-template <int NC, int N>
+// DOT: acc gains this item's share of (p, Gamma p) = sum_k Re(conj p_k (Gamma p)_k)
+// over the full spectrum (the table carries 1/V, the transforms are unnormalised):
+// columns other than kx = 0 and nx/2 stand for their mirror images too.
+template <int NC, int N, bool DOT>
 __device__ __forceinline__ void zp_fused_item(const OpArgs<float>& a, float2* B, int item, bool nyq, int yp,
-                                              int kx0) {
+                                              int kx0, Acc<float>& acc) {
   typedef ZPipe<NC, N, true> ZC;
   constexpr int TZ = ZC::TZ, P = ZC::P, R1 = ZC::R1, NX = ZC::NX;
   const int li = item & (TZ - 1), k1 = item / TZ, kb = k1 & 1;
@@ -90,6 +93,16 @@ __device__ __forceinline__ void zp_fused_item(const OpArgs<float>& a, float2* B,
   float2* const od = B + (4 * k1 - kb) * TZ + li;
   const int kx = nyq ? kx0 : kx0 + li, ypos = nyq ? yp + li : yp;
   float2 d[NC][P];
+  const float w = (nyq || kx == 0) ? 1.f : 2.f;
+  auto put = [&](int k2, const float2* g) {  // the product's result in place of d[.][k2]
+    float q = 0.f;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      if (DOT) q = fmaf(d[c][k2].x, g[c].x, fmaf(d[c][k2].y, g[c].y, q));
+      d[c][k2] = g[c];
+    }
+    if (DOT) acc.add(w * q);
+  };
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
 #pragma unroll
@@ -104,8 +117,7 @@ __device__ __forceinline__ void zp_fused_item(const OpArgs<float>& a, float2* B,
 #pragma unroll
       for (int c = 0; c < NC; ++c) g[c] = d[c][k2];
       gamma_trunc_onfly<float, NC>(a, kx, ky, k1 + R1 * k2, g);
-#pragma unroll
-      for (int c = 0; c < NC; ++c) d[c][k2] = g[c];
+      put(k2, g);
     }
   } else {
     constexpr int NCO = GammaPack<NC>::NCO;
@@ -122,8 +134,7 @@ __device__ __forceinline__ void zp_fused_item(const OpArgs<float>& a, float2* B,
       if (a.fdphase) fd_rotate<float, NC>(a, kx, a.kofy[ypos], k1 + R1 * k2, g, -1.f);
       gamma_coef_apply<float, NC>(gc[k2 & 1], g);
       if (a.fdphase) fd_rotate<float, NC>(a, kx, a.kofy[ypos], k1 + R1 * k2, g, 1.f);
-#pragma unroll
-      for (int c = 0; c < NC; ++c) d[c][k2] = g[c];
+      put(k2, g);
     }
   }
 #pragma unroll
@@ -134,10 +145,13 @@ __device__ __forceinline__ void zp_fused_item(const OpArgs<float>& a, float2* B,
   }
 }
 
-template <int NC, int N, bool FUSED>
+// DOT (FUSED only): each tile's share of (p, Gamma p) goes to partials[s per_sys + tile
+// of the system], regular tiles first; k_cg_alpha sums them in that order.
+template <int NC, int N, bool FUSED, bool DOT>
 __global__ void __launch_bounds__(ZPipe<NC, N, FUSED>::THREADS, ZPipe<NC, N, FUSED>::MINB)
     k_zgamma_pipe(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtensorMap tmQ, OpArgs<float> a,
-                  const SolverState* __restrict__ st, int nkt, int nregular, int total) {
+                  const SolverState* __restrict__ st, int nkt, int nregular, int total,
+                  double* __restrict__ partials) {
   typedef ZPipe<NC, N, FUSED> ZC;
   constexpr int TZ = ZC::TZ, P = ZC::P, R1 = ZC::R1, Q = ZC::Q, NX = ZC::NX, THREADS = ZC::THREADS;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -146,6 +160,7 @@ __global__ void __launch_bounds__(ZPipe<NC, N, FUSED>::THREADS, ZPipe<NC, N, FUS
   float2* const tw = buf0 + 2 * ZC::BUF;  // buffer b at buf0 + b BUF
   __shared__ __align__(8) uint64_t bar[2];
   __shared__ int fault;
+  __shared__ float dot_sh[2][ZC::THREADS / 32];
   // the tile each buffer holds, published by warp 0: live, system, y position, first kx
   __shared__ int tile_live[2], tile_s[2], tile_yp[2], tile_kx0[2];
   for (int u = threadIdx.x; u < N; u += THREADS) tw[u] = a.twz[u];
@@ -242,7 +257,16 @@ __global__ void __launch_bounds__(ZPipe<NC, N, FUSED>::THREADS, ZPipe<NC, N, FUS
     for (int k1 = 0; k1 < R1; ++k1) B[xa(k1)] = v[k1];
     __syncthreads();
     if constexpr (FUSED) {
-      for (int item = threadIdx.x; item < R1 * TZ; item += THREADS) zp_fused_item<NC, N>(a, B, item, nyq, yp, kx0);
+      Acc<float> acc;
+      for (int item = threadIdx.x; item < R1 * TZ; item += THREADS)
+        zp_fused_item<NC, N, DOT>(a, B, item, nyq, yp, kx0, acc);
+      if constexpr (DOT) {
+        warp_merge_pair(acc.s, acc.c);
+        if ((threadIdx.x & 31) == 0) {
+          dot_sh[0][threadIdx.x >> 5] = acc.s;
+          dot_sh[1][threadIdx.x >> 5] = acc.c;
+        }
+      }
     } else {
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
@@ -324,6 +348,15 @@ __global__ void __launch_bounds__(ZPipe<NC, N, FUSED>::THREADS, ZPipe<NC, N, FUS
     }
     }  // !FUSED
     __syncthreads();
+    if constexpr (DOT) {
+      if (threadIdx.x == THREADS - 1) {  // not the thread that requests the next box
+        double sum = 0.0;
+#pragma unroll
+        for (int w = 0; w < THREADS / 32; ++w) sum += (double)dot_sh[0][w] - (double)dot_sh[1][w];
+        const int tile = nyq ? a.ny * nkt + yp / TZ : yp * nkt + kx0 / TZ;
+        partials[(long long)s * (a.ny * nkt + a.ny / TZ) + tile] = sum;
+      }
+    }
 #pragma unroll
     for (int k1 = 0; k1 < R1; ++k1) v[k1] = B[xa(k1)];
 #pragma unroll
@@ -355,13 +388,14 @@ __global__ void __launch_bounds__(ZPipe<NC, N, FUSED>::THREADS, ZPipe<NC, N, FUS
 // ------------------------------------------------------------------ host side
 namespace {
 
-template <int NC, int N, bool FUSED> int zpipe_blocks_per_sm() {
+template <int NC, int N, bool FUSED, bool DOT> int zpipe_blocks_per_sm() {
   typedef ZPipe<NC, N, FUSED> ZC;
   static int n = []() {
     int v = 0;
     if constexpr (ZC::FITS) {
-      cudaFuncSetAttribute(k_zgamma_pipe<NC, N, FUSED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ZC::SMEM);
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_zgamma_pipe<NC, N, FUSED>, ZC::THREADS, ZC::SMEM) !=
+      cudaFuncSetAttribute(k_zgamma_pipe<NC, N, FUSED, DOT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)ZC::SMEM);
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_zgamma_pipe<NC, N, FUSED, DOT>, ZC::THREADS, ZC::SMEM) !=
           cudaSuccess) {
         cudaGetLastError();
         v = 0;
@@ -372,13 +406,13 @@ template <int NC, int N, bool FUSED> int zpipe_blocks_per_sm() {
   return n;
 }
 
-template <int NC, int N, bool FUSED>
-bool launch_zpipe_n(const OpArgs<float>& a, const SolverState* st, cudaStream_t s) {
+template <int NC, int N, bool FUSED, bool DOT>
+bool launch_zpipe_n(const OpArgs<float>& a, const SolverState* st, double* partials, cudaStream_t s) {
   typedef ZPipe<NC, N, FUSED> ZC;
   if constexpr (!ZC::FITS) {
     return false;
   } else {
-    const int bpsm = zpipe_blocks_per_sm<NC, N, FUSED>();
+    const int bpsm = zpipe_blocks_per_sm<NC, N, FUSED, DOT>();
     if (bpsm < 1) return false;
     if (a.S < 1) return true;
     const int nkt = (a.nx / 2) / ZC::TZ;
@@ -386,21 +420,22 @@ bool launch_zpipe_n(const OpArgs<float>& a, const SolverState* st, cudaStream_t 
     const long long total = nregular + (long long)a.S * (a.ny / ZC::TZ);
     const long long grid = std::max<long long>(1, std::min<long long>(total, (long long)multiprocessors() * bpsm));
     if (total + grid >= (1ll << 31)) return false;
-    k_zgamma_pipe<NC, N, FUSED><<<(unsigned)grid, ZC::THREADS, ZC::SMEM, s>>>(*a.tmzp, *a.tmzq, a, st, nkt,
-                                                                              (int)nregular, (int)total);
+    k_zgamma_pipe<NC, N, FUSED, DOT><<<(unsigned)grid, ZC::THREADS, ZC::SMEM, s>>>(*a.tmzp, *a.tmzq, a, st, nkt,
+                                                                                   (int)nregular, (int)total, partials);
     return true;
   }
 }
 
-template <int NC, bool FUSED> bool launch_zpipe_nc(const OpArgs<float>& a, const SolverState* st, cudaStream_t s) {
+template <int NC, bool FUSED, bool DOT>
+bool launch_zpipe_nc(const OpArgs<float>& a, const SolverState* st, double* partials, cudaStream_t s) {
   switch (a.nz) {
-    case 16: return launch_zpipe_n<NC, 16, FUSED>(a, st, s);
-    case 32: return launch_zpipe_n<NC, 32, FUSED>(a, st, s);
-    case 48: return launch_zpipe_n<NC, 48, FUSED>(a, st, s);
-    case 64: return launch_zpipe_n<NC, 64, FUSED>(a, st, s);
-    case 96: return launch_zpipe_n<NC, 96, FUSED>(a, st, s);
-    case 128: return launch_zpipe_n<NC, 128, FUSED>(a, st, s);
-    case 256: return launch_zpipe_n<NC, 256, FUSED>(a, st, s);
+    case 16: return launch_zpipe_n<NC, 16, FUSED, DOT>(a, st, partials, s);
+    case 32: return launch_zpipe_n<NC, 32, FUSED, DOT>(a, st, partials, s);
+    case 48: return launch_zpipe_n<NC, 48, FUSED, DOT>(a, st, partials, s);
+    case 64: return launch_zpipe_n<NC, 64, FUSED, DOT>(a, st, partials, s);
+    case 96: return launch_zpipe_n<NC, 96, FUSED, DOT>(a, st, partials, s);
+    case 128: return launch_zpipe_n<NC, 128, FUSED, DOT>(a, st, partials, s);
+    case 256: return launch_zpipe_n<NC, 256, FUSED, DOT>(a, st, partials, s);
     default: return false;
   }
 }
@@ -425,14 +460,25 @@ PFN_cuTensorMapEncodeTiled_v12000 zp_encode_fn() {
 // takes the level-b DFTs and Gamma^h in one register phase); false (nothing launched) when
 // the spectrum is not ky-major, the maps are missing, the geometry has no
 // tiling or the kernel does not fit.  With a.S = 0 it only answers whether it
-// would launch.
-bool launch_zgamma_pipe(const OpArgs<float>& a, bool fused, const SolverState* st, cudaStream_t s) {
+// would launch.  partials (fused only): also the tiles' shares of (p, Gamma p),
+// zdot_count() of them per system.
+bool launch_zgamma_pipe(const OpArgs<float>& a, bool fused, const SolverState* st, cudaStream_t s, double* partials) {
   if (!a.tlay || a.nq == nullptr || a.tmzp == nullptr || a.tmzq == nullptr) return false;
   if ((a.nx & 15) != 0 || (a.ny & 7) != 0) return false;  // whole 8-column tiles of kx < nx/2 and of ky
-  if (a.c == 6) return fused ? launch_zpipe_nc<6, true>(a, st, s) : launch_zpipe_nc<6, false>(a, st, s);
-  if (a.c == 3) return fused ? launch_zpipe_nc<3, true>(a, st, s) : launch_zpipe_nc<3, false>(a, st, s);
+  if (partials != nullptr) {
+    if (!fused) return false;
+    if (a.c == 6) return launch_zpipe_nc<6, true, true>(a, st, partials, s);
+    if (a.c == 3) return launch_zpipe_nc<3, true, true>(a, st, partials, s);
+    return false;
+  }
+  if (a.c == 6)
+    return fused ? launch_zpipe_nc<6, true, false>(a, st, nullptr, s) : launch_zpipe_nc<6, false, false>(a, st, nullptr, s);
+  if (a.c == 3)
+    return fused ? launch_zpipe_nc<3, true, false>(a, st, nullptr, s) : launch_zpipe_nc<3, false, false>(a, st, nullptr, s);
   return false;
 }
+
+int zdot_count(const OpArgs<float>& a) { return a.ny * ((a.nx / 2) / 8) + a.ny / 8; }
 
 // Tensor maps of the ky-major FP32 spectrum H[S c][ky][z][hs] ({2 hs, nz, ny, S c}
 // floats, box {16, nz, 1, c}) and of its Nyquist columns NQ[S c][z][ky]
@@ -461,21 +507,23 @@ bool encode_zpipe_maps(CUtensorMap* th, CUtensorMap* tq, void* H, void* NQ, int 
          CUDA_SUCCESS;
 }
 
-template <int NC, bool FUSED> void zpipe_prepare_nc() {
-  zpipe_blocks_per_sm<NC, 16, FUSED>();
-  zpipe_blocks_per_sm<NC, 32, FUSED>();
-  zpipe_blocks_per_sm<NC, 48, FUSED>();
-  zpipe_blocks_per_sm<NC, 64, FUSED>();
-  zpipe_blocks_per_sm<NC, 96, FUSED>();
-  zpipe_blocks_per_sm<NC, 128, FUSED>();
-  zpipe_blocks_per_sm<NC, 256, FUSED>();
+template <int NC, bool FUSED, bool DOT> void zpipe_prepare_nc() {
+  zpipe_blocks_per_sm<NC, 16, FUSED, DOT>();
+  zpipe_blocks_per_sm<NC, 32, FUSED, DOT>();
+  zpipe_blocks_per_sm<NC, 48, FUSED, DOT>();
+  zpipe_blocks_per_sm<NC, 64, FUSED, DOT>();
+  zpipe_blocks_per_sm<NC, 96, FUSED, DOT>();
+  zpipe_blocks_per_sm<NC, 128, FUSED, DOT>();
+  zpipe_blocks_per_sm<NC, 256, FUSED, DOT>();
 }
 
 void zpipe_prepare() {
-  zpipe_prepare_nc<3, false>();
-  zpipe_prepare_nc<6, false>();
-  zpipe_prepare_nc<3, true>();
-  zpipe_prepare_nc<6, true>();
+  zpipe_prepare_nc<3, false, false>();
+  zpipe_prepare_nc<6, false, false>();
+  zpipe_prepare_nc<3, true, false>();
+  zpipe_prepare_nc<6, true, false>();
+  zpipe_prepare_nc<3, true, true>();
+  zpipe_prepare_nc<6, true, true>();
 }
 
 }  // namespace lsh

@@ -427,7 +427,7 @@ Layout make_layout(const Derived& d) {
                                       (long long)S * d.c * d.nz});
   l.nparts = np;
   l.off_state = take(sizeof(SolverState) * (size_t)(3 * S + d.B));
-  l.off_partials = take(sizeof(double) * 2 * (size_t)np);  // two sums per block where a kernel forms two
+  l.off_partials = take(sizeof(double) * 4 * (size_t)np);  // up to four sums per block
   l.off_phase = take((size_t)(d.B * d.V));
   l.off_scale = take(d.has_scale ? sizeof(float) * (size_t)(d.B * d.V) : 0);
   l.off_act = take(256);
@@ -652,6 +652,7 @@ void init_prec(lsh_handle* h, PrecBufs<T>& P, const size_t* off_f, size_t off_H,
   a.xreg = 0;  // lsh_autotune measures the register x passes against the shared-memory ones
   a.xfreg = 0;
   a.plane = 0;
+  a.fuse = 0;
   a.tlay = 0;
   a.nq = nullptr;
   // measured on the batched workload: the inverse pass gains (0.61 -> 0.66 of the
@@ -869,6 +870,27 @@ template <typename T> void enqueue_cg_iteration(lsh_handle* h, PrecBufs<T>& P, c
   cudaEvent_t* e = timed ? &h->ev[h->ev_used] : nullptr;
   // inside a capture the records become graph nodes that record at replay
   const unsigned rf = h->capturing ? cudaEventRecordExternal : cudaEventRecordDefault;
+  if constexpr (sizeof(T) == 4) {
+    if (a.plane && a.fuse) {
+      // five launches: xy forward, z, alpha, xy inverse with the update of z, beta
+      if (timed) cudaEventRecordWithFlags(e[0], s, rf);
+      launch_xyfwd(a, 1, nullptr, P.x, P.r, P.p, P.st, s);
+      if (timed) cudaEventRecordWithFlags(e[1], s, rf);
+      if (timed) cudaEventRecordWithFlags(e[2], s, rf);
+      launch_zgamma_pipe(a, true, P.st, s, h->partials);
+      if (timed) cudaEventRecordWithFlags(e[3], s, rf);
+      if (timed) cudaEventRecordWithFlags(e[4], s, rf);
+      launch_cg_alpha(P.st, h->partials, zdot_count(a), a.S, s);
+      launch_xyinv_update(a, P.p, P.r, P.st, h->partials, h->lay.nparts, s);
+      if (timed) {
+        cudaEventRecordWithFlags(e[5], s, rf);
+        cudaEventRecordWithFlags(e[6], s, rf);
+        h->ev_used += 7;
+      }
+      h->launches += 5;
+      return;
+    }
+  }
   if (timed) cudaEventRecordWithFlags(e[0], s, rf);
   launch_xfwd<T>(a, P.L, 1, nullptr, P.x, P.r, P.p, P.st, s);
   if (timed) cudaEventRecordWithFlags(e[1], s, rf);
@@ -938,11 +960,12 @@ lsh_status chunk_graph(lsh_handle* h, PrecBufs<T>& P, const OpArgs<T>& a, int ch
 // After a host synchronisation: add the pass times of the first `real`
 // recorded iterations (later ones returned at once because every system of
 // the wave was done).
-void harvest_profile(lsh_handle* h, int real, bool plane) {
+void harvest_profile(lsh_handle* h, int real, bool plane, bool fuse) {
   const int groups = h->ev_used / 7;
   for (int g = 0; g < groups && g < real; ++g) {
     for (int k = 0; k < 6; ++k) {
       if (plane && (k == 1 || k == 3)) continue;  // no separate y passes
+      if (plane && fuse && k == 5) continue;      // the inverse pass updates z
       float ms = 0.f;
       if (cudaEventElapsedTime(&ms, h->ev[7 * g + k], h->ev[7 * g + k + 1]) == cudaSuccess) {
         h->pass_ms[k] += ms;
@@ -997,7 +1020,7 @@ lsh_status cg_run(lsh_handle* h, PrecBufs<T>& P, const OpArgs<T>& a, int maxit, 
     if (h->prof_now) {
       for (int k = 0; k < S; ++k) h->timed_sys_iters += out[k].iter;
       h->timed_sys_iters -= live0;
-      harvest_profile(h, max_iter() - before, a.plane != 0);
+      harvest_profile(h, max_iter() - before, a.plane != 0, a.fuse != 0);
     }
     h->prof_now = false;
   }
@@ -1491,7 +1514,10 @@ lsh_status lsh_setup(const lsh_problem* prob, void* workspace, size_t bytes, voi
     // else the register kernel
     OpArgs<float> az = h->pf.a;
     az.S = 0;
-    if (d.precision == LSH_MIXED && launch_zgamma_pipe(az, true, nullptr, 0)) h->pf.a.ztma = 11;
+    if (d.precision == LSH_MIXED && launch_zgamma_pipe(az, true, nullptr, 0)) {
+      h->pf.a.ztma = 11;
+      h->pf.a.fuse = 1;
+    }
   }
   if (l.df) df_prepare();
   launch_gamma_table<double>(h->pd.a, d.dim, d.physics, d.green, d.ref_user, h->kofy, h->kofz, st,
@@ -1769,6 +1795,7 @@ lsh_status lsh_autotune(lsh_handle* h, lsh_tune_report* rep) {
     cudaStream_t s = h->stream;
     LSH_CK(cudaMemsetAsync(P.H, 0, sizeof(float2) * (size_t)d.Smax * d.c * d.nz * d.ny * d.hs, s));
     OpArgs<float> a = P.a;
+    a.fuse = 0;
     cudaEvent_t e0, e1;
     LSH_CK(cudaEventCreate(&e0));
     if (cudaEventCreate(&e1) != cudaSuccess) {
@@ -1869,7 +1896,7 @@ lsh_status lsh_autotune(lsh_handle* h, lsh_tune_report* rep) {
       b.plane = 1;
       b.tlay = 1;
       const int zc[7] = {0, 6, 8, 9, 7, 10, 11};
-      int bz = 0;
+      int bz = 0;  // the fastest of the variants that leave the update of r a kernel of its own
       for (int k = 0; k < 7; ++k) {
         b.ztma = zc[k];
         r.zp_ms[k] = timeit([&]() {
@@ -1878,18 +1905,43 @@ lsh_status lsh_autotune(lsh_handle* h, lsh_tune_report* rep) {
           launch_zgamma<float>(b, P.L, nullptr, s);
           return true;
         });
-        if (r.zp_ms[k] > 0.f && (r.zp_ms[bz] < 0.f || r.zp_ms[k] < r.zp_ms[bz])) bz = k;
+        if (zc[k] != 11 && r.zp_ms[k] > 0.f && (r.zp_ms[bz] < 0.f || r.zp_ms[k] < r.zp_ms[bz])) bz = k;
       }
       b.ztma = zc[bz];
       const float f = timeit([&]() {
         cudaMemcpyAsync(P.st, fake.data(), sizeof(SolverState) * d.Smax, cudaMemcpyHostToDevice, s);
         return launch_xyfwd(b, 1, nullptr, P.x, P.r, P.p, P.st, s);
       });
-      const float i = timeit([&]() {
+      float i = timeit([&]() {
         cudaMemcpyAsync(P.st, fake.data(), sizeof(SolverState) * d.Smax, cudaMemcpyHostToDevice, s);
         return launch_xyinv(b, 1, P.p, P.q, P.st, h->partials, s);
       });
-      r.xy_ms[1] = (f > 0.f && i > 0.f && r.zp_ms[bz] > 0.f) ? f + r.zp_ms[bz] + i : -1.f;
+      const float u = timeit([&]() {
+        cudaMemcpyAsync(P.st, fake.data(), sizeof(SolverState) * d.Smax, cudaMemcpyHostToDevice, s);
+        launch_cg_update<float>(b, P.r, P.q, P.st, h->partials, h->lay.nparts, P.L.ew_per_sys, s);
+        return true;
+      });
+      float z = r.zp_ms[bz];
+      if (r.zp_ms[6] > 0.f) {
+        // z variant 11 leaves (p, Gamma p), so that the inverse pass can update z
+        b.ztma = 11;
+        const float zf = timeit([&]() { return launch_zgamma_pipe(b, true, nullptr, s, h->partials); });
+        const float jf = timeit([&]() {
+          cudaMemcpyAsync(P.st, fake.data(), sizeof(SolverState) * d.Smax, cudaMemcpyHostToDevice, s);
+          // the pass first: on the arbitrary data alpha may flag a breakdown that would stop it
+          const bool ok = launch_xyinv_update(b, P.p, P.r, P.st, h->partials, h->lay.nparts, s);
+          launch_cg_alpha(P.st, h->partials, zdot_count(b), b.S, s);
+          return ok;
+        });
+        if (zf > 0.f && jf > 0.f && zf + jf < z + i + u) {
+          b.fuse = 1;
+          z = zf;
+          i = jf - u;  // comparable with the separate schedule's sum, which has no update kernel either
+        } else {
+          b.ztma = zc[bz];
+        }
+      }
+      r.xy_ms[1] = (f > 0.f && z > 0.f) ? f + z + i : -1.f;
       if (sep_ok) {
         const float xf = r.xf_ms[a.xfreg] > 0.f ? r.xf_ms[a.xfreg] : r.xf_ms[0];
         const float yy = r.y_ms[a.ytma] > 0.f ? r.y_ms[a.ytma] : -1.f;
@@ -1913,6 +1965,7 @@ lsh_status lsh_autotune(lsh_handle* h, lsh_tune_report* rep) {
     P.a.ztma = a.ztma;
     P.a.plane = a.plane;
     P.a.tlay = a.tlay;
+    P.a.fuse = a.fuse;
     h->drop_graphs();  // captured with the previous choices
   }
   if (rep) *rep = r;
@@ -1939,6 +1992,7 @@ lsh_status lsh_set_variants(lsh_handle* h, int xf_variant, int x_variant, int y_
     P.a.plane = 1;
     P.a.tlay = 1;
     P.a.ztma = z_variant;
+    P.a.fuse = z_variant == 11;
     h->drop_graphs();
     return LSH_OK;
   }
@@ -1966,6 +2020,7 @@ lsh_status lsh_set_variants(lsh_handle* h, int xf_variant, int x_variant, int y_
   P.a.ztma = z_variant;
   P.a.plane = 0;
   P.a.tlay = 0;
+  P.a.fuse = 0;
   h->drop_graphs();
   return LSH_OK;
 }
