@@ -115,8 +115,17 @@ __device__ __forceinline__ double block_reduce(const Acc<float>& a) {
   return out;
 }
 
-// a / d with a shift when d is a power of two (d is uniform across the block).
-__device__ __forceinline__ int fdiv(int a, int d) { return (d & (d - 1)) == 0 ? (a >> (__ffs(d) - 1)) : a / d; }
+// Quotients by a divisor that is uniform across the block: one multiplication with
+// ceil(2^32 / d), exact for dividends and divisors below 2^16 (every index inside a
+// block's shared-memory tile).  The mixed-radix stages spend most of their integer
+// work on such splits; an integer division is some twenty instructions.
+struct FastDiv {
+  unsigned d, m;
+  __host__ __device__ __forceinline__ static unsigned magic(int d) { return d == 1 ? 0u : 0xffffffffu / (unsigned)d + 1u; }
+  __device__ __forceinline__ explicit FastDiv(int d_) : d((unsigned)d_), m(magic(d_)) {}
+  __device__ __forceinline__ FastDiv(int d_, unsigned m_) : d((unsigned)d_), m(m_) {}
+  __device__ __forceinline__ int div(int a) const { return d == 1u ? a : (int)__umulhi((unsigned)a, m); }
+};
 
 // FFT plan of one axis: length n = product of the radices, DIF stage order.
 #define LSH_MAX_STAGES 8
@@ -124,7 +133,73 @@ struct Plan1D {
   int n;
   int nst;
   int radix[LSH_MAX_STAGES];
+  int m[LSH_MAX_STAGES];             // distance between a butterfly's inputs: span / radix
+  int tws[LSH_MAX_STAGES];           // twiddle stride n / span
+  unsigned mag_m[LSH_MAX_STAGES];    // FastDiv factors of m and of n / radix
+  unsigned mag_nb[LSH_MAX_STAGES];
 };
+
+// Plan of length n (factors 2, 3, 5, 7), false if there is none.  Every stage is a
+// round trip through shared memory with a barrier, so the fewest stages win, then
+// the fewest operations; larger radices first.  Radices up to 12 keep an FP64
+// butterfly in 128 registers.  The lengths with compile-time schedules (fft.cuh) come
+// out as those expect.  A length whose factors 8, 4, 2, 3, 5, 7 number more than
+// LSH_MAX_STAGES is not taken.
+inline bool lsh_make_plan(int n, Plan1D* p) {
+  if (n < 1) return false;
+  int m = n, small = 0;
+  for (int q : {8, 4, 2, 3, 5, 7})
+    while (m % q == 0) { m /= q; ++small; }
+  if (m != 1 || small > LSH_MAX_STAGES) return false;
+  // radix and cost per point: a stage's own cost (shared-memory round trip, indices,
+  // twiddles) of 16 and the butterfly's operations
+  const int rad[] = {12, 10, 9, 8, 7, 6, 5, 4, 3, 2};
+  const int cost[] = {26, 25, 28, 22, 26, 23, 23, 20, 21, 18};
+  int best = 1 << 30, cur[16], nbest = 0;
+  int bestr[LSH_MAX_STAGES];
+  struct Search {
+    static void run(int left, int from, int k, int c, const int* rad, const int* cost, int* cur, int* best, int* bestr,
+                    int* nbest) {
+      if (left == 1) {
+        if (c < *best) {
+          *best = c;
+          *nbest = k;
+          for (int i = 0; i < k; ++i) bestr[i] = cur[i];
+        }
+        return;
+      }
+      if (k == LSH_MAX_STAGES) return;
+      for (int i = from; i < 10; ++i)
+        if (left % rad[i] == 0) {
+          cur[k] = rad[i];
+          run(left / rad[i], i, k + 1, c + cost[i], rad, cost, cur, best, bestr, nbest);
+        }
+    }
+  };
+  switch (n) {
+    case 128: nbest = 3; bestr[0] = 4; bestr[1] = 8; bestr[2] = 4; break;
+    case 256: nbest = 3; bestr[0] = 8; bestr[1] = 8; bestr[2] = 4; break;
+    case 96: nbest = 2; bestr[0] = 12; bestr[1] = 8; break;
+    case 64: nbest = 2; bestr[0] = bestr[1] = 8; break;
+    case 48: nbest = 2; bestr[0] = 8; bestr[1] = 6; break;
+    case 32: nbest = 2; bestr[0] = 8; bestr[1] = 4; break;
+    case 16: nbest = 2; bestr[0] = bestr[1] = 4; break;
+    default: Search::run(n, 0, 0, 0, rad, cost, cur, &best, bestr, &nbest);
+  }
+  p->n = n;
+  p->nst = nbest;
+  int span = n;
+  for (int i = 0; i < nbest; ++i) {
+    const int r = bestr[i];
+    p->radix[i] = r;
+    p->m[i] = span / r;
+    p->tws[i] = n / span;
+    p->mag_m[i] = FastDiv::magic(p->m[i]);
+    p->mag_nb[i] = FastDiv::magic(n / r);
+    span /= r;
+  }
+  return true;
+}
 
 // ---------------------------------------------------------------- reductions
 // Sum of one double per thread; result valid in thread 0.  Deterministic for a

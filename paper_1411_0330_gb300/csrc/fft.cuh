@@ -176,90 +176,59 @@ template <typename T, bool INV> struct Dft<T, 32, INV> {
   }
 };
 
-// Direct DFT for the remaining small prime (7), from the twiddle table.
+// 7 points from the sums and differences of the pairs (q, 7 - q)
 template <typename T, bool INV> struct Dft<T, 7, INV> {
-  static __device__ __forceinline__ void run(C2<T>* a, const C2<T>* tw, int n) {
-    const int st = n / 7;
-    C2<T> y[7];
+  static __device__ __forceinline__ void run(C2<T>* a, const C2<T>*, int) {
+    const T c[3] = {(T)0.62348980185873353052500488400424, (T)-0.22252093395631440428890256449679,
+                    (T)-0.90096886790241912623610231950745};  // cos(2 pi k / 7)
+    const T s[3] = {(T)0.78183148246802980870844452667406, (T)0.97492791218182360701813168299393,
+                    (T)0.43388373911755812047576833284836};  // sin(2 pi k / 7)
+    C2<T> p[3], m[3];
 #pragma unroll
-    for (int p = 0; p < 7; ++p) {
-      C2<T> s = a[0];
-#pragma unroll
-      for (int q = 1; q < 7; ++q) {
-        C2<T> w = tw[((p * q) % 7) * st];
-        s = cadd<T>(s, INV ? cmulc<T>(a[q], w) : cmul<T>(a[q], w));
-      }
-      y[p] = s;
+    for (int q = 0; q < 3; ++q) {
+      p[q] = cadd<T>(a[q + 1], a[6 - q]);
+      m[q] = csub<T>(a[q + 1], a[6 - q]);
     }
+    const C2<T> a0 = a[0];
+    a[0] = mkc<T>(a0.x + p[0].x + p[1].x + p[2].x, a0.y + p[0].y + p[1].y + p[2].y);
 #pragma unroll
-    for (int p = 0; p < 7; ++p) a[p] = y[p];
+    for (int k = 1; k <= 3; ++k) {
+      C2<T> b = a0, u = mkc<T>((T)0, (T)0);
+#pragma unroll
+      for (int q = 1; q <= 3; ++q) {
+        const int e = (k * q) % 7, f = e <= 3 ? e : 7 - e;  // angle 2 pi e / 7, folded
+        const T sn = e <= 3 ? s[f - 1] : -s[f - 1];
+        b.x += c[f - 1] * p[q - 1].x;
+        b.y += c[f - 1] * p[q - 1].y;
+        u.x += sn * m[q - 1].x;
+        u.y += sn * m[q - 1].y;
+      }
+      const C2<T> iu = INV ? cmul_pi<T>(u) : cmul_mi<T>(u);
+      a[k] = cadd<T>(b, iu);
+      a[7 - k] = csub<T>(b, iu);
+    }
   }
 };
 
-// cos and sin of 2 pi m / 24 (multiples of 15 degrees) from the closed forms
-// cos 15 = (sqrt 6 + sqrt 2) / 4, sin 15 = (sqrt 6 - sqrt 2) / 4, cos 30 = sqrt 3 / 2,
-// cos 45 = sqrt 2 / 2; once the loops are unrolled m is a constant and these fold.
-__host__ __device__ constexpr double cos24(int m) {
-  constexpr double c15 = 0.96592582628906828674974319972889736763, s15 = 0.25881904510252076234889883762404832835;
-  constexpr double c30 = 0.86602540378443864676372317075293618347, c45 = 0.70710678118654752440084436210484903928;
-  switch (((m % 24) + 24) % 24) {
-    case 0: return 1.0;
-    case 1: return c15;
-    case 2: return c30;
-    case 3: return c45;
-    case 4: return 0.5;
-    case 5: return s15;
-    case 6: return 0.0;
-    case 7: return -s15;
-    case 8: return -0.5;
-    case 9: return -c45;
-    case 10: return -c30;
-    case 11: return -c15;
-    case 12: return -1.0;
-    case 13: return -c15;
-    case 14: return -c30;
-    case 15: return -c45;
-    case 16: return -0.5;
-    case 17: return -s15;
-    case 18: return 0.0;
-    case 19: return s15;
-    case 20: return 0.5;
-    case 21: return c45;
-    case 22: return c30;
-    default: return c15;
-  }
+// Composite lengths with coprime factors R = A * B in registers, by the Chinese
+// remainder theorem (Good-Thomas): with n = (B n1 + A n2) mod R and k = (B B' k1 +
+// A A' k2) mod R, B' = B^{-1} mod A and A' = A^{-1} mod B, w_R^(nk) = w_A^(n1 k1)
+// w_B^(n2 k2): A- and B-point DFTs with no twiddles between them.
+__host__ __device__ constexpr int inverse_mod(int a, int m) {
+  for (int x = 1; x < m; ++x)
+    if ((a * x) % m == 1) return x;
+  return 0;
 }
-__host__ __device__ constexpr double sin24(int m) { return cos24(m - 6); }
-
-// Composite lengths R = A * B in registers (Cooley-Tukey with B-point outer
-// and A-point inner DFTs): x[B n1 + n2] -> X[k1 + A k2] =
-//   sum_n2 w_B^(n2 k2) [ w_R^(n2 k1) sum_n1 x[B n1 + n2] w_A^(n1 k1) ];
-// the twiddles w_R^m are constants for R dividing 24 (the radix-3 lengths 6,
-// 12, 24), else they come from the line's table tw of length n (stride n / R).
-template <typename T, int A, int B, bool INV> struct DftAB {
-  static __device__ __forceinline__ C2<T> twiddle(const C2<T>& c, int m, const C2<T>* tw, int st) {
-    constexpr int R = A * B;
-    if constexpr (24 % R == 0) {
-      const int m24 = m * (24 / R);
-      const C2<T> w = mkc<T>((T)cos24(m24), (T)(INV ? sin24(m24) : -sin24(m24)));
-      return cmul<T>(c, w);
-    } else {
-      return INV ? cmulc<T>(c, tw[m * st]) : cmul<T>(c, tw[m * st]);
-    }
-  }
+template <typename T, int A, int B, bool INV> struct DftPFA {
   static __device__ __forceinline__ void run(C2<T>* a, const C2<T>* tw, int n) {
     constexpr int R = A * B;
-    const int st = n / R;
+    constexpr int eb = B * inverse_mod(B % A, A), ea = A * inverse_mod(A % B, B);
     C2<T> b[B][A];
 #pragma unroll
     for (int n2 = 0; n2 < B; ++n2) {
-      C2<T> c[A];
 #pragma unroll
-      for (int n1 = 0; n1 < A; ++n1) c[n1] = a[B * n1 + n2];
-      Dft<T, A, INV>::run(c, tw, n);
-#pragma unroll
-      for (int k1 = 0; k1 < A; ++k1)
-        b[n2][k1] = (n2 == 0 || k1 == 0) ? c[k1] : twiddle(c[k1], n2 * k1, tw, st);
+      for (int n1 = 0; n1 < A; ++n1) b[n2][n1] = a[(B * n1 + A * n2) % R];
+      Dft<T, A, INV>::run(b[n2], tw, n);
     }
 #pragma unroll
     for (int k1 = 0; k1 < A; ++k1) {
@@ -268,13 +237,43 @@ template <typename T, int A, int B, bool INV> struct DftAB {
       for (int n2 = 0; n2 < B; ++n2) d[n2] = b[n2][k1];
       Dft<T, B, INV>::run(d, tw, n);
 #pragma unroll
-      for (int k2 = 0; k2 < B; ++k2) a[k1 + A * k2] = d[k2];
+      for (int k2 = 0; k2 < B; ++k2) a[(eb * k1 + ea * k2) % R] = d[k2];
     }
   }
 };
-template <typename T, bool INV> struct Dft<T, 6, INV> : DftAB<T, 2, 3, INV> {};
-template <typename T, bool INV> struct Dft<T, 12, INV> : DftAB<T, 4, 3, INV> {};
-template <typename T, bool INV> struct Dft<T, 24, INV> : DftAB<T, 8, 3, INV> {};
+template <typename T, bool INV> struct Dft<T, 6, INV> : DftPFA<T, 2, 3, INV> {};
+template <typename T, bool INV> struct Dft<T, 10, INV> : DftPFA<T, 2, 5, INV> {};
+template <typename T, bool INV> struct Dft<T, 12, INV> : DftPFA<T, 4, 3, INV> {};
+template <typename T, bool INV> struct Dft<T, 24, INV> : DftPFA<T, 8, 3, INV> {};
+
+// 9 = 3 x 3: x[3 n1 + n2] -> X[k1 + 3 k2] = sum_n2 w3^(n2 k2) w9^(n2 k1) sum_n1 x w3^(n1 k1)
+template <typename T, bool INV> struct Dft<T, 9, INV> {
+  static __device__ __forceinline__ void run(C2<T>* a, const C2<T>* tw, int n) {
+    const T sg = INV ? (T)1 : (T)-1;
+    // w9^1, w9^2, w9^4
+    const C2<T> w1 = mkc<T>((T)0.76604444311897803520239265055542, sg * (T)0.64278760968653932632264340990726);
+    const C2<T> w2 = mkc<T>((T)0.17364817766693034885171662676931, sg * (T)0.98480775301220805936674302458952);
+    const C2<T> w4 = mkc<T>((T)-0.93969262078590838405410927732473, sg * (T)0.34202014332566873304409961468226);
+    C2<T> b[3][3];
+#pragma unroll
+    for (int n2 = 0; n2 < 3; ++n2) {
+#pragma unroll
+      for (int n1 = 0; n1 < 3; ++n1) b[n2][n1] = a[3 * n1 + n2];
+      Dft<T, 3, INV>::run(b[n2], tw, n);
+    }
+    b[1][1] = cmul<T>(b[1][1], w1);
+    b[1][2] = cmul<T>(b[1][2], w2);
+    b[2][1] = cmul<T>(b[2][1], w2);
+    b[2][2] = cmul<T>(b[2][2], w4);
+#pragma unroll
+    for (int k1 = 0; k1 < 3; ++k1) {
+      C2<T> d[3] = {b[0][k1], b[1][k1], b[2][k1]};
+      Dft<T, 3, INV>::run(d, tw, n);
+#pragma unroll
+      for (int k2 = 0; k2 < 3; ++k2) a[k1 + 3 * k2] = d[k2];
+    }
+  }
+};
 
 template <typename T, int R, bool INV>
 __device__ __forceinline__ void butterfly(C2<T>* base, int m, int te, const C2<T>* tw, int n) {
@@ -298,32 +297,41 @@ __device__ __forceinline__ void butterfly(C2<T>* base, int m, int te, const C2<T
   for (int q = 0; q < R; ++q) base[q * m] = a[q];
 }
 
-// One stage over `nlines` lines of length n (line stride ls, element stride 1).
-template <typename T, bool INV>
-__device__ __forceinline__ void fft_stage(C2<T>* __restrict__ buf, int nlines, int ls, int n, int r, int L,
-                                          const C2<T>* __restrict__ tw) {
-  const int m = L / r, nb = n / r, total = nb * nlines, tws = n / L;
+// Stage `st` of plan pl (radix R) over nlines lines (line stride ls, element stride 1).
+template <typename T, bool INV, int R>
+__device__ __forceinline__ void fft_stage_r(C2<T>* __restrict__ buf, int nlines, const FastDiv& dl, int ls,
+                                            const Plan1D& pl, int st, const C2<T>* __restrict__ tw) {
+  const int m = pl.m[st], nb = pl.n / R, total = nb * nlines, tws = pl.tws[st];
   const bool jmajor = m >= 16;
+  const FastDiv dm(m, pl.mag_m[st]), dnb(nb, pl.mag_nb[st]);
   for (int w = threadIdx.x; w < total; w += blockDim.x) {
     int line, b;
     if (jmajor) {
-      line = fdiv(w, nb);
+      line = dnb.div(w);
       b = w - line * nb;
     } else {
-      b = fdiv(w, nlines);
+      b = dl.div(w);
       line = w - b * nlines;
     }
-    const int sp = fdiv(b, m), j = b - sp * m;
-    C2<T>* base = buf + line * ls + sp * L + j;
-    const int te = j * tws;
-    switch (r) {
-      case 8: butterfly<T, 8, INV>(base, m, te, tw, n); break;
-      case 4: butterfly<T, 4, INV>(base, m, te, tw, n); break;
-      case 2: butterfly<T, 2, INV>(base, m, te, tw, n); break;
-      case 3: butterfly<T, 3, INV>(base, m, te, tw, n); break;
-      case 5: butterfly<T, 5, INV>(base, m, te, tw, n); break;
-      default: butterfly<T, 7, INV>(base, m, te, tw, n); break;
-    }
+    const int sp = dm.div(b), j = b - sp * m;
+    butterfly<T, R, INV>(buf + line * ls + sp * (m * R) + j, m, j * tws, tw, pl.n);
+  }
+}
+
+template <typename T, bool INV>
+__device__ __forceinline__ void fft_stage(C2<T>* __restrict__ buf, int nlines, const FastDiv& dl, int ls,
+                                          const Plan1D& pl, int st, const C2<T>* __restrict__ tw) {
+  switch (pl.radix[st]) {
+    case 12: fft_stage_r<T, INV, 12>(buf, nlines, dl, ls, pl, st, tw); break;
+    case 10: fft_stage_r<T, INV, 10>(buf, nlines, dl, ls, pl, st, tw); break;
+    case 9: fft_stage_r<T, INV, 9>(buf, nlines, dl, ls, pl, st, tw); break;
+    case 8: fft_stage_r<T, INV, 8>(buf, nlines, dl, ls, pl, st, tw); break;
+    case 7: fft_stage_r<T, INV, 7>(buf, nlines, dl, ls, pl, st, tw); break;
+    case 6: fft_stage_r<T, INV, 6>(buf, nlines, dl, ls, pl, st, tw); break;
+    case 5: fft_stage_r<T, INV, 5>(buf, nlines, dl, ls, pl, st, tw); break;
+    case 4: fft_stage_r<T, INV, 4>(buf, nlines, dl, ls, pl, st, tw); break;
+    case 3: fft_stage_r<T, INV, 3>(buf, nlines, dl, ls, pl, st, tw); break;
+    default: fft_stage_r<T, INV, 2>(buf, nlines, dl, ls, pl, st, tw); break;
   }
 }
 
@@ -335,13 +343,14 @@ __device__ __forceinline__ void stage_ct(C2<T>* __restrict__ buf, int nlines, in
   constexpr int m = L / R, nb = N / R, tws = N / L;
   constexpr bool jmajor = m >= 16;
   const int total = nb * nlines;
+  const FastDiv dl(nlines);
   for (int w = threadIdx.x; w < total; w += blockDim.x) {
     int line, b;
     if (jmajor) {
       line = w / nb;
       b = w - line * nb;
     } else {
-      b = fdiv(w, nlines);
+      b = dl.div(w);
       line = w - b * nlines;
     }
     const int sp = b / m, j = b - sp * m;
@@ -396,37 +405,26 @@ template <typename T, bool INV>
 __device__ void fft_lines_generic(C2<T>* buf, int nlines, int ls, const Plan1D& pl, const C2<T>* tw);
 
 // Forward (DIF) or inverse (DIT) transform of nlines lines; ends synchronised.
-// The fixed schedules mirror the host's radix choice (8s first, an 8*2 pair
-// becomes 4*4, then 3, 5, 7); any other plan runs the generic stage loop.
+// The fixed schedules mirror the host's radix choice (lsh_make_plan); any other
+// plan runs the generic stage loop.
 template <typename T, bool INV>
 __device__ void fft_lines(C2<T>* buf, int nlines, int ls, const Plan1D& pl, const C2<T>* tw) {
   if (try_fixed<T, INV, 128, 4, 8, 4>(buf, nlines, ls, pl, tw)) return;
   if (try_fixed<T, INV, 64, 8, 8>(buf, nlines, ls, pl, tw)) return;
   if (try_fixed<T, INV, 256, 8, 8, 4>(buf, nlines, ls, pl, tw)) return;
   if (try_fixed<T, INV, 32, 8, 4>(buf, nlines, ls, pl, tw)) return;
-  if (try_fixed<T, INV, 96, 8, 4, 3>(buf, nlines, ls, pl, tw)) return;
-  if (try_fixed<T, INV, 48, 4, 4, 3>(buf, nlines, ls, pl, tw)) return;
+  if (try_fixed<T, INV, 96, 12, 8>(buf, nlines, ls, pl, tw)) return;
+  if (try_fixed<T, INV, 48, 8, 6>(buf, nlines, ls, pl, tw)) return;
   if (try_fixed<T, INV, 16, 4, 4>(buf, nlines, ls, pl, tw)) return;
   fft_lines_generic<T, INV>(buf, nlines, ls, pl, tw);
 }
 
 template <typename T, bool INV>
 __device__ void fft_lines_generic(C2<T>* buf, int nlines, int ls, const Plan1D& pl, const C2<T>* tw) {
-  const int n = pl.n;
-  if (!INV) {
-    int L = n;
-    for (int s = 0; s < pl.nst; ++s) {
-      fft_stage<T, false>(buf, nlines, ls, n, pl.radix[s], L, tw);
-      L /= pl.radix[s];
-      __syncthreads();
-    }
-  } else {
-    int L = 1;
-    for (int s = pl.nst - 1; s >= 0; --s) {
-      L *= pl.radix[s];
-      fft_stage<T, true>(buf, nlines, ls, n, pl.radix[s], L, tw);
-      __syncthreads();
-    }
+  const FastDiv dl(nlines);
+  for (int k = 0; k < pl.nst; ++k) {
+    fft_stage<T, INV>(buf, nlines, dl, ls, pl, INV ? pl.nst - 1 - k : k, tw);
+    __syncthreads();
   }
 }
 

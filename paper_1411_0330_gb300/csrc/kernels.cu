@@ -34,6 +34,7 @@ template <typename T> struct MinBlocks { static constexpr int value = sizeof(T) 
 
 template <typename T, int VEC> struct VecOf;
 template <> struct VecOf<float, 4> { typedef float4 type; };
+template <> struct VecOf<float, 2> { typedef float2 type; };
 template <> struct VecOf<double, 2> { typedef double2 type; };
 
 template <typename T, int VEC> __device__ __forceinline__ void vload(const T* __restrict__ p, T* v) {
@@ -71,6 +72,23 @@ __device__ __forceinline__ T local_coef(const OpArgs<T>& a, long long pv, int co
   return (T)1 / (s * a.modtab[ph * a.c + comp] - a.ref[comp]);
 }
 
+// Component and row inside its plane of the rows of a block that starts at row rloc of
+// a system (a block may span components): one division per block, then subtractions.
+struct RowComp {
+  int rpc, comp0, off0;
+  template <typename T> __device__ __forceinline__ RowComp(const OpArgs<T>& a, int rloc)
+      : rpc(a.nz * a.ny), comp0(rloc / (a.nz * a.ny)), off0(rloc - comp0 * rpc) {}
+  __device__ __forceinline__ int row(int r, int* comp) const {
+    int off = off0 + r, c = comp0;
+    while (off >= rpc) {
+      off -= rpc;
+      ++c;
+    }
+    *comp = c;
+    return off;
+  }
+};
+
 // ------------------------------------------------------------------ x forward
 // MODE 0: input field `in` (masked by I0).  MODE 1: CG prologue.
 // Each thread handles VEC consecutive x of a row pair and writes complete
@@ -102,10 +120,11 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_xfwd(OpArgs<T
     beta = (T)st[s].beta;
   }
   const int nxv = nx / VEC;
-  const int rows_per_comp = a.nz * a.ny;
+  const FastDiv dxv(nxv), dxh(a.nxh);
+  const RowComp rc(a, rloc);
   const long long pbase = (long long)((a.sys0 + s) / a.sys_per_ms) * a.V;
   for (int idx = threadIdx.x; idx < npair * nxv; idx += blockDim.x) {
-    const int lp = fdiv(idx, nxv);
+    const int lp = dxv.div(idx);
     const int xx = (idx - lp * nxv) * VEC;
     T v0[VEC], v1[VEC];
 #pragma unroll
@@ -120,9 +139,8 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_xfwd(OpArgs<T
       const long long g = (row0 + row) * nx + xx;
       if (MODE == 0) {
         vload<T, VEC>(in + g, v);
-        const int rs = rloc + row;
-        const int comp = rs / rows_per_comp;
-        const long long vox = (long long)(rs - comp * rows_per_comp) * nx + xx;
+        int comp;
+        const long long vox = (long long)rc.row(row, &comp) * nx + xx;
 #pragma unroll
         for (int u = 0; u < VEC; ++u)
           if (!a.act[a.phase[pbase + vox + u]]) v[u] = (T)0;
@@ -151,7 +169,7 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_xfwd(OpArgs<T
   // split Z = X_a + i X_b into the two Hermitian half rows
   const T h = (T)0.5;
   for (int idx = threadIdx.x; idx < npair * a.nxh; idx += blockDim.x) {
-    const int lp = fdiv(idx, a.nxh), kx = idx - lp * a.nxh;
+    const int lp = dxh.div(idx), kx = idx - lp * a.nxh;
     const C2<T> z1 = Z[lp * a.lsx + pos[kx]];
     const C2<T> z2 = Z[lp * a.lsx + pos[kx == 0 ? 0 : nx - kx]];
     const long long hrow = row0 + 2 * lp;
@@ -174,6 +192,7 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_yfft(OpArgs<T
   const int kx0 = blockIdx.x * a.TY;
   const int nt = min(a.TY, a.nxh - kx0);
   const int TY = a.TY;
+  const FastDiv dty(TY);
   C2<T>* __restrict__ Hp = a.H + plane * a.ny * a.hs + kx0;
   const int tot = a.ny * TY;
   for (int base = threadIdx.x; base < tot; base += 4 * blockDim.x) {
@@ -181,20 +200,20 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_yfft(OpArgs<T
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int idx = base + u * blockDim.x;
-      const int y = fdiv(idx, TY), t = idx - y * TY;
+      const int y = dty.div(idx), t = idx - y * TY;
       if (idx < tot && t < nt) v[u] = Hp[(long long)y * a.hs + t];
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int idx = base + u * blockDim.x;
-      const int y = fdiv(idx, TY), t = idx - y * TY;
+      const int y = dty.div(idx), t = idx - y * TY;
       if (idx < tot && t < nt) buf[t * a.lsy + y] = v[u];
     }
   }
   __syncthreads();
   fft_lines<T, INV>(buf, nt, a.lsy, a.py, tw);
   for (int idx = threadIdx.x; idx < tot; idx += blockDim.x) {
-    const int y = fdiv(idx, TY), t = idx - y * TY;
+    const int y = dty.div(idx), t = idx - y * TY;
     if (t < nt) Hp[(long long)y * a.hs + t] = buf[t * a.lsy + y];
   }
 }
@@ -215,6 +234,7 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_zgamma(OpArgs
   const int kx0 = blockIdx.y * a.TZ;
   const int nt = min(a.TZ, a.nxh - kx0);
   const int nz = a.nz, TZ = a.TZ;
+  const FastDiv dtz(TZ), dnz(nz);
   const long long zstride = (long long)a.ny * a.hs;  // distance between z planes of H
   const long long cstride = zstride * nz;
   C2<T>* __restrict__ Hp = a.H + (long long)s * NC * cstride + (long long)yp * a.hs + kx0;
@@ -224,16 +244,16 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_zgamma(OpArgs
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int idx = base + u * blockDim.x;
-      const int rest = fdiv(idx, TZ), t = idx - rest * TZ;
-      const int comp = fdiv(rest, nz), z = rest - comp * nz;
+      const int rest = dtz.div(idx), t = idx - rest * TZ;
+      const int comp = dnz.div(rest), z = rest - comp * nz;
       v[u] = mkc<T>(0, 0);
       if (idx < tot && t < nt) v[u] = Hp[comp * cstride + z * zstride + t];
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int idx = base + u * blockDim.x;
-      const int rest = fdiv(idx, TZ), t = idx - rest * TZ;
-      const int comp = fdiv(rest, nz), z = rest - comp * nz;
+      const int rest = dtz.div(idx), t = idx - rest * TZ;
+      const int comp = dnz.div(rest), z = rest - comp * nz;
       if (idx < tot) buf[(comp * TZ + t) * a.lsz + z] = v[u];
     }
   }
@@ -242,7 +262,7 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_zgamma(OpArgs
   // per-frequency product with Gamma^h_k
   const int ky = (a.onfly || a.fdphase) ? a.kofy[yp] : 0;
   for (int idx = threadIdx.x; idx < nz * TZ; idx += blockDim.x) {
-    const int zp = fdiv(idx, TZ), t = idx - zp * TZ;
+    const int zp = dtz.div(idx), t = idx - zp * TZ;
     if (t >= nt) continue;
     C2<T> v[NC];
 #pragma unroll
@@ -260,10 +280,36 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_zgamma(OpArgs
   __syncthreads();
   if (nz > 1) fft_lines<T, true>(buf, NC * TZ, a.lsz, a.pz, tw);
   for (int idx = threadIdx.x; idx < tot; idx += blockDim.x) {
-    const int rest = fdiv(idx, TZ), t = idx - rest * TZ;
-    const int comp = fdiv(rest, nz), z = rest - comp * nz;
+    const int rest = dtz.div(idx), t = idx - rest * TZ;
+    const int comp = dnz.div(rest), z = rest - comp * nz;
     if (t < nt) Hp[comp * cstride + z * zstride + t] = buf[(comp * TZ + t) * a.lsz + z];
   }
+}
+
+// The z pass of a 2D grid: no transform, Gamma^h at every (kx, y position) of the NC
+// components in place.  The tiles of k_zgamma would leave 256 threads with the 8
+// columns of one y position (600 x 500, FP64: 287 us against 6).
+template <typename T, int NC>
+__global__ void __launch_bounds__(kThreads) k_gamma2d(OpArgs<T> a, const SolverState* __restrict__ st) {
+  const int s = blockIdx.z;
+  if (st != nullptr && st[s].done) return;
+  const int kx = blockIdx.x * blockDim.x + threadIdx.x, yp = blockIdx.y * blockDim.y + threadIdx.y;
+  if (kx >= a.nxh || yp >= a.ny) return;
+  const long long cstride = (long long)a.ny * a.hs;
+  C2<T>* __restrict__ Hp = a.H + (long long)s * NC * cstride + (long long)yp * a.hs + kx;
+  C2<T> v[NC];
+#pragma unroll
+  for (int i = 0; i < NC; ++i) v[i] = Hp[i * cstride];
+  if (a.onfly) {
+    gamma_trunc_onfly<T, NC>(a, kx, a.kofy[yp], 0, v);
+  } else {
+    const int ky = a.fdphase ? a.kofy[yp] : 0;
+    if (a.fdphase) fd_rotate<T, NC>(a, kx, ky, 0, v, (T)-1);
+    gamma_table_apply<T, NC>(a.gtab, (long long)yp * a.ts + kx, v);
+    if (a.fdphase) fd_rotate<T, NC>(a, kx, ky, 0, v, (T)1);
+  }
+#pragma unroll
+  for (int i = 0; i < NC; ++i) Hp[i * cstride] = v[i];
 }
 
 // ------------------------------------------------------------------ x inverse + local term
@@ -299,6 +345,7 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_xinv(OpArgs<T
   const C2<T>* __restrict__ Hb = a.H + row0 * a.hs;
   // Z = X_a + i X_b over the full line, X(nx - k) = conj X(k) beyond the half
   const int nz_items = npair * a.nxh;
+  const FastDiv dxh(a.nxh);
   for (int base = threadIdx.x; base < nz_items; base += 4 * blockDim.x) {
     C2<T> xa[4], xb[4];
 #pragma unroll
@@ -306,7 +353,7 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_xinv(OpArgs<T
       const int idx = base + u * blockDim.x;
       xa[u] = xb[u] = mkc<T>(0, 0);
       if (idx < nz_items) {
-        const int lp = fdiv(idx, a.nxh), kx = idx - lp * a.nxh;
+        const int lp = dxh.div(idx), kx = idx - lp * a.nxh;
         xa[u] = Hb[(2 * lp) * a.hs + kx];
         if (2 * lp + 1 < nr) xb[u] = Hb[(2 * lp + 1) * a.hs + kx];
       }
@@ -315,7 +362,7 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_xinv(OpArgs<T
     for (int u = 0; u < 4; ++u) {
       const int idx = base + u * blockDim.x;
       if (idx < nz_items) {
-        const int lp = fdiv(idx, a.nxh), kx = idx - lp * a.nxh;
+        const int lp = dxh.div(idx), kx = idx - lp * a.nxh;
         Z[lp * a.lsx + pos[kx]] = mkc<T>(xa[u].x - xb[u].y, xa[u].y + xb[u].x);
         if (kx >= 1 && kx <= nx - a.nxh) Z[lp * a.lsx + pos[nx - kx]] = mkc<T>(xa[u].x + xb[u].y, xb[u].x - xa[u].y);
       }
@@ -323,12 +370,13 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_xinv(OpArgs<T
   }
   __syncthreads();
   fft_lines<T, true>(Z, npair, a.lsx, a.px, tw);
-  const int rows_per_comp = a.nz * a.ny;
+  const RowComp rc(a, rloc);
   const long long pbase = (long long)((a.sys0 + s) / a.sys_per_ms) * a.V;
   const int nxv = nx / VEC;
+  const FastDiv dxv(nxv);
   Acc<T> acc;
   for (int idx = threadIdx.x; idx < npair * nxv; idx += blockDim.x) {
-    const int lp = fdiv(idx, nxv);
+    const int lp = dxv.div(idx);
     const int xx = (idx - lp * nxv) * VEC;
     // issue every global load of the row pair first
     T xv[2][VEC];
@@ -338,9 +386,7 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_xinv(OpArgs<T
 #pragma unroll
     for (int h2 = 0; h2 < 2; ++h2) {
       const int row = 2 * lp + h2;
-      const int rs = rloc + min(row, nr - 1);
-      comp[h2] = rs / rows_per_comp;
-      const long long vox = (long long)(rs - comp[h2] * rows_per_comp) * nx + xx;
+      const long long vox = (long long)rc.row(min(row, nr - 1), &comp[h2]) * nx + xx;
       voxs[h2] = pbase + vox;
       if (row < nr) {
         vload<T, VEC>(xin + (row0 + row) * nx + xx, xv[h2]);
@@ -1323,21 +1369,21 @@ __global__ void k_scale_grad(const double* __restrict__ tau_all, const double* _
 // ------------------------------------------------------------------ launchers
 // The attribute is a per-function upper bound shared by every handle: always
 // allow the full 227 KB so that one handle never shrinks another's limit.
+template <typename T, int VEC> void set_smem_attrs_x(int mx) {
+  cudaFuncSetAttribute(k_xfwd<T, 0, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+  cudaFuncSetAttribute(k_xfwd<T, 1, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+  cudaFuncSetAttribute(k_xinv<T, 0, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+  cudaFuncSetAttribute(k_xinv<T, 1, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+  if constexpr (sizeof(T) == 8) {
+    cudaFuncSetAttribute(k_xinv<T, 2, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+    cudaFuncSetAttribute(k_xinv<T, 3, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+  }
+}
 template <typename T> void set_smem_attrs() {
   const int mx = 227 * 1024;
-  constexpr int VV = 16 / sizeof(T);
-  cudaFuncSetAttribute(k_xinv<T, 3, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_xinv<T, 3, VV>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_xfwd<T, 0, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_xfwd<T, 1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_xfwd<T, 0, VV>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_xfwd<T, 1, VV>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_xinv<T, 0, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_xinv<T, 1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_xinv<T, 2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_xinv<T, 0, VV>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_xinv<T, 1, VV>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_xinv<T, 2, VV>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+  set_smem_attrs_x<T, 1>(mx);
+  set_smem_attrs_x<T, 2>(mx);
+  if constexpr (sizeof(T) == 4) set_smem_attrs_x<T, 4>(mx);
   cudaFuncSetAttribute(k_yfft<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
   cudaFuncSetAttribute(k_yfft<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
   cudaFuncSetAttribute(k_zgamma<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
@@ -1355,13 +1401,18 @@ void launch_xfwd(const OpArgs<T>& a, const LaunchCfg& L, int mode, const T* in, 
   }
   const int grid = a.S * a.bps;
   constexpr int VV = 16 / sizeof(T);
+#define LSH_XFWD(MODE, VEC) k_xfwd<T, MODE, VEC><<<grid, L.threads, L.smem_x, s>>>(a, in, x, r, p, st)
   if (L.VEC == VV) {
-    if (mode == 0) k_xfwd<T, 0, VV><<<grid, L.threads, L.smem_x, s>>>(a, in, x, r, p, st);
-    else k_xfwd<T, 1, VV><<<grid, L.threads, L.smem_x, s>>>(a, in, x, r, p, st);
+    if (mode == 0) LSH_XFWD(0, VV);
+    else LSH_XFWD(1, VV);
+  } else if (L.VEC == 2) {
+    if (mode == 0) LSH_XFWD(0, 2);
+    else LSH_XFWD(1, 2);
   } else {
-    if (mode == 0) k_xfwd<T, 0, 1><<<grid, L.threads, L.smem_x, s>>>(a, in, x, r, p, st);
-    else k_xfwd<T, 1, 1><<<grid, L.threads, L.smem_x, s>>>(a, in, x, r, p, st);
+    if (mode == 0) LSH_XFWD(0, 1);
+    else LSH_XFWD(1, 1);
   }
+#undef LSH_XFWD
 }
 
 template <typename T>
@@ -1396,6 +1447,12 @@ void launch_zgamma(const OpArgs<T>& a, const LaunchCfg& L, const SolverState* st
     launch_zgamma_reg<T>(a, st, s, tz);
     return;
   }
+  if (a.nz == 1 && a.c != 6) {
+    const dim3 b(32, kThreads / 32), g2((a.nxh + 31) / 32, (a.ny + b.y - 1) / b.y, a.S);
+    if (a.c == 3) k_gamma2d<T, 3><<<g2, b, 0, s>>>(a, st);
+    else k_gamma2d<T, 2><<<g2, b, 0, s>>>(a, st);
+    return;
+  }
   dim3 g(a.S, L.grid_zx, L.grid_zy);
   if (a.c == 6) k_zgamma<T, 6><<<g, L.threads, L.smem_z, s>>>(a, st);
   else if (a.c == 3) k_zgamma<T, 3><<<g, L.threads, L.smem_z, s>>>(a, st);
@@ -1411,17 +1468,21 @@ void launch_xinv(const OpArgs<T>& a, const LaunchCfg& L, int mode, const T* xin,
   }
   const int grid = a.S * a.bps;
   constexpr int VV = 16 / sizeof(T);
-  if (L.VEC == VV) {
-    if (mode == 0) k_xinv<T, 0, VV><<<grid, L.threads, L.smem_x, s>>>(a, xin, out, st, partials);
-    else if (mode == 1) k_xinv<T, 1, VV><<<grid, L.threads, L.smem_x, s>>>(a, xin, out, st, partials);
-    else if (mode == 3) k_xinv<T, 3, VV><<<grid, L.threads, L.smem_x, s>>>(a, xin, out, st, partials);
-    else k_xinv<T, 2, VV><<<grid, L.threads, L.smem_x, s>>>(a, xin, out, st, partials);
-  } else {
-    if (mode == 0) k_xinv<T, 0, 1><<<grid, L.threads, L.smem_x, s>>>(a, xin, out, st, partials);
-    else if (mode == 1) k_xinv<T, 1, 1><<<grid, L.threads, L.smem_x, s>>>(a, xin, out, st, partials);
-    else if (mode == 3) k_xinv<T, 3, 1><<<grid, L.threads, L.smem_x, s>>>(a, xin, out, st, partials);
-    else k_xinv<T, 2, 1><<<grid, L.threads, L.smem_x, s>>>(a, xin, out, st, partials);
-  }
+#define LSH_XINV(MODE, VEC) k_xinv<T, MODE, VEC><<<grid, L.threads, L.smem_x, s>>>(a, xin, out, st, partials)
+#define LSH_XINV_MODES(VEC)                              \
+  do {                                                   \
+    if (mode == 0) LSH_XINV(0, VEC);                     \
+    else if (mode == 1) LSH_XINV(1, VEC);                \
+    else if constexpr (sizeof(T) == 8) { /* FP64 only */ \
+      if (mode == 3) LSH_XINV(3, VEC);                   \
+      else LSH_XINV(2, VEC);                             \
+    }                                                    \
+  } while (0)
+  if (L.VEC == VV) LSH_XINV_MODES(VV);
+  else if (L.VEC == 2) LSH_XINV_MODES(2);
+  else LSH_XINV_MODES(1);
+#undef LSH_XINV_MODES
+#undef LSH_XINV
 }
 
 void launch_dot_finalize(SolverState* st, const double* partials, int nb, int S, cudaStream_t s) {

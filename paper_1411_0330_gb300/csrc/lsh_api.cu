@@ -40,29 +40,6 @@ bool getenv_flag(const char* name) {
 }
 
 // ---------------------------------------------------------------- FFT plans
-bool make_plan(int n, Plan1D* p) {
-  p->n = n;
-  p->nst = 0;
-  std::vector<int> r;
-  int m = n;
-  while (m % 8 == 0) { r.push_back(8); m /= 8; }
-  if (m % 4 == 0) { r.push_back(4); m /= 4; }
-  if (m % 2 == 0) {
-    // 8 * 2 -> 4 * 4 keeps every stage at radix >= 4 where possible
-    bool swapped = false;
-    for (auto& v : r)
-      if (v == 8) { v = 4; r.push_back(4); swapped = true; break; }
-    if (!swapped) r.push_back(2);
-    m /= 2;
-  }
-  for (int q : {3, 5, 7})
-    while (m % q == 0) { r.push_back(q); m /= q; }
-  if (m != 1 || (int)r.size() > LSH_MAX_STAGES) return false;
-  p->nst = (int)r.size();
-  for (int i = 0; i < p->nst; ++i) p->radix[i] = r[i];
-  return true;
-}
-
 // position of frequency k after the DIF stages of plan p
 int dif_position(const Plan1D& p, int k) {
   int pos = 0, kk = k, L = p.n;
@@ -191,7 +168,7 @@ lsh_status derive(const lsh_problem* pr, Derived* d) {
   if (pr->scale_kind != 0 && pr->scale_kind != 1) return LSH_ERR_INVALID_ARG;
   d->frac = d->has_scale && pr->scale_kind == 1;
   if (d->frac && pr->nphase != 2) return LSH_ERR_INVALID_ARG;
-  if (!make_plan(d->nx, &d->px) || !make_plan(d->ny, &d->py) || !make_plan(d->nz, &d->pz))
+  if (!lsh_make_plan(d->nx, &d->px) || !lsh_make_plan(d->ny, &d->py) || !lsh_make_plan(d->nz, &d->pz))
     return LSH_ERR_UNSUPPORTED_SIZE;
   d->plane = d->precision == LSH_MIXED && d->dim == 3 && d->nx == d->ny && plane_length(d->nx) &&
              (reg_length(d->nz) || d->nz == 48 || d->nz == 96) && !getenv_flag("LSH_NO_PLANE");
@@ -351,9 +328,15 @@ template <typename T> LaunchCfg make_cfg(const Derived& d) {
   const int lsx = d.nx | 1, lsy = d.ny | 1, lsz = d.nz | 1;
   const int rps = d.c * d.nz * d.ny;
   L.RY = choose_ry(rps, lsx, cs, d.Smax);
-  L.VEC = (d.nx % (16 / (int)sizeof(T)) == 0) ? 16 / (int)sizeof(T) : 1;
+  L.VEC = (d.nx % (16 / (int)sizeof(T)) == 0) ? 16 / (int)sizeof(T) : (d.nx % 2 == 0 ? 2 : 1);
   L.smem_x = d.nx * cs + (size_t)((L.RY + 1) / 2) * lsx * cs + d.nx * sizeof(int);
-  L.TY = std::min(sizeof(T) == 8 ? 8 : 16, d.nxh);
+  // y columns per block: up to 16 (8 in FP64), fewer where that leaves too few blocks,
+  // evenly shared among the blocks of a plane
+  int TY = std::min(sizeof(T) == 8 ? 8 : 16, d.nxh);
+  const long long planes = (long long)d.Smax * d.c * d.nz;
+  while (TY > 2 && planes * ((d.nxh + TY - 1) / TY) < 608) TY /= 2;
+  const int nty = (d.nxh + TY - 1) / TY;
+  L.TY = (d.nxh + nty - 1) / nty;
   L.smem_y = d.ny * cs + (size_t)L.TY * lsy * cs;
   int TZ = std::min(8, d.nxh);
   while (TZ > 1 && (size_t)d.c * TZ * lsz * cs > 100 * 1024) TZ /= 2;
@@ -1607,25 +1590,33 @@ lsh_status lsh_apply(lsh_handle* h, int dtype, const void* x, void* y) {
       if (el) launch_rotate<TT>(in, out, d.V, S, to_internal, h->stream);
       else launch_rotate_scalar<TT>(in, out, d.V, S, d.c, d.R, to_internal, h->stream);
     };
+    // the passes move fields in pieces of up to 16 bytes: caller buffers that start
+    // between go through the handle's own
+    auto unaligned = [](const void* p, const void* q) { return (((uintptr_t)p | (uintptr_t)q) & 15) != 0; };
     if (dtype != LSH_F32) {
       PrecBufs<double>& P = h->pd;
       const double* in = (const double*)x + b0 * n;
       double* o = (double*)y + b0 * n;
+      const bool stage = !rot && unaligned(in, o);
       if (rot) {
         rotate(in, P.p, 1);
         in = P.p;
+      } else if (stage) {
+        LSH_CK(cudaMemcpyAsync(P.p, in, sizeof(double) * (size_t)(S * n), cudaMemcpyDeviceToDevice, h->stream));
+        in = P.p;
       }
-      lsh_status s = dtype == LSH_F64_DF ? apply_df(h, wave_args<double>(h, w), in, rot ? P.q : o)
-                                         : apply_internal<double>(h, wave_args<double>(h, w), in, rot ? P.q : o);
+      double* to = rot || stage ? P.q : o;
+      lsh_status s = dtype == LSH_F64_DF ? apply_df(h, wave_args<double>(h, w), in, to)
+                                         : apply_internal<double>(h, wave_args<double>(h, w), in, to);
       if (s) return s;
       if (rot) rotate((const double*)P.q, o, 0);
+      else if (stage)
+        LSH_CK(cudaMemcpyAsync(o, P.q, sizeof(double) * (size_t)(S * n), cudaMemcpyDeviceToDevice, h->stream));
     } else {
       PrecBufs<float>& P = h->pf;
       const float* in = (const float*)x + b0 * n;
       float* o = (float*)y + b0 * n;
-      // the plane passes move fields in 16-byte pieces: unaligned caller buffers
-      // go through the handle's own
-      const bool stage = !rot && P.a.plane && (((uintptr_t)in | (uintptr_t)o) & 15) != 0;
+      const bool stage = !rot && unaligned(in, o);
       if (rot) {
         rotate(in, P.p, 1);
         in = P.p;

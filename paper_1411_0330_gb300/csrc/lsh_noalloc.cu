@@ -32,6 +32,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <cstdint>
 #include <mutex>
 
 #include "internal.h"
@@ -67,28 +68,6 @@ lsh_status scratch_address(void** out) {
   }
   *out = g_ptr[dev];
   return LSH_OK;
-}
-
-bool plan_axis(int n, Plan1D* p) {
-  int r[LSH_MAX_STAGES * 4];
-  int k = 0, m = n;
-  while (m % 8 == 0 && k < 32) { r[k++] = 8; m /= 8; }
-  if (m % 4 == 0) { r[k++] = 4; m /= 4; }
-  if (m % 2 == 0) {
-    bool swapped = false;
-    for (int i = 0; i < k; ++i)
-      if (r[i] == 8) { r[i] = 4; r[k++] = 4; swapped = true; break; }
-    if (!swapped) r[k++] = 2;
-    m /= 2;
-  }
-  const int qs[3] = {3, 5, 7};
-  for (int qi = 0; qi < 3; ++qi)
-    while (m % qs[qi] == 0 && k < 32) { r[k++] = qs[qi]; m /= qs[qi]; }
-  if (m != 1 || k > LSH_MAX_STAGES) return false;
-  p->n = n;
-  p->nst = k;
-  for (int i = 0; i < k; ++i) p->radix[i] = r[i];
-  return true;
 }
 
 // Twiddles exp(-2 i pi t / n), DIF positions of x frequencies, frequencies of
@@ -145,7 +124,7 @@ extern "C" lsh_status lsh_apply_noalloc(const lsh_problem* pr, const double* x, 
   const int c = el ? 6 : dim, ncoef = c * (c + 1) / 2, nxh = nx / 2 + 1;
   const long long V = (long long)nx * ny * nz;
   Plan1D px, py, pz;
-  if (!plan_axis(nx, &px) || !plan_axis(ny, &py) || !plan_axis(nz, &pz)) return LSH_ERR_UNSUPPORTED_SIZE;
+  if (!lsh_make_plan(nx, &px) || !lsh_make_plan(ny, &py) || !lsh_make_plan(nz, &pz)) return LSH_ERR_UNSUPPORTED_SIZE;
 
   // reference medium and per-phase diagonal tables in the internal basis
   double ref_user[6] = {0, 0, 0, 0, 0, 0}, ref_in[6] = {0, 0, 0, 0, 0, 0};
@@ -232,7 +211,7 @@ extern "C" lsh_status lsh_apply_noalloc(const lsh_problem* pr, const double* x, 
   LaunchCfg L{};
   L.threads = 256;
   L.RY = RY;
-  L.VEC = (nx % 2 == 0) ? 2 : 1;
+  L.VEC = (nx % 2 == 0 && (((uintptr_t)x | (uintptr_t)y) & 15) == 0) ? 2 : 1;
   L.smem_x = nx * cs + (size_t)((RY + 1) / 2) * lsx * cs + nx * sizeof(int);
   L.TY = std::min(8, nxh);
   L.smem_y = ny * cs + (size_t)L.TY * lsy * cs;
