@@ -4,6 +4,8 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace lsh {
@@ -51,6 +53,14 @@ template <typename T> struct OpArgs {
   // holds z = D r, so that p = z + beta p needs no phase map.
   int pre;
   const T* dtab;               // per phase * c: D (1 outside I0)
+  const T* etab;               // per phase * c: 1 / D
+  // per-voxel local operator of handles with a scale or fraction field, formed once when
+  // the field is set (a division per voxel instead of one per voxel, component, system
+  // and pass): M, and D in FP64; [class][nbatch * V], class 0 / 1 the spherical /
+  // deviatoric components of elasticity, else the component.  Null: formed where used.
+  const T* mfld;
+  const T* dfld;
+  long long fstride;           // nbatch * V
   T gpre[6];                   // share of the diagonal of the Green operator, per component
   const T* loads;              // [S][6] macroscopic load per system (internal basis)
   // Green operator computed in the z pass instead of read from gtab (truncated
@@ -96,12 +106,95 @@ template <typename T> struct OpArgs {
 
 // Thread-block sizes and tile shapes, chosen at setup for one system count.
 struct LaunchCfg {
-  int threads;
+  int thr_x, thr_y, thr_z;  // threads per block of the shared-memory x, y and z passes
   int RY, TY, TZ, VEC;
   size_t smem_x, smem_y, smem_z;
   int grid_x, grid_yx, grid_yy, grid_zx, grid_zy, grid_zz;
   int ew_per_sys;  // blocks per system of the elementwise kernels
 };
+
+// Threads per block of a shared-memory pass over nlines lines of plan p, `blocks` of them
+// in the launch: the largest number of blocks in flight per SM over the time of one,
+// where a stage of radix R takes ceil(butterflies / threads) rounds of R values.  Larger
+// radices leave few butterflies per block, and 256 threads for 56 of them hold the
+// registers of 200 idle ones.
+inline int pass_threads(int nlines, const Plan1D& p, size_t smem, int max_resident, long long blocks) {
+  int best = 256;
+  double best_rate = 0.0;
+  const long long share = (blocks + 151) / 152;  // blocks an SM gets
+  for (int t = 256; t >= 64; t -= 32) {
+    const long long fit = std::min<long long>(
+        {32LL, (long long)(max_resident / t), (long long)(226 * 1024 / (smem + 1024)), share});
+    if (fit < 1) continue;
+    const long long pts = (long long)nlines * p.n;
+    double time = 8.0 + 2.0 * 4.0 * (double)((pts / 4 + t) / t);  // barriers; loads and stores, four in flight
+    for (int s = 0; s < p.nst; ++s) time += (double)p.radix[s] * (double)((pts / p.radix[s] + t - 1) / t);
+    const double rate = (double)fit / time;
+    if (rate > best_rate * 1.02) {
+      best_rate = rate;
+      best = t;
+    }
+  }
+  return best;
+}
+
+// Tiles and block sizes of the shared-memory passes for S systems: blocks of about 32 KB,
+// fewer lines where that would leave the 152 SMs without some four blocks each (two for
+// the FP32 x passes, whose tables and barriers cost more than the idle SMs).
+template <typename T>
+LaunchCfg pass_cfg(int nx, int ny, int nz, int c, const Plan1D& px, const Plan1D& py, const Plan1D& pz, int S) {
+  LaunchCfg L{};
+  const size_t cs = sizeof(C2<T>);
+  const int nxh = nx / 2 + 1, lsx = nx | 1, lsy = ny | 1, lsz = nz | 1;
+  const int rps = c * nz * ny;
+  const int resident = sizeof(T) == 8 ? 512 : 768;  // threads per SM at the passes' register counts
+  constexpr long long kBlocks = 608;                // four per SM
+  // rows per x block: an even divisor of the rows of a system where there is one
+  int target = std::max(2, 2 * (int)(32768 / (lsx * cs)));
+  target = std::min(target, std::max(2, (int)((long long)rps * S / (sizeof(T) == 4 ? kBlocks / 2 : kBlocks))));
+  if (target >= rps) {
+    L.RY = rps;
+  } else {
+    int odd = 1;
+    L.RY = 0;
+    for (int d = target; d >= 1 && !L.RY; --d)
+      if (rps % d == 0) {
+        if (d % 2 == 0) L.RY = d;
+        else if (odd == 1) odd = d;
+      }
+    if (!L.RY) L.RY = odd;
+  }
+  constexpr int VV = 16 / (int)sizeof(T);
+  L.VEC = nx % VV == 0 ? VV : (nx % 2 == 0 ? 2 : 1);
+  const int npair = (L.RY + 1) / 2;
+  L.smem_x = nx * cs + (size_t)npair * lsx * cs + nx * sizeof(int);
+  // the FP32 x passes stream three fields in and two out: the loads want every thread; the
+  // lengths with a compile-time schedule are bound by the FP64 pipe at any block size
+  const bool fixed = nx == 16 || nx == 32 || nx == 48 || nx == 64 || nx == 96 || nx == 128 || nx == 256;
+  L.thr_x = sizeof(T) == 4 || fixed ? 256 : pass_threads(npair, px, L.smem_x, resident, (long long)S * (rps / L.RY));
+  // y columns per block: up to 16 (8 in FP64), evenly shared among a plane's blocks
+  int TY = std::min(sizeof(T) == 8 ? 8 : 16, nxh);
+  while (TY > 2 && (long long)S * c * nz * ((nxh + TY - 1) / TY) < kBlocks) TY /= 2;
+  const int nty = (nxh + TY - 1) / TY;
+  L.TY = (nxh + nty - 1) / nty;
+  L.smem_y = ny * cs + (size_t)L.TY * lsy * cs;
+  L.thr_y = pass_threads(L.TY, py, L.smem_y, resident, (long long)S * c * nz * nty);
+  // z columns per block (32-byte segments at least)
+  int TZ = std::min(8, nxh);
+  while (TZ > 1 && (size_t)c * TZ * lsz * cs > 100 * 1024) TZ /= 2;
+  while (TZ > 32 / (int)cs && (long long)S * ny * ((nxh + TZ - 1) / TZ) < kBlocks) TZ /= 2;
+  L.TZ = TZ;
+  L.smem_z = nz * cs + (size_t)c * TZ * lsz * cs;
+  L.thr_z = pass_threads(c * TZ, pz, L.smem_z, resident, (long long)S * ny * ((nxh + TZ - 1) / TZ));
+  L.grid_x = rps / L.RY;  // per system
+  L.grid_yx = nty;
+  L.grid_yy = c * nz;  // per system
+  L.grid_zx = (nxh + TZ - 1) / TZ;
+  L.grid_zy = ny;
+  const long long n = (long long)rps * nx, want = (n + 2047) / 2048;
+  L.ew_per_sys = (int)std::max(1LL, std::min(want, std::max(1LL, 2432LL / S)));
+  return L;
+}
 
 template <typename T>
 void launch_xfwd(const OpArgs<T>& a, const LaunchCfg& L, int mode, const T* in, T* x, const T* r, T* p,
@@ -134,6 +227,7 @@ void launch_gamma_table(const OpArgs<T>& a, int dim, int physics, int green, con
 template <typename T>
 void launch_rotate_scalar(const T* in, T* out, long long V, int nsys, int d, const double* R, int to_internal,
                           cudaStream_t s);
+template <typename T> void launch_voxel_fields(const OpArgs<T>& a, T* mfld, T* dfld, int B, cudaStream_t s);
 void launch_gamma_diag(const OpArgs<double>& a, double* partials, int nblk, double* out, cudaStream_t s);
 void launch_d2f_begin(const OpArgs<float>& a, const double* r64, bool df_pairs, float* r32, float* x32, SolverState* st,
                       double* partials, long long off2, double tol, const unsigned char* active, int G,

@@ -61,12 +61,17 @@ template <typename T, int VEC> __device__ __forceinline__ void vstore(T* __restr
   }
 }
 
+template <typename T> __device__ __forceinline__ int field_class(const OpArgs<T>& a, int comp) {
+  return a.physics != 0 ? (comp > 0) : comp;
+}
+
 // Local coefficient m = (A_beta - A0)^{-1} of component `comp` at voxel index
 // `pv` of the stacked phase map; *active = voxel in I0.
 template <typename T>
 __device__ __forceinline__ T local_coef(const OpArgs<T>& a, long long pv, int comp, int* active) {
   const int ph = a.phase[pv];
   *active = a.act[ph];
+  if (a.mfld) return a.mfld[field_class(a, comp) * a.fstride + pv];
   if (a.scale == nullptr) return a.mtab[ph * a.c + comp];
   const T s = (T)a.scale[pv];
   return (T)1 / (s * a.modtab[ph * a.c + comp] - a.ref[comp]);
@@ -415,7 +420,9 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_xinv(OpArgs<T
         const int p = ph[h2][u];
         const bool active = aloc[p] != 0;
         T m = mloc[p * a.c + comp[h2]];
-        if (a.scale) {
+        if (a.mfld) {
+          m = a.mfld[field_class(a, comp[h2]) * a.fstride + voxs[h2] + u];
+        } else if (a.scale) {
           const T f = (T)a.scale[voxs[h2] + u];
           m = a.frac ? f * mloc[a.c + comp[h2]] + ((T)1 - f) * mloc[comp[h2]]  // Eq. (def_ah)
                      : (T)1 / (f * m - a.ref[comp[h2]]);
@@ -785,16 +792,17 @@ template <typename T, typename F> __device__ __forceinline__ void sweep_planes(i
 // FP32 iterations to 5e-6 (and 1e-10), 32^3 spheres at f = 0.3: contrast 10
 // truncated 46 (88) -> 22 (39), filtered 38 (75) -> 24 (46); contrast 1000
 // truncated 415 (850) -> 223 (400), filtered 116 (232) -> 72 (144).
+// *e = 1 / D.
 template <typename T, int PRE>
-__device__ __forceinline__ T precond(const OpArgs<T>& a, const T* __restrict__ dloc, int comp, int ph, long long pv) {
-  if constexpr (PRE == 1) return dloc[ph * a.c + comp];
-  const T f = (T)a.scale[pv];
-  if (a.frac) {
-    const T m = f * a.mtab[a.c + comp] + ((T)1 - f) * a.mtab[comp];  // Eq. (def_ah)
-    return (T)1 / (fabs(m) + a.gpre[comp]);
+__device__ __forceinline__ T precond(const OpArgs<T>& a, const T* __restrict__ dloc, const T* __restrict__ eloc,
+                                     int comp, int ph, long long pv, T* e) {
+  if constexpr (PRE == 1) {
+    *e = eloc[ph * a.c + comp];
+    return dloc[ph * a.c + comp];
   }
-  const T d = fabs(f * a.modtab[ph * a.c + comp] - a.ref[comp]);
-  return a.gpre[comp] == (T)0 ? d : d / ((T)1 + a.gpre[comp] * d);
+  const long long at = field_class(a, comp) * a.fstride + pv;
+  *e = fabs(a.mfld[at]) + a.gpre[comp];
+  return sizeof(T) == 8 ? a.dfld[at] : (T)1 / *e;
 }
 
 template <int VEC> __device__ __forceinline__ void phase_load(const unsigned char* __restrict__ p, int* ph) {
@@ -818,9 +826,12 @@ __global__ void __launch_bounds__(kThreads) k_cg_update(OpArgs<T> a, T* __restri
   const int s = blockIdx.y;
   SolverState* sst = st + s;
   if (sst->done) return;
-  __shared__ T dloc[PRE == 1 ? 256 * 6 : 1];
+  __shared__ T dloc[PRE == 1 ? 256 * 6 : 1], eloc[PRE == 1 ? 256 * 6 : 1];
   if (PRE == 1) {
-    for (int i = threadIdx.x; i < a.nphase * a.c; i += blockDim.x) dloc[i] = a.dtab[i];
+    for (int i = threadIdx.x; i < a.nphase * a.c; i += blockDim.x) {
+      dloc[i] = a.dtab[i];
+      eloc[i] = a.etab[i];
+    }
     __syncthreads();
   }
   const T al = (T)sst->alpha;
@@ -844,9 +855,10 @@ __global__ void __launch_bounds__(kThreads) k_cg_update(OpArgs<T> a, T* __restri
         rv[u] -= al * qv[u];
         acc.add(rv[u] * rv[u]);
       } else {
-        const T d = precond<T, PRE>(a, dloc, comp, ph[u], pbase + i + u);
+        T e;
+        const T d = precond<T, PRE>(a, dloc, eloc, comp, ph[u], pbase + i + u, &e);
         rv[u] -= al * (d * qv[u]);
-        const T ru = rv[u] / d;
+        const T ru = rv[u] * e;
         acc.add(ru * ru);
         accz.add(ru * rv[u]);
       }
@@ -914,7 +926,8 @@ __global__ void __launch_bounds__(kThreads) k_cg_begin(OpArgs<T> a, T* __restric
     for (int u = 0; u < VEC; ++u) {
       acc.add(rv[u] * rv[u]);
       if constexpr (PRE != 0) {
-        const T z = precond<T, PRE>(a, a.dtab, comp, ph[u], pbase + i + u) * rv[u];
+        T e;
+        const T z = precond<T, PRE>(a, a.dtab, a.etab, comp, ph[u], pbase + i + u, &e) * rv[u];
         accz.add(z * rv[u]);
         rv[u] = z;
       }
@@ -1228,17 +1241,14 @@ __global__ void __launch_bounds__(kThreads) k_d2f_begin(OpArgs<float> a, const d
       zero[u] = 0.0f;
       acc.add(v[u] * v[u]);
       if constexpr (PRE != 0) {
-        const float z = precond<float, PRE>(a, a.dtab, comp, ph[u], pbase + i + u) * v[u];
+        float e;
+        const float z = precond<float, PRE>(a, a.dtab, a.etab, comp, ph[u], pbase + i + u, &e) * v[u];
         accz.add(z * v[u]);
         v[u] = z;
       }
       if (zmz) {
         int active;
-        float m = local_coef<float>(a, pbase + i + u, comp, &active);
-        if (a.frac) {
-          const float f = a.scale[pbase + i + u];
-          m = f * a.mtab[a.c + comp] + (1.f - f) * a.mtab[comp];
-        }
+        const float m = local_coef<float>(a, pbase + i + u, comp, &active);
         accm.add(m * v[u] * v[u]);
       }
     }
@@ -1269,6 +1279,22 @@ __global__ void __launch_bounds__(kThreads) k_d2f_begin(OpArgs<float> a, const d
       sst->status = 0;
       sst->done = (!active[s] || rr <= sst->tol2) ? 1 : 0;
     }
+  }
+}
+
+// M (and D) of every voxel of a handle with a scale or fraction field, per class of
+// components (see OpArgs): grid (G, classes).
+template <typename T>
+__global__ void __launch_bounds__(kThreads) k_voxel_fields(OpArgs<T> a, T* __restrict__ mfld, T* __restrict__ dfld) {
+  const int cls = blockIdx.y;  // also the first component of the class
+  const double g = (double)a.gpre[cls];
+  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < a.fstride;
+       v += (long long)gridDim.x * blockDim.x) {
+    const T f = (T)a.scale[v];
+    const T m = a.frac ? f * a.mtab[a.c + cls] + ((T)1 - f) * a.mtab[cls]  // Eq. (def_ah)
+                       : (T)1 / (f * a.modtab[a.phase[v] * a.c + cls] - a.ref[cls]);
+    mfld[cls * a.fstride + v] = m;
+    if (dfld) dfld[cls * a.fstride + v] = (T)(1.0 / (fabs((double)m) + g));
   }
 }
 
@@ -1401,7 +1427,7 @@ void launch_xfwd(const OpArgs<T>& a, const LaunchCfg& L, int mode, const T* in, 
   }
   const int grid = a.S * a.bps;
   constexpr int VV = 16 / sizeof(T);
-#define LSH_XFWD(MODE, VEC) k_xfwd<T, MODE, VEC><<<grid, L.threads, L.smem_x, s>>>(a, in, x, r, p, st)
+#define LSH_XFWD(MODE, VEC) k_xfwd<T, MODE, VEC><<<grid, L.thr_x, L.smem_x, s>>>(a, in, x, r, p, st)
   if (L.VEC == VV) {
     if (mode == 0) LSH_XFWD(0, VV);
     else LSH_XFWD(1, VV);
@@ -1429,8 +1455,8 @@ void launch_yfft(const OpArgs<T>& a, const LaunchCfg& L, bool inv, const SolverS
     return;
   }
   dim3 g(L.grid_yx, a.S * a.c * a.nz);
-  if (inv) k_yfft<T, true><<<g, L.threads, L.smem_y, s>>>(a, st);
-  else k_yfft<T, false><<<g, L.threads, L.smem_y, s>>>(a, st);
+  if (inv) k_yfft<T, true><<<g, L.thr_y, L.smem_y, s>>>(a, st);
+  else k_yfft<T, false><<<g, L.thr_y, L.smem_y, s>>>(a, st);
 }
 
 template <typename T>
@@ -1454,9 +1480,9 @@ void launch_zgamma(const OpArgs<T>& a, const LaunchCfg& L, const SolverState* st
     return;
   }
   dim3 g(a.S, L.grid_zx, L.grid_zy);
-  if (a.c == 6) k_zgamma<T, 6><<<g, L.threads, L.smem_z, s>>>(a, st);
-  else if (a.c == 3) k_zgamma<T, 3><<<g, L.threads, L.smem_z, s>>>(a, st);
-  else k_zgamma<T, 2><<<g, L.threads, L.smem_z, s>>>(a, st);
+  if (a.c == 6) k_zgamma<T, 6><<<g, L.thr_z, L.smem_z, s>>>(a, st);
+  else if (a.c == 3) k_zgamma<T, 3><<<g, L.thr_z, L.smem_z, s>>>(a, st);
+  else k_zgamma<T, 2><<<g, L.thr_z, L.smem_z, s>>>(a, st);
 }
 
 template <typename T>
@@ -1468,7 +1494,7 @@ void launch_xinv(const OpArgs<T>& a, const LaunchCfg& L, int mode, const T* xin,
   }
   const int grid = a.S * a.bps;
   constexpr int VV = 16 / sizeof(T);
-#define LSH_XINV(MODE, VEC) k_xinv<T, MODE, VEC><<<grid, L.threads, L.smem_x, s>>>(a, xin, out, st, partials)
+#define LSH_XINV(MODE, VEC) k_xinv<T, MODE, VEC><<<grid, L.thr_x, L.smem_x, s>>>(a, xin, out, st, partials)
 #define LSH_XINV_MODES(VEC)                              \
   do {                                                   \
     if (mode == 0) LSH_XINV(0, VEC);                     \
@@ -1590,6 +1616,10 @@ void launch_d2f_begin(const OpArgs<float>& a, const double* r64, bool df_pairs, 
   else { if (df_pairs) LSH_D2F(true, 2); else LSH_D2F(false, 2); }
 #undef LSH_D2F
 }
+template <typename T> void launch_voxel_fields(const OpArgs<T>& a, T* mfld, T* dfld, int B, cudaStream_t s) {
+  const int G = (int)std::max(1LL, std::min((B * a.V + kThreads - 1) / kThreads, 152LL * 8));
+  k_voxel_fields<T><<<dim3(G, a.physics != 0 ? 2 : a.c), kThreads, 0, s>>>(a, mfld, dfld);
+}
 void launch_gamma_diag(const OpArgs<double>& a, double* partials, int nblk, double* out, cudaStream_t s) {
   k_gamma_diag<<<dim3(nblk, a.c), kThreads, 0, s>>>(a, partials);
   k_comp_final<<<a.c, kThreads, 0, s>>>(partials, nblk, out);
@@ -1627,6 +1657,7 @@ void launch_scale_grad(const double* tau_all, const double* W, const unsigned ch
   template void launch_comp_sums<T>(const T*, int, long long, int, double*, int, double*, cudaStream_t);           \
   template void launch_gamma_table<T>(const OpArgs<T>&, int, int, int, const double*, const int*, const int*,      \
                                       cudaStream_t, const double*, const double*);                                 \
+  template void launch_voxel_fields<T>(const OpArgs<T>&, T*, T*, int, cudaStream_t);                               \
   template void launch_rotate_scalar<T>(const T*, T*, long long, int, int, const double*, int, cudaStream_t);
 
 LSH_INSTANTIATE(double)

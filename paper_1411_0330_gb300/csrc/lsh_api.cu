@@ -307,50 +307,8 @@ lsh_status derive(const lsh_problem* pr, Derived* d) {
 }
 
 // ---------------------------------------------------------------- launch configuration
-int choose_ry(int rps, int lsx, size_t cs, int S) {
-  int target = std::max(2, 2 * (int)(32768 / (lsx * cs)));
-  // keep at least ~4 blocks per SM in flight for small problems
-  target = std::min(target, std::max(2, (int)((long long)rps * S / 608)));
-  if (target >= rps) return rps;
-  int best = 1;
-  for (int d = target; d >= 1; --d)
-    if (rps % d == 0) {
-      if (d % 2 == 0) return d;
-      if (best == 1) best = d;
-    }
-  return best;
-}
-
-template <typename T> LaunchCfg make_cfg(const Derived& d) {
-  LaunchCfg L{};
-  L.threads = kThreads;
-  const size_t cs = sizeof(C2<T>);
-  const int lsx = d.nx | 1, lsy = d.ny | 1, lsz = d.nz | 1;
-  const int rps = d.c * d.nz * d.ny;
-  L.RY = choose_ry(rps, lsx, cs, d.Smax);
-  L.VEC = (d.nx % (16 / (int)sizeof(T)) == 0) ? 16 / (int)sizeof(T) : (d.nx % 2 == 0 ? 2 : 1);
-  L.smem_x = d.nx * cs + (size_t)((L.RY + 1) / 2) * lsx * cs + d.nx * sizeof(int);
-  // y columns per block: up to 16 (8 in FP64), fewer where that leaves too few blocks,
-  // evenly shared among the blocks of a plane
-  int TY = std::min(sizeof(T) == 8 ? 8 : 16, d.nxh);
-  const long long planes = (long long)d.Smax * d.c * d.nz;
-  while (TY > 2 && planes * ((d.nxh + TY - 1) / TY) < 608) TY /= 2;
-  const int nty = (d.nxh + TY - 1) / TY;
-  L.TY = (d.nxh + nty - 1) / nty;
-  L.smem_y = d.ny * cs + (size_t)L.TY * lsy * cs;
-  int TZ = std::min(8, d.nxh);
-  while (TZ > 1 && (size_t)d.c * TZ * lsz * cs > 100 * 1024) TZ /= 2;
-  L.TZ = TZ;
-  L.smem_z = d.nz * cs + (size_t)d.c * TZ * lsz * cs;
-  L.grid_x = rps / L.RY;  // per system
-  L.grid_yx = (d.nxh + L.TY - 1) / L.TY;
-  L.grid_yy = d.c * d.nz;  // per system
-  L.grid_zx = (d.nxh + TZ - 1) / TZ;
-  L.grid_zy = d.ny;
-  const long long n = (long long)d.c * d.V;
-  const long long want = (n + kThreads * 8 - 1) / (kThreads * 8);
-  L.ew_per_sys = (int)std::max(1LL, std::min(want, std::max(1LL, 2432LL / d.Smax)));
-  return L;
+template <typename T> LaunchCfg make_cfg(const Derived& d, int S) {
+  return pass_cfg<T>(d.nx, d.ny, d.nz, d.c, d.px, d.py, d.pz, S);
 }
 
 bool cfg_fits(const LaunchCfg& L) {
@@ -369,6 +327,7 @@ struct Layout {
   size_t off_ff[4], off_Hf, off_gf;
   size_t off_wa, off_wb, off_ms;  // MINRES: two direction fields (FP64) and per-system scalars
   size_t off_gdf, off_twdf;       // double-float Gamma table and twiddles (mixed handles)
+  size_t off_mfd, off_mff;        // per-voxel local operator (handles with a voxel field)
   size_t off_nq;                  // FP32 Nyquist columns of the plane passes
   size_t off_kofy32, off_kofz32;  // frequency of each y / z position in the FP32 spectrum
   bool df;                        // double-float residual passes available
@@ -403,16 +362,19 @@ Layout make_layout(const Derived& d) {
   const long long n = (long long)d.c * d.V;  // elements per system
   const long long nf = (long long)d.nz * d.ny * d.ts;    // Gamma table frequencies (rows padded to ts)
   const long long nfh = (long long)d.nz * d.ny * d.hs;  // half spectrum per component
-  LaunchCfg Ld = make_cfg<double>(d), Lf = make_cfg<float>(d);
-  long long np = std::max<long long>({(long long)S * Ld.grid_x, (long long)S * Lf.grid_x, (long long)S * Ld.ew_per_sys,
-                                      (long long)S * Lf.ew_per_sys, (long long)S * d.c * 152,
-                                      (long long)d.B * 1216, (long long)S * (rps_of(d) / 2 + 1),
+  // block partials: x passes have at most one block per row (two rows where their number
+  // is even), the elementwise kernels 2432 blocks or one per system
+  const long long xblocks = rps_of(d) % 2 == 0 ? rps_of(d) / 2 + 1 : rps_of(d);
+  long long np = std::max<long long>({2432LL + S, (long long)S * d.c * 152, (long long)d.B * 1216, (long long)S * xblocks,
                                       (long long)S * d.c * d.nz});
   l.nparts = np;
   l.off_state = take(sizeof(SolverState) * (size_t)(3 * S + d.B));
   l.off_partials = take(sizeof(double) * 4 * (size_t)np);  // up to four sums per block
   l.off_phase = take((size_t)(d.B * d.V));
   l.off_scale = take(d.has_scale ? sizeof(float) * (size_t)(d.B * d.V) : 0);
+  const long long nfield = (d.physics == LSH_ELASTIC_ISO ? 2LL : d.c) * d.B * d.V;  // per-voxel M (and D)
+  l.off_mfd = take(d.has_scale ? sizeof(double) * 2 * (size_t)nfield : 0);
+  l.off_mff = take(d.has_scale && d.precision == LSH_MIXED ? sizeof(float) * (size_t)nfield : 0);
   l.off_act = take(256);
   l.off_posx = take(sizeof(int) * d.nx);
   l.off_kofy = take(sizeof(int) * d.ny);
@@ -421,8 +383,8 @@ Layout make_layout(const Derived& d) {
   l.off_kofz32 = take(sizeof(int) * d.nz);
   l.off_sums = take(sizeof(double) * (size_t)S * d.c);
   l.off_W = take(sizeof(double) * 64);
-  l.off_tabd = take(sizeof(double) * 3 * 256 * 6);
-  l.off_tabf = take(sizeof(float) * 3 * 256 * 6);
+  l.off_tabd = take(sizeof(double) * 4 * 256 * 6);
+  l.off_tabf = take(sizeof(float) * 4 * 256 * 6);
   l.off_loads_d = take(sizeof(double) * 6 * (size_t)S);
   l.off_loads_f = take(sizeof(float) * 6 * (size_t)S);
   l.off_bb = take(sizeof(double) * (size_t)S);
@@ -575,7 +537,7 @@ void init_prec(lsh_handle* h, PrecBufs<T>& P, const size_t* off_f, size_t off_H,
   P.modtab = P.mtab + 256 * 6;
   P.loads = (T*)(b + off_loads);
   P.st = st;
-  P.L = make_cfg<T>(d);
+  P.L = make_cfg<T>(d, d.Smax);
   OpArgs<T>& a = P.a;
   a.nx = d.nx;
   a.ny = d.ny;
@@ -617,6 +579,13 @@ void init_prec(lsh_handle* h, PrecBufs<T>& P, const size_t* off_f, size_t off_H,
   // definite, and FP64 CG with a per-voxel field.  FP64 CG on phase maps is the plain
   // method the mixed solver is measured against.
   a.dtab = P.modtab + 256 * 6;
+  a.etab = a.dtab + 256 * 6;
+  a.mfld = a.dfld = nullptr;
+  a.fstride = (long long)d.B * d.V;
+  if (d.has_scale) {
+    a.mfld = (const T*)(b + (sizeof(T) == 8 ? h->lay.off_mfd : h->lay.off_mff));
+    if (sizeof(T) == 8) a.dfld = a.mfld + (d.physics == LSH_ELASTIC_ISO ? 2 : d.c) * a.fstride;
+  }
   a.pre = (d.definite == 0 || (sizeof(T) == 8 && !d.has_scale)) ? 0 : (d.has_scale ? 2 : 1);
   for (int i = 0; i < 6; ++i) a.gpre[i] = (T)0;
   for (int i = 0; i < 6; ++i) a.ref[i] = (T)(i < d.c ? d.ref_in[i] : 0.0);
@@ -751,6 +720,13 @@ template <typename T> OpArgs<T> wave_args(lsh_handle* h, const Wave& w) {
   a.S = w.S;
   a.sys0 = w.sys0;
   a.sys_per_ms = w.sys_per_ms;
+  // tiles for the wave's own number of systems (an apply runs one where a solve runs all)
+  LaunchCfg& L = bufs<T>(h).L;
+  L = make_cfg<T>(h->d, w.S);
+  a.RY = L.RY;
+  a.bps = a.rps / a.RY;
+  a.TY = L.TY;
+  a.TZ = L.TZ;
   return a;
 }
 
@@ -1327,6 +1303,16 @@ lsh_status scan_microstructure(lsh_handle* h) {
   return LSH_OK;
 }
 
+// per-voxel M and D from the scale (fraction) field on the device
+lsh_status set_voxel_fields(lsh_handle* h) {
+  if (!h->d.has_scale) return LSH_OK;
+  launch_voxel_fields<double>(h->pd.a, const_cast<double*>(h->pd.a.mfld), const_cast<double*>(h->pd.a.dfld), h->d.B,
+                              h->stream);
+  if (h->d.precision == LSH_MIXED)
+    launch_voxel_fields<float>(h->pf.a, const_cast<float*>(h->pf.a.mfld), nullptr, h->d.B, h->stream);
+  return last_launch();
+}
+
 lsh_status copy_microstructure(lsh_handle* h, const unsigned char* phase, const float* scale, int on_host) {
   const cudaMemcpyKind k = on_host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
   const size_t nv = (size_t)(h->d.B * h->d.V);
@@ -1380,7 +1366,7 @@ lsh_status lsh_workspace_size(const lsh_problem* prob, size_t* bytes) {
   Derived d;
   lsh_status s = derive(prob, &d);
   if (s) return s;
-  if (!cfg_fits(make_cfg<double>(d)) || !cfg_fits(make_cfg<float>(d))) return LSH_ERR_UNSUPPORTED_SIZE;
+  if (!cfg_fits(make_cfg<double>(d, d.Smax)) || !cfg_fits(make_cfg<float>(d, d.Smax))) return LSH_ERR_UNSUPPORTED_SIZE;
   *bytes = make_layout(d).total;
   return LSH_OK;
 }
@@ -1393,7 +1379,7 @@ lsh_status lsh_setup(const lsh_problem* prob, void* workspace, size_t bytes, voi
   lsh_status s = derive(prob, &h->d);
   if (s) { delete h; return s; }
   Derived& d = h->d;
-  if (!cfg_fits(make_cfg<double>(d)) || !cfg_fits(make_cfg<float>(d))) {
+  if (!cfg_fits(make_cfg<double>(d, d.Smax)) || !cfg_fits(make_cfg<float>(d, d.Smax))) {
     delete h;
     return LSH_ERR_UNSUPPORTED_SIZE;
   }
@@ -1461,8 +1447,8 @@ lsh_status lsh_setup(const lsh_problem* prob, void* workspace, size_t bytes, voi
   twiddles<double>(d.nz, tmpd); twd.insert(twd.end(), tmpd.begin(), tmpd.end());
   std::vector<float> twf(twd.size());
   for (size_t i = 0; i < twd.size(); ++i) twf[i] = (float)twd[i];
-  std::vector<double> tabd(3 * 256 * 6, 0.0);
-  std::vector<float> tabf(3 * 256 * 6, 0.0f);
+  std::vector<double> tabd(2 * 256 * 6, 0.0);
+  std::vector<float> tabf(2 * 256 * 6, 0.0f);
   for (int ph = 0; ph < d.nphase; ++ph)
     for (int i = 0; i < d.c; ++i) {
       tabd[ph * d.c + i] = d.m_in[ph * d.c + i];
@@ -1517,11 +1503,19 @@ lsh_status lsh_setup(const lsh_problem* prob, void* workspace, size_t bytes, voi
       SETUP_CK(cudaMemcpyAsync(g, h->sums, sizeof(double) * d.c, cudaMemcpyDeviceToHost, st));
       SETUP_CK(cudaStreamSynchronize(st));
     }
-    std::vector<double> dd(256 * 6, 1.0);
-    std::vector<float> df(256 * 6, 1.0f);
+    if (d.has_scale && d.physics == LSH_ELASTIC_ISO) {
+      // the per-voxel fields hold one value for all deviatoric components
+      const double mean = (g[1] + g[2] + g[3] + g[4] + g[5]) / 5.0;
+      for (int i = 1; i < 6; ++i) g[i] = mean;
+    }
+    std::vector<double> dd(2 * 256 * 6, 1.0);  // D, then 1 / D
+    std::vector<float> df(2 * 256 * 6, 1.0f);
     for (int ph = 0; ph < d.nphase; ++ph)
       for (int i = 0; i < d.c; ++i)
-        if (d.act[ph] && !d.has_scale) dd[ph * d.c + i] = 1.0 / (std::fabs(d.m_in[ph * d.c + i]) + g[i]);
+        if (d.act[ph] && !d.has_scale) {
+          dd[256 * 6 + ph * d.c + i] = std::fabs(d.m_in[ph * d.c + i]) + g[i];
+          dd[ph * d.c + i] = 1.0 / dd[256 * 6 + ph * d.c + i];
+        }
     for (size_t i = 0; i < dd.size(); ++i) df[i] = (float)dd[i];
     for (int i = 0; i < 6; ++i) {
       h->pd.a.gpre[i] = g[i];
@@ -1553,6 +1547,7 @@ lsh_status lsh_setup(const lsh_problem* prob, void* workspace, size_t bytes, voi
     launch_d2df((const double*)(h->base + l.off_tw_d), reinterpret_cast<DF*>(h->twdf), 2ll * (d.nx + d.ny + d.nz), st);
   }
   if (last_launch() != LSH_OK) { delete h; return LSH_ERR_CUDA; }
+  if (set_voxel_fields(h) != LSH_OK) { delete h; return LSH_ERR_CUDA; }
   s = scan_microstructure(h);  // synchronises the stream (host vectors may go)
   if (s) { delete h; return s; }
 #undef SETUP_CK
@@ -1565,6 +1560,7 @@ lsh_status lsh_set_microstructure(lsh_handle* h, const unsigned char* phase, con
   h->drop_graphs();  // the scale pointer in the captured arguments may change
   lsh_status s = copy_microstructure(h, phase, scale, on_host);
   if (s) return s;
+  if ((s = set_voxel_fields(h))) return s;
   return scan_microstructure(h);
 }
 
@@ -1787,6 +1783,7 @@ lsh_status lsh_autotune(lsh_handle* h, lsh_tune_report* rep) {
     LSH_CK(cudaMemsetAsync(P.H, 0, sizeof(float2) * (size_t)d.Smax * d.c * d.nz * d.ny * d.hs, s));
     OpArgs<float> a = P.a;
     a.fuse = 0;
+    P.L = make_cfg<float>(d, d.Smax);  // the tiles that a holds
     cudaEvent_t e0, e1;
     LSH_CK(cudaEventCreate(&e0));
     if (cudaEventCreate(&e1) != cudaSuccess) {

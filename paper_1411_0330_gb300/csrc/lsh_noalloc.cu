@@ -193,37 +193,10 @@ extern "C" lsh_status lsh_apply_noalloc(const lsh_problem* pr, const double* x, 
   }
 
   // tile shapes (same rules as the workspace path, one system)
-  const size_t cs = sizeof(double2);
   const int lsx = nx | 1, lsy = ny | 1, lsz = nz | 1, rps = c * nz * ny;
-  int RY = std::max(2, 2 * (int)(32768 / (lsx * cs)));
-  RY = std::min(RY, std::max(2, rps / 608));
-  if (RY >= rps) {
-    RY = rps;
-  } else {
-    int best = 1, pick = 0;
-    for (int dv = RY; dv >= 1 && !pick; --dv)
-      if (rps % dv == 0) {
-        if (dv % 2 == 0) pick = dv;
-        else if (best == 1) best = dv;
-      }
-    RY = pick ? pick : best;
-  }
-  LaunchCfg L{};
-  L.threads = 256;
-  L.RY = RY;
-  L.VEC = (nx % 2 == 0 && (((uintptr_t)x | (uintptr_t)y) & 15) == 0) ? 2 : 1;
-  L.smem_x = nx * cs + (size_t)((RY + 1) / 2) * lsx * cs + nx * sizeof(int);
-  L.TY = std::min(8, nxh);
-  L.smem_y = ny * cs + (size_t)L.TY * lsy * cs;
-  int TZ = std::min(8, nxh);
-  while (TZ > 1 && (size_t)c * TZ * lsz * cs > 100 * 1024) TZ /= 2;
-  L.TZ = TZ;
-  L.smem_z = nz * cs + (size_t)c * TZ * lsz * cs;
-  L.grid_x = rps / RY;
-  L.grid_yx = (nxh + L.TY - 1) / L.TY;
-  L.grid_yy = c * nz;
-  L.grid_zx = (nxh + TZ - 1) / TZ;
-  L.grid_zy = ny;
+  LaunchCfg L = pass_cfg<double>(nx, ny, nz, c, px, py, pz, 1);
+  const int RY = L.RY;
+  if ((((uintptr_t)x | (uintptr_t)y) & 15) != 0) L.VEC = 1;
   const size_t kMax = 227 * 1024;
   if (L.smem_x > kMax || L.smem_y > kMax || L.smem_z > kMax || ny > 65535 || (long long)c * nz > 65535)
     return LSH_ERR_UNSUPPORTED_SIZE;
