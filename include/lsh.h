@@ -135,7 +135,10 @@ typedef struct lsh_solve_opts {
   int warm_start;    /* lsh_solve: tau holds the initial guess on entry                  */
   int no_graphs;     /* 0: each block of check_every CG iterations is captured once in a
                         CUDA graph (per handle, wave and precision) and replayed;
-                        1: the kernels are launched one by one.  Results are identical. */
+                        1: the kernels are launched one by one.  Results are identical.
+                        (Small grids run a whole CG solve in one launch, one thread-block
+                        cluster per system, unless the environment has LSH_NO_CLUSTER=1
+                        at lsh_setup or lsh_set_variants chose the passes.)              */
 } lsh_solve_opts;
 
 typedef struct lsh_solve_info {
@@ -296,7 +299,8 @@ lsh_status lsh_apply_noalloc(const lsh_problem *prob, const double *x, double *y
 /* Diagnostics (no counterpart in the paper): kernel launches issued by the
  * handle, and, when enabled, the device time of each pass of the CG
  * iteration measured with CUDA events recorded on the handle's stream
- * between consecutive launches.  Pass kinds: 0 x-forward (with the CG
+ * between consecutive launches (solves in one launch: with the device's timer
+ * between the phases of the first system).  Pass kinds: 0 x-forward (with the CG
  * prologue), 1 y-forward, 2 z-forward + Gamma^h product + z-inverse,
  * 3 y-inverse, 4 x-inverse (with local term and (p, Kp)), 5 CG update.  The
  * plane passes with z variant 11 update the residual in the inverse pass: kind

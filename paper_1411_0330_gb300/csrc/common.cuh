@@ -139,58 +139,42 @@ struct Plan1D {
   unsigned mag_nb[LSH_MAX_STAGES];
 };
 
-// Plan of length n (factors 2, 3, 5, 7), false if there is none.  Every stage is a
-// round trip through shared memory with a barrier, so the fewest stages win, then
-// the fewest operations; larger radices first.  Radices up to 12 keep an FP64
-// butterfly in 128 registers.  The lengths with compile-time schedules (fft.cuh) come
-// out as those expect.  A length whose factors 8, 4, 2, 3, 5, 7 number more than
-// LSH_MAX_STAGES is not taken.
-inline bool lsh_make_plan(int n, Plan1D* p) {
-  if (n < 1) return false;
-  int m = n, small = 0;
-  for (int q : {8, 4, 2, 3, 5, 7})
-    while (m % q == 0) { m /= q; ++small; }
-  if (m != 1 || small > LSH_MAX_STAGES) return false;
-  // radix and cost per point: a stage's own cost (shared-memory round trip, indices,
-  // twiddles) of 16 and the butterfly's operations
-  const int rad[] = {12, 10, 9, 8, 7, 6, 5, 4, 3, 2};
-  const int cost[] = {26, 25, 28, 22, 26, 23, 23, 20, 21, 18};
-  int best = 1 << 30, cur[16], nbest = 0;
-  int bestr[LSH_MAX_STAGES];
-  struct Search {
-    static void run(int left, int from, int k, int c, const int* rad, const int* cost, int* cur, int* best, int* bestr,
-                    int* nbest) {
-      if (left == 1) {
-        if (c < *best) {
-          *best = c;
-          *nbest = k;
-          for (int i = 0; i < k; ++i) bestr[i] = cur[i];
-        }
-        return;
-      }
-      if (k == LSH_MAX_STAGES) return;
-      for (int i = from; i < 10; ++i)
-        if (left % rad[i] == 0) {
-          cur[k] = rad[i];
-          run(left / rad[i], i, k + 1, c + cost[i], rad, cost, cur, best, bestr, nbest);
-        }
+// The cheapest sequence of radices (descending, each at most 12) whose product is n, by
+// the sum of cost(radix) over the stages; its length in *nst, 0 if there is none.
+template <typename Cost> inline void lsh_best_radices(int left, int from, int k, double c, const Cost& cost, int* cur,
+                                                      double* best, int* bestr, int* nst) {
+  if (left == 1) {
+    if (c < *best) {
+      *best = c;
+      *nst = k;
+      for (int i = 0; i < k; ++i) bestr[i] = cur[i];
     }
-  };
-  switch (n) {
-    case 128: nbest = 3; bestr[0] = 4; bestr[1] = 8; bestr[2] = 4; break;
-    case 256: nbest = 3; bestr[0] = 8; bestr[1] = 8; bestr[2] = 4; break;
-    case 96: nbest = 2; bestr[0] = 12; bestr[1] = 8; break;
-    case 64: nbest = 2; bestr[0] = bestr[1] = 8; break;
-    case 48: nbest = 2; bestr[0] = 8; bestr[1] = 6; break;
-    case 32: nbest = 2; bestr[0] = 8; bestr[1] = 4; break;
-    case 16: nbest = 2; bestr[0] = bestr[1] = 4; break;
-    default: Search::run(n, 0, 0, 0, rad, cost, cur, &best, bestr, &nbest);
+    return;
   }
+  if (k == LSH_MAX_STAGES) return;
+  for (int r = from; r >= 2; --r) {
+    if (r == 11 || left % r != 0) continue;
+    cur[k] = r;
+    lsh_best_radices(left / r, r, k + 1, c + cost(r), cost, cur, best, bestr, nst);
+  }
+}
+
+// A length whose factors 8, 4, 2, 3, 5, 7 number more than LSH_MAX_STAGES is not taken.
+inline bool lsh_plan_length(int n) {
+  if (n < 1) return false;
+  int small = 0;
+  for (int q : {8, 4, 2, 3, 5, 7})
+    while (n % q == 0) { n /= q; ++small; }
+  return n == 1 && small <= LSH_MAX_STAGES;
+}
+
+inline void lsh_fill_plan(int n, const int* radix, int nst, Plan1D* p) {
+  *p = Plan1D{};
   p->n = n;
-  p->nst = nbest;
+  p->nst = nst;
   int span = n;
-  for (int i = 0; i < nbest; ++i) {
-    const int r = bestr[i];
+  for (int i = 0; i < nst; ++i) {
+    const int r = radix[i];
     p->radix[i] = r;
     p->m[i] = span / r;
     p->tws[i] = n / span;
@@ -198,6 +182,52 @@ inline bool lsh_make_plan(int n, Plan1D* p) {
     p->mag_nb[i] = FastDiv::magic(n / r);
     span /= r;
   }
+}
+
+// Plan of length n (factors 2, 3, 5, 7), false if there is none.  Every stage is a
+// round trip through shared memory with a barrier, so the fewest stages win, then
+// the fewest operations; larger radices first.  Radices up to 12 keep an FP64
+// butterfly in 128 registers.  The lengths with compile-time schedules (fft.cuh) come
+// out as those expect.
+inline bool lsh_make_plan(int n, Plan1D* p) {
+  if (!lsh_plan_length(n)) return false;
+  // cost per point: a stage's own (shared-memory round trip, indices, twiddles) of 16 and
+  // the butterfly's operations
+  const auto cost = [](int r) {
+    const double c[13] = {0, 0, 18, 21, 20, 23, 23, 26, 22, 28, 25, 0, 26};
+    return c[r];
+  };
+  double best = 1e30;
+  int cur[LSH_MAX_STAGES], r[LSH_MAX_STAGES] = {0}, nst = 0;
+  switch (n) {
+    case 128: nst = 3; r[0] = 4; r[1] = 8; r[2] = 4; break;
+    case 256: nst = 3; r[0] = 8; r[1] = 8; r[2] = 4; break;
+    case 96: nst = 2; r[0] = 12; r[1] = 8; break;
+    case 64: nst = 2; r[0] = r[1] = 8; break;
+    case 48: nst = 2; r[0] = 8; r[1] = 6; break;
+    case 32: nst = 2; r[0] = 8; r[1] = 4; break;
+    case 16: nst = 2; r[0] = r[1] = 4; break;
+    default: lsh_best_radices(n, 12, 0, 0.0, cost, cur, &best, r, &nst);
+  }
+  lsh_fill_plan(n, r, nst, p);
+  return true;
+}
+
+// Plan for `lines` lines in one block of `threads` threads, by the cycles of a stage: a
+// barrier and the shared-memory round trip, and the instructions of a butterfly times
+// the warps (FP64: 16 cycles each of the SM's one unit) or the rounds of the threads.
+inline bool lsh_make_plan_lines(int n, int lines, int threads, bool fp64, Plan1D* p) {
+  if (!lsh_plan_length(n)) return false;
+  const auto cost = [&](int r) {
+    const double instr[13] = {0, 0, 16, 30, 36, 60, 66, 100, 92, 130, 140, 0, 160};
+    const double items = (double)lines * n / r, warps = (double)(long long)((items + 31) / 32);
+    const double rounds = (double)(long long)((items + threads - 1) / threads);
+    return 200.0 + (fp64 ? 16.0 * instr[r] * warps : instr[r] * (4.0 * rounds + warps / 4.0));
+  };
+  double best = 1e30;
+  int cur[LSH_MAX_STAGES], r[LSH_MAX_STAGES] = {0}, nst = 0;
+  lsh_best_radices(n, 12, 0, 0.0, cost, cur, &best, r, &nst);
+  lsh_fill_plan(n, r, nst, p);
   return true;
 }
 

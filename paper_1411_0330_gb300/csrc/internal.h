@@ -117,7 +117,9 @@ struct LaunchCfg {
 // in the launch: the largest number of blocks in flight per SM over the time of one,
 // where a stage of radix R takes ceil(butterflies / threads) rounds of R values.  Larger
 // radices leave few butterflies per block, and 256 threads for 56 of them hold the
-// registers of 200 idle ones.
+// registers of 200 idle ones: at 90 x 100 x 84, six systems, the y pass went from 89 to
+// 65 us in FP32 and from 755 to 707 us in FP64 with blocks of 64, at 63 x 45 x 50 the FP64
+// z pass from 81 to 61 us with tiles of 2 columns in blocks of 96.
 inline int pass_threads(int nlines, const Plan1D& p, size_t smem, int max_resident, long long blocks) {
   int best = 256;
   double best_rate = 0.0;
@@ -140,7 +142,7 @@ inline int pass_threads(int nlines, const Plan1D& p, size_t smem, int max_reside
 
 // Tiles and block sizes of the shared-memory passes for S systems: blocks of about 32 KB,
 // fewer lines where that would leave the 152 SMs without some four blocks each (two for
-// the FP32 x passes, whose tables and barriers cost more than the idle SMs).
+// the x passes, whose tables and barriers cost more than the idle SMs).
 template <typename T>
 LaunchCfg pass_cfg(int nx, int ny, int nz, int c, const Plan1D& px, const Plan1D& py, const Plan1D& pz, int S) {
   LaunchCfg L{};
@@ -151,7 +153,7 @@ LaunchCfg pass_cfg(int nx, int ny, int nz, int c, const Plan1D& px, const Plan1D
   constexpr long long kBlocks = 608;                // four per SM
   // rows per x block: an even divisor of the rows of a system where there is one
   int target = std::max(2, 2 * (int)(32768 / (lsx * cs)));
-  target = std::min(target, std::max(2, (int)((long long)rps * S / (sizeof(T) == 4 ? kBlocks / 2 : kBlocks))));
+  target = std::min(target, std::max(2, (int)((long long)rps * S / (kBlocks / 2))));
   if (target >= rps) {
     L.RY = rps;
   } else {
@@ -195,6 +197,28 @@ LaunchCfg pass_cfg(int nx, int ny, int nz, int c, const Plan1D& px, const Plan1D
   L.ew_per_sys = (int)std::max(1LL, std::min(want, std::max(1LL, 2432LL / S)));
   return L;
 }
+
+// A CG solve of every system of a wave in one cluster each (kernels_cluster.cu).
+template <typename T> struct ClusterCg {
+  OpArgs<T> a;
+  Plan1D qx, qy, qs;  // the kernel's own plans: x, y (3D), slowest axis
+  int flat;           // 2D grid: y is the slowest axis
+  int ns, ry;         // slices along the slowest axis, rows per slice
+  int CS, ps, pp;     // cluster size, slices and (row, kx) positions per CTA
+  int hs, LP;         // half rows and row pairs in shared memory (complex elements)
+  int threads;
+  size_t smem;
+  T* x;
+  const T* z;
+  SolverState* st;
+  int maxit;
+  // per-pass device time of system 0's iterations in every prof_every-th chunk of `check`
+  unsigned long long* prof;
+  int check, prof_every;
+  long long chunk0;
+};
+template <typename T> bool cluster_plan(const OpArgs<T>& a, int nsys, ClusterCg<T>* out);
+template <typename T> bool launch_cluster_cg(const ClusterCg<T>& c, cudaStream_t s);
 
 template <typename T>
 void launch_xfwd(const OpArgs<T>& a, const LaunchCfg& L, int mode, const T* in, T* x, const T* r, T* p,

@@ -321,7 +321,7 @@ int rps_of(const Derived& d) { return d.c * d.nz * d.ny; }
 // ---------------------------------------------------------------- workspace layout
 struct Layout {
   size_t off_state, off_partials, off_phase, off_scale, off_act, off_posx, off_kofy, off_kofz, off_sums, off_W;
-  size_t off_tabd, off_tabf, off_loads_d, off_loads_f, off_bb, off_flags, off_fault;
+  size_t off_tabd, off_tabf, off_loads_d, off_loads_f, off_bb, off_flags, off_fault, off_prof;
   size_t off_tw_d, off_tw_f;
   size_t off_fd[4], off_Hd, off_gd;
   size_t off_ff[4], off_Hf, off_gf;
@@ -390,6 +390,7 @@ Layout make_layout(const Derived& d) {
   l.off_bb = take(sizeof(double) * (size_t)S);
   l.off_flags = take((size_t)S);
   l.off_fault = take(sizeof(int));
+  l.off_prof = take(6 * sizeof(unsigned long long));
   l.off_tw_d = take(sizeof(double2) * (size_t)(d.nx + d.ny + d.nz));
   l.off_tw_f = take(sizeof(float2) * (size_t)(d.nx + d.ny + d.nz));
   // FP64 fields: x, r always; p, q for the FP64 CG (one system's worth of p, q
@@ -437,6 +438,8 @@ template <typename T> struct PrecBufs {
   CUtensorMap tmzp{};         // ky-major spectrum and its Nyquist columns (plane passes)
   CUtensorMap tmzq{};
   bool ytma_ok = false, ztma_ok = false, zpipe_ok = false;
+  ClusterCg<T> cl{};          // whole solves in one cluster per system, where cl_ok
+  bool cl_ok = false;
 };
 
 }  // namespace
@@ -450,6 +453,7 @@ struct lsh_handle {
   SymmlqScalars* sq = nullptr;  // after the S MinresScalars
   int* fault = nullptr;  // device word set by a kernel whose bounded wait ran out
   bool no_tma = false;
+  bool no_cluster = false;  // kernel variants chosen by hand, or LSH_NO_CLUSTER=1
   Layout lay;
   cudaStream_t stream;
   unsigned char* base;
@@ -937,11 +941,53 @@ void harvest_profile(lsh_handle* h, int real, bool plane, bool fuse) {
   h->ev_used = 0;
 }
 
+// The whole solve of every system of the wave in one launch (small problems).
+template <typename T>
+lsh_status cg_run_cluster(lsh_handle* h, PrecBufs<T>& P, const OpArgs<T>& a, int maxit, int check_every,
+                          std::vector<SolverState>& out) {
+  ClusterCg<T> c = P.cl;
+  c.a = a;
+  c.x = P.x;
+  c.z = P.r;
+  c.st = P.st;
+  c.maxit = maxit;
+  c.check = check_every;
+  c.prof_every = h->prof_every;
+  c.chunk0 = h->prof_chunk;
+  c.prof = h->prof ? (unsigned long long*)(h->base + h->lay.off_prof) : nullptr;
+  if (c.prof) LSH_CK(cudaMemsetAsync(c.prof, 0, 6 * sizeof(unsigned long long), h->stream));
+  if (!launch_cluster_cg<T>(c, h->stream)) {
+    cudaGetLastError();
+    return LSH_ERR_CUDA;
+  }
+  h->launches += 1;
+  unsigned long long ns[6] = {0, 0, 0, 0, 0, 0};
+  if (c.prof) LSH_CK(cudaMemcpyAsync(ns, c.prof, sizeof(ns), cudaMemcpyDeviceToHost, h->stream));
+  out.resize(a.S);
+  lsh_status stt = read_states(h, P.st, a.S, out.data());
+  if (stt) return stt;
+  if (h->prof) {
+    int most = 0;
+    for (int s = 0; s < a.S; ++s) {
+      most = std::max(most, out[s].iter);
+      h->timed_sys_iters += out[s].pad;
+    }
+    for (int k = 0; k < 6; ++k) {
+      h->pass_ms[k] += 1e-6 * (double)ns[k];
+      h->pass_n[k] += out[0].pad;
+    }
+    h->timed_iters += out[0].pad;
+    h->prof_chunk += (most + check_every - 1) / check_every;
+  }
+  return LSH_OK;
+}
+
 // CG on the states already begun for the wave; finalises x.  `out` receives
 // the S states.
 template <typename T>
 lsh_status cg_run(lsh_handle* h, PrecBufs<T>& P, const OpArgs<T>& a, int maxit, int check_every, bool graphs,
                   std::vector<SolverState>& out) {
+  if (P.cl_ok && !h->no_cluster) return cg_run_cluster<T>(h, P, a, maxit, check_every, out);
   const int S = a.S;
   out.resize(S);
   lsh_status stt = read_states(h, P.st, S, out.data());
@@ -1419,6 +1465,7 @@ lsh_status lsh_setup(const lsh_problem* prob, void* workspace, size_t bytes, voi
   {
     const char* e = getenv("LSH_NO_TMA");
     h->no_tma = e && e[0] == '1';
+    h->no_cluster = getenv_flag("LSH_NO_CLUSTER");
     const char* f = getenv("LSH_NO_DF");
     h->dfres = l.df && !(f && f[0] == '1');
     if (l.df) {
@@ -1489,6 +1536,8 @@ lsh_status lsh_setup(const lsh_problem* prob, void* workspace, size_t bytes, voi
     }
   }
   if (l.df) df_prepare();
+  h->pd.cl_ok = d.precision == LSH_FP64 && cluster_plan<double>(h->pd.a, d.B * d.c, &h->pd.cl);
+  h->pf.cl_ok = d.precision == LSH_MIXED && cluster_plan<float>(h->pf.a, d.B * d.c, &h->pf.cl);
   launch_gamma_table<double>(h->pd.a, d.dim, d.physics, d.green, d.ref_user, h->kofy, h->kofz, st,
                              d.rotated ? d.A0full : nullptr, d.rotated ? d.R : nullptr);
   if (d.precision == LSH_MIXED)
@@ -1982,6 +2031,7 @@ lsh_status lsh_set_variants(lsh_handle* h, int xf_variant, int x_variant, int y_
     P.a.ztma = z_variant;
     P.a.fuse = z_variant == 11;
     h->drop_graphs();
+    h->no_cluster = true;  // a choice made by hand runs the passes it names
     return LSH_OK;
   }
   if (h->d.plane && !reg_length(h->d.ny)) return LSH_ERR_UNSUPPORTED;  // radix-3 planes: plane passes only
@@ -2010,6 +2060,7 @@ lsh_status lsh_set_variants(lsh_handle* h, int xf_variant, int x_variant, int y_
   P.a.tlay = 0;
   P.a.fuse = 0;
   h->drop_graphs();
+  h->no_cluster = true;  // a choice made by hand runs the passes it names
   return LSH_OK;
 }
 
