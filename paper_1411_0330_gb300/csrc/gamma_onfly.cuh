@@ -96,6 +96,26 @@ __device__ __forceinline__ void gamma_trunc_onfly(const OpArgs<T>& a, int kx, in
   v[5] = cscale<T>(S12, r2);
 }
 
+// Normal components of one frequency between Mandel and the internal basis (hydrostatic,
+// two deviators; orthonormal, so that the inverse is the transpose).
+__device__ __forceinline__ void normals_to_internal(float2* v) {
+  const float s3 = 0.57735026918962576450914878050195745565f, s2 = 0.70710678118654752440084436210484903928f,
+              s6 = 0.40824829046386301636621401245098189866f;
+  const float2 p = cadd<float>(v[0], v[1]), m = csub<float>(v[0], v[1]), c = v[2];
+  v[0] = make_float2((p.x + c.x) * s3, (p.y + c.y) * s3);
+  v[1] = make_float2(m.x * s2, m.y * s2);
+  v[2] = make_float2((p.x - 2.f * c.x) * s6, (p.y - 2.f * c.y) * s6);
+}
+__device__ __forceinline__ void normals_to_mandel(float2* v) {
+  const float s3 = 0.57735026918962576450914878050195745565f, s2 = 0.70710678118654752440084436210484903928f,
+              s6 = 0.40824829046386301636621401245098189866f;
+  const float2 h = cscale<float>(v[0], s3), d = cscale<float>(v[1], s2), q = cscale<float>(v[2], s6);
+  const float2 e = cadd<float>(h, q);
+  v[0] = cadd<float>(e, d);
+  v[1] = csub<float>(e, d);
+  v[2] = make_float2(h.x - 2.f * q.x, h.y - 2.f * q.y);
+}
+
 // Finite-difference operator: rotate component i (axis i) by sign * pi k_i / N_i
 // (k unsigned, as in the table), before (sign -1) and after (+1) the real table.
 template <typename T, int NC>

@@ -99,6 +99,8 @@ template <typename T> struct OpArgs {
   int plane;
   int tlay;
   C2<T>* nq;
+  int mandel;  // apply on the plane passes: fields are Mandel components, the z pass takes
+               // the internal basis around Gamma^h and the local term couples the normals
   int fuse;  // plane passes with z variant 11: the CG update runs in the inverse pass
   int l2pf;  // plane passes, input planes requested into L2 at a block's start: bit 0 the
              // forward pass's x, r, p; bit 1 the inverse pass's p and phase planes

@@ -452,6 +452,55 @@ __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyinv(Op
     }
   };
   plane_x_inv<N>(PL, tw);
+  if (MODE == 0 && a.mandel) {
+    // Mandel components: M acts as m_d on the deviatoric part and m_h on the spherical
+    // part, so a normal component takes (m_h - m_d) / 3 of the trace too
+    __syncthreads();
+    const long long nv = (long long)a.nz * N * N;  // one component
+    const float* x0 = xin + plane - (comp < 3 ? (long long)comp * nv : 0);
+    constexpr int MB = PC::IT % 2 == 0 ? 2 : 1;
+#pragma unroll 1
+    for (int it0 = 0; it0 < PC::IT; it0 += MB) {
+      float4 v[MB][3];
+      uchar4 hc[MB];
+#pragma unroll
+      for (int b = 0; b < MB; ++b) {
+        const int idx = threadIdx.x + (it0 + b) * TH;
+        const int row = idx / NV, xx = (idx - row * NV) * 4;
+        const long long o = (long long)row * N + xx;
+        hc[b] = *reinterpret_cast<const uchar4*>(a.phase + pbase + o);
+        v[b][0] = *reinterpret_cast<const float4*>(x0 + o);
+        v[b][1] = v[b][2] = v[b][0];
+        if (comp < 3) {
+          v[b][1] = *reinterpret_cast<const float4*>(x0 + nv + o);
+          v[b][2] = *reinterpret_cast<const float4*>(x0 + 2 * nv + o);
+        }
+      }
+#pragma unroll
+      for (int b = 0; b < MB; ++b) {
+        const int idx = threadIdx.x + (it0 + b) * TH;
+        const int row = idx / NV, xx = (idx - row * NV) * 4;
+        const long long o = (long long)row * N + xx, vox = pbase + o;
+        const float4 g4 = *reinterpret_cast<const float4*>(PR + 2 * RS * row + xx);
+        const float4 q4 = comp == 1 ? v[b][1] : (comp == 2 ? v[b][2] : v[b][0]);
+        const float xq[4] = {q4.x, q4.y, q4.z, q4.w}, gv[4] = {g4.x, g4.y, g4.z, g4.w};
+        const float tr[4] = {v[b][0].x + v[b][1].x + v[b][2].x, v[b][0].y + v[b][1].y + v[b][2].y,
+                             v[b][0].z + v[b][1].z + v[b][2].z, v[b][0].w + v[b][1].w + v[b][2].w};
+        const unsigned char ph[4] = {hc[b].x, hc[b].y, hc[b].z, hc[b].w};
+        float ov[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int pp = ph[u];
+          const float mh = a.mfld ? a.mfld[vox + u] : a.mtab[pp * 6];
+          const float md = a.mfld ? a.mfld[a.fstride + vox + u] : a.mtab[pp * 6 + 1];
+          const float local = comp < 3 ? fmaf((mh - md) * (1.f / 3.f), tr[u], md * xq[u]) : md * xq[u];
+          ov[u] = aloc[pp] ? local + gv[u] : 0.f;
+        }
+        *reinterpret_cast<float4*>(out + plane + o) = make_float4(ov[0], ov[1], ov[2], ov[3]);
+      }
+    }
+    return;
+  }
   load_batch(0, xb0, hb0, zb0);
   __syncthreads();
   Acc<float> acc, accz, accm, accp;

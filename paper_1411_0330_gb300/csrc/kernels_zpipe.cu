@@ -116,7 +116,11 @@ __device__ __forceinline__ void zp_fused_item(const OpArgs<float>& a, float2* B,
       float2 g[NC];
 #pragma unroll
       for (int c = 0; c < NC; ++c) g[c] = d[c][k2];
+      if constexpr (NC == 6 && !DOT)
+        if (a.mandel) normals_to_internal(g);
       gamma_trunc_onfly<float, NC>(a, kx, ky, k1 + R1 * k2, g);
+      if constexpr (NC == 6 && !DOT)
+        if (a.mandel) normals_to_mandel(g);
       put(k2, g);
     }
   } else {
@@ -132,7 +136,11 @@ __device__ __forceinline__ void zp_fused_item(const OpArgs<float>& a, float2* B,
 #pragma unroll
       for (int c = 0; c < NC; ++c) g[c] = d[c][k2];
       if (a.fdphase) fd_rotate<float, NC>(a, kx, a.kofy[ypos], k1 + R1 * k2, g, -1.f);
+      if constexpr (NC == 6 && !DOT)
+        if (a.mandel) normals_to_internal(g);
       gamma_coef_apply<float, NC>(gc[k2 & 1], g);
+      if constexpr (NC == 6 && !DOT)
+        if (a.mandel) normals_to_mandel(g);
       if (a.fdphase) fd_rotate<float, NC>(a, kx, a.kofy[ypos], k1 + R1 * k2, g, 1.f);
       put(k2, g);
     }

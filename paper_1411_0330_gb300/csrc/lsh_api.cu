@@ -609,6 +609,7 @@ void init_prec(lsh_handle* h, PrecBufs<T>& P, const size_t* off_f, size_t off_H,
   a.xfreg = 0;
   a.plane = 0;
   a.fuse = 0;
+  a.mandel = 0;
   a.tlay = 0;
   a.nq = nullptr;
   // measured on the batched workload: the inverse pass gains (0.61 -> 0.66 of the
@@ -1661,6 +1662,12 @@ lsh_status lsh_apply(lsh_handle* h, int dtype, const void* x, void* y) {
       PrecBufs<float>& P = h->pf;
       const float* in = (const float*)x + b0 * n;
       float* o = (float*)y + b0 * n;
+      // elastic fields on the plane passes with z variant 11 stay in Mandel components: the
+      // change of basis commutes with the transforms and takes a few instructions per
+      // frequency there, against two passes over the field (128^3: 285 -> 180 us)
+      OpArgs<float> af = wave_args<float>(h, w);
+      af.mandel = el && af.plane && af.ztma == 11;
+      const bool rot = (el || d.rotated) && !af.mandel;
       const bool stage = !rot && unaligned(in, o);
       if (rot) {
         rotate(in, P.p, 1);
@@ -1669,7 +1676,7 @@ lsh_status lsh_apply(lsh_handle* h, int dtype, const void* x, void* y) {
         LSH_CK(cudaMemcpyAsync(P.p, in, sizeof(float) * (size_t)(S * n), cudaMemcpyDeviceToDevice, h->stream));
         in = P.p;
       }
-      lsh_status s = apply_internal<float>(h, wave_args<float>(h, w), in, (rot || stage) ? P.q : o);
+      lsh_status s = apply_internal<float>(h, af, in, (rot || stage) ? P.q : o);
       if (s) return s;
       if (rot) rotate((const float*)P.q, o, 0);
       else if (stage)

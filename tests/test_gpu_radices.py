@@ -55,3 +55,29 @@ def test_unaligned_caller_buffers(shape, dtype):
     xu, yu = x[1:].view(h.field_shape), y[1:].view(h.field_shape)
     h.apply(xu, out=yu)
     assert torch.equal(yu, h.apply(xu.clone()))
+
+
+@pytest.mark.parametrize("shape", [(16, 16, 16), (32, 48, 48), (16, 64, 64), (128, 16, 16), (16, 128, 128)])
+@pytest.mark.parametrize("kind", ["phase", "scale", "fraction"])
+@pytest.mark.parametrize("green", [0, 1])
+def test_elastic_apply_in_mandel_components(shape, kind, green):
+    """FP32 apply whose fields stay in Mandel components (z variant 11) against the one through the internal
+    basis (variant 10), two microstructures, voxels outside I0: both are the operator to FP32 rounding, each
+    2e-5 of the largest value from the oracle's, and from each other by the FFT's rounding (2e-6)."""
+    rng = np.random.default_rng(sum(shape) + green)
+    K, mu = 0.8333, 0.3846
+    ref = np.array([0.25 * K, 0.25 * mu])
+    mods = np.array([[K, mu], [6.7 * K, 10.8 * mu]] if kind == "fraction" else [[K, mu], list(ref), [6.7 * K, 10.8 * mu]])
+    ph = rng.integers(0, len(mods), (2,) + shape).astype(np.uint8)
+    kw = {}
+    if kind != "phase":
+        f = rng.uniform(0.5, 2.0, ph.shape) if kind == "scale" else rng.uniform(0.0, 1.0, ph.shape)
+        kw = {kind: torch.from_numpy(f.astype(np.float32)).cuda()}
+    h = lsh.Handle(torch.from_numpy(ph).cuda(), mods, physics=lsh.ELASTIC, green=green, precision=lsh.MIXED, ref=ref,
+                   batch=True, **kw)
+    x = torch.randn(h.field_shape, dtype=torch.float32, device="cuda")
+    h.set_variants(0, 0, 2, 11)
+    a = h.apply(x).double()
+    h.set_variants(0, 0, 2, 10)
+    b = h.apply(x).double()
+    assert float((a - b).abs().max()) < 2e-6 * float(b.abs().max())
