@@ -10,6 +10,22 @@
 
 namespace lsh {
 
+// Launch with or without programmatic dependence on the kernel ahead in the stream.
+template <typename... P, typename... A>
+inline void launch_dep(bool pdl, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = pdl ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, k, args...);
+}
+
 // Everything an operator pass needs, passed by value to the kernels.
 //
 // A launch covers S independent systems (one microstructure, one load each)
@@ -45,6 +61,7 @@ template <typename T> struct OpArgs {
   int frac;                    // 1: scale holds the volume fraction of phase 1 (Eq. (def_ah))
   const unsigned char* act;    // per phase: 1 if A_phase != A0 (voxel in I0)
   int nphase;
+  int both;                    // two phases, both in I0, no voxel field (the common case)
   const T* mtab;               // per phase * c: diagonal of M (no scale field)
   const T* modtab;             // per phase * c: diagonal of A_phase (scale field)
   T ref[6];                    // diagonal of A0 (internal basis)
@@ -101,6 +118,7 @@ template <typename T> struct OpArgs {
   C2<T>* nq;
   int mandel;  // apply on the plane passes: fields are Mandel components, the z pass takes
                // the internal basis around Gamma^h and the local term couples the normals
+  int pdl;     // the kernels of the fused plane iteration start before the one ahead has drained
   int fuse;  // plane passes with z variant 11: the CG update runs in the inverse pass
   int l2pf;  // plane passes, input planes requested into L2 at a block's start: bit 0 the
              // forward pass's x, r, p; bit 1 the inverse pass's p and phase planes
@@ -319,7 +337,7 @@ bool launch_xyfwd(const OpArgs<float>& a, int mode, const float* in, float* x, c
 bool launch_xyinv(const OpArgs<float>& a, int mode, const float* xin, float* out, SolverState* st, double* partials,
                   cudaStream_t s);
 // CG iteration with the update of z fused into the inverse pass (kernels_plane.cu)
-void launch_cg_alpha(SolverState* st, const double* partials, int nb, int S, cudaStream_t s);
+void launch_cg_alpha(SolverState* st, const double* partials, int nb, int S, bool pdl, cudaStream_t s);
 bool launch_xyinv_update(const OpArgs<float>& a, const float* p, float* z, SolverState* st, double* partials,
                          long long off, cudaStream_t s);
 void plane_prepare();

@@ -253,10 +253,17 @@ __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyfwd(Op
   const int s = blockIdx.x / cnz;
   const int blk = blockIdx.x - s * cnz;  // comp * nz + z
   const int comp = blk / a.nz, z = blk - comp * a.nz;
-  if (MODE == 1 && st[s].done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* PL = reinterpret_cast<float2*>(smem_raw);  // [N][RS]
   float2* tw = PL + N * RS;
+  // the state is written by the kernel ahead: read after the wait, never from a cache of
+  // invariant data
+  const volatile SolverState* vst = st + s;
+  if (MODE == 1) {
+    griddep_wait();
+    griddep_launch();
+    if (vst->done) return;
+  }
   float* PR = reinterpret_cast<float*>(PL);  // real row y at PR + 2 RS y
   __shared__ unsigned char aloc[256];
   for (int u = threadIdx.x; u < N; u += TH) tw[u] = a.twx[u];
@@ -267,9 +274,9 @@ __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyfwd(Op
   int k = 0;
   float alpha = 0.f, beta = 0.f;
   if (MODE == 1) {
-    k = st[s].iter;
-    alpha = (float)st[s].alpha;
-    beta = (float)st[s].beta;
+    k = vst->iter;
+    alpha = (float)vst->alpha;
+    beta = (float)vst->beta;
   }
   if (MODE == 0) {
     __syncthreads();  // aloc
@@ -375,7 +382,8 @@ __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyfwd(Op
 // (r, r), (r, z), (z, M z), (z, M p) go to partials + {0, 1, 2, 3} off; k_cg_beta sums
 // them.  Against MODE 4 and the CG update kernel the q field is neither written nor read
 // and r is read where p and the phases already are: 12.5 instead of 14.25 field passes
-// per iteration.
+// per iteration.  MODE 6: the same for two phases that are both in I0 and no voxel field,
+// without the general forms of the local term in its epilogue.
 template <int N, int MODE>
 __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyinv(OpArgs<float> a, const float* __restrict__ xin,
                                                            float* __restrict__ out, const SolverState* __restrict__ st,
@@ -386,7 +394,12 @@ __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyinv(Op
   const int s = blockIdx.x / cnz;
   const int blk = blockIdx.x - s * cnz;
   const int comp = blk / a.nz, z = blk - comp * a.nz;
-  if (MODE >= 4 && st[s].done) return;
+  if (MODE >= 5) {
+    griddep_wait();
+    griddep_launch();
+  }
+  const volatile SolverState* vst = st + s;  // as in the forward pass
+  if (MODE >= 4 && vst->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* PL = reinterpret_cast<float2*>(smem_raw);
   float2* tw = PL + N * RS;
@@ -409,13 +422,13 @@ __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyinv(Op
   for (int u = threadIdx.x; u < N; u += TH) tw[u] = a.twx[u];
   for (int u = threadIdx.x; u < a.nphase; u += TH) {
     mloc[u] = (a.scale && !a.frac) ? a.modtab[u * a.c + comp] : a.mtab[u * a.c + comp];
-    dloc[u] = MODE == 5 && a.pre == 1 ? a.dtab[u * a.c + comp] : 1.f;
+    dloc[u] = MODE >= 5 && a.pre == 1 ? a.dtab[u * a.c + comp] : 1.f;
     aloc[u] = a.act[u];
   }
   // the epilogue's p plane and phase plane go to L2 while the transforms run
   const long long plane = (long long)blockIdx.x * N * N;
   const long long pbase = (long long)((a.sys0 + s) / a.sys_per_ms) * a.V + (long long)z * N * N;
-  if ((a.l2pf & 2) && threadIdx.x < (MODE == 5 ? 17 : 9)) {
+  if ((a.l2pf & 2) && threadIdx.x < (MODE >= 5 ? 17 : 9)) {
     constexpr uint32_t PB = (uint32_t)(sizeof(float) * N * N);
     if (threadIdx.x < 8) bulk_prefetch_l2(reinterpret_cast<const char*>(xin + plane) + threadIdx.x * (PB / 8), PB / 8);
     else if (threadIdx.x > 8) bulk_prefetch_l2(reinterpret_cast<const char*>(out + plane) + (threadIdx.x - 9) * (PB / 8), PB / 8);
@@ -437,8 +450,8 @@ __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyinv(Op
   // the epilogue's p and phase loads go out in batches of B groups of four
   // voxels, each batch in flight while the previous one is worked on; two
   // register sets take the batches in turn (no copies between them)
-  constexpr int B = PC::IT % 2 == 0 && MODE != 5 ? 2 : 1;
-  constexpr int ZB = MODE == 5 ? B : 1;
+  constexpr int B = PC::IT % 2 == 0 && MODE < 5 ? 2 : 1;
+  constexpr int ZB = MODE >= 5 ? B : 1;
   float4 xb0[B], xb1[B], zb0[ZB], zb1[ZB];
   uchar4 hb0[B], hb1[B];
   auto load_batch = [&](int it0, float4* xb, uchar4* hb, float4* zb) {
@@ -448,7 +461,7 @@ __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyinv(Op
       const int row = idx / NV, xx = (idx - row * NV) * 4;
       xb[b] = *reinterpret_cast<const float4*>(xin + plane + (long long)row * N + xx);
       hb[b] = *reinterpret_cast<const uchar4*>(a.phase + pbase + (long long)row * N + xx);
-      if (MODE == 5) zb[b] = *reinterpret_cast<const float4*>(out + plane + (long long)row * N + xx);
+      if (MODE >= 5) zb[b] = *reinterpret_cast<const float4*>(out + plane + (long long)row * N + xx);
     }
   };
   plane_x_inv<N>(PL, tw);
@@ -504,16 +517,16 @@ __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyinv(Op
   load_batch(0, xb0, hb0, zb0);
   __syncthreads();
   Acc<float> acc, accz, accm, accp;
-  const float al = MODE == 5 ? (float)st[s].alpha : 0.f;
+  const float al = MODE >= 5 ? (float)vst->alpha : 0.f;
   // two phases without a voxel field (the common case): both phases' M and
   // activity in registers, selected per voxel instead of read from the tables;
   // both active (A0 differs from both phases): no projection to apply
-  const bool two = a.nphase <= 2 && !a.scale;
+  const bool two = MODE == 6 || (a.nphase <= 2 && !a.scale);
   const float m0 = mloc[0], m1 = a.nphase > 1 ? mloc[1] : m0;
   const float d0 = dloc[0], d1 = a.nphase > 1 ? dloc[1] : d0;
   const float e0 = 1.f / d0, e1 = 1.f / d1;
   const bool act0 = aloc[0] != 0, act1 = a.nphase > 1 ? aloc[1] != 0 : act0;
-  const bool both = two && act0 && act1;
+  const bool both = MODE == 6 || (two && act0 && act1);
   auto work = [&](int it0, const float4* xc, const uchar4* hc, const float4* zc) {
 #pragma unroll
     for (int b = 0; b < B; ++b) {
@@ -526,7 +539,7 @@ __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyinv(Op
       const unsigned char ph[4] = {hc[b].x, hc[b].y, hc[b].z, hc[b].w};
       const float gv[4] = {g4.x, g4.y, g4.z, g4.w};
       float ov[4];
-      if constexpr (MODE == 5) {
+      if constexpr (MODE >= 5) {
         float z[4] = {zc[b].x, zc[b].y, zc[b].z, zc[b].w};
         float srr = 0.f, srz = 0.f, szm = 0.f, spm = 0.f;
 #pragma unroll
@@ -605,7 +618,7 @@ __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyinv(Op
     if (it0 + 2 * B < PC::IT) load_batch(it0 + 2 * B, xb0, hb0, zb0);
     work(it0 + B, xb1, hb1, zb1);
   }
-  if constexpr (MODE == 5) {
+  if constexpr (MODE >= 5) {
     double* part = partials + (long long)s * cnz + blk;
     auto store = [&](const Acc<float>& v, long long at) {
       const double tot = block_reduce(v);
@@ -634,10 +647,12 @@ __global__ void __launch_bounds__(256) k_cg_alpha(SolverState* __restrict__ st, 
                                                   int nb) {
   const int s = blockIdx.x;
   SolverState* sst = st + s;
+  griddep_wait();
+  griddep_launch();
   if (sst->done) return;
   const double* part = partials + (long long)s * nb;
   double v = 0.0;
-  for (int i = threadIdx.x; i < nb; i += blockDim.x) v += part[i];
+  for (int i = threadIdx.x; i < nb; i += blockDim.x) v += __ldcg(part + i);
   const double sum = block_sum(v);
   if (threadIdx.x == 0) {
     const double b = sst->beta;
@@ -660,17 +675,20 @@ __global__ void __launch_bounds__(256) k_cg_beta(SolverState* __restrict__ st, c
                                                  long long off, int nb) {
   const int s = blockIdx.x;
   SolverState* sst = st + s;
+  griddep_wait();
+  griddep_launch();
   if (sst->done) return;
-  double v[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int i = threadIdx.x; i < nb; i += blockDim.x)
+  // two warps per sum, one barrier
+  __shared__ double part[8];
+  const int w = threadIdx.x >> 5, k = w & 3;
+  double t = 0.0;
+  for (int i = threadIdx.x & 31 | (w >> 2) << 5; i < nb; i += 64) t += __ldcg(partials + k * off + (long long)s * nb + i);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] += partials[k * off + (long long)s * nb + i];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    v[k] = block_sum(v[k]);
-    __syncthreads();
-  }
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+  if ((threadIdx.x & 31) == 0) part[w] = t;
+  __syncthreads();
   if (threadIdx.x == 0) {
+    const double v[4] = {part[0] + part[4], part[1] + part[5], part[2] + part[6], part[3] + part[7]};
     sst->beta = v[1] / sst->rz;
     sst->rr = v[0];
     sst->rz = v[1];
@@ -701,6 +719,7 @@ template <int N> void plane_attrs() {
   cudaFuncSetAttribute(k_xyinv<N, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, smi);
   cudaFuncSetAttribute(k_xyinv<N, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smi);
   cudaFuncSetAttribute(k_xyinv<N, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize, smi);
+  cudaFuncSetAttribute(k_xyinv<N, 6>, cudaFuncAttributeMaxDynamicSharedMemorySize, smi);
 }
 
 template <int N> bool plane_fwd_n(const OpArgs<float>& a, int mode, const float* in, float* x, const float* r,
@@ -709,7 +728,7 @@ template <int N> bool plane_fwd_n(const OpArgs<float>& a, int mode, const float*
   if (a.hs < PC::RS || (a.hs & 1) != 0) return false;
   const unsigned grid = (unsigned)((long long)a.S * a.c * a.nz);
   if (mode == 0) k_xyfwd<N, 0><<<grid, PC::TH, PC::SMEM, s>>>(a, in, x, r, p, st);
-  else k_xyfwd<N, 1><<<grid, PC::TH, PC::SMEM, s>>>(a, in, x, r, p, st);
+  else launch_dep(a.pdl != 0, k_xyfwd<N, 1>, dim3(grid), dim3(PC::TH), PC::SMEM, s, a, in, x, r, p, st);
   return true;
 }
 
@@ -725,8 +744,9 @@ template <int N> bool plane_inv_n(const OpArgs<float>& a, int mode, const float*
     k_xyinv<N, 4><<<grid, PC::TH, smem, s>>>(a, xin, out, st, partials, 0);
     launch_dot_finalize(st, partials, a.c * a.nz, a.S, s);
   } else {
-    k_xyinv<N, 5><<<grid, PC::TH, smem, s>>>(a, xin, out, st, partials, off);
-    k_cg_beta<<<a.S, 256, 0, s>>>(st, partials, off, a.c * a.nz);
+    launch_dep(a.pdl != 0, a.both ? k_xyinv<N, 6> : k_xyinv<N, 5>, dim3(grid), dim3(PC::TH), smem, s, a, xin, out,
+               (const SolverState*)st, partials, off);
+    launch_dep(a.pdl != 0, k_cg_beta, dim3(a.S), dim3(256), 0, s, st, (const double*)partials, off, a.c * a.nz);
   }
   return true;
 }
@@ -775,8 +795,8 @@ bool launch_xyinv_update(const OpArgs<float>& a, const float* p, float* z, Solve
   return xyinv_n(a, 2, p, z, st, partials, off, s);
 }
 
-void launch_cg_alpha(SolverState* st, const double* partials, int nb, int S, cudaStream_t s) {
-  k_cg_alpha<<<S, 256, 0, s>>>(st, partials, nb);
+void launch_cg_alpha(SolverState* st, const double* partials, int nb, int S, bool pdl, cudaStream_t s) {
+  launch_dep(pdl, k_cg_alpha, dim3(S), dim3(256), 0, s, st, partials, nb);
 }
 
 void plane_prepare() {

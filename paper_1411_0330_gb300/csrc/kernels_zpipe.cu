@@ -178,6 +178,10 @@ __global__ void __launch_bounds__(ZPipe<NC, N, FUSED>::THREADS, ZPipe<NC, N, FUS
     mbar_init_fence();
     fault = 0;
   }
+  if constexpr (DOT) {
+    griddep_wait();
+    griddep_launch();
+  }
   __syncthreads();
 
   // Warp 0 walks the block's tiles (grid stride, skipping converged systems),
@@ -428,8 +432,8 @@ bool launch_zpipe_n(const OpArgs<float>& a, const SolverState* st, double* parti
     const long long total = nregular + (long long)a.S * (a.ny / ZC::TZ);
     const long long grid = std::max<long long>(1, std::min<long long>(total, (long long)multiprocessors() * bpsm));
     if (total + grid >= (1ll << 31)) return false;
-    k_zgamma_pipe<NC, N, FUSED, DOT><<<(unsigned)grid, ZC::THREADS, ZC::SMEM, s>>>(*a.tmzp, *a.tmzq, a, st, nkt,
-                                                                                   (int)nregular, (int)total, partials);
+    launch_dep(DOT && a.pdl, k_zgamma_pipe<NC, N, FUSED, DOT>, dim3((unsigned)grid), dim3(ZC::THREADS), ZC::SMEM, s,
+               *a.tmzp, *a.tmzq, a, st, nkt, (int)nregular, (int)total, partials);
     return true;
   }
 }

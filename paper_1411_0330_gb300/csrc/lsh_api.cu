@@ -577,6 +577,7 @@ void init_prec(lsh_handle* h, PrecBufs<T>& P, const size_t* off_f, size_t off_H,
   a.frac = d.frac ? 1 : 0;
   a.act = h->act;
   a.nphase = d.nphase;
+  a.both = d.nphase == 2 && !d.has_scale && d.act[0] && d.act[1];
   a.mtab = P.mtab;
   a.modtab = P.modtab;
   // preconditioner of the CG iterations: the FP32 ones of the mixed solver wherever K is
@@ -610,6 +611,7 @@ void init_prec(lsh_handle* h, PrecBufs<T>& P, const size_t* off_f, size_t off_H,
   a.plane = 0;
   a.fuse = 0;
   a.mandel = 0;
+  a.pdl = 0;
   a.tlay = 0;
   a.nq = nullptr;
   // measured on the batched workload: the inverse pass gains (0.61 -> 0.66 of the
@@ -836,16 +838,19 @@ template <typename T> void enqueue_cg_iteration(lsh_handle* h, PrecBufs<T>& P, c
   const unsigned rf = h->capturing ? cudaEventRecordExternal : cudaEventRecordDefault;
   if constexpr (sizeof(T) == 4) {
     if (a.plane && a.fuse) {
-      // five launches: xy forward, z, alpha, xy inverse with the update of z, beta
+      // five launches: xy forward, z, alpha, xy inverse with the update of z, beta; each
+      // is set up while the one ahead drains (not with events between them)
+      OpArgs<T> b = a;
+      b.pdl = timed ? 0 : 1;
       if (timed) cudaEventRecordWithFlags(e[0], s, rf);
-      launch_xyfwd(a, 1, nullptr, P.x, P.r, P.p, P.st, s);
+      launch_xyfwd(b, 1, nullptr, P.x, P.r, P.p, P.st, s);
       if (timed) cudaEventRecordWithFlags(e[1], s, rf);
       if (timed) cudaEventRecordWithFlags(e[2], s, rf);
-      launch_zgamma_pipe(a, true, P.st, s, h->partials);
+      launch_zgamma_pipe(b, true, P.st, s, h->partials);
       if (timed) cudaEventRecordWithFlags(e[3], s, rf);
       if (timed) cudaEventRecordWithFlags(e[4], s, rf);
-      launch_cg_alpha(P.st, h->partials, zdot_count(a), a.S, s);
-      launch_xyinv_update(a, P.p, P.r, P.st, h->partials, h->lay.nparts, s);
+      launch_cg_alpha(P.st, h->partials, zdot_count(b), b.S, b.pdl != 0, s);
+      launch_xyinv_update(b, P.p, P.r, P.st, h->partials, h->lay.nparts, s);
       if (timed) {
         cudaEventRecordWithFlags(e[5], s, rf);
         cudaEventRecordWithFlags(e[6], s, rf);
@@ -1974,7 +1979,7 @@ lsh_status lsh_autotune(lsh_handle* h, lsh_tune_report* rep) {
           cudaMemcpyAsync(P.st, fake.data(), sizeof(SolverState) * d.Smax, cudaMemcpyHostToDevice, s);
           // the pass first: on the arbitrary data alpha may flag a breakdown that would stop it
           const bool ok = launch_xyinv_update(b, P.p, P.r, P.st, h->partials, h->lay.nparts, s);
-          launch_cg_alpha(P.st, h->partials, zdot_count(b), b.S, s);
+          launch_cg_alpha(P.st, h->partials, zdot_count(b), b.S, false, s);
           return ok;
         });
         if (zf > 0.f && jf > 0.f && zf + jf < z + i + u) {

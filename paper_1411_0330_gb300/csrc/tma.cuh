@@ -113,6 +113,12 @@ __device__ __forceinline__ void bulk_store_1d(void* dst, const void* src, uint32
                : "memory");
 }
 
+// Programmatic dependent launch: everything the kernel before produced is visible after
+// the wait (at once if the launch does not depend on one); from the other call on, the
+// kernel after may take the SMs' free places and run up to its own wait.
+__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 
 // the shared-memory sources of all committed stores have been read
