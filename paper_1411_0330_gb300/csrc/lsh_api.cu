@@ -991,13 +991,12 @@ lsh_status cg_run_cluster(lsh_handle* h, PrecBufs<T>& P, const OpArgs<T>& a, int
 // CG on the states already begun for the wave; finalises x.  `out` receives
 // the S states.
 template <typename T>
-lsh_status cg_run(lsh_handle* h, PrecBufs<T>& P, const OpArgs<T>& a, int maxit, int check_every, bool graphs,
-                  std::vector<SolverState>& out) {
+lsh_status cg_run(lsh_handle* h, PrecBufs<T>& P, const OpArgs<T>& a, int maxit, int check_every, bool check_given,
+                  bool graphs, std::vector<SolverState>& out) {
   if (P.cl_ok && !h->no_cluster) return cg_run_cluster<T>(h, P, a, maxit, check_every, out);
   const int S = a.S;
-  out.resize(S);
-  lsh_status stt = read_states(h, P.st, S, out.data());
-  if (stt) return stt;
+  out.assign(S, SolverState{});
+  lsh_status stt;
   auto all_done = [&]() {
     for (int s = 0; s < S; ++s)
       if (!out[s].done) return false;
@@ -1008,25 +1007,43 @@ lsh_status cg_run(lsh_handle* h, PrecBufs<T>& P, const OpArgs<T>& a, int maxit, 
     for (int s = 0; s < S; ++s) m = std::max(m, out[s].iter);
     return m;
   };
-  int it = 0;
-  while (!all_done() && it < maxit) {
-    const int chunk = std::min(check_every, maxit - it);
-    const int before = max_iter();
-    h->prof_now = h->prof && (h->prof_chunk++ % h->prof_every) == 0;
-    if (graphs && chunk == check_every) {
-      lsh_handle::Graph* g = nullptr;
-      if ((stt = chunk_graph<T>(h, P, a, chunk, &g))) return stt;
-      if (h->prof_now) h->ev_used = 0;
-      LSH_CK(cudaGraphLaunch(g->exec, h->stream));
-      h->launches += g->launches;
-      if (h->prof_now) h->ev_used = (int)std::min<size_t>(7 * (size_t)chunk, h->ev.size() / 7 * 7);
-    } else {
-      for (int j = 0; j < chunk; ++j) enqueue_cg_iteration<T>(h, P, a);
+  // Chunks to enqueue before the states are read again.  Each reading leaves the device
+  // idle for a round trip to the host (some 12 us, a third of an iteration of 32^3), and
+  // iterations enqueued past convergence return at once.  With the default interval the
+  // residual's decrease so far says how many more the slowest system needs; 0.7 of them
+  // are enqueued in one go, because CG speeds up.  Beyond 2^23 elements an iteration is
+  // long against the round trip and the blocks of idle ones cost as much (90 x 100 x 84).
+  auto chunks_ahead = [&]() {
+    if (check_given || h->prof || (long long)S * a.c * a.V > (1ll << 23)) return 1;
+    double most = 0.0;
+    for (int s = 0; s < S; ++s) {
+      const SolverState& t = out[s];
+      if (t.done || t.iter < 1 || !(t.rr > 0.0) || !(t.bb > t.rr) || !(t.tol2 > 0.0)) continue;
+      most = std::max(most, t.iter * std::log(t.rr / t.tol2) / std::log(t.bb / t.rr));
     }
-    if ((stt = last_launch())) return stt;
-    it += chunk;
+    return (int)std::max(1.0, std::min(64.0, 0.7 * most / check_every));
+  };
+  int it = 0;
+  do {
+    const int before = max_iter();
     long long live0 = 0;
     for (int k = 0; k < S; ++k) live0 += out[k].iter;
+    for (int ahead = chunks_ahead(); ahead > 0 && it < maxit; --ahead) {
+      const int chunk = std::min(check_every, maxit - it);
+      h->prof_now = h->prof && (h->prof_chunk++ % h->prof_every) == 0;
+      if (graphs && chunk == check_every) {
+        lsh_handle::Graph* g = nullptr;
+        if ((stt = chunk_graph<T>(h, P, a, chunk, &g))) return stt;
+        if (h->prof_now) h->ev_used = 0;
+        LSH_CK(cudaGraphLaunch(g->exec, h->stream));
+        h->launches += g->launches;
+        if (h->prof_now) h->ev_used = (int)std::min<size_t>(7 * (size_t)chunk, h->ev.size() / 7 * 7);
+      } else {
+        for (int j = 0; j < chunk; ++j) enqueue_cg_iteration<T>(h, P, a);
+      }
+      if ((stt = last_launch())) return stt;
+      it += chunk;
+    }
     if ((stt = read_states(h, P.st, S, out.data()))) return stt;
     if (h->prof_now) {
       for (int k = 0; k < S; ++k) h->timed_sys_iters += out[k].iter;
@@ -1034,11 +1051,10 @@ lsh_status cg_run(lsh_handle* h, PrecBufs<T>& P, const OpArgs<T>& a, int maxit, 
       harvest_profile(h, max_iter() - before, a.plane != 0, a.fuse != 0);
     }
     h->prof_now = false;
-  }
+  } while (!all_done() && it < maxit);
   launch_cg_finalize<T>(P.x, P.p, (long long)a.c * a.V, S, P.st, P.L.ew_per_sys, h->stream);
   h->launches += 1;
-  if ((stt = last_launch())) return stt;
-  return read_states(h, P.st, S, out.data());
+  return last_launch();
 }
 
 // MINRES on the FP64 operator for the systems of a wave, whose right-hand
@@ -1167,7 +1183,8 @@ lsh_status solve_wave(lsh_handle* h, const Wave& w, bool warm, const lsh_solve_o
   const long long n = (long long)d.c * d.V;
   const double tol = o && o->tol > 0 ? o->tol : 1e-10;
   const int maxit = o && o->maxit > 0 ? o->maxit : 10000;
-  const int check = o && o->check_every > 0 ? o->check_every : 8;
+  const bool check_given = o && o->check_every > 0;
+  const int check = check_given ? o->check_every : 8;
   const bool graphs = !(o && o->no_graphs);
   lsh_status stt;
   if ((stt = upload_loads(h, w))) return stt;
@@ -1243,7 +1260,7 @@ lsh_status solve_wave(lsh_handle* h, const Wave& w, bool warm, const lsh_solve_o
       h->launches += 1;
     }
     if ((stt = last_launch())) return stt;
-    if ((stt = cg_run<double>(h, Pd, ad, maxit, check, graphs, st))) return stt;
+    if ((stt = cg_run<double>(h, Pd, ad, maxit, check, check_given, graphs, st))) return stt;
     for (int s = 0; s < S; ++s) {
       infos[s].iters = st[s].iter;
       infos[s].applies64 += st[s].iter;
@@ -1306,7 +1323,7 @@ lsh_status solve_wave(lsh_handle* h, const Wave& w, bool warm, const lsh_solve_o
       launch_d2f_begin(af, Pd.r, rdf, Pf.r, Pf.x, Pf.st, h->partials, h->lay.nparts, itol_k, h->flags,
                        Pf.L.ew_per_sys, h->stream);
       h->launches += 1;
-      if ((stt = cg_run<float>(h, Pf, af, maxit - total_max, check, graphs, st))) return stt;
+      if ((stt = cg_run<float>(h, Pf, af, maxit - total_max, check, check_given, graphs, st))) return stt;
       launch_f2d_axpy(Pd.x, Pf.x, n * S, h->stream);
       h->launches += 1;
       if ((stt = residual64(h, ad, Pd.x, Pd.r, h->dfres))) return stt;
@@ -1612,7 +1629,6 @@ lsh_status lsh_setup(const lsh_problem* prob, void* workspace, size_t bytes, voi
 
 lsh_status lsh_set_microstructure(lsh_handle* h, const unsigned char* phase, const float* scale, int on_host) {
   if (!h || !phase) return LSH_ERR_INVALID_ARG;
-  h->drop_graphs();  // the scale pointer in the captured arguments may change
   lsh_status s = copy_microstructure(h, phase, scale, on_host);
   if (s) return s;
   if ((s = set_voxel_fields(h))) return s;
