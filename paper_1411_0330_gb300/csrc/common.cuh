@@ -55,6 +55,11 @@ struct SolverState {
   unsigned int counter[4];  // last-block counters, reset by the last block
 };
 
+// the flag as the kernel ahead left it (not from a cache of invariant data)
+__device__ __forceinline__ bool is_done(const SolverState* st) {
+  return *reinterpret_cast<const volatile int*>(&st->done) != 0;
+}
+
 // Per-thread accumulator for inner products.  FP64 fields: plain double sum.
 // FP32 fields: Kahan-compensated float sum (the FP64 pipe of GB300 is 64x
 // slower than the FP32 one), handed to the FP64 block / grid reduction.

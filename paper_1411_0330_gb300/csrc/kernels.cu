@@ -23,6 +23,7 @@
 #include "fft.cuh"
 #include "internal.h"
 #include "gamma_onfly.cuh"
+#include "tma.cuh"
 
 namespace lsh {
 
@@ -103,7 +104,6 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_xfwd(OpArgs<T
                                                    const T* __restrict__ r, T* __restrict__ p,
                                                    const SolverState* __restrict__ st) {
   const int s = blockIdx.x / a.bps;
-  if (MODE == 1 && st[s].done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2<T>* tw = reinterpret_cast<C2<T>*>(smem_raw);
   C2<T>* Z = tw + a.nx;
@@ -113,6 +113,8 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_xfwd(OpArgs<T
     tw[i] = a.twx[i];
     pos[i] = a.posx[i];
   }
+  chain_wait();
+  if (MODE == 1 && is_done(st + s)) return;
   const int rloc = (blockIdx.x - s * a.bps) * a.RY;  // first row inside the system
   const int nr = a.RY;
   const int npair = (nr + 1) >> 1;
@@ -189,11 +191,12 @@ template <typename T, bool INV>
 __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_yfft(OpArgs<T> a, const SolverState* __restrict__ st) {
   const long long plane = blockIdx.y;
   const int s = (int)(plane / (a.c * a.nz));
-  if (st != nullptr && st[s].done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2<T>* tw = reinterpret_cast<C2<T>*>(smem_raw);
   C2<T>* buf = tw + a.ny;
   for (int i = threadIdx.x; i < a.ny; i += blockDim.x) tw[i] = a.twy[i];
+  chain_wait();
+  if (st != nullptr && is_done(st + s)) return;
   const int kx0 = blockIdx.x * a.TY;
   const int nt = min(a.TY, a.nxh - kx0);
   const int TY = a.TY;
@@ -230,11 +233,12 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_yfft(OpArgs<T
 template <typename T, int NC>
 __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_zgamma(OpArgs<T> a, const SolverState* __restrict__ st) {
   const int s = blockIdx.x;
-  if (st != nullptr && st[s].done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2<T>* tw = reinterpret_cast<C2<T>*>(smem_raw);
   C2<T>* buf = tw + a.nz;
   for (int i = threadIdx.x; i < a.nz; i += blockDim.x) tw[i] = a.twz[i];
+  chain_wait();
+  if (st != nullptr && is_done(st + s)) return;
   const int yp = blockIdx.z;
   const int kx0 = blockIdx.y * a.TZ;
   const int nt = min(a.TZ, a.nxh - kx0);
@@ -297,7 +301,8 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_zgamma(OpArgs
 template <typename T, int NC>
 __global__ void __launch_bounds__(kThreads) k_gamma2d(OpArgs<T> a, const SolverState* __restrict__ st) {
   const int s = blockIdx.z;
-  if (st != nullptr && st[s].done) return;
+  chain_wait();
+  if (st != nullptr && is_done(st + s)) return;
   const int kx = blockIdx.x * blockDim.x + threadIdx.x, yp = blockIdx.y * blockDim.y + threadIdx.y;
   if (kx >= a.nxh || yp >= a.ny) return;
   const long long cstride = (long long)a.ny * a.hs;
@@ -326,7 +331,6 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_xinv(OpArgs<T
                                                                         SolverState* __restrict__ st,
                                                                         double* __restrict__ partials) {
   const int s = blockIdx.x / a.bps;
-  if ((MODE == 1 || MODE == 3) && st[s].done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ T mloc[256 * 6];  // local coefficients (no scale field) or A_phase diagonal
   __shared__ unsigned char aloc[256];
@@ -341,6 +345,8 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_xinv(OpArgs<T
   const int ntab = a.nphase * a.c;
   for (int i = threadIdx.x; i < ntab; i += blockDim.x) mloc[i] = (a.scale && !a.frac) ? a.modtab[i] : a.mtab[i];
   for (int i = threadIdx.x; i < a.nphase; i += blockDim.x) aloc[i] = a.act[i];
+  chain_wait();
+  if ((MODE == 1 || MODE == 3) && is_done(st + s)) return;
   __syncthreads();
   const int blk = blockIdx.x - s * a.bps;
   const int rloc = blk * a.RY;
@@ -825,15 +831,15 @@ __global__ void __launch_bounds__(kThreads) k_cg_update(OpArgs<T> a, T* __restri
                                                         long long off2) {
   const int s = blockIdx.y;
   SolverState* sst = st + s;
-  if (sst->done) return;
   __shared__ T dloc[PRE == 1 ? 256 * 6 : 1], eloc[PRE == 1 ? 256 * 6 : 1];
-  if (PRE == 1) {
+  if (PRE == 1)
     for (int i = threadIdx.x; i < a.nphase * a.c; i += blockDim.x) {
       dloc[i] = a.dtab[i];
       eloc[i] = a.etab[i];
     }
-    __syncthreads();
-  }
+  chain_wait();
+  if (is_done(sst)) return;
+  __syncthreads();
   const T al = (T)sst->alpha;
   const long long n = (long long)a.c * a.V;
   T* rs = r + s * n;
@@ -1427,7 +1433,7 @@ void launch_xfwd(const OpArgs<T>& a, const LaunchCfg& L, int mode, const T* in, 
   }
   const int grid = a.S * a.bps;
   constexpr int VV = 16 / sizeof(T);
-#define LSH_XFWD(MODE, VEC) k_xfwd<T, MODE, VEC><<<grid, L.thr_x, L.smem_x, s>>>(a, in, x, r, p, st)
+#define LSH_XFWD(MODE, VEC) launch_dep(a.pdl != 0, k_xfwd<T, MODE, VEC>, dim3(grid), dim3(L.thr_x), L.smem_x, s, a, in, x, r, p, st)
   if (L.VEC == VV) {
     if (mode == 0) LSH_XFWD(0, VV);
     else LSH_XFWD(1, VV);
@@ -1455,8 +1461,7 @@ void launch_yfft(const OpArgs<T>& a, const LaunchCfg& L, bool inv, const SolverS
     return;
   }
   dim3 g(L.grid_yx, a.S * a.c * a.nz);
-  if (inv) k_yfft<T, true><<<g, L.thr_y, L.smem_y, s>>>(a, st);
-  else k_yfft<T, false><<<g, L.thr_y, L.smem_y, s>>>(a, st);
+  launch_dep(a.pdl != 0, inv ? k_yfft<T, true> : k_yfft<T, false>, g, dim3(L.thr_y), L.smem_y, s, a, st);
 }
 
 template <typename T>
@@ -1475,14 +1480,12 @@ void launch_zgamma(const OpArgs<T>& a, const LaunchCfg& L, const SolverState* st
   }
   if (a.nz == 1 && a.c != 6) {
     const dim3 b(32, kThreads / 32), g2((a.nxh + 31) / 32, (a.ny + b.y - 1) / b.y, a.S);
-    if (a.c == 3) k_gamma2d<T, 3><<<g2, b, 0, s>>>(a, st);
-    else k_gamma2d<T, 2><<<g2, b, 0, s>>>(a, st);
+    launch_dep(a.pdl != 0, a.c == 3 ? k_gamma2d<T, 3> : k_gamma2d<T, 2>, g2, b, 0, s, a, st);
     return;
   }
   dim3 g(a.S, L.grid_zx, L.grid_zy);
-  if (a.c == 6) k_zgamma<T, 6><<<g, L.thr_z, L.smem_z, s>>>(a, st);
-  else if (a.c == 3) k_zgamma<T, 3><<<g, L.thr_z, L.smem_z, s>>>(a, st);
-  else k_zgamma<T, 2><<<g, L.thr_z, L.smem_z, s>>>(a, st);
+  launch_dep(a.pdl != 0, a.c == 6 ? k_zgamma<T, 6> : (a.c == 3 ? k_zgamma<T, 3> : k_zgamma<T, 2>), g, dim3(L.thr_z),
+             L.smem_z, s, a, st);
 }
 
 template <typename T>
@@ -1494,7 +1497,8 @@ void launch_xinv(const OpArgs<T>& a, const LaunchCfg& L, int mode, const T* xin,
   }
   const int grid = a.S * a.bps;
   constexpr int VV = 16 / sizeof(T);
-#define LSH_XINV(MODE, VEC) k_xinv<T, MODE, VEC><<<grid, L.thr_x, L.smem_x, s>>>(a, xin, out, st, partials)
+#define LSH_XINV(MODE, VEC) \
+  launch_dep(a.pdl != 0, k_xinv<T, MODE, VEC>, dim3(grid), dim3(L.thr_x), L.smem_x, s, a, xin, out, st, partials)
 #define LSH_XINV_MODES(VEC)                              \
   do {                                                   \
     if (mode == 0) LSH_XINV(0, VEC);                     \
@@ -1555,9 +1559,8 @@ template <typename T>
 void launch_cg_update(const OpArgs<T>& a, T* r, const T* q, SolverState* st, double* partials, long long off2, int G,
                       cudaStream_t s) {
   const dim3 g(G, a.S);
-  if (a.pre == 0) k_cg_update<T, 0><<<g, kThreads, 0, s>>>(a, r, q, st, partials, off2);
-  else if (a.pre == 1) k_cg_update<T, 1><<<g, kThreads, 0, s>>>(a, r, q, st, partials, off2);
-  else k_cg_update<T, 2><<<g, kThreads, 0, s>>>(a, r, q, st, partials, off2);
+  launch_dep(a.pdl != 0, a.pre == 0 ? k_cg_update<T, 0> : (a.pre == 1 ? k_cg_update<T, 1> : k_cg_update<T, 2>), g,
+             dim3(kThreads), 0, s, a, r, q, st, partials, off2);
 }
 template <typename T>
 void launch_cg_finalize(T* x, const T* p, long long n, int S, const SolverState* st, int G, cudaStream_t s) {

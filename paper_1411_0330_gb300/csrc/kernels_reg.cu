@@ -28,6 +28,7 @@ __global__ void __launch_bounds__(16 * RegPlan<N>::P) k_yfft_reg(OpArgs<T> a, co
   C2<T>* tw = reinterpret_cast<C2<T>*>(smem_raw);
   C2<T>* ex = tw + N;
   for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = a.twy[i];
+  chain_wait();
   const int i = threadIdx.x % TY, t = threadIdx.x / TY;
   const long long nplanes = (long long)a.S * a.c * a.nz;
   const int nleft = a.nxh - nreg;
@@ -37,13 +38,13 @@ __global__ void __launch_bounds__(16 * RegPlan<N>::P) k_yfft_reg(OpArgs<T> a, co
   if ((long long)blockIdx.x < nplanes * nrt) {
     plane = blockIdx.x / nrt;
     kx = (int)(blockIdx.x - plane * nrt) * TY + i;
-    if (st != nullptr && st[plane / (a.c * a.nz)].done) return;  // uniform: one plane per block
+    if (st != nullptr && is_done(st + plane / (a.c * a.nz))) return;  // uniform: one plane per block
   } else {
     const long long l = (blockIdx.x - nplanes * nrt) * (long long)TY + i;
     valid = l < nplanes * nleft;
     plane = valid ? l / nleft : 0;
     kx = valid ? nreg + (int)(l - plane * nleft) : 0;
-    if (valid && st != nullptr && st[plane / (a.c * a.nz)].done) valid = false;
+    if (valid && st != nullptr && is_done(st + plane / (a.c * a.nz))) valid = false;
   }
   C2<T>* __restrict__ Hl = a.H + plane * a.ny * a.hs + kx;
   const int rs = a.hs;  // row stride
@@ -198,8 +199,9 @@ __global__ void __launch_bounds__(ZCfg<T, NC, N, TZV>::THREADS,
     s = blockIdx.x;
     tile = blockIdx.y;
   }
-  if (st != nullptr && st[s].done) return;
   for (int u = threadIdx.x; u < N; u += blockDim.x) tw[u] = a.twz[u];
+  chain_wait();
+  if (st != nullptr && is_done(st + s)) return;
   if (threadIdx.x < TZ) {
     const int i = threadIdx.x;
     int yp = -1, kx = 0;
@@ -435,7 +437,7 @@ template <typename T, bool INV, int N> void launch_y_n(const OpArgs<T>& a, const
   const long long nleft_lines = nplanes * (a.nxh - nreg);
   const long long grid = nplanes * nrt + (nleft_lines + TY - 1) / TY;
   const size_t smem = sizeof(C2<T>) * (N + TY * RegLine<T, N>::LS);
-  k_yfft_reg<T, INV, N><<<(unsigned)grid, TY * RegPlan<N>::P, smem, s>>>(a, st, nrt, nreg);
+  launch_dep(a.pdl != 0, k_yfft_reg<T, INV, N>, dim3((unsigned)grid), dim3(TY * RegPlan<N>::P), smem, s, a, st, nrt, nreg);
 }
 
 template <typename T, bool INV> void launch_y_reg(const OpArgs<T>& a, const SolverState* st, cudaStream_t s) {
@@ -474,9 +476,10 @@ template <typename T, int NC, int N, int TZV> void launch_z_n(const OpArgs<T>& a
   const int ntiles = a.ny * nrt + (a.ny * (a.nxh - nreg) + ZC::TZ - 1) / ZC::TZ;
   const size_t smem = sizeof(C2<T>) * (N + ZC::BUF);
   if (a.tlay)
-    k_zgamma_reg<T, NC, N, TZV><<<(unsigned)((long long)a.S * ntiles), ZC::THREADS, smem, s>>>(a, st, nrt, nreg);
+    launch_dep(a.pdl != 0, k_zgamma_reg<T, NC, N, TZV>, dim3((unsigned)((long long)a.S * ntiles)), dim3(ZC::THREADS), smem,
+               s, a, st, nrt, nreg);
   else
-    k_zgamma_reg<T, NC, N, TZV><<<dim3(a.S, ntiles), ZC::THREADS, smem, s>>>(a, st, nrt, nreg);
+    launch_dep(a.pdl != 0, k_zgamma_reg<T, NC, N, TZV>, dim3(a.S, ntiles), dim3(ZC::THREADS), smem, s, a, st, nrt, nreg);
 }
 
 template <typename T, int NC, int TZV> void launch_z_nc(const OpArgs<T>& a, const SolverState* st, cudaStream_t s) {

@@ -734,6 +734,7 @@ template <typename T> OpArgs<T> wave_args(lsh_handle* h, const Wave& w) {
   a.bps = a.rps / a.RY;
   a.TY = L.TY;
   a.TZ = L.TZ;
+  a.pdl = 1;
   return a;
 }
 
@@ -830,27 +831,27 @@ lsh_status residual64(lsh_handle* h, const OpArgs<double>& a, const double* x, d
   return last_launch();
 }
 
-template <typename T> void enqueue_cg_iteration(lsh_handle* h, PrecBufs<T>& P, const OpArgs<T>& a) {
+template <typename T> void enqueue_cg_iteration(lsh_handle* h, PrecBufs<T>& P, const OpArgs<T>& wave) {
   cudaStream_t s = h->stream;
   const bool timed = h->prof_now && h->ev_used + 7 <= (int)h->ev.size();
+  OpArgs<T> a = wave;
+  if (timed) a.pdl = 0;  // events between the kernels
   cudaEvent_t* e = timed ? &h->ev[h->ev_used] : nullptr;
   // inside a capture the records become graph nodes that record at replay
   const unsigned rf = h->capturing ? cudaEventRecordExternal : cudaEventRecordDefault;
   if constexpr (sizeof(T) == 4) {
     if (a.plane && a.fuse) {
       // five launches: xy forward, z, alpha, xy inverse with the update of z, beta; each
-      // is set up while the one ahead drains (not with events between them)
-      OpArgs<T> b = a;
-      b.pdl = timed ? 0 : 1;
+      // is set up while the one ahead drains
       if (timed) cudaEventRecordWithFlags(e[0], s, rf);
-      launch_xyfwd(b, 1, nullptr, P.x, P.r, P.p, P.st, s);
+      launch_xyfwd(a, 1, nullptr, P.x, P.r, P.p, P.st, s);
       if (timed) cudaEventRecordWithFlags(e[1], s, rf);
       if (timed) cudaEventRecordWithFlags(e[2], s, rf);
-      launch_zgamma_pipe(b, true, P.st, s, h->partials);
+      launch_zgamma_pipe(a, true, P.st, s, h->partials);
       if (timed) cudaEventRecordWithFlags(e[3], s, rf);
       if (timed) cudaEventRecordWithFlags(e[4], s, rf);
-      launch_cg_alpha(P.st, h->partials, zdot_count(b), b.S, b.pdl != 0, s);
-      launch_xyinv_update(b, P.p, P.r, P.st, h->partials, h->lay.nparts, s);
+      launch_cg_alpha(P.st, h->partials, zdot_count(a), a.S, a.pdl != 0, s);
+      launch_xyinv_update(a, P.p, P.r, P.st, h->partials, h->lay.nparts, s);
       if (timed) {
         cudaEventRecordWithFlags(e[5], s, rf);
         cudaEventRecordWithFlags(e[6], s, rf);
