@@ -85,6 +85,7 @@ template <typename T> struct OpArgs {
   int onfly;                   // 1: compute Gamma^h_k on the fly
   int fdphase;                 // finite-difference operator: the table holds the real part
                                // u u^T / (u^T A0 u); components rotate by -/+ pi k_i / N_i around it
+  const C2<T>* fdw;            // its factors (cos, sin)(pi k / N), x then y then z (null: computed)
   int physics;
   const int* kofy;             // y position -> frequency
   const int* kofz;             // z position -> frequency

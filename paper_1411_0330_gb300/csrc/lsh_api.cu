@@ -323,6 +323,7 @@ struct Layout {
   size_t off_state, off_partials, off_phase, off_scale, off_act, off_posx, off_kofy, off_kofz, off_sums, off_W;
   size_t off_tabd, off_tabf, off_loads_d, off_loads_f, off_bb, off_flags, off_fault, off_prof;
   size_t off_tw_d, off_tw_f;
+  size_t off_fd_d, off_fd_f;      // finite-difference phase factors
   size_t off_fd[4], off_Hd, off_gd;
   size_t off_ff[4], off_Hf, off_gf;
   size_t off_wa, off_wb, off_ms;  // MINRES: two direction fields (FP64) and per-system scalars
@@ -393,6 +394,8 @@ Layout make_layout(const Derived& d) {
   l.off_prof = take(6 * sizeof(unsigned long long));
   l.off_tw_d = take(sizeof(double2) * (size_t)(d.nx + d.ny + d.nz));
   l.off_tw_f = take(sizeof(float2) * (size_t)(d.nx + d.ny + d.nz));
+  l.off_fd_d = take(d.green == LSH_GREEN_FD ? sizeof(double2) * (size_t)(d.nx + d.ny + d.nz) : 0);
+  l.off_fd_f = take(d.green == LSH_GREEN_FD ? sizeof(float2) * (size_t)(d.nx + d.ny + d.nz) : 0);
   // FP64 fields: x, r always; p, q for the FP64 CG (one system's worth of p, q
   // suffices for the Mandel rotations of lsh_apply on a mixed handle)
   const bool mixed = d.precision == LSH_MIXED;
@@ -598,6 +601,7 @@ void init_prec(lsh_handle* h, PrecBufs<T>& P, const size_t* off_f, size_t off_H,
   // FP32 truncated operator: computed on the fly in the z pass (no table read)
   a.onfly = (sizeof(T) == 4 && d.green == LSH_GREEN_TRUNCATED && !d.rotated) ? 1 : 0;
   a.fdphase = d.green == LSH_GREEN_FD ? 1 : 0;
+  a.fdw = a.fdphase ? (const C2<T>*)(b + (sizeof(T) == 8 ? h->lay.off_fd_d : h->lay.off_fd_f)) : nullptr;
   a.physics = d.physics;
   a.kofy = h->kofy;
   a.kofz = h->kofz;
@@ -789,6 +793,7 @@ OpArgs<DF> df_args(lsh_handle* h, const OpArgs<double>& a) {
   b.invV = DF(a.invV);
   b.onfly = 0;
   b.fdphase = 0;
+  b.fdw = nullptr;
   return b;
 }
 
@@ -1518,6 +1523,17 @@ lsh_status lsh_setup(const lsh_problem* prob, void* workspace, size_t bytes, voi
   twiddles<double>(d.nz, tmpd); twd.insert(twd.end(), tmpd.begin(), tmpd.end());
   std::vector<float> twf(twd.size());
   for (size_t i = 0; i < twd.size(); ++i) twf[i] = (float)twd[i];
+  std::vector<double> fdd;
+  std::vector<float> fdf;
+  if (d.green == LSH_GREEN_FD) {
+    for (int n : {d.nx, d.ny, d.nz})
+      for (int k = 0; k < n; ++k) {
+        const long double t = 3.141592653589793238462643383279502884L * (long double)k / (long double)n;
+        fdd.push_back((double)cosl(t));
+        fdd.push_back((double)sinl(t));
+      }
+    for (double v : fdd) fdf.push_back((float)v);
+  }
   std::vector<double> tabd(2 * 256 * 6, 0.0);
   std::vector<float> tabf(2 * 256 * 6, 0.0f);
   for (int ph = 0; ph < d.nphase; ++ph)
@@ -1539,6 +1555,10 @@ lsh_status lsh_setup(const lsh_problem* prob, void* workspace, size_t bytes, voi
   SETUP_CK(cudaMemcpyAsync(h->kofz32, kofz32.data(), sizeof(int) * d.nz, cudaMemcpyHostToDevice, st));
   SETUP_CK(cudaMemcpyAsync(h->base + l.off_tw_d, twd.data(), sizeof(double) * twd.size(), cudaMemcpyHostToDevice, st));
   SETUP_CK(cudaMemcpyAsync(h->base + l.off_tw_f, twf.data(), sizeof(float) * twf.size(), cudaMemcpyHostToDevice, st));
+  if (!fdd.empty()) {
+    SETUP_CK(cudaMemcpyAsync(h->base + l.off_fd_d, fdd.data(), sizeof(double) * fdd.size(), cudaMemcpyHostToDevice, st));
+    SETUP_CK(cudaMemcpyAsync(h->base + l.off_fd_f, fdf.data(), sizeof(float) * fdf.size(), cudaMemcpyHostToDevice, st));
+  }
   SETUP_CK(cudaMemcpyAsync(h->base + l.off_tabd, tabd.data(), sizeof(double) * tabd.size(), cudaMemcpyHostToDevice, st));
   SETUP_CK(cudaMemcpyAsync(h->base + l.off_tabf, tabf.data(), sizeof(float) * tabf.size(), cudaMemcpyHostToDevice, st));
   if (copy_microstructure(h, prob->phase, prob->scale, prob->phase_on_host) != LSH_OK) { delete h; return LSH_ERR_CUDA; }
