@@ -127,7 +127,7 @@ __device__ __forceinline__ void fd_rotate(const OpArgs<T>& a, int kx, int ky, in
   for (int i = 0; i < NC && i < 3; ++i) {
     T s, c;
     if (a.fdw) {
-      // tabulated (96 x 80 x 64 in FP64: sine and cosine were two thirds of the z pass's 187 us)
+      // tabulated (96 x 80 x 64 in FP64: sine and cosine were most of the z pass's 187 us)
       const C2<T> w = a.fdw[(i == 0 ? 0 : (i == 1 ? a.nx : a.nx + a.ny)) + kk[i]];
       c = w.x;
       s = w.y;

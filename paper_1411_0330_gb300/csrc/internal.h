@@ -119,8 +119,11 @@ template <typename T> struct OpArgs {
   C2<T>* nq;
   int mandel;  // apply on the plane passes: fields are Mandel components, the z pass takes
                // the internal basis around Gamma^h and the local term couples the normals
+  double* dot; // FP32 z passes: each block's share of (p, Gamma p), zdot_blocks() of them per
+               // system (null: not wanted)
   int pdl;     // the kernels of the fused plane iteration start before the one ahead has drained
-  int fuse;  // plane passes with z variant 11: the CG update runs in the inverse pass
+  int fuse;  // the CG update runs in the inverse pass: plane passes with z variant 11; other
+             // grids with the shared-memory inverse x pass and z variants 0 and 9
   int l2pf;  // plane passes, input planes requested into L2 at a block's start: bit 0 the
              // forward pass's x, r, p; bit 1 the inverse pass's p and phase planes
 };
@@ -284,6 +287,11 @@ void launch_scale_grad(const double* tau_all, const double* W, const unsigned ch
                        const double* modtab, const double* ref, int c, int elastic, long long V, int B,
                        double* grad, cudaStream_t s);
 
+// FP32 CG iteration of the separate passes with the update of z in the inverse x pass
+int zdot_blocks(const OpArgs<float>& a, const LaunchCfg& L);
+void launch_xinv_update(const OpArgs<float>& a, const LaunchCfg& L, const float* p, float* z, SolverState* st,
+                        double* partials, long long off, cudaStream_t s);
+void launch_cg_beta(SolverState* st, const double* partials, long long off, int nb, int S, bool pdl, cudaStream_t s);
 void launch_dot_finalize(SolverState* st, const double* partials, int nb, int S, cudaStream_t s);
 void launch_basic_update(const OpArgs<double>& a, double* x, const double* r, const unsigned char* flags, int G,
                          cudaStream_t s);

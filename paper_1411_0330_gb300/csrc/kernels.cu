@@ -269,6 +269,7 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_zgamma(OpArgs
   __syncthreads();
   if (nz > 1) fft_lines<T, false>(buf, NC * TZ, a.lsz, a.pz, tw);
   // per-frequency product with Gamma^h_k
+  Acc<float> accd;
   const int ky = (a.onfly || a.fdphase) ? a.kofy[yp] : 0;
   for (int idx = threadIdx.x; idx < nz * TZ; idx += blockDim.x) {
     const int zp = dtz.div(idx), t = idx - zp * TZ;
@@ -283,9 +284,26 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_zgamma(OpArgs
       gamma_table_apply<T, NC>(a.gtab, ((long long)zp * a.ny + yp) * a.ts + kx0 + t, v);
       if (a.fdphase) fd_rotate<T, NC>(a, kx0 + t, ky, a.kofz[zp], v, (T)1);
     }
+    if constexpr (sizeof(T) == 4)
+      if (a.dot) {
+        T q = 0;
+#pragma unroll
+        for (int i = 0; i < NC; ++i) {
+          const C2<T> u = buf[(i * TZ + t) * a.lsz + zp];
+          q += u.x * v[i].x + u.y * v[i].y;
+        }
+        accd.add((kx0 + t == 0 || 2 * (kx0 + t) == a.nx) ? q : q + q);
+      }
 #pragma unroll
     for (int i = 0; i < NC; ++i) buf[(i * TZ + t) * a.lsz + zp] = v[i];
   }
+  if constexpr (sizeof(T) == 4)
+    if (a.dot) {
+      // the block's share of (p, Gamma p) (see k_xinv, MODE 5)
+      const double d = block_reduce(accd);
+      if (threadIdx.x == 0)
+        a.dot[((long long)s * gridDim.z + blockIdx.z) * gridDim.y + blockIdx.y] = d;
+    }
   __syncthreads();
   if (nz > 1) fft_lines<T, true>(buf, NC * TZ, a.lsz, a.pz, tw);
   for (int idx = threadIdx.x; idx < tot; idx += blockDim.x) {
@@ -303,37 +321,52 @@ __global__ void __launch_bounds__(kThreads) k_gamma2d(OpArgs<T> a, const SolverS
   const int s = blockIdx.z;
   chain_wait();
   if (st != nullptr && is_done(st + s)) return;
-  const int kx = blockIdx.x * blockDim.x + threadIdx.x, yp = blockIdx.y * blockDim.y + threadIdx.y;
-  if (kx >= a.nxh || yp >= a.ny) return;
-  const long long cstride = (long long)a.ny * a.hs;
-  C2<T>* __restrict__ Hp = a.H + (long long)s * NC * cstride + (long long)yp * a.hs + kx;
-  C2<T> v[NC];
+  const int kx = blockIdx.x * 32 + (threadIdx.x & 31), yp = blockIdx.y * (kThreads / 32) + (threadIdx.x >> 5);
+  Acc<float> accd;
+  if (kx < a.nxh && yp < a.ny) {
+    const long long cstride = (long long)a.ny * a.hs;
+    C2<T>* __restrict__ Hp = a.H + (long long)s * NC * cstride + (long long)yp * a.hs + kx;
+    C2<T> v[NC], u[NC];
 #pragma unroll
-  for (int i = 0; i < NC; ++i) v[i] = Hp[i * cstride];
-  if (a.onfly) {
-    gamma_trunc_onfly<T, NC>(a, kx, a.kofy[yp], 0, v);
-  } else {
-    const int ky = a.fdphase ? a.kofy[yp] : 0;
-    if (a.fdphase) fd_rotate<T, NC>(a, kx, ky, 0, v, (T)-1);
-    gamma_table_apply<T, NC>(a.gtab, (long long)yp * a.ts + kx, v);
-    if (a.fdphase) fd_rotate<T, NC>(a, kx, ky, 0, v, (T)1);
+    for (int i = 0; i < NC; ++i) v[i] = u[i] = Hp[i * cstride];
+    if (a.onfly) {
+      gamma_trunc_onfly<T, NC>(a, kx, a.kofy[yp], 0, v);
+    } else {
+      const int ky = a.fdphase ? a.kofy[yp] : 0;
+      if (a.fdphase) fd_rotate<T, NC>(a, kx, ky, 0, v, (T)-1);
+      gamma_table_apply<T, NC>(a.gtab, (long long)yp * a.ts + kx, v);
+      if (a.fdphase) fd_rotate<T, NC>(a, kx, ky, 0, v, (T)1);
+    }
+    T q = 0;
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+      q += u[i].x * v[i].x + u[i].y * v[i].y;
+      Hp[i * cstride] = v[i];
+    }
+    if (sizeof(T) == 4) accd.add((float)((kx == 0 || 2 * kx == a.nx) ? q : q + q));
   }
-#pragma unroll
-  for (int i = 0; i < NC; ++i) Hp[i * cstride] = v[i];
+  if constexpr (sizeof(T) == 4)
+    if (a.dot) {
+      const double d = block_reduce(accd);
+      if (threadIdx.x == 0) a.dot[((long long)s * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = d;
+    }
 }
 
 // ------------------------------------------------------------------ x inverse + local term
 // MODE 0: out = P (M xin + g).  MODE 1 (CG): q = P (M p + g), (p, q) -> alpha.
 // MODE 2 (residual): out = P (load - M xin - g), (r, r) -> st[s].aux[0].
+// MODE 5 (FP32 CG, alpha known from the z pass): q = P (M p + g) is not stored, out = z is
+// updated, z -= alpha D q, and the four sums of k_cg_beta go to partials + {0, 1, 2, 3} off.
 template <typename T, int MODE, int VEC>
 __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_xinv(OpArgs<T> a, const T* __restrict__ xin,
                                                                         T* __restrict__ out,
                                                                         SolverState* __restrict__ st,
-                                                                        double* __restrict__ partials) {
+                                                                        double* __restrict__ partials, long long off) {
   const int s = blockIdx.x / a.bps;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ T mloc[256 * 6];  // local coefficients (no scale field) or A_phase diagonal
   __shared__ unsigned char aloc[256];
+  __shared__ T dloc[MODE == 5 ? 256 * 6 : 1], eloc[MODE == 5 ? 256 * 6 : 1];
   C2<T>* tw = reinterpret_cast<C2<T>*>(smem_raw);
   C2<T>* Z = tw + a.nx;
   int* pos = reinterpret_cast<int*>(Z + ((a.RY + 1) >> 1) * a.lsx);
@@ -342,12 +375,18 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_xinv(OpArgs<T
     tw[i] = a.twx[i];
     pos[i] = a.posx[i];
   }
+  if (MODE == 5)
+    for (int i = threadIdx.x; i < a.nphase * a.c; i += blockDim.x) {
+      dloc[i] = a.pre == 1 ? a.dtab[i] : (T)1;
+      eloc[i] = a.pre == 1 ? a.etab[i] : (T)1;
+    }
   const int ntab = a.nphase * a.c;
   for (int i = threadIdx.x; i < ntab; i += blockDim.x) mloc[i] = (a.scale && !a.frac) ? a.modtab[i] : a.mtab[i];
   for (int i = threadIdx.x; i < a.nphase; i += blockDim.x) aloc[i] = a.act[i];
   chain_wait();
-  if ((MODE == 1 || MODE == 3) && is_done(st + s)) return;
+  if ((MODE == 1 || MODE == 3 || MODE == 5) && is_done(st + s)) return;
   __syncthreads();
+  const T al = MODE == 5 ? (T)*const_cast<const volatile double*>(&st[s].alpha) : (T)0;
   const int blk = blockIdx.x - s * a.bps;
   const int rloc = blk * a.RY;
   const int nr = a.RY;
@@ -385,12 +424,12 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_xinv(OpArgs<T
   const long long pbase = (long long)((a.sys0 + s) / a.sys_per_ms) * a.V;
   const int nxv = nx / VEC;
   const FastDiv dxv(nxv);
-  Acc<T> acc;
+  Acc<T> acc, accz, accm, accp;
   for (int idx = threadIdx.x; idx < npair * nxv; idx += blockDim.x) {
     const int lp = dxv.div(idx);
     const int xx = (idx - lp * nxv) * VEC;
     // issue every global load of the row pair first
-    T xv[2][VEC];
+    T xv[2][VEC], zv[2][VEC];
     unsigned char ph[2][VEC];
     int comp[2];
     long long voxs[2];
@@ -401,6 +440,7 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_xinv(OpArgs<T
       voxs[h2] = pbase + vox;
       if (row < nr) {
         vload<T, VEC>(xin + (row0 + row) * nx + xx, xv[h2]);
+        if (MODE == 5) vload<T, VEC>(out + (row0 + row) * nx + xx, zv[h2]);
         if constexpr (VEC == 4) {
           const uchar4 q = *reinterpret_cast<const uchar4*>(a.phase + pbase + vox);
           ph[h2][0] = q.x; ph[h2][1] = q.y; ph[h2][2] = q.z; ph[h2][3] = q.w;
@@ -435,7 +475,18 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_xinv(OpArgs<T
         }
         const T gv = h2 ? zc[u].y : zc[u].x;
         const T xq = xv[h2][u];
-        if (MODE == 0) {
+        if (MODE == 5) {
+          const int k = p * a.c + comp[h2];
+          const T e = a.mfld ? (a.pre ? fabs(m) + a.gpre[comp[h2]] : (T)1) : eloc[k];
+          const T d = a.mfld ? (T)1 / e : dloc[k];
+          const T q = active ? m * xq + gv : (T)0;
+          const T z = zv[h2][u] - al * (d * q), r = z * e, zm = z * m;
+          ov[u] = z;
+          acc.add(r * r);
+          accz.add(r * z);
+          accm.add(zm * z);
+          accp.add(zm * xq);
+        } else if (MODE == 0) {
           ov[u] = active ? m * xq + gv : (T)0;
         } else if (MODE == 1 || MODE == 3) {
           ov[u] = active ? m * xq + gv : (T)0;
@@ -448,7 +499,18 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_xinv(OpArgs<T
       vstore<T, VEC>(out + g, ov);
     }
   }
-  if (MODE != 0) {
+  if constexpr (MODE == 5) {
+    double* part = partials + (long long)s * a.bps + blk;
+    auto store = [&](const Acc<T>& v, long long at) {
+      const double tot = block_reduce(v);
+      if (threadIdx.x == 0) part[at] = tot;
+      __syncthreads();
+    };
+    store(acc, 0);
+    store(accz, off);
+    store(accm, 2 * off);
+    store(accp, 3 * off);
+  } else if (MODE != 0) {
     const double tot = block_reduce(acc);
     double* part = partials + (long long)s * a.bps;
     SolverState* sst = st + s;
@@ -1227,7 +1289,7 @@ __global__ void __launch_bounds__(kThreads) k_d2f_begin(OpArgs<float> a, const d
   float* x32s = x32 + s * n;
   const long long pbase = (long long)((a.sys0 + s) / a.sys_per_ms) * a.V;
   Acc<float> acc, accz, accm;
-  const bool zmz = a.plane && a.fuse;  // (z, M z) for the fused plane schedule
+  const bool zmz = a.fuse != 0;  // (z, M z) for the iterations whose inverse pass updates z
   sweep_planes<float>(a.c, a.V, [&](int comp, long long i, auto vec) {
     constexpr int VEC = decltype(vec)::value;
     const long long g = comp * a.V + i;
@@ -1406,6 +1468,8 @@ template <typename T, int VEC> void set_smem_attrs_x(int mx) {
   cudaFuncSetAttribute(k_xfwd<T, 1, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
   cudaFuncSetAttribute(k_xinv<T, 0, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
   cudaFuncSetAttribute(k_xinv<T, 1, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+  if constexpr (sizeof(T) == 4)  // less its larger static tables
+    cudaFuncSetAttribute(k_xinv<T, 5, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx - 24 * 1024);
   if constexpr (sizeof(T) == 8) {
     cudaFuncSetAttribute(k_xinv<T, 2, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
     cudaFuncSetAttribute(k_xinv<T, 3, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
@@ -1479,8 +1543,8 @@ void launch_zgamma(const OpArgs<T>& a, const LaunchCfg& L, const SolverState* st
     return;
   }
   if (a.nz == 1 && a.c != 6) {
-    const dim3 b(32, kThreads / 32), g2((a.nxh + 31) / 32, (a.ny + b.y - 1) / b.y, a.S);
-    launch_dep(a.pdl != 0, a.c == 3 ? k_gamma2d<T, 3> : k_gamma2d<T, 2>, g2, b, 0, s, a, st);
+    const dim3 g2((a.nxh + 31) / 32, (a.ny + kThreads / 32 - 1) / (kThreads / 32), a.S);
+    launch_dep(a.pdl != 0, a.c == 3 ? k_gamma2d<T, 3> : k_gamma2d<T, 2>, g2, dim3(kThreads), 0, s, a, st);
     return;
   }
   dim3 g(a.S, L.grid_zx, L.grid_zy);
@@ -1498,7 +1562,7 @@ void launch_xinv(const OpArgs<T>& a, const LaunchCfg& L, int mode, const T* xin,
   const int grid = a.S * a.bps;
   constexpr int VV = 16 / sizeof(T);
 #define LSH_XINV(MODE, VEC) \
-  launch_dep(a.pdl != 0, k_xinv<T, MODE, VEC>, dim3(grid), dim3(L.thr_x), L.smem_x, s, a, xin, out, st, partials)
+  launch_dep(a.pdl != 0, k_xinv<T, MODE, VEC>, dim3(grid), dim3(L.thr_x), L.smem_x, s, a, xin, out, st, partials, 0LL)
 #define LSH_XINV_MODES(VEC)                              \
   do {                                                   \
     if (mode == 0) LSH_XINV(0, VEC);                     \
@@ -1513,6 +1577,22 @@ void launch_xinv(const OpArgs<T>& a, const LaunchCfg& L, int mode, const T* xin,
   else LSH_XINV_MODES(1);
 #undef LSH_XINV_MODES
 #undef LSH_XINV
+}
+
+int zdot_blocks(const OpArgs<float>& a, const LaunchCfg& L) {
+  if (a.zreg) {
+    const int TZ = a.nz >= 256 ? 4 : 8, nrt = a.nxh / TZ;  // z variants 0 and 9
+    return a.ny * nrt + (a.ny * (a.nxh - nrt * TZ) + TZ - 1) / TZ;
+  }
+  if (a.nz == 1 && a.c != 6) return ((a.nxh + 31) / 32) * ((a.ny + kThreads / 32 - 1) / (kThreads / 32));
+  return L.grid_zx * L.grid_zy;
+}
+
+void launch_xinv_update(const OpArgs<float>& a, const LaunchCfg& L, const float* p, float* z, SolverState* st,
+                        double* partials, long long off, cudaStream_t s) {
+  launch_dep(a.pdl != 0, L.VEC == 4 ? k_xinv<float, 5, 4> : (L.VEC == 2 ? k_xinv<float, 5, 2> : k_xinv<float, 5, 1>),
+             dim3(a.S * a.bps), dim3(L.thr_x), L.smem_x, s, a, p, z, st, partials, off);
+  launch_cg_beta(st, partials, off, a.bps, a.S, a.pdl != 0, s);
 }
 
 void launch_dot_finalize(SolverState* st, const double* partials, int nb, int S, cudaStream_t s) {

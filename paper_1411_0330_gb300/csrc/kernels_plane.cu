@@ -795,6 +795,10 @@ bool launch_xyinv_update(const OpArgs<float>& a, const float* p, float* z, Solve
   return xyinv_n(a, 2, p, z, st, partials, off, s);
 }
 
+void launch_cg_beta(SolverState* st, const double* partials, long long off, int nb, int S, bool pdl, cudaStream_t s) {
+  launch_dep(pdl, k_cg_beta, dim3(S), dim3(256), 0, s, st, partials, off, nb);
+}
+
 void launch_cg_alpha(SolverState* st, const double* partials, int nb, int S, bool pdl, cudaStream_t s) {
   launch_dep(pdl, k_cg_alpha, dim3(S), dim3(256), 0, s, st, partials, nb);
 }

@@ -366,7 +366,12 @@ Layout make_layout(const Derived& d) {
   // block partials: x passes have at most one block per row (two rows where their number
   // is even), the elementwise kernels 2432 blocks or one per system
   const long long xblocks = rps_of(d) % 2 == 0 ? rps_of(d) / 2 + 1 : rps_of(d);
-  long long np = std::max<long long>({2432LL + S, (long long)S * d.c * 152, (long long)d.B * 1216, (long long)S * xblocks,
+  // (p, Gamma p) of the FP32 z pass: one partial per block, most with one system's tiles
+  const LaunchCfg L1 = make_cfg<float>(d, 1);
+  const long long zblocks = d.nz == 1 ? (d.nxh / 32 + 1LL) * (d.ny / 8 + 1)
+                                      : std::max<long long>((long long)L1.grid_zx * L1.grid_zy,
+                                                            (long long)d.ny * (d.nxh / 4 + 2));
+  long long np = std::max<long long>({2432LL + S, d.precision == LSH_MIXED ? (long long)S * zblocks : 0LL, (long long)S * d.c * 152, (long long)d.B * 1216, (long long)S * xblocks,
                                       (long long)S * d.c * d.nz});
   l.nparts = np;
   l.off_state = take(sizeof(SolverState) * (size_t)(3 * S + d.B));
@@ -616,12 +621,16 @@ void init_prec(lsh_handle* h, PrecBufs<T>& P, const size_t* off_f, size_t off_H,
   a.fuse = 0;
   a.mandel = 0;
   a.pdl = 0;
+  a.dot = nullptr;
   a.tlay = 0;
   a.nq = nullptr;
   // measured on the batched workload: the inverse pass gains (0.61 -> 0.66 of the
   // copy bandwidth), the forward pass loses (0.81 -> 0.70); LSH_L2PF overrides
   a.l2pf = 2;
   if (const char* e = getenv("LSH_L2PF")) a.l2pf = atoi(e) & 3;
+  // off the plane grids the shared-memory inverse x pass can update z (its tables take
+  // 12 KB more of shared memory)
+  if (sizeof(T) == 4 && !d.plane) a.fuse = P.L.smem_x <= 200 * 1024 ? 1 : 0;
   if (sizeof(T) == 4 && d.plane) {
     // natural frequency order along y and z in every FP32 pass; the plane
     // passes (ky-major spectrum) are the default
@@ -866,6 +875,30 @@ template <typename T> void enqueue_cg_iteration(lsh_handle* h, PrecBufs<T>& P, c
       return;
     }
   }
+  if constexpr (sizeof(T) == 4) {
+    if (!a.plane && a.fuse) {
+      // seven launches: x forward, y, z, alpha, y inverse, x inverse with the update of z, beta
+      a.dot = h->partials;
+      if (timed) cudaEventRecordWithFlags(e[0], s, rf);
+      launch_xfwd<T>(a, P.L, 1, nullptr, P.x, P.r, P.p, P.st, s);
+      if (timed) cudaEventRecordWithFlags(e[1], s, rf);
+      launch_yfft<T>(a, P.L, false, P.st, s);
+      if (timed) cudaEventRecordWithFlags(e[2], s, rf);
+      launch_zgamma<T>(a, P.L, P.st, s);
+      launch_cg_alpha(P.st, h->partials, zdot_blocks(a, P.L), a.S, a.pdl != 0, s);
+      if (timed) cudaEventRecordWithFlags(e[3], s, rf);
+      launch_yfft<T>(a, P.L, true, P.st, s);
+      if (timed) cudaEventRecordWithFlags(e[4], s, rf);
+      launch_xinv_update(a, P.L, P.p, P.r, P.st, h->partials, h->lay.nparts, s);
+      if (timed) {
+        cudaEventRecordWithFlags(e[5], s, rf);
+        cudaEventRecordWithFlags(e[6], s, rf);
+        h->ev_used += 7;
+      }
+      h->launches += 7;
+      return;
+    }
+  }
   if (timed) cudaEventRecordWithFlags(e[0], s, rf);
   launch_xfwd<T>(a, P.L, 1, nullptr, P.x, P.r, P.p, P.st, s);
   if (timed) cudaEventRecordWithFlags(e[1], s, rf);
@@ -940,7 +973,7 @@ void harvest_profile(lsh_handle* h, int real, bool plane, bool fuse) {
   for (int g = 0; g < groups && g < real; ++g) {
     for (int k = 0; k < 6; ++k) {
       if (plane && (k == 1 || k == 3)) continue;  // no separate y passes
-      if (plane && fuse && k == 5) continue;      // the inverse pass updates z
+      if (fuse && k == 5) continue;               // the inverse pass updates z
       float ms = 0.f;
       if (cudaEventElapsedTime(&ms, h->ev[7 * g + k], h->ev[7 * g + k + 1]) == cudaSuccess) {
         h->pass_ms[k] += ms;
@@ -1397,6 +1430,14 @@ lsh_status copy_microstructure(lsh_handle* h, const unsigned char* phase, const 
     LSH_CK(cudaMemcpyAsync(h->scale, scale, sizeof(float) * nv, k, h->stream));
   }
   return LSH_OK;
+}
+
+// Separate passes: whether the inverse x pass can update z with these variants.
+int can_fuse(const lsh_handle* h, int x_variant, int z_variant) {
+  return h->d.precision == LSH_MIXED && x_variant == 0 && (z_variant == 0 || z_variant == 9) &&
+                 make_cfg<float>(h->d, h->d.Smax).smem_x <= 200 * 1024
+             ? 1
+             : 0;
 }
 
 lsh_status rotate_or_copy(lsh_handle* h, const double* in, double* out, int nsys, int to_internal) {
@@ -1960,6 +2001,10 @@ lsh_status lsh_autotune(lsh_handle* h, lsh_tune_report* rep) {
     if (sep_ok && a.zreg) {
       int best = 0;
       for (int v = 0; v < 10; ++v) {
+        // with the shared-memory inverse x pass only the variants that give (p, Gamma p):
+        // its update of z saves more than the others gain (96 x 80 x 64: 16 us of update
+        // kernel against 1 us)
+        if (can_fuse(h, a.xreg, 0) && !can_fuse(h, a.xreg, v)) continue;
         if (v >= 1 && v <= 5 && !P.ztma_ok) continue;  // TMA tiles need the tensor map
         a.ztma = v;
         r.z_ms[v] = timeit([&]() {
@@ -2045,6 +2090,7 @@ lsh_status lsh_autotune(lsh_handle* h, lsh_tune_report* rep) {
     lsh_status st = last_launch();
     if (st) return st;
     if (h->fault && (st = check_fault(h))) return st;
+    if (!a.plane) a.fuse = can_fuse(h, a.xreg, a.ztma);
     P.a.xreg = a.xreg;
     P.a.xfreg = a.xfreg;
     P.a.ytma = a.ytma;
@@ -2107,7 +2153,7 @@ lsh_status lsh_set_variants(lsh_handle* h, int xf_variant, int x_variant, int y_
   P.a.ztma = z_variant;
   P.a.plane = 0;
   P.a.tlay = 0;
-  P.a.fuse = 0;
+  P.a.fuse = can_fuse(h, x_variant, z_variant);
   h->drop_graphs();
   h->no_cluster = true;  // a choice made by hand runs the passes it names
   return LSH_OK;
