@@ -277,10 +277,11 @@ void launch_rotate_scalar(const T* in, T* out, long long V, int nsys, int d, con
                           cudaStream_t s);
 template <typename T> void launch_voxel_fields(const OpArgs<T>& a, T* mfld, T* dfld, int B, cudaStream_t s);
 void launch_gamma_diag(const OpArgs<double>& a, double* partials, int nblk, double* out, cudaStream_t s);
-void launch_d2f_begin(const OpArgs<float>& a, const double* r64, bool df_pairs, float* r32, float* x32, SolverState* st,
+void launch_d2f_begin(const OpArgs<float>& a, const double* r64, int src, float* r32, float* x32, SolverState* st,
                       double* partials, long long off2, double tol, const unsigned char* active, int G,
                       cudaStream_t s);
-void launch_f2d_axpy(double* x64, const float* x32, long long n, cudaStream_t s);
+void launch_f2d_axpy(double* x64, const float* x32, const float* p, long long n, int S, const SolverState* st,
+                     bool first, int G, cudaStream_t s);
 void launch_scan_phase(const unsigned char* phase, long long V, int B, const unsigned char* act, int nphase,
                        SolverState* st, double* partials, int G, cudaStream_t s);
 void launch_scale_grad(const double* tau_all, const double* W, const unsigned char* phase, const float* scale,

@@ -1275,8 +1275,9 @@ __global__ void k_gamma_table(OpArgs<T> a, GammaCtx g, const int* __restrict__ k
 // ------------------------------------------------------------------ mixed precision helpers
 // r32 = (float) r64 (PRE: z32 = D r32), x32 = 0, inner CG state begun with tolerance
 // tol relative to the new right-hand side; systems with active[s] == 0 start done.
-// DFIN: r64's elements hold double-float pairs (h, l); the FP32 residual is h
-template <bool DFIN, int PRE>
+// SRC: where the residual comes from: 0 r64, 1 r64's elements as double-float pairs (h, l),
+// of which the FP32 residual is h, 2 the load on I0 (first step from x = 0).
+template <int SRC, int PRE>
 __global__ void __launch_bounds__(kThreads) k_d2f_begin(OpArgs<float> a, const double* __restrict__ r64,
                                                         float* __restrict__ r32, float* __restrict__ x32,
                                                         SolverState* __restrict__ st, double* __restrict__ partials,
@@ -1296,13 +1297,17 @@ __global__ void __launch_bounds__(kThreads) k_d2f_begin(OpArgs<float> a, const d
     float v[VEC], zero[VEC];
     int ph[VEC];
     phase_load<VEC>(a.phase + pbase + i, ph);
-    if constexpr (VEC == 4) {
+    if constexpr (SRC == 2) {
+      const float ld = a.loads[s * 6 + comp];
+#pragma unroll
+      for (int u = 0; u < VEC; ++u) v[u] = a.act[ph[u]] ? ld : 0.0f;
+    } else if constexpr (VEC == 4) {
       const double2 d0 = *reinterpret_cast<const double2*>(r64s + g), d1 = *reinterpret_cast<const double2*>(r64s + g + 2);
       const double d[4] = {d0.x, d0.y, d1.x, d1.y};
 #pragma unroll
-      for (int u = 0; u < 4; ++u) v[u] = DFIN ? __int_as_float(__double2loint(d[u])) : (float)d[u];
+      for (int u = 0; u < 4; ++u) v[u] = SRC == 1 ? __int_as_float(__double2loint(d[u])) : (float)d[u];
     } else {
-      v[0] = DFIN ? reinterpret_cast<const float2*>(r64s)[g].x : (float)r64s[g];
+      v[0] = SRC == 1 ? reinterpret_cast<const float2*>(r64s)[g].x : (float)r64s[g];
     }
 #pragma unroll
     for (int u = 0; u < VEC; ++u) {
@@ -1385,9 +1390,36 @@ __global__ void __launch_bounds__(kThreads) k_gamma_diag(OpArgs<double> a, doubl
   if (threadIdx.x == 0) partials[(long long)comp * gridDim.x + blockIdx.x] = acc;
 }
 
-__global__ void k_f2d_axpy(double* __restrict__ x64, const float* __restrict__ x32, long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    x64[i] += (double)x32[i];
+// x64 += x32 + alpha p, the inner solve's iterate with its last step (FIRST: x64 = ...,
+// the first step from x = 0).  Grid (G, S).
+template <bool FIRST>
+__global__ void __launch_bounds__(kThreads) k_f2d_axpy(double* __restrict__ x64, const float* __restrict__ x32,
+                                                       const float* __restrict__ p, long long n,
+                                                       const SolverState* __restrict__ st) {
+  const int s = blockIdx.y;
+  const float al = (float)st[s].alpha;
+  double* xs = x64 + s * n;
+  const float *ys = x32 + s * n, *ps = p + s * n;
+  const long long nv = n % 4 == 0 ? n / 4 : 0;
+  const long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x, di = (long long)gridDim.x * blockDim.x;
+  for (long long i = i0; i < nv; i += di) {
+    float4 y = reinterpret_cast<const float4*>(ys)[i];
+    if (al != 0.f) {
+      const float4 q = reinterpret_cast<const float4*>(ps)[i];
+      y = make_float4(y.x + al * q.x, y.y + al * q.y, y.z + al * q.z, y.w + al * q.w);
+    }
+    double2 *o = reinterpret_cast<double2*>(xs) + 2 * i, a = make_double2(0.0, 0.0), b = a;
+    if (!FIRST) {
+      a = o[0];
+      b = o[1];
+    }
+    o[0] = make_double2(a.x + (double)y.x, a.y + (double)y.y);
+    o[1] = make_double2(b.x + (double)y.z, b.y + (double)y.w);
+  }
+  for (long long i = nv * 4 + i0; i < n; i += di) {
+    const float y = al != 0.f ? ys[i] + al * ps[i] : ys[i];
+    xs[i] = (FIRST ? 0.0 : xs[i]) + (double)y;
+  }
 }
 
 // Phase scan at setup, grid (G, B): voxels in I0 per microstructure (st[b].aux[1])
@@ -1688,16 +1720,16 @@ void launch_gamma_table(const OpArgs<T>& a, int dim, int physics, int green, con
   const int grid = (int)std::min<long long>((nf + 127) / 128, 152LL * 16);
   k_gamma_table<T><<<grid, 128, 0, s>>>(a, g, kofy, kofz);
 }
-void launch_d2f_begin(const OpArgs<float>& a, const double* r64, bool df_pairs, float* r32, float* x32, SolverState* st,
+void launch_d2f_begin(const OpArgs<float>& a, const double* r64, int src, float* r32, float* x32, SolverState* st,
                       double* partials, long long off2, double tol, const unsigned char* active, int G,
                       cudaStream_t s) {
   const dim3 g(G, a.S);
-#define LSH_D2F(DFIN, PRE) \
-  k_d2f_begin<DFIN, PRE><<<g, kThreads, 0, s>>>(a, r64, r32, x32, st, partials, off2, tol, active)
-  if (a.pre == 0) { if (df_pairs) LSH_D2F(true, 0); else LSH_D2F(false, 0); }
-  else if (a.pre == 1) { if (df_pairs) LSH_D2F(true, 1); else LSH_D2F(false, 1); }
-  else { if (df_pairs) LSH_D2F(true, 2); else LSH_D2F(false, 2); }
-#undef LSH_D2F
+  typedef void (*K)(OpArgs<float>, const double*, float*, float*, SolverState*, double*, long long, double,
+                    const unsigned char*);
+  static const K k[3][3] = {{k_d2f_begin<0, 0>, k_d2f_begin<0, 1>, k_d2f_begin<0, 2>},
+                            {k_d2f_begin<1, 0>, k_d2f_begin<1, 1>, k_d2f_begin<1, 2>},
+                            {k_d2f_begin<2, 0>, k_d2f_begin<2, 1>, k_d2f_begin<2, 2>}};
+  k[src][a.pre]<<<g, kThreads, 0, s>>>(a, r64, r32, x32, st, partials, off2, tol, active);
 }
 template <typename T> void launch_voxel_fields(const OpArgs<T>& a, T* mfld, T* dfld, int B, cudaStream_t s) {
   const int G = (int)std::max(1LL, std::min((B * a.V + kThreads - 1) / kThreads, 152LL * 8));
@@ -1707,9 +1739,10 @@ void launch_gamma_diag(const OpArgs<double>& a, double* partials, int nblk, doub
   k_gamma_diag<<<dim3(nblk, a.c), kThreads, 0, s>>>(a, partials);
   k_comp_final<<<a.c, kThreads, 0, s>>>(partials, nblk, out);
 }
-void launch_f2d_axpy(double* x64, const float* x32, long long n, cudaStream_t s) {
-  const int grid = (int)std::max(1LL, std::min((n + kThreads - 1) / kThreads, 152LL * 16));
-  k_f2d_axpy<<<grid, kThreads, 0, s>>>(x64, x32, n);
+void launch_f2d_axpy(double* x64, const float* x32, const float* p, long long n, int S, const SolverState* st,
+                     bool first, int G, cudaStream_t s) {
+  if (first) k_f2d_axpy<true><<<dim3(G, S), kThreads, 0, s>>>(x64, x32, p, n, st);
+  else k_f2d_axpy<false><<<dim3(G, S), kThreads, 0, s>>>(x64, x32, p, n, st);
 }
 void launch_scan_phase(const unsigned char* phase, long long V, int B, const unsigned char* act, int nphase,
                        SolverState* st, double* partials, int G, cudaStream_t s) {

@@ -1027,8 +1027,8 @@ lsh_status cg_run_cluster(lsh_handle* h, PrecBufs<T>& P, const OpArgs<T>& a, int
   return LSH_OK;
 }
 
-// CG on the states already begun for the wave; finalises x.  `out` receives
-// the S states.
+// CG on the states already begun for the wave; finalises x (FP64; in FP32 x lacks the last
+// step alpha p).  `out` receives the S states.
 template <typename T>
 lsh_status cg_run(lsh_handle* h, PrecBufs<T>& P, const OpArgs<T>& a, int maxit, int check_every, bool check_given,
                   bool graphs, std::vector<SolverState>& out) {
@@ -1091,8 +1091,10 @@ lsh_status cg_run(lsh_handle* h, PrecBufs<T>& P, const OpArgs<T>& a, int maxit, 
     }
     h->prof_now = false;
   } while (!all_done() && it < maxit);
-  launch_cg_finalize<T>(P.x, P.p, (long long)a.c * a.V, S, P.st, P.L.ew_per_sys, h->stream);
-  h->launches += 1;
+  if (sizeof(T) == 8) {  // in FP32 the caller adds the last step as it takes the result
+    launch_cg_finalize<T>(P.x, P.p, (long long)a.c * a.V, S, P.st, P.L.ew_per_sys, h->stream);
+    h->launches += 1;
+  }
   return last_launch();
 }
 
@@ -1316,14 +1318,12 @@ lsh_status solve_wave(lsh_handle* h, const Wave& w, bool warm, const lsh_solve_o
     const int max_outer = o && o->max_outer > 0 ? o->max_outer : 30;
     std::vector<double> rr(S);
     SolverState* sres = h->st + 2 * d.Smax;
-    bool rdf = false;  // Pd.r holds double-float pairs (else FP64)
+    int src = 2;  // the first step's right-hand side is the load; later Pd.r as FP64 or double-float pairs
     if (!warm) {
-      launch_fill_rhs<double>(ad, Pd.r, Pd.x, G, h->stream);
-      h->launches += 1;
       rr = bb;
     } else {
       if ((stt = residual64(h, ad, Pd.x, Pd.r, h->dfres))) return stt;
-      rdf = h->dfres;
+      src = h->dfres ? 1 : 0;
       for (int s = 0; s < S; ++s) infos[s].applies64 += 1;
       std::vector<SolverState> s2(S);
       if ((stt = read_states(h, sres, S, s2.data()))) return stt;
@@ -1342,6 +1342,10 @@ lsh_status solve_wave(lsh_handle* h, const Wave& w, bool warm, const lsh_solve_o
         active[s] = (!conv && !failed) ? 1 : 0;
         nact += active[s];
       }
+      if (nact == 0 || outer >= max_outer || total_max >= maxit) {
+        // no step taken: x is still to be set
+        if (src == 2) LSH_CK(cudaMemsetAsync(Pd.x, 0, sizeof(double) * (size_t)(S * n), h->stream));
+      }
       if (nact == 0) break;
       if (outer >= max_outer || total_max >= maxit) {
         for (int s = 0; s < S; ++s)
@@ -1359,14 +1363,14 @@ lsh_status solve_wave(lsh_handle* h, const Wave& w, bool warm, const lsh_solve_o
           if (active[s] && bb[s] > 0) worst = std::max(worst, std::sqrt(rr[s] / bb[s]));
         if (worst > 0.0) itol_k = std::min(1e-3, std::max(itol, 0.5 * tol / worst));
       }
-      launch_d2f_begin(af, Pd.r, rdf, Pf.r, Pf.x, Pf.st, h->partials, h->lay.nparts, itol_k, h->flags,
+      launch_d2f_begin(af, Pd.r, src, Pf.r, Pf.x, Pf.st, h->partials, h->lay.nparts, itol_k, h->flags,
                        Pf.L.ew_per_sys, h->stream);
       h->launches += 1;
       if ((stt = cg_run<float>(h, Pf, af, maxit - total_max, check, check_given, graphs, st))) return stt;
-      launch_f2d_axpy(Pd.x, Pf.x, n * S, h->stream);
+      launch_f2d_axpy(Pd.x, Pf.x, Pf.p, n, S, Pf.st, src == 2, G, h->stream);
       h->launches += 1;
       if ((stt = residual64(h, ad, Pd.x, Pd.r, h->dfres))) return stt;
-      rdf = h->dfres;
+      src = h->dfres ? 1 : 0;
       std::vector<SolverState> s2(S);
       if ((stt = read_states(h, sres, S, s2.data()))) return stt;
       ++outer;
