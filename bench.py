@@ -160,8 +160,8 @@ PROF_EVERY = 8  # per-pass events in one CG chunk of this many
 # plane-pass summary under profiles/ (filtered operator); to be retaken
 # whenever one of these kernels changes (None: not captured for the current
 # kernel).
-NCU_TRAFFIC_FP32 = {"x_forward": 1774.9e6, "y_forward": None, "z_gamma": 724.2e6, "y_inverse": None,
-                    "x_inverse_local": 909.1e6, "cg_update": 861.8e6}
+NCU_TRAFFIC_FP32 = {"x_forward": 1774.9e6, "y_forward": None, "z_gamma": 713.9e6, "y_inverse": None,
+                    "x_inverse_local": 909.1e6, "x_inverse_update": 1248.6e6, "cg_update": 861.8e6}
 NCU_TRAFFIC_SOURCE = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch over 6 systems at 128^3 "
                       "(filtered), scaled to the batch's average launch by its algorithmic bytes")
 
@@ -482,7 +482,7 @@ def run_batch(args, rank, world, local):
             cg_ms += sum(p["pass_ms"].values()) * live * args.steps / p["timed_sys_iters"]
     step_split = {"inner_cg_ms_est": cg_ms / args.steps, "other_ms_est": ms_mx - cg_ms / args.steps}
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
-                "frac": achieved / peaks["hbm_gbs"], "traffic": ncu_traffic_per_launch(dom, tot_b[dom] / tot_n[dom]),
+                "frac": achieved / peaks["hbm_gbs"], "traffic": ncu_traffic_per_launch(pass_kind(prof_mx[0], dom), tot_b[dom] / tot_n[dom]),
                 "traffic_source": NCU_TRAFFIC_SOURCE,
                 "kernel": f"{dom} (FP32, all grids)", "avg_launch_ms": tot_ms[dom] / tot_n[dom],
                 "algorithmic_bytes_per_launch": tot_b[dom] / tot_n[dom],

@@ -1765,10 +1765,6 @@ void launch_scale_grad(const double* tau_all, const double* W, const unsigned ch
                                cudaStream_t);                                                                      \
   template void launch_cg_update<T>(const OpArgs<T>&, T*, const T*, SolverState*, double*, long long, int,         \
                                     cudaStream_t);                                                                 \
-  template void launch_cg_finalize<T>(T*, const T*, long long, int, const SolverState*, int, cudaStream_t);        \
-  template void launch_cg_begin<T>(const OpArgs<T>&, T*, SolverState*, double*, long long, double, const double*,  \
-                                   int, cudaStream_t);                                                             \
-  template void launch_fill_rhs<T>(const OpArgs<T>&, T*, T*, int, cudaStream_t);                                   \
   template void launch_rotate<T>(const T*, T*, long long, int, int, cudaStream_t);                                 \
   template void launch_comp_sums<T>(const T*, int, long long, int, double*, int, double*, cudaStream_t);           \
   template void launch_gamma_table<T>(const OpArgs<T>&, int, int, int, const double*, const int*, const int*,      \
@@ -1778,5 +1774,10 @@ void launch_scale_grad(const double* tau_all, const double* W, const unsigned ch
 
 LSH_INSTANTIATE(double)
 LSH_INSTANTIATE(float)
+// FP64 solves only: the mixed solver starts and ends its FP32 solves with conversions
+template void launch_cg_finalize<double>(double*, const double*, long long, int, const SolverState*, int, cudaStream_t);
+template void launch_cg_begin<double>(const OpArgs<double>&, double*, SolverState*, double*, long long, double,
+                                      const double*, int, cudaStream_t);
+template void launch_fill_rhs<double>(const OpArgs<double>&, double*, double*, int, cudaStream_t);
 
 }  // namespace lsh
