@@ -220,14 +220,21 @@ inline bool lsh_make_plan(int n, Plan1D* p) {
 
 // Plan for `lines` lines in one block of `threads` threads, by the cycles of a stage: a
 // barrier and the shared-memory round trip, and the instructions of a butterfly times
-// the warps (FP64: 16 cycles each of the SM's one unit) or the rounds of the threads.
+// the rounds of the threads.  FP64: a warp instruction holds its scheduler's share of the
+// unit for 64 cycles, and radix 2 runs on two lanes per butterfly.  Measured, us per
+// iteration of the cluster solver: 32 x 32 in radices 4, 4, 2 23.7, in 2s 20.9; 64 x 64
+// rows in 8, 8 30.5, in 2s 29.5, in 4, 4, 4 26.9; 96 x 96 columns in 12, 8 42.8, in
+// 6, 4, 4 39.8; 16^3 in 4, 4 27.8, in 8, 2 35.
 inline bool lsh_make_plan_lines(int n, int lines, int threads, bool fp64, Plan1D* p) {
   if (!lsh_plan_length(n)) return false;
   const auto cost = [&](int r) {
     const double instr[13] = {0, 0, 16, 30, 36, 60, 66, 100, 92, 130, 140, 0, 160};
-    const double items = (double)lines * n / r, warps = (double)(long long)((items + 31) / 32);
+    const double instr64[13] = {0, 0, 5, 24, 28, 56, 60, 100, 84, 150, 136, 0, 156};
+    const double items = (double)lines * n / r * (fp64 && r == 2 ? 2 : 1);
+    const double warps = (double)(long long)((items + 31) / 32);
     const double rounds = (double)(long long)((items + threads - 1) / threads);
-    return 200.0 + (fp64 ? 16.0 * instr[r] * warps : instr[r] * (4.0 * rounds + warps / 4.0));
+    if (fp64) return 250.0 + 100.0 * rounds + 16.0 * instr64[r] * (warps > 4.0 ? warps : 4.0);
+    return 200.0 + instr[r] * (4.0 * rounds + warps / 4.0);
   };
   double best = 1e30;
   int cur[LSH_MAX_STAGES], r[LSH_MAX_STAGES] = {0}, nst = 0;

@@ -67,6 +67,48 @@ __device__ __forceinline__ void line_stage_r(C2<T>* __restrict__ buf, int nlines
   }
 }
 
+// Radix 2 in FP64 on two lanes per butterfly, one for the real and one for the imaginary
+// parts.  A scheduler's FP64 unit is busy some 64 cycles with any warp instruction; where
+// a stage is a warp or two, four times as many instructions per butterfly are on the
+// critical path of a radix-4 stage as here per level (32 x 32, two systems: 23.7 -> 20.9 us
+// per iteration; 12^3, radices 3, 2, 2 for one 12: 30.5 -> 28.3).
+template <bool INV, typename A>
+__device__ __forceinline__ void line_stage_pair(double2* __restrict__ buf, int nlines, const FastDiv& dl, const A& at,
+                                                const Plan1D& pl, int st, const double2* __restrict__ tw) {
+  const int m = pl.m[st], total = pl.n * nlines, tws = pl.tws[st];  // lanes: two per butterfly
+  const FastDiv dm(m, pl.mag_m[st]);
+  double* f = reinterpret_cast<double*>(buf);
+  const int im = threadIdx.x & 1;  // the block is a whole number of warps
+  const double sg = im ? 1.0 : -1.0;
+  for (int w = threadIdx.x; w < total; w += blockDim.x) {
+    const int i = w >> 1, b = dl.div(i), line = i - b * nlines;
+    const int sp = dm.div(b), j = b - sp * m, e0 = sp * (2 * m) + j, te = j * tws;
+    const int i0 = 2 * at(line, e0), i1 = 2 * at(line, e0 + m);
+    const double a = f[i0 + im], c = f[i1 + im];
+    double y0, y1;
+    if (te == 0) {
+      y0 = a + c;
+      y1 = a - c;
+    } else if (INV) {
+      // t = b conj(w): re b.x w.x + b.y w.y, im b.y w.x - b.x w.y
+      const double o = f[i1 + (im ^ 1)];
+      const double2 wv = tw[te];
+      const double t = fma(-sg * o, wv.y, c * wv.x);
+      y0 = a + t;
+      y1 = a - t;
+    } else {
+      // (a - b) w: re d.x w.x - d.y w.y, im d.y w.x + d.x w.y
+      const double ao = f[i0 + (im ^ 1)], co = f[i1 + (im ^ 1)];
+      const double2 wv = tw[te];
+      y0 = a + c;
+      y1 = fma(sg * (ao - co), wv.y, (a - c) * wv.x);
+    }
+    __syncwarp(__activemask());  // both lanes have read before either writes
+    f[i0 + im] = y0;
+    f[i1 + im] = y1;
+  }
+}
+
 // In-place transform of nlines lines, element e of a line at buf[at(line, e)]: DIF
 // (natural in, digit-reversed out) or DIT.  Ends synchronised.
 template <typename T, bool INV, typename A>
@@ -85,7 +127,10 @@ __device__ __forceinline__ void line_fft(C2<T>* __restrict__ buf, int nlines, co
       case 5: line_stage_r<T, INV, 5>(buf, nlines, dl, at, pl, st, tw); break;
       case 4: line_stage_r<T, INV, 4>(buf, nlines, dl, at, pl, st, tw); break;
       case 3: line_stage_r<T, INV, 3>(buf, nlines, dl, at, pl, st, tw); break;
-      default: line_stage_r<T, INV, 2>(buf, nlines, dl, at, pl, st, tw); break;
+      default:
+        if constexpr (sizeof(T) == 8) line_stage_pair<INV>(buf, nlines, dl, at, pl, st, tw);
+        else line_stage_r<T, INV, 2>(buf, nlines, dl, at, pl, st, tw);
+        break;
     }
     __syncthreads();
   }
@@ -611,12 +656,12 @@ template <typename T> bool cluster_plan(const OpArgs<T>& a, int nsys, ClusterCg<
     c.ps = (c.ns + CS - 1) / CS;
     c.pp = (npos + CS - 1) / CS;
     const int npair = (a.c * c.ps * c.ry + 1) / 2;
-    c.threads = std::min(kThreadsOf<T>, std::max(64, (npair * a.nx / 2 + 31) / 32 * 32));
+    c.threads = std::min(kThreadsOf<T>, std::max(sizeof(T) == 8 ? 128 : 64, (npair * a.nx / 2 + 31) / 32 * 32));
     c.smem = cluster_smem(a, c);
     if (c.smem > 223 * 1024) return false;  // smaller clusters need more still
     // elements a CTA carries through an iteration: beyond these the separate passes,
     // which use the whole chip, are as fast.  us per iteration, cluster / separate: FP64
-    // 32^2 conductivity 24 / 42, 16^3 28 / 69, 16^3 elasticity (1536 a CTA) 40 / 66; FP32
+    // 32^2 conductivity 21 / 42, 16^3 28 / 69, 16^3 elasticity (1536 a CTA) 40 / 66; FP32
     // 24^3 elasticity 39 / 58; on grids with the plane passes 32^3 conductivity (6144) 34
     // / 36, 32^3 elasticity (12288) 51 / 49; off them 20^3 elasticity, four
     // microstructures (12000) 68 / 93.
