@@ -174,10 +174,11 @@ typedef struct lsh_tune_report {
                      brought in and written back by TMA, double-buffered, with the
                      FFT and Gamma exchanges in the tile's buffer; 11 the same on
                      the plan N = R1 x 4 with the 4-point FFT level and Gamma in one
-                     register phase (z lengths up to 128), which also leaves
-                     (p, Gamma p): the CG update then runs in the inverse pass       */
+                     register phase (z lengths up to 128).  0, 9 and 11 also leave
+                     (p, Gamma p): the CG update then runs in the inverse pass (the
+                     plane pass after 11, x variants 0, 1 and 3 after 0 and 9)       */
   float xf_ms[2]; /* measured time of one launch per candidate (-1: not available)   */
-  float x_ms[4];
+  float x_ms[4];  /* as the pass runs when a kernel of its own updates z             */
   float y_ms[2];
   float z_ms[10];
   float xy_ms[2]; /* one CG iteration's passes without the CG update summed: separate

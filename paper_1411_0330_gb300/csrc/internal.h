@@ -128,6 +128,12 @@ template <typename T> struct OpArgs {
              // forward pass's x, r, p; bit 1 the inverse pass's p and phase planes
 };
 
+// Row of the voxel fields for component comp: one per component, or the bulk and the
+// shear part of isotropic elasticity.
+template <typename T> __host__ __device__ __forceinline__ int field_class(const OpArgs<T>& a, int comp) {
+  return a.physics != 0 ? (comp > 0) : comp;
+}
+
 // Thread-block sizes and tile shapes, chosen at setup for one system count.
 struct LaunchCfg {
   int thr_x, thr_y, thr_z;  // threads per block of the shared-memory x, y and z passes
@@ -335,7 +341,7 @@ bool encode_z_map(CUtensorMap* out, void* H, int hs, int ny, int nz, int c, long
 void tma_prepare();
 void launch_wait_probe(int* fault, unsigned long long limit_ns, cudaStream_t s);
 bool launch_xinv_reg(const OpArgs<float>& a, int mode, const float* xin, float* out, SolverState* st,
-                     double* partials, cudaStream_t s, bool persistent, bool small = false);
+                     double* partials, cudaStream_t s, bool persistent, bool small = false, long long off = 0);
 void xreg_prepare();
 bool xinv_reg_fits(const OpArgs<float>& a);
 bool launch_xfwd_reg(const OpArgs<float>& a, int mode, const float* in, float* x, const float* r, float* p,

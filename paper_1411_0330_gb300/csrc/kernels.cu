@@ -62,10 +62,6 @@ template <typename T, int VEC> __device__ __forceinline__ void vstore(T* __restr
   }
 }
 
-template <typename T> __device__ __forceinline__ int field_class(const OpArgs<T>& a, int comp) {
-  return a.physics != 0 ? (comp > 0) : comp;
-}
-
 // Local coefficient m = (A_beta - A0)^{-1} of component `comp` at voxel index
 // `pv` of the stacked phase map; *active = voxel in I0.
 template <typename T>
@@ -1613,7 +1609,7 @@ void launch_xinv(const OpArgs<T>& a, const LaunchCfg& L, int mode, const T* xin,
 
 int zdot_blocks(const OpArgs<float>& a, const LaunchCfg& L) {
   if (a.zreg) {
-    const int TZ = a.nz >= 256 ? 4 : 8, nrt = a.nxh / TZ;  // z variants 0 and 9
+    const int TZ = 8, nrt = a.nxh / TZ;  // z variants 0 and 9
     return a.ny * nrt + (a.ny * (a.nxh - nrt * TZ) + TZ - 1) / TZ;
   }
   if (a.nz == 1 && a.c != 6) return ((a.nxh + 31) / 32) * ((a.ny + kThreads / 32 - 1) / (kThreads / 32));
@@ -1622,6 +1618,7 @@ int zdot_blocks(const OpArgs<float>& a, const LaunchCfg& L) {
 
 void launch_xinv_update(const OpArgs<float>& a, const LaunchCfg& L, const float* p, float* z, SolverState* st,
                         double* partials, long long off, cudaStream_t s) {
+  if ((a.xreg == 1 || a.xreg == 3) && launch_xinv_reg(a, 5, p, z, st, partials, s, false, a.xreg == 3, off)) return;
   launch_dep(a.pdl != 0, L.VEC == 4 ? k_xinv<float, 5, 4> : (L.VEC == 2 ? k_xinv<float, 5, 2> : k_xinv<float, 5, 1>),
              dim3(a.S * a.bps), dim3(L.thr_x), L.smem_x, s, a, p, z, st, partials, off);
   launch_cg_beta(st, partials, off, a.bps, a.S, a.pdl != 0, s);

@@ -75,9 +75,10 @@ __global__ void __launch_bounds__(16 * RegPlan<N>::P) k_yfft_reg(OpArgs<T> a, co
 
 // ------------------------------------------------------------------ z pass + Gamma
 template <typename T, int NC, int N, int TZV = 0> struct ZCfg {
-  // TZV <= 0: 8 columns per block (4 in FP64 or for length 256); else TZV columns.
+  // TZV <= 0: 8 columns per block (4 in FP64); else TZV columns.  At length 256 rows of
+  // 64 bytes: six components, six systems at 256^3 2.66 (4 columns) -> 2.13 ms.
   // TZV < 0: the Gamma coefficients are loaded when used, not one frequency ahead.
-  static constexpr int TZ = TZV > 0 ? TZV : ((sizeof(T) == 8 || N >= 256) ? 4 : 8);
+  static constexpr int TZ = TZV > 0 ? TZV : (sizeof(T) == 8 ? 4 : 8);
   static constexpr int W = 128 / (int)sizeof(C2<T>);  // complex values per shared wavefront
   static constexpr int KS0 = NC * TZ;
   static constexpr int KS = KS0 + ((TZ - KS0 % W) % W + W) % W;  // KS = TZ (mod W)
@@ -297,7 +298,7 @@ __global__ void __launch_bounds__(ZCfg<T, NC, N, TZV>::THREADS,
 // copies issued right after the current tile has left it, so the strided reads
 // along z run under the FFTs and the Gamma^h product of the current tile.
 template <int NC, int N> struct ZPCfg {
-  typedef ZCfg<float, NC, N, 0> ZC;
+  typedef ZCfg<float, NC, N, N >= 256 ? 4 : 0> ZC;
   static constexpr int TZ = ZC::TZ, THREADS = ZC::THREADS;
   static constexpr int STAGE = N * NC * TZ;  // complex values of one tile
   static constexpr size_t SMEM = sizeof(float2) * (STAGE + N + ZC::BUF);
@@ -308,7 +309,7 @@ template <int NC, int N>
 __global__ void __launch_bounds__(ZPCfg<NC, N>::THREADS, ZPCfg<NC, N>::THREADS <= 192 ? 4 : 2)
     k_zgamma_regp(OpArgs<float> a, const SolverState* __restrict__ st, int nrt, int nreg, int ntiles) {
   typedef RegLine<float, N> RL;
-  typedef ZCfg<float, NC, N, 0> ZC;
+  typedef ZCfg<float, NC, N, N >= 256 ? 4 : 0> ZC;
   constexpr int TZ = ZC::TZ, P = RL::P, R1 = RL::R1, KS = ZC::KS, THREADS = ZC::THREADS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* stage = reinterpret_cast<float2*>(smem_raw);  // [z][comp][li]

@@ -177,31 +177,45 @@ __device__ __forceinline__ bool xinv_rows(const OpArgs<float>& a, const float* _
 
 // One block per RY rows (standalone body; the persistent kernel below runs the
 // same arithmetic through xinv_rows).
-// MODE 0: out = P (M xin + g).  MODE 1 (CG): q = P (M p + g), (p, q) -> alpha.
+// MODE 0: out = P (M xin + g).  MODE 4 (CG): q = P (M p + g), per-block partials of (p, q).
 // MODE 2 (residual): out = P (load - M xin - g), (r, r) -> st[s].aux[0].
+// MODE 5 (CG, alpha known from the z pass): q = P (M p + g) is not stored, out = z is
+// updated, z -= alpha D q, and the four sums of k_cg_beta go to partials + {0, 1, 2, 3} off.
+// Bound by HBM latency at 17 B per voxel-component: with the loads of the whole block held
+// in registers through the FFT (128 of them, 16 warps an SM, as in the other modes) 2.82 ms
+// at 256^3, six systems; with p and z in L2 meanwhile and 80 registers (24 warps) 2.28 ms,
+// 0.66 of the copy bandwidth, against 1.61 for MODE 4 and 1.23 for k_cg_update.  The tables
+// are sized by the phases, so that the blocks fit.
 template <int MODE, int N, int TH = 256>
-__global__ void __launch_bounds__(TH, TH == 256 ? 2 : 4) k_xinv_reg(OpArgs<float> a, const float* __restrict__ xin,
+__global__ void __launch_bounds__(TH, (MODE == 5 ? 768 : 512) / TH) k_xinv_reg(OpArgs<float> a, const float* __restrict__ xin,
                                                                    float* __restrict__ out,
                                                                    SolverState* __restrict__ st,
                                                                    double* __restrict__ partials, int bps,
-                                                                   size_t rows_bytes) {
+                                                                   size_t rows_bytes, long long off) {
   typedef RegLine<float, N> RL;
   typedef XReg<N, TH> XC;
   constexpr int P = XC::P, R1 = RL::R1, Q = RL::Q, RY = XC::RY, OSTR = XC::OSTR;
   const int s = blockIdx.x / bps;
-  if ((MODE == 1 || MODE == 4) && st[s].done) return;
+  if ((MODE == 4 || MODE == 5) && st[s].done) return;
+  const float al = MODE == 5 ? (float)st[s].alpha : 0.f;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ float mloc[256 * 6];
-  __shared__ unsigned char aloc[256];
   __shared__ __align__(8) uint64_t bar;
   float2* HS = reinterpret_cast<float2*>(smem_raw);  // [RY][hs] spectrum rows, later [RY][OSTR] real rows
   float* OS = reinterpret_cast<float*>(smem_raw);
   float2* ex = reinterpret_cast<float2*>(smem_raw + rows_bytes);
   float2* tw = ex + XC::LINES * XC::LS;
-  for (int u = threadIdx.x; u < N; u += blockDim.x) tw[u] = a.twx[u];
   const int ntab = a.nphase * a.c;
+  float* mloc = reinterpret_cast<float*>(tw + N);
+  float *dloc = mloc + ntab, *eloc = dloc + ntab;  // MODE 5: D, 1 / D
+  unsigned char* aloc = reinterpret_cast<unsigned char*>(MODE == 5 ? eloc + ntab : dloc);
+  for (int u = threadIdx.x; u < N; u += blockDim.x) tw[u] = a.twx[u];
   for (int u = threadIdx.x; u < ntab; u += blockDim.x) mloc[u] = (a.scale && !a.frac) ? a.modtab[u] : a.mtab[u];
   for (int u = threadIdx.x; u < a.nphase; u += blockDim.x) aloc[u] = a.act[u];
+  if (MODE == 5)
+    for (int u = threadIdx.x; u < ntab; u += blockDim.x) {
+      dloc[u] = a.pre == 1 ? a.dtab[u] : 1.f;
+      eloc[u] = a.pre == 1 ? a.etab[u] : 1.f;
+    }
   const int blk = blockIdx.x - s * bps;
   const int rloc = blk * RY;                            // first row inside the system
   const long long row0 = (long long)s * a.rps + rloc;  // global row
@@ -213,25 +227,36 @@ __global__ void __launch_bounds__(TH, TH == 256 ? 2 : 4) k_xinv_reg(OpArgs<float
     const uint32_t bytes = (uint32_t)(sizeof(float2) * (size_t)RY * hs);
     mbar_expect_tx(&bar, bytes);
     bulk_load_1d(HS, a.H + row0 * hs, bytes, &bar);
+    if (MODE == 5) {
+      bulk_prefetch_l2(xin + row0 * N, (uint32_t)(sizeof(float) * RY * N));
+      bulk_prefetch_l2(out + row0 * N, (uint32_t)(sizeof(float) * RY * N));
+    }
   }
   const int rows_per_comp = a.nz * a.ny;
   const long long pbase = (long long)((a.sys0 + s) / a.sys_per_ms) * a.V;
   constexpr int NV = N / 4;
   constexpr int IT = RY * NV / XC::THREADS;  // float4 groups per thread
   static_assert(RY * NV % XC::THREADS == 0, "epilogue tiling");
-  // the epilogue's global loads go out while the copy and the FFT run
-  float4 xq4s[IT];
-  uchar4 ph4s[IT];
-#pragma unroll
-  for (int it = 0; it < IT; ++it) {
+  // the epilogue's global loads go out while the copy and the FFT run (MODE 5: to L2
+  // only, EB groups at a time in registers; 80 registers a thread keep 24 warps on an SM)
+  constexpr int EB = MODE == 5 ? (IT % 4 == 0 ? 4 : IT) : IT;
+  float4 xq4s[EB];
+  uchar4 ph4s[EB];
+  float4 zq4s[MODE == 5 ? EB : 1];
+  auto load = [&](int b, int it) {
     const int idx = threadIdx.x + it * XC::THREADS;
     const int row = idx / NV;
     const int xx = (idx - row * NV) * 4;
     const int rs = rloc + row;
     const int comp = rs / rows_per_comp;
     const long long vox = (long long)(rs - comp * rows_per_comp) * N + xx;
-    xq4s[it] = *reinterpret_cast<const float4*>(xin + (row0 + row) * N + xx);
-    ph4s[it] = *reinterpret_cast<const uchar4*>(a.phase + pbase + vox);
+    xq4s[b] = *reinterpret_cast<const float4*>(xin + (row0 + row) * N + xx);
+    ph4s[b] = *reinterpret_cast<const uchar4*>(a.phase + pbase + vox);
+    if constexpr (MODE == 5) zq4s[b] = *reinterpret_cast<const float4*>(out + (row0 + row) * N + xx);
+  };
+  if constexpr (MODE != 5) {
+#pragma unroll
+    for (int it = 0; it < IT; ++it) load(it, it);
   }
   __syncthreads();
   if (__syncthreads_or(!mbar_wait(&bar, 0))) {
@@ -269,47 +294,84 @@ __global__ void __launch_bounds__(TH, TH == 256 ? 2 : 4) k_xinv_reg(OpArgs<float
     OS[(2 * l) * OSTR + t + P * j] = v[j].x;
     OS[(2 * l + 1) * OSTR + t + P * j] = v[j].y;
   }
-  __syncthreads();
-  Acc<float> acc;
+  if constexpr (MODE == 5) {
 #pragma unroll
-  for (int it = 0; it < IT; ++it) {
-    const int idx = threadIdx.x + it * XC::THREADS;
-    const int row = idx / NV;
-    const int xx = (idx - row * NV) * 4;
-    const int rs = rloc + row;
-    const int comp = rs / rows_per_comp;
-    const long long vox = (long long)(rs - comp * rows_per_comp) * N + xx;
-    const long long g = (row0 + row) * N + xx;
-    const float4 xq4 = xq4s[it];
-    const uchar4 ph4 = ph4s[it];
-    const float4 g4 = *reinterpret_cast<const float4*>(OS + row * OSTR + xx);
-    const float xq[4] = {xq4.x, xq4.y, xq4.z, xq4.w};
-    const unsigned char ph[4] = {ph4.x, ph4.y, ph4.z, ph4.w};
-    const float gv[4] = {g4.x, g4.y, g4.z, g4.w};
-    float ov[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int p = ph[u];
-      const bool active = aloc[p] != 0;
-      float m = mloc[p * a.c + comp];
-      if (a.scale) {
-        const float f = a.scale[pbase + vox + u];
-        m = a.frac ? f * mloc[a.c + comp] + (1.f - f) * mloc[comp]  // Eq. (def_ah)
-                   : 1.f / (f * m - a.ref[comp]);
-      }
-      if (MODE == 0) {
-        ov[u] = active ? m * xq[u] + gv[u] : 0.f;
-      } else if (MODE == 1 || MODE == 4) {
-        ov[u] = active ? m * xq[u] + gv[u] : 0.f;
-        acc.add(xq[u] * ov[u]);
-      } else {
-        ov[u] = active ? a.loads[s * 6 + comp] - (m * xq[u] + gv[u]) : 0.f;
-        acc.add(ov[u] * ov[u]);
-      }
-    }
-    *reinterpret_cast<float4*>(out + g) = make_float4(ov[0], ov[1], ov[2], ov[3]);
+    for (int b = 0; b < EB; ++b) load(b, b);
   }
-  if (MODE == 4) {
+  __syncthreads();
+  Acc<float> acc, accz, accm, accp;
+#pragma unroll 1
+  for (int it0 = 0; it0 < IT; it0 += EB) {
+    if (MODE == 5 && it0 > 0) {
+#pragma unroll
+      for (int b = 0; b < EB; ++b) load(b, it0 + b);
+    }
+#pragma unroll
+    for (int b = 0; b < EB; ++b) {
+      const int it = it0 + b;
+      const int idx = threadIdx.x + it * XC::THREADS;
+      const int row = idx / NV;
+      const int xx = (idx - row * NV) * 4;
+      const int rs = rloc + row;
+      const int comp = rs / rows_per_comp;
+      const long long vox = (long long)(rs - comp * rows_per_comp) * N + xx;
+      const long long g = (row0 + row) * N + xx;
+      const float4 xq4 = xq4s[b];
+      const uchar4 ph4 = ph4s[b];
+      const float4 g4 = *reinterpret_cast<const float4*>(OS + row * OSTR + xx);
+      const float xq[4] = {xq4.x, xq4.y, xq4.z, xq4.w};
+      const unsigned char ph[4] = {ph4.x, ph4.y, ph4.z, ph4.w};
+      const float gv[4] = {g4.x, g4.y, g4.z, g4.w};
+      float ov[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int p = ph[u];
+        const bool active = aloc[p] != 0;
+        float m = mloc[p * a.c + comp];
+        if (MODE == 5 && a.mfld) {
+          m = a.mfld[field_class(a, comp) * a.fstride + pbase + vox + u];
+        } else if (a.scale) {
+          const float f = a.scale[pbase + vox + u];
+          m = a.frac ? f * mloc[a.c + comp] + (1.f - f) * mloc[comp]  // Eq. (def_ah)
+                     : 1.f / (f * m - a.ref[comp]);
+        }
+        if constexpr (MODE == 5) {
+          const int k = p * a.c + comp;
+          const float e = a.mfld ? (a.pre ? fabsf(m) + a.gpre[comp] : 1.f) : eloc[k];
+          const float d = a.mfld ? 1.f / e : dloc[k];
+          const float q = active ? m * xq[u] + gv[u] : 0.f;
+          const float zo[4] = {zq4s[b].x, zq4s[b].y, zq4s[b].z, zq4s[b].w};
+          const float z = zo[u] - al * (d * q), r = z * e, zm = z * m;
+          ov[u] = z;
+          acc.add(r * r);
+          accz.add(r * z);
+          accm.add(zm * z);
+          accp.add(zm * xq[u]);
+        } else if (MODE == 0) {
+          ov[u] = active ? m * xq[u] + gv[u] : 0.f;
+        } else if (MODE == 4) {
+          ov[u] = active ? m * xq[u] + gv[u] : 0.f;
+          acc.add(xq[u] * ov[u]);
+        } else {
+          ov[u] = active ? a.loads[s * 6 + comp] - (m * xq[u] + gv[u]) : 0.f;
+          acc.add(ov[u] * ov[u]);
+        }
+      }
+      *reinterpret_cast<float4*>(out + g) = make_float4(ov[0], ov[1], ov[2], ov[3]);
+    }
+  }
+  if constexpr (MODE == 5) {
+    double* part = partials + (long long)s * bps + blk;
+    auto store = [&](const Acc<float>& v, long long at) {
+      const double tot = block_reduce(v);
+      if (threadIdx.x == 0) part[at] = tot;
+      __syncthreads();
+    };
+    store(acc, 0);
+    store(accz, off);
+    store(accm, 2 * off);
+    store(accp, 3 * off);
+  } else if (MODE == 4) {
     // (p, Kp) partial of this block only; k_dot_finalize sums them (no fence, no ticket)
     const double tot = block_reduce(acc);
     if (threadIdx.x == 0) partials[(long long)s * bps + blk] = tot;
@@ -319,20 +381,7 @@ __global__ void __launch_bounds__(TH, TH == 256 ? 2 : 4) k_xinv_reg(OpArgs<float
     SolverState* sst = st + s;
     if (publish_partial_sys(part, blk, bps, tot, &sst->counter[0])) {
       const double sum = gather_partials_sys(part, bps, &sst->counter[0]);
-      if (threadIdx.x == 0) {
-        if (MODE == 1) {
-          sst->pq = sum;
-          if (!(fabs(sum) > 0.0) || !isfinite(sum) || !isfinite(sst->rr)) {
-            sst->status = 5;  // LSH_ERR_BREAKDOWN
-            sst->alpha = 0.0;
-            sst->done = 1;
-          } else {
-            sst->alpha = sst->rz / sum;
-          }
-        } else {
-          sst->aux[0] = sum;
-        }
-      }
+      if (threadIdx.x == 0) sst->aux[0] = sum;
     }
   }
 }
@@ -580,21 +629,24 @@ template <int N> bool launch_xfwd_reg_n(const OpArgs<float>& a, int mode, const 
 }
 
 template <int N, int TH = 256> bool launch_xinv_reg_n(const OpArgs<float>& a, int mode, const float* xin, float* out,
-                                                      SolverState* st, double* partials, cudaStream_t s) {
+                                                      SolverState* st, double* partials, long long off, cudaStream_t s) {
   typedef XReg<N, TH> XC;
   if (a.rps % XC::RY != 0 || (a.hs & 1)) return false;
   const int bps = a.rps / XC::RY;
   const size_t rows = std::max(sizeof(float2) * (size_t)XC::RY * a.hs, sizeof(float) * (size_t)XC::RY * XC::OSTR);
   const size_t rows16 = (rows + 15) & ~(size_t)15;
-  const size_t smem = xreg_smem<N, TH>(a.hs);
-  if (smem > 200 * 1024) return false;
+  const size_t smem = xreg_smem<N, TH>(a.hs) + (size_t)a.nphase * (sizeof(float) * a.c * (mode == 5 ? 3 : 1) + 1);
+  if (xreg_smem<N, TH>(a.hs) > 180 * 1024) return false;
   const int grid = a.S * bps;
-  if (mode == 0) k_xinv_reg<0, N, TH><<<grid, XC::THREADS, smem, s>>>(a, xin, out, st, partials, bps, rows16);
+  if (mode == 5) {
+    k_xinv_reg<5, N, TH><<<grid, XC::THREADS, smem, s>>>(a, xin, out, st, partials, bps, rows16, off);
+    launch_cg_beta(st, partials, off, bps, a.S, a.pdl != 0, s);
+  } else if (mode == 0) k_xinv_reg<0, N, TH><<<grid, XC::THREADS, smem, s>>>(a, xin, out, st, partials, bps, rows16, 0LL);
   else if (mode == 1) {
     // CG: partials per block, then one small kernel per system turns them into alpha
-    k_xinv_reg<4, N, TH><<<grid, XC::THREADS, smem, s>>>(a, xin, out, st, partials, bps, rows16);
+    k_xinv_reg<4, N, TH><<<grid, XC::THREADS, smem, s>>>(a, xin, out, st, partials, bps, rows16, 0LL);
     launch_dot_finalize(st, partials, bps, a.S, s);
-  } else k_xinv_reg<2, N, TH><<<grid, XC::THREADS, smem, s>>>(a, xin, out, st, partials, bps, rows16);
+  } else k_xinv_reg<2, N, TH><<<grid, XC::THREADS, smem, s>>>(a, xin, out, st, partials, bps, rows16, 0LL);
   return true;
 }
 
@@ -639,10 +691,11 @@ template <int N> bool launch_xinv_regp_n(const OpArgs<float>& a, int mode, const
 
 template <int N> void xreg_attrs() {
   const int mx = 200 * 1024;
+  cudaFuncSetAttribute(k_xinv_reg<5, N, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+  cudaFuncSetAttribute(k_xinv_reg<5, N, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
   cudaFuncSetAttribute(k_xinv_reg<4, N, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
   cudaFuncSetAttribute(k_xinv_reg<4, N, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
   cudaFuncSetAttribute(k_xinv_reg<0, N, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_xinv_reg<1, N, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
   cudaFuncSetAttribute(k_xinv_reg<2, N, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
   cudaFuncSetAttribute(k_xinv_regp<0, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
   cudaFuncSetAttribute(k_xinv_regp<1, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
@@ -650,7 +703,6 @@ template <int N> void xreg_attrs() {
   cudaFuncSetAttribute(k_xfwd_reg<0, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
   cudaFuncSetAttribute(k_xfwd_reg<1, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
   cudaFuncSetAttribute(k_xinv_reg<0, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_xinv_reg<1, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
   cudaFuncSetAttribute(k_xinv_reg<2, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
 }
 
@@ -693,16 +745,16 @@ bool xinv_reg_fits(const OpArgs<float>& a) {
 }
 
 // False when this grid has no register inverse x pass (the caller keeps the
-// shared-memory kernel).  persistent: the double-buffered persistent kernel.
+// shared-memory kernel).  persistent: the double-buffered persistent kernel (modes 0 to 2).
 bool launch_xinv_reg(const OpArgs<float>& a, int mode, const float* xin, float* out, SolverState* st,
-                     double* partials, cudaStream_t s, bool persistent, bool small) {
+                     double* partials, cudaStream_t s, bool persistent, bool small, long long off) {
   if (small) {
     switch (a.nx) {
-      case 16: return launch_xinv_reg_n<16, 128>(a, mode, xin, out, st, partials, s);
-      case 32: return launch_xinv_reg_n<32, 128>(a, mode, xin, out, st, partials, s);
-      case 64: return launch_xinv_reg_n<64, 128>(a, mode, xin, out, st, partials, s);
-      case 128: return launch_xinv_reg_n<128, 128>(a, mode, xin, out, st, partials, s);
-      case 256: return launch_xinv_reg_n<256, 128>(a, mode, xin, out, st, partials, s);
+      case 16: return launch_xinv_reg_n<16, 128>(a, mode, xin, out, st, partials, off, s);
+      case 32: return launch_xinv_reg_n<32, 128>(a, mode, xin, out, st, partials, off, s);
+      case 64: return launch_xinv_reg_n<64, 128>(a, mode, xin, out, st, partials, off, s);
+      case 128: return launch_xinv_reg_n<128, 128>(a, mode, xin, out, st, partials, off, s);
+      case 256: return launch_xinv_reg_n<256, 128>(a, mode, xin, out, st, partials, off, s);
       default: return false;
     }
   }
@@ -717,11 +769,11 @@ bool launch_xinv_reg(const OpArgs<float>& a, int mode, const float* xin, float* 
     }
   }
   switch (a.nx) {
-    case 16: return launch_xinv_reg_n<16>(a, mode, xin, out, st, partials, s);
-    case 32: return launch_xinv_reg_n<32>(a, mode, xin, out, st, partials, s);
-    case 64: return launch_xinv_reg_n<64>(a, mode, xin, out, st, partials, s);
-    case 128: return launch_xinv_reg_n<128>(a, mode, xin, out, st, partials, s);
-    case 256: return launch_xinv_reg_n<256>(a, mode, xin, out, st, partials, s);
+    case 16: return launch_xinv_reg_n<16>(a, mode, xin, out, st, partials, off, s);
+    case 32: return launch_xinv_reg_n<32>(a, mode, xin, out, st, partials, off, s);
+    case 64: return launch_xinv_reg_n<64>(a, mode, xin, out, st, partials, off, s);
+    case 128: return launch_xinv_reg_n<128>(a, mode, xin, out, st, partials, off, s);
+    case 256: return launch_xinv_reg_n<256>(a, mode, xin, out, st, partials, off, s);
     default: return false;
   }
 }

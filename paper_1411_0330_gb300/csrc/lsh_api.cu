@@ -1438,8 +1438,8 @@ lsh_status copy_microstructure(lsh_handle* h, const unsigned char* phase, const 
 
 // Separate passes: whether the inverse x pass can update z with these variants.
 int can_fuse(const lsh_handle* h, int x_variant, int z_variant) {
-  return h->d.precision == LSH_MIXED && x_variant == 0 && (z_variant == 0 || z_variant == 9) &&
-                 make_cfg<float>(h->d, h->d.Smax).smem_x <= 200 * 1024
+  return h->d.precision == LSH_MIXED && x_variant != 2 && (z_variant == 0 || z_variant == 9) &&
+                 (x_variant != 0 || make_cfg<float>(h->d, h->d.Smax).smem_x <= 200 * 1024)
              ? 1
              : 0;
 }
@@ -1934,19 +1934,22 @@ lsh_status lsh_autotune(lsh_handle* h, lsh_tune_report* rep) {
       cudaGetLastError();
       return LSH_ERR_CUDA;
     }
-    // average of 5 launches after 2 untimed ones; -1 if the variant does not run here
+    // average of 5 launches after 2 untimed ones, of 2 after one where a launch takes a
+    // sizeable part of a millisecond or more; -1 if the variant does not run here
+    const bool big = (long long)d.Smax * d.c * d.V >= 1ll << 27;
+    const int warm = big ? 1 : 2, reps = big ? 2 : 5;
     auto timeit = [&](auto launch) -> float {
-      for (int k = 0; k < 2; ++k)
+      for (int k = 0; k < warm; ++k)
         if (!launch()) return -1.f;
       cudaEventRecord(e0, s);
-      for (int k = 0; k < 5; ++k) launch();
+      for (int k = 0; k < reps; ++k) launch();
       cudaEventRecord(e1, s);
       float ms = -1.f;
       if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) {
         cudaGetLastError();
         return -1.f;
       }
-      return ms / 5.f;
+      return ms / (float)reps;
     };
     // the x passes are timed as in a CG iteration, on states of a running solve
     std::vector<SolverState> fake(d.Smax);
@@ -1956,6 +1959,14 @@ lsh_status lsh_autotune(lsh_handle* h, lsh_tune_report* rep) {
       f.rr = f.rz = 1.0;
     }
     LSH_CK(cudaMemcpyAsync(P.st, fake.data(), sizeof(SolverState) * d.Smax, cudaMemcpyHostToDevice, s));
+    int fx = -1;  // the fastest inverse x pass that updates z, and its time
+    float fx_ms = -1.f;
+    bool fused = false;
+    const float upd = timeit([&]() {
+      cudaMemcpyAsync(P.st, fake.data(), sizeof(SolverState) * d.Smax, cudaMemcpyHostToDevice, s);
+      launch_cg_update<float>(a, P.r, P.q, P.st, h->partials, h->lay.nparts, P.L.ew_per_sys, s);
+      return true;
+    });
     // the separate x and y passes need natural y order for the FP32 table on
     // plane grids (powers of two); radix-3 planes have the plane passes only
     const bool sep_ok = !d.plane || reg_length(d.ny);
@@ -1987,6 +1998,16 @@ lsh_status lsh_autotune(lsh_handle* h, lsh_tune_report* rep) {
           return true;
         });
         if (r.x_ms[v] > 0.f && r.x_ms[v] < r.x_ms[bx]) bx = v;
+        if (!can_fuse(h, v, 0) || (v != 0 && !xinv_reg_fits(a))) continue;
+        const float t = timeit([&]() {
+          cudaMemcpyAsync(P.st, fake.data(), sizeof(SolverState) * d.Smax, cudaMemcpyHostToDevice, s);
+          launch_xinv_update(a, P.L, P.p, P.r, P.st, h->partials, h->lay.nparts, s);
+          return true;
+        });
+        if (t > 0.f && (fx < 0 || t < fx_ms)) {
+          fx = v;
+          fx_ms = t;
+        }
       }
       r.x_variant = bx;
       a.xreg = r.x_variant;
@@ -2005,10 +2026,6 @@ lsh_status lsh_autotune(lsh_handle* h, lsh_tune_report* rep) {
     if (sep_ok && a.zreg) {
       int best = 0;
       for (int v = 0; v < 10; ++v) {
-        // with the shared-memory inverse x pass only the variants that give (p, Gamma p):
-        // its update of z saves more than the others gain (96 x 80 x 64: 16 us of update
-        // kernel against 1 us)
-        if (can_fuse(h, a.xreg, 0) && !can_fuse(h, a.xreg, v)) continue;
         if (v >= 1 && v <= 5 && !P.ztma_ok) continue;  // TMA tiles need the tensor map
         a.ztma = v;
         r.z_ms[v] = timeit([&]() {
@@ -2022,7 +2039,20 @@ lsh_status lsh_autotune(lsh_handle* h, lsh_tune_report* rep) {
         if (r.z_ms[v] > 0.f && (r.z_ms[best] < 0.f || r.z_ms[v] < r.z_ms[best])) best = v;
       }
       r.z_variant = best;
-      a.ztma = best;
+    }
+    if (sep_ok) {
+      // the fastest passes with an update kernel, or the fastest inverse pass that updates
+      // z behind a z pass that leaves (p, Gamma p).  256^3, six systems: 1.61 + 1.23 ms
+      // against 2.28; 64 x 64 x 16: a z variant 1 us faster does not pay for the kernel
+      const int zd = a.zreg && r.z_ms[9] > 0.f && r.z_ms[9] < r.z_ms[0] ? 9 : 0;
+      const float zdiff = a.zreg ? r.z_ms[zd] - r.z_ms[r.z_variant] : 0.f;
+      if (fx >= 0 && fx_ms + zdiff < r.x_ms[r.x_variant] + upd) {
+        fused = true;
+        r.x_variant = fx;
+        r.z_variant = zd;
+      }
+      a.xreg = r.x_variant;
+      a.ztma = r.z_variant;
     }
     if (d.plane) {
       // the plane passes with the register z kernels on the ky-major spectrum,
@@ -2051,11 +2081,6 @@ lsh_status lsh_autotune(lsh_handle* h, lsh_tune_report* rep) {
         cudaMemcpyAsync(P.st, fake.data(), sizeof(SolverState) * d.Smax, cudaMemcpyHostToDevice, s);
         return launch_xyinv(b, 1, P.p, P.q, P.st, h->partials, s);
       });
-      const float u = timeit([&]() {
-        cudaMemcpyAsync(P.st, fake.data(), sizeof(SolverState) * d.Smax, cudaMemcpyHostToDevice, s);
-        launch_cg_update<float>(b, P.r, P.q, P.st, h->partials, h->lay.nparts, P.L.ew_per_sys, s);
-        return true;
-      });
       float z = r.zp_ms[bz];
       if (r.zp_ms[6] > 0.f) {
         // z variant 11 leaves (p, Gamma p), so that the inverse pass can update z
@@ -2068,10 +2093,10 @@ lsh_status lsh_autotune(lsh_handle* h, lsh_tune_report* rep) {
           launch_cg_alpha(P.st, h->partials, zdot_count(b), b.S, false, s);
           return ok;
         });
-        if (zf > 0.f && jf > 0.f && zf + jf < z + i + u) {
+        if (zf > 0.f && jf > 0.f && zf + jf < z + i + upd) {
           b.fuse = 1;
           z = zf;
-          i = jf - u;  // comparable with the separate schedule's sum, which has no update kernel either
+          i = jf - upd;  // comparable with the separate schedule's sum, which has no update kernel either
         } else {
           b.ztma = zc[bz];
         }
@@ -2080,7 +2105,7 @@ lsh_status lsh_autotune(lsh_handle* h, lsh_tune_report* rep) {
       if (sep_ok) {
         const float xf = r.xf_ms[a.xfreg] > 0.f ? r.xf_ms[a.xfreg] : r.xf_ms[0];
         const float yy = r.y_ms[a.ytma] > 0.f ? r.y_ms[a.ytma] : -1.f;
-        const float zz = r.z_ms[a.ztma], xi = r.x_ms[a.xreg];
+        const float zz = r.z_ms[a.ztma], xi = fused ? fx_ms - upd : r.x_ms[a.xreg];
         if (xf > 0.f && yy > 0.f && zz > 0.f && xi > 0.f) r.xy_ms[0] = xf + 2.f * yy + zz + xi;
       }
       if (!sep_ok || (r.xy_ms[1] > 0.f && (r.xy_ms[0] < 0.f || r.xy_ms[1] < r.xy_ms[0]))) {
@@ -2094,7 +2119,7 @@ lsh_status lsh_autotune(lsh_handle* h, lsh_tune_report* rep) {
     lsh_status st = last_launch();
     if (st) return st;
     if (h->fault && (st = check_fault(h))) return st;
-    if (!a.plane) a.fuse = can_fuse(h, a.xreg, a.ztma);
+    if (!a.plane) a.fuse = fused;
     P.a.xreg = a.xreg;
     P.a.xfreg = a.xfreg;
     P.a.ytma = a.ytma;
