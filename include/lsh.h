@@ -209,7 +209,8 @@ lsh_status lsh_set_microstructure(lsh_handle *h, const unsigned char *phase, con
  * x, y: device, nbatch*c*V elements of `dtype` (LSH_F64; LSH_F32 for
  * LSH_MIXED handles; LSH_F64_DF, FP64 fields evaluated in double-float, for
  * LSH_MIXED handles of the grids listed at LSH_F64_DF -- else
- * LSH_ERR_UNSUPPORTED), layout [nbatch][c][n2][n1][n0].  Asynchronous. */
+ * LSH_ERR_UNSUPPORTED), layout [nbatch][c][n2][n1][n0].  y may be x (in
+ * place); buffers that overlap in part are not supported.  Asynchronous. */
 lsh_status lsh_apply(lsh_handle *h, int dtype, const void *x, void *y);
 
 /* Solve Eq. (13) for one macroscopic load p (host, c doubles; Mandel

@@ -1756,10 +1756,13 @@ lsh_status lsh_apply(lsh_handle* h, int dtype, const void* x, void* y) {
       af.mandel = el && af.plane && af.ztma == 11;
       const bool rot = (el || d.rotated) && !af.mandel;
       const bool stage = !rot && unaligned(in, o);
+      // in Mandel components a block reads all three normal components of x while other
+      // blocks write them to y: an x that y overlaps is read from a copy
+      const bool shared = af.mandel && in < o + S * n && o < in + S * n;
       if (rot) {
         rotate(in, P.p, 1);
         in = P.p;
-      } else if (stage) {
+      } else if (stage || shared) {
         LSH_CK(cudaMemcpyAsync(P.p, in, sizeof(float) * (size_t)(S * n), cudaMemcpyDeviceToDevice, h->stream));
         in = P.p;
       }
