@@ -1489,30 +1489,36 @@ __global__ void k_scale_grad(const double* __restrict__ tau_all, const double* _
 }
 
 // ------------------------------------------------------------------ launchers
-// The attribute is a per-function upper bound shared by every handle: always
-// allow the full 227 KB so that one handle never shrinks another's limit.
-template <typename T, int VEC> void set_smem_attrs_x(int mx) {
-  cudaFuncSetAttribute(k_xfwd<T, 0, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_xfwd<T, 1, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_xinv<T, 0, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_xinv<T, 1, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  if constexpr (sizeof(T) == 4)  // less its larger static tables
-    cudaFuncSetAttribute(k_xinv<T, 5, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx - 24 * 1024);
+// The attribute is a per-function upper bound shared by every handle: always allow as much
+// as the 227 KB leave beside the kernel's own static arrays, so that one handle never
+// shrinks another's limit.  A request for more is refused as a whole, and the kernel then
+// keeps to 48 KB, static and dynamic together.
+constexpr int kSmemMax = 227 * 1024;
+constexpr int kReduceSmem = 512;  // block_reduce and the flag of the last block
+template <typename T, int MODE> constexpr int kXinvSmem = 256 * 6 * (int)sizeof(T) * (MODE == 5 ? 3 : 1) + 256 + 2 * kReduceSmem;
+template <typename T, int MODE, int VEC> void set_smem_attr_xinv() {
+  cudaFuncSetAttribute(k_xinv<T, MODE, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - kXinvSmem<T, MODE>);
+}
+template <typename T, int VEC> void set_smem_attrs_x() {
+  cudaFuncSetAttribute(k_xfwd<T, 0, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+  cudaFuncSetAttribute(k_xfwd<T, 1, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+  set_smem_attr_xinv<T, 0, VEC>();
+  set_smem_attr_xinv<T, 1, VEC>();
+  if constexpr (sizeof(T) == 4) set_smem_attr_xinv<T, 5, VEC>();
   if constexpr (sizeof(T) == 8) {
-    cudaFuncSetAttribute(k_xinv<T, 2, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    cudaFuncSetAttribute(k_xinv<T, 3, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+    set_smem_attr_xinv<T, 2, VEC>();
+    set_smem_attr_xinv<T, 3, VEC>();
   }
 }
 template <typename T> void set_smem_attrs() {
-  const int mx = 227 * 1024;
-  set_smem_attrs_x<T, 1>(mx);
-  set_smem_attrs_x<T, 2>(mx);
-  if constexpr (sizeof(T) == 4) set_smem_attrs_x<T, 4>(mx);
-  cudaFuncSetAttribute(k_yfft<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_yfft<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_zgamma<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_zgamma<T, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  cudaFuncSetAttribute(k_zgamma<T, 6>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+  set_smem_attrs_x<T, 1>();
+  set_smem_attrs_x<T, 2>();
+  if constexpr (sizeof(T) == 4) set_smem_attrs_x<T, 4>();
+  cudaFuncSetAttribute(k_yfft<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+  cudaFuncSetAttribute(k_yfft<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+  cudaFuncSetAttribute(k_zgamma<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - kReduceSmem);
+  cudaFuncSetAttribute(k_zgamma<T, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - kReduceSmem);
+  cudaFuncSetAttribute(k_zgamma<T, 6>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - kReduceSmem);
   set_smem_attrs_reg<T>();
 }
 
