@@ -294,8 +294,20 @@ void launch_scale_grad(const double* tau_all, const double* W, const unsigned ch
                        const double* modtab, const double* ref, int c, int elastic, long long V, int B,
                        double* grad, cudaStream_t s);
 
-// FP32 CG iteration of the separate passes with the update of z in the inverse x pass
-int zdot_blocks(const OpArgs<float>& a, const LaunchCfg& L);
+// FP32 CG iteration of the separate passes with the update of z in the inverse x pass.
+// Blocks per system of the z pass, each of which leaves its share of (p, Gamma p): register
+// kernel in tiles of 8 columns (z variants 0 and 9), pointwise kernel of a scalar 2D grid,
+// else the shared-memory tiles, grids of one z layer with six components among them.  The
+// workspace holds as many partials for every system, at the tiles of a single one (the
+// most): the layout asks the same function.
+inline long long zdot_blocks(bool zreg, int nxh, int ny, int nz, int c, const LaunchCfg& L) {
+  if (zreg) {
+    const int TZ = 8, nrt = nxh / TZ;
+    return (long long)ny * nrt + ((long long)ny * (nxh - nrt * TZ) + TZ - 1) / TZ;
+  }
+  if (nz == 1 && c != 6) return ((nxh + 31) / 32) * (long long)((ny + 7) / 8);
+  return (long long)L.grid_zx * L.grid_zy;
+}
 void launch_xinv_update(const OpArgs<float>& a, const LaunchCfg& L, const float* p, float* z, SolverState* st,
                         double* partials, long long off, cudaStream_t s);
 void launch_cg_beta(SolverState* st, const double* partials, long long off, int nb, int S, bool pdl, cudaStream_t s);

@@ -1613,15 +1613,6 @@ void launch_xinv(const OpArgs<T>& a, const LaunchCfg& L, int mode, const T* xin,
 #undef LSH_XINV
 }
 
-int zdot_blocks(const OpArgs<float>& a, const LaunchCfg& L) {
-  if (a.zreg) {
-    const int TZ = 8, nrt = a.nxh / TZ;  // z variants 0 and 9
-    return a.ny * nrt + (a.ny * (a.nxh - nrt * TZ) + TZ - 1) / TZ;
-  }
-  if (a.nz == 1 && a.c != 6) return ((a.nxh + 31) / 32) * ((a.ny + kThreads / 32 - 1) / (kThreads / 32));
-  return L.grid_zx * L.grid_zy;
-}
-
 void launch_xinv_update(const OpArgs<float>& a, const LaunchCfg& L, const float* p, float* z, SolverState* st,
                         double* partials, long long off, cudaStream_t s) {
   if ((a.xreg == 1 || a.xreg == 3) && launch_xinv_reg(a, 5, p, z, st, partials, s, false, a.xreg == 3, off)) return;

@@ -367,10 +367,9 @@ Layout make_layout(const Derived& d) {
   // is even), the elementwise kernels 2432 blocks or one per system
   const long long xblocks = rps_of(d) % 2 == 0 ? rps_of(d) / 2 + 1 : rps_of(d);
   // (p, Gamma p) of the FP32 z pass: one partial per block, most with one system's tiles
-  const LaunchCfg L1 = make_cfg<float>(d, 1);
-  const long long zblocks = d.nz == 1 ? (d.nxh / 32 + 1LL) * (d.ny / 8 + 1)
-                                      : std::max<long long>((long long)L1.grid_zx * L1.grid_zy,
-                                                            (long long)d.ny * (d.nxh / 4 + 2));
+  // (fewer on the plane passes)
+  const long long zblocks =
+      zdot_blocks(d.plane || reg_length(d.nz), d.nxh, d.ny, d.nz, d.c, make_cfg<float>(d, 1));
   long long np = std::max<long long>({2432LL + S, d.precision == LSH_MIXED ? (long long)S * zblocks : 0LL, (long long)S * d.c * 152, (long long)d.B * 1216, (long long)S * xblocks,
                                       (long long)S * d.c * d.nz});
   l.nparts = np;
@@ -885,7 +884,7 @@ template <typename T> void enqueue_cg_iteration(lsh_handle* h, PrecBufs<T>& P, c
       launch_yfft<T>(a, P.L, false, P.st, s);
       if (timed) cudaEventRecordWithFlags(e[2], s, rf);
       launch_zgamma<T>(a, P.L, P.st, s);
-      launch_cg_alpha(P.st, h->partials, zdot_blocks(a, P.L), a.S, a.pdl != 0, s);
+      launch_cg_alpha(P.st, h->partials, (int)zdot_blocks(a.zreg != 0, a.nxh, a.ny, a.nz, a.c, P.L), a.S, a.pdl != 0, s);
       if (timed) cudaEventRecordWithFlags(e[3], s, rf);
       launch_yfft<T>(a, P.L, true, P.st, s);
       if (timed) cudaEventRecordWithFlags(e[4], s, rf);
