@@ -51,7 +51,7 @@ struct SolverState {
   int iter;         // completed CG iterations
   int done;         // nonzero: converged or failed, later kernels return at once
   int status;       // lsh_status-compatible code set on device (0, breakdown)
-  int pad;
+  int pad;          // setup scan: largest phase id; solves in a cluster: timed iterations
   unsigned int counter[4];  // last-block counters, reset by the last block
 };
 

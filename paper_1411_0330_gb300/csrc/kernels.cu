@@ -1017,6 +1017,7 @@ __global__ void __launch_bounds__(kThreads) k_cg_begin(OpArgs<T> a, T* __restric
       sst->pq = 0.0;
       sst->iter = 0;
       sst->status = 0;
+      sst->pad = 0;
       sst->done = (rr <= sst->tol2) ? 1 : 0;
     }
   }
@@ -1346,6 +1347,7 @@ __global__ void __launch_bounds__(kThreads) k_d2f_begin(OpArgs<float> a, const d
       sst->alpha = sst->beta = sst->pq = 0.0;
       sst->iter = 0;
       sst->status = 0;
+      sst->pad = 0;
       sst->done = (!active[s] || rr <= sst->tol2) ? 1 : 0;
     }
   }
