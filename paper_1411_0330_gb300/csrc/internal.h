@@ -182,19 +182,40 @@ LaunchCfg pass_cfg(int nx, int ny, int nz, int c, const Plan1D& px, const Plan1D
   const int resident = sizeof(T) == 8 ? 512 : 768;  // threads per SM at the passes' register counts
   constexpr long long kBlocks = 608;                // four per SM
   // rows per x block: an even divisor of the rows of a system where there is one
-  int target = std::max(2, 2 * (int)(32768 / (lsx * cs)));
-  target = std::min(target, std::max(2, (int)((long long)rps * S / (kBlocks / 2))));
-  if (target >= rps) {
-    L.RY = rps;
-  } else {
-    int odd = 1;
-    L.RY = 0;
-    for (int d = target; d >= 1 && !L.RY; --d)
-      if (rps % d == 0) {
-        if (d % 2 == 0) L.RY = d;
-        else if (odd == 1) odd = d;
+  const int cap = std::max(2, 2 * (int)(32768 / (lsx * cs)));
+  const bool fixed = nx == 16 || nx == 32 || nx == 48 || nx == 64 || nx == 96 || nx == 128 || nx == 256;
+  L.RY = 0;
+  if (sizeof(T) == 8 && fixed && cap < rps) {
+    // FP64 at the lengths with a compile-time schedule, blocks of 256 threads, two to an SM:
+    // the divisor of the least time, a wave of blocks costing its chain of barriers (the
+    // time of some 1280 elements) and an SM the elements of its blocks; among equals the
+    // larger.  us per iteration with RY = 8 (384 blocks, two waves) / 12 (256, one): 32^3
+    // conductivity, one load, 68 / 55; 16 x 64 x 64 75 / 61; 32^3 elasticity, six loads, 96
+    // (384) / 64 (576) 180 / 173; 96^3 conductivity 36 (768) / 32 (864) 502 / 474.
+    long long best = 0;
+    for (int d = cap & ~1; d >= 2; d -= 2) {
+      if (rps % d != 0) continue;
+      const long long blocks = (long long)S * (rps / d);
+      const long long t = (blocks + 303) / 304 * 1280 + (blocks + 151) / 152 * d * nx;
+      if (!L.RY || t < best) {
+        best = t;
+        L.RY = d;
       }
-    if (!L.RY) L.RY = odd;
+    }
+  }
+  if (!L.RY) {
+    const int target = std::min(cap, std::max(2, (int)((long long)rps * S / (kBlocks / 2))));
+    if (target >= rps) {
+      L.RY = rps;
+    } else {
+      int odd = 1;
+      for (int d = target; d >= 1 && !L.RY; --d)
+        if (rps % d == 0) {
+          if (d % 2 == 0) L.RY = d;
+          else if (odd == 1) odd = d;
+        }
+      if (!L.RY) L.RY = odd;
+    }
   }
   constexpr int VV = 16 / (int)sizeof(T);
   L.VEC = nx % VV == 0 ? VV : (nx % 2 == 0 ? 2 : 1);
@@ -202,7 +223,6 @@ LaunchCfg pass_cfg(int nx, int ny, int nz, int c, const Plan1D& px, const Plan1D
   L.smem_x = nx * cs + (size_t)npair * lsx * cs + nx * sizeof(int);
   // the FP32 x passes stream three fields in and two out: the loads want every thread; the
   // lengths with a compile-time schedule are bound by the FP64 pipe at any block size
-  const bool fixed = nx == 16 || nx == 32 || nx == 48 || nx == 64 || nx == 96 || nx == 128 || nx == 256;
   L.thr_x = sizeof(T) == 4 || fixed ? 256 : pass_threads(npair, px, L.smem_x, resident, (long long)S * (rps / L.RY));
   // y columns per block: up to 16 (8 in FP64), evenly shared among a plane's blocks
   int TY = std::min(sizeof(T) == 8 ? 8 : 16, nxh);
