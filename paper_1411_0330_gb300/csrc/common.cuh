@@ -67,6 +67,7 @@ template <typename T> struct Acc;
 template <> struct Acc<double> {
   double s = 0.0;
   __device__ __forceinline__ void add(double v) { s += v; }
+  __device__ __forceinline__ void mac(double a, double b) { s = fma(a, b, s); }
   __device__ __forceinline__ double get() const { return s; }
 };
 template <> struct Acc<float> {
@@ -77,7 +78,38 @@ template <> struct Acc<float> {
     c = (t - s) - y;
     s = t;
   }
+  // add(a * b) with one rounding for the product and the compensation together
+  __device__ __forceinline__ void mac(float a, float b) {
+    const float y = fmaf(a, b, -c);
+    const float t = s + y;
+    c = (t - s) - y;
+    s = t;
+  }
   __device__ __forceinline__ double get() const { return (double)s - (double)c; }
+};
+
+// Two FP32 accumulators side by side for products that come in pairs (the two parts of a
+// complex value, neighbouring voxels): the operations of Acc<float>::mac on both halves of
+// packed registers.
+struct Acc2 {
+  float2 s = {0.0f, 0.0f}, n = {0.0f, 0.0f};  // n: minus the compensation
+  __device__ __forceinline__ void mac(float2 a, float2 b) {
+    const float2 m = make_float2(-1.0f, -1.0f);
+    const float2 y = __ffma2_rn(a, b, n);
+    const float2 t = __fadd2_rn(s, y);
+    n = __ffma2_rn(m, __ffma2_rn(m, s, t), y);  // y - (t - s)
+    s = t;
+  }
+  // both sums times w (a power of two) as one compensated pair
+  __device__ __forceinline__ Acc<float> fold(float w = 1.0f) const {
+    Acc<float> a;
+    a.s = s.x + s.y;
+    const float bp = a.s - s.x;
+    a.c = -(n.x + n.y) - ((s.x - (a.s - bp)) + (s.y - bp));  // s.x + s.y = a.s + the bracket exactly
+    a.s *= w;
+    a.c *= w;
+    return a;
+  }
 };
 
 // Block sum of per-thread accumulators; result valid in thread 0.  FP32

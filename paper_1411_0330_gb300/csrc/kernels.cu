@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_zgamma(OpArgs
   __syncthreads();
   if (nz > 1) fft_lines<T, false>(buf, NC * TZ, a.lsz, a.pz, tw);
   // per-frequency product with Gamma^h_k
-  Acc<float> accd;
+  Acc2 accd;
   const int ky = (a.onfly || a.fdphase) ? a.kofy[yp] : 0;
   for (int idx = threadIdx.x; idx < nz * TZ; idx += blockDim.x) {
     const int zp = dtz.div(idx), t = idx - zp * TZ;
@@ -282,13 +282,9 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_zgamma(OpArgs
     }
     if constexpr (sizeof(T) == 4)
       if (a.dot) {
-        T q = 0;
+        const T w = (kx0 + t == 0 || 2 * (kx0 + t) == a.nx) ? (T)1 : (T)2;
 #pragma unroll
-        for (int i = 0; i < NC; ++i) {
-          const C2<T> u = buf[(i * TZ + t) * a.lsz + zp];
-          q += u.x * v[i].x + u.y * v[i].y;
-        }
-        accd.add((kx0 + t == 0 || 2 * (kx0 + t) == a.nx) ? q : q + q);
+        for (int i = 0; i < NC; ++i) accd.mac(cscale<T>(buf[(i * TZ + t) * a.lsz + zp], w), v[i]);
       }
 #pragma unroll
     for (int i = 0; i < NC; ++i) buf[(i * TZ + t) * a.lsz + zp] = v[i];
@@ -296,7 +292,7 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_zgamma(OpArgs
   if constexpr (sizeof(T) == 4)
     if (a.dot) {
       // the block's share of (p, Gamma p) (see k_xinv, MODE 5)
-      const double d = block_reduce(accd);
+      const double d = block_reduce(accd.fold());
       if (threadIdx.x == 0)
         a.dot[((long long)s * gridDim.z + blockIdx.z) * gridDim.y + blockIdx.y] = d;
     }
@@ -318,7 +314,7 @@ __global__ void __launch_bounds__(kThreads) k_gamma2d(OpArgs<T> a, const SolverS
   chain_wait();
   if (st != nullptr && is_done(st + s)) return;
   const int kx = blockIdx.x * 32 + (threadIdx.x & 31), yp = blockIdx.y * (kThreads / 32) + (threadIdx.x >> 5);
-  Acc<float> accd;
+  Acc2 accd;
   if (kx < a.nxh && yp < a.ny) {
     const long long cstride = (long long)a.ny * a.hs;
     C2<T>* __restrict__ Hp = a.H + (long long)s * NC * cstride + (long long)yp * a.hs + kx;
@@ -333,17 +329,15 @@ __global__ void __launch_bounds__(kThreads) k_gamma2d(OpArgs<T> a, const SolverS
       gamma_table_apply<T, NC>(a.gtab, (long long)yp * a.ts + kx, v);
       if (a.fdphase) fd_rotate<T, NC>(a, kx, ky, 0, v, (T)1);
     }
-    T q = 0;
 #pragma unroll
     for (int i = 0; i < NC; ++i) {
-      q += u[i].x * v[i].x + u[i].y * v[i].y;
+      if constexpr (sizeof(T) == 4) accd.mac(u[i], v[i]);
       Hp[i * cstride] = v[i];
     }
-    if (sizeof(T) == 4) accd.add((float)((kx == 0 || 2 * kx == a.nx) ? q : q + q));
   }
   if constexpr (sizeof(T) == 4)
     if (a.dot) {
-      const double d = block_reduce(accd);
+      const double d = block_reduce(accd.fold((kx == 0 || 2 * kx == a.nx) ? 1.f : 2.f));
       if (threadIdx.x == 0) a.dot[((long long)s * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = d;
     }
 }

@@ -173,14 +173,14 @@ __device__ __forceinline__ void cluster_gamma(const OpArgs<T>& a, C2<T>* __restr
       gamma_table_apply<T, NC>(a.gtab, f, v);
       if (a.fdphase) fd_rotate<T, NC>(a, kx, ky, kz, v, (T)1);
     }
-    T q = 0;
+    // columns other than kx = 0 and nx/2 stand for their mirror images too
+    const T w2 = (kx == 0 || 2 * kx == a.nx) ? (T)1 : (T)2;
 #pragma unroll
     for (int i = 0; i < NC; ++i) {
-      q += u[i].x * v[i].x + u[i].y * v[i].y;
+      acc.mac(w2 * u[i].x, v[i].x);
+      acc.mac(w2 * u[i].y, v[i].y);
       G[(i * ns + sp) * pp + t] = v[i];
     }
-    // columns other than kx = 0 and nx/2 stand for their mirror images too
-    acc.add((kx == 0 || 2 * kx == a.nx) ? q : q + q);
   }
 }
 

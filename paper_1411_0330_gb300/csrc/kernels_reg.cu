@@ -92,21 +92,17 @@ template <typename T, int NC, int N, int TZV = 0> struct ZCfg {
 // in place in buf[kz KS + comp TZ + li]; line_yp/line_kx give each line's y
 // position (-1: no line) and kx.  PIPE: a thread loads the table coefficients
 // of its next frequency while it applies the current ones.
-// accd (FP32 with a.dot): gains the block's share of (p, Gamma p).
+// accd (FP32 with a.dot): gains this thread's share of (p, Gamma p), each frequency counted
+// once; a thread's frequencies lie in one column, its number mod TZ.
 template <typename T, int NC, int N, int TZ, int KS, bool PIPE = true>
 __device__ __forceinline__ void z_gamma_block(const OpArgs<T>& a, C2<T>* buf, const int* line_yp,
-                                              const int* line_kx, Acc<float>& accd) {
+                                              const int* line_kx, Acc2& accd) {
   // the product's result g in place of the frequency's values in buf
-  auto put = [&](C2<T>* at, int kx, const C2<T>* g) {
+  auto put = [&](C2<T>* at, const C2<T>* g) {
     if constexpr (sizeof(T) == 4)
       if (a.dot) {
-        float q = 0.f;
 #pragma unroll
-        for (int c2 = 0; c2 < NC; ++c2) {
-          const C2<T> u = at[c2 * TZ];
-          q += u.x * g[c2].x + u.y * g[c2].y;
-        }
-        accd.add((kx == 0 || 2 * kx == a.nx) ? q : q + q);
+        for (int c2 = 0; c2 < NC; ++c2) accd.mac(at[c2 * TZ], g[c2]);
       }
 #pragma unroll
     for (int c2 = 0; c2 < NC; ++c2) at[c2 * TZ] = g[c2];
@@ -123,7 +119,7 @@ __device__ __forceinline__ void z_gamma_block(const OpArgs<T>& a, C2<T>* buf, co
 #pragma unroll
         for (int c2 = 0; c2 < NC; ++c2) g[c2] = buf[kz * KS + c2 * TZ + li];
         gamma_trunc_onfly<T, NC>(a, line_kx[li], a.kofy[lyp], kz, g);
-        put(buf + kz * KS + li, line_kx[li], g);
+        put(buf + kz * KS + li, g);
       }
     }
   } else if constexpr (!PIPE) {
@@ -139,7 +135,7 @@ __device__ __forceinline__ void z_gamma_block(const OpArgs<T>& a, C2<T>* buf, co
       gamma_table_apply<T, NC>(a.gtab, ((long long)kz * a.ny + lyp) * a.ts + line_kx[li], g);
       if constexpr (FLY)
         if (a.fdphase) fd_rotate<T, NC>(a, line_kx[li], a.kofy[lyp], kz, g, (T)1);
-      put(buf + kz * KS + li, line_kx[li], g);
+      put(buf + kz * KS + li, g);
     }
   } else {
     // tabulated Gamma^h_k: the coefficients of a thread's next frequency are
@@ -169,7 +165,7 @@ __device__ __forceinline__ void z_gamma_block(const OpArgs<T>& a, C2<T>* buf, co
         gamma_coef_apply<T, NC>(gc, g);
         if constexpr (FLY)
           if (a.fdphase) fd_rotate<T, NC>(a, line_kx[li], a.kofy[line_yp[li]], kz, g, (T)1);
-        put(buf + kz * KS + li, line_kx[li], g);
+        put(buf + kz * KS + li, g);
       }
 #pragma unroll
       for (int c = 0; c < NCO; ++c) gc[c] = gn[c];
@@ -271,11 +267,14 @@ __global__ void __launch_bounds__(ZCfg<T, NC, N, TZV>::THREADS,
 #pragma unroll
   for (int m = 0; m < R1; ++m) buf[RL::freq(t, m) * KS + comp * TZ + i] = v[m];
   __syncthreads();
-  Acc<float> accd;
+  Acc2 accd;
   z_gamma_block<T, NC, N, TZ, KS, (TZV >= 0)>(a, buf, line_yp, line_kx, accd);
   if constexpr (sizeof(T) == 4)
     if (a.dot) {
-      const double d = block_reduce(accd);
+      // columns other than kx = 0 and nx/2 stand for their mirror images too
+      static_assert(ZC::THREADS % TZ == 0, "columns of a thread");
+      const int kx = line_kx[threadIdx.x % TZ];
+      const double d = block_reduce(accd.fold(kx == 0 || 2 * kx == a.nx ? 1.f : 2.f));
       if (threadIdx.x == 0) a.dot[(long long)s * gridDim.y + tile] = d;
     }
   __syncthreads();
@@ -428,7 +427,7 @@ __global__ void __launch_bounds__(ZPCfg<NC, N>::THREADS, ZPCfg<NC, N>::THREADS <
 #pragma unroll
     for (int m = 0; m < R1; ++m) buf[RL::freq(t, m) * KS + comp * TZ + i] = v[m];
     __syncthreads();
-    Acc<float> unused;
+    Acc2 unused;
     z_gamma_block<float, NC, N, TZ, KS, false>(a, buf, line_yp, line_kx, unused);
     __syncthreads();
 #pragma unroll

@@ -80,11 +80,11 @@ template <int Q> __device__ __forceinline__ int zp_grow(int kz) {
 // of each k2, transforms back and writes the same rows.  The coefficients of
 // the next k2 load while the current ones are applied.
 // DOT: acc gains this item's share of (p, Gamma p) = sum_k Re(conj p_k (Gamma p)_k)
-// over the full spectrum (the table carries 1/V, the transforms are unnormalised):
-// columns other than kx = 0 and nx/2 stand for their mirror images too.
+// (the table carries 1/V, the transforms are unnormalised), each frequency once: columns
+// other than kx = 0 and nx/2 stand for their mirror images too, which the caller weights.
 template <int NC, int N, bool DOT>
 __device__ __forceinline__ void zp_fused_item(const OpArgs<float>& a, float2* B, int item, bool nyq, int yp,
-                                              int kx0, Acc<float>& acc) {
+                                              int kx0, Acc2& acc) {
   typedef ZPipe<NC, N, true> ZC;
   constexpr int TZ = ZC::TZ, P = ZC::P, R1 = ZC::R1, NX = ZC::NX;
   const int li = item & (TZ - 1), k1 = item / TZ, kb = k1 & 1;
@@ -93,15 +93,12 @@ __device__ __forceinline__ void zp_fused_item(const OpArgs<float>& a, float2* B,
   float2* const od = B + (4 * k1 - kb) * TZ + li;
   const int kx = nyq ? kx0 : kx0 + li, ypos = nyq ? yp + li : yp;
   float2 d[NC][P];
-  const float w = (nyq || kx == 0) ? 1.f : 2.f;
   auto put = [&](int k2, const float2* g) {  // the product's result in place of d[.][k2]
-    float q = 0.f;
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-      if (DOT) q = fmaf(d[c][k2].x, g[c].x, fmaf(d[c][k2].y, g[c].y, q));
+      if (DOT) acc.mac(d[c][k2], g[c]);
       d[c][k2] = g[c];
     }
-    if (DOT) acc.add(w * q);
   };
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
@@ -269,10 +266,13 @@ __global__ void __launch_bounds__(ZPipe<NC, N, FUSED>::THREADS, ZPipe<NC, N, FUS
     for (int k1 = 0; k1 < R1; ++k1) B[xa(k1)] = v[k1];
     __syncthreads();
     if constexpr (FUSED) {
-      Acc<float> acc;
+      Acc2 acc2;
       for (int item = threadIdx.x; item < R1 * TZ; item += THREADS)
-        zp_fused_item<NC, N, DOT>(a, B, item, nyq, yp, kx0, acc);
+        zp_fused_item<NC, N, DOT>(a, B, item, nyq, yp, kx0, acc2);
       if constexpr (DOT) {
+        // a thread's items lie in one column (its number mod TZ): one weight for all of them
+        static_assert(THREADS % TZ == 0, "columns of a thread");
+        Acc<float> acc = acc2.fold(nyq || kx0 + (int)(threadIdx.x & (TZ - 1)) == 0 ? 1.f : 2.f);
         warp_merge_pair(acc.s, acc.c);
         if ((threadIdx.x & 31) == 0) {
           dot_sh[0][threadIdx.x >> 5] = acc.s;
