@@ -63,10 +63,11 @@ enum { LSH_GREEN_TRUNCATED = 0, LSH_GREEN_FILTERED = 1, LSH_GREEN_FD = 2 };
  * residual b - K x is computed to double-precision accuracy: in double-float
  * arithmetic (see LSH_F64_DF) where the grid allows it, else with the FP64
  * operator.  Where K is definite the FP32 CG is preconditioned by a diagonal
- * (1 / (|M_beta| + g), g the diagonal of the filtered Green operator, 0 for the
- * others), and so is FP64 CG on handles with a per-voxel field; FP64 CG on
- * phase maps is not.  The stopping rule is on the residual itself either way.  The environment variable LSH_NO_DF=1 at lsh_setup forces the
- * FP64 operator. */
+ * 1 / (|M_beta| + g), and so is FP64 CG on handles with a per-voxel field; FP64
+ * CG on phase maps is not.  g is the diagonal of the filtered Green operator;
+ * for the others it is 0 or, where |M| spreads far, a share of A0^{-1}.  The
+ * stopping rule is on the residual itself either way.  The environment variable
+ * LSH_NO_DF=1 at lsh_setup forces the FP64 operator. */
 enum { LSH_FP64 = 0, LSH_MIXED = 1 };
 /* element type of fields passed to lsh_apply.  LSH_F64_DF: FP64 fields, the
  * operator evaluated in double-float arithmetic (pairs of FP32 values, 48

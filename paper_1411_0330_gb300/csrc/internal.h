@@ -301,7 +301,8 @@ void launch_gamma_table(const OpArgs<T>& a, int dim, int physics, int green, con
 template <typename T>
 void launch_rotate_scalar(const T* in, T* out, long long V, int nsys, int d, const double* R, int to_internal,
                           cudaStream_t s);
-template <typename T> void launch_voxel_fields(const OpArgs<T>& a, T* mfld, T* dfld, int B, cudaStream_t s);
+template <typename T>
+void launch_voxel_fields(const OpArgs<T>& a, T* mfld, T* dfld, unsigned* range, int B, cudaStream_t s);
 void launch_gamma_diag(const OpArgs<double>& a, double* partials, int nblk, double* out, cudaStream_t s);
 void launch_d2f_begin(const OpArgs<float>& a, const double* r64, int src, float* r32, float* x32, SolverState* st,
                       double* partials, long long off2, double tol, const unsigned char* active, int G,

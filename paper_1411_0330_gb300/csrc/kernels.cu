@@ -846,7 +846,8 @@ template <typename T, typename F> __device__ __forceinline__ void sweep_planes(i
 // projector times A0^{-1/2}; with D = |M|^{-1} (gpre = 0) the preconditioned
 // operator is the identity plus a compression of (A - A0), whose condition number
 // is the contrast itself instead of the contrast times that of Gamma.  The
-// filtered operator has no kernel of that size, there D is the diagonal of K.
+// filtered operator has no kernel of that size, there D is the diagonal of K; so it is
+// where |M| spreads too far for |M|^{-1} (full_diagonal in lsh_api.cu).
 // FP32 iterations to 5e-6 (and 1e-10), 32^3 spheres at f = 0.3: contrast 10
 // truncated 46 (88) -> 22 (39), filtered 38 (75) -> 24 (46); contrast 1000
 // truncated 415 (850) -> 223 (400), filtered 116 (232) -> 72 (144).
@@ -1348,11 +1349,14 @@ __global__ void __launch_bounds__(kThreads) k_d2f_begin(OpArgs<float> a, const d
 }
 
 // M (and D) of every voxel of a handle with a scale or fraction field, per class of
-// components (see OpArgs): grid (G, classes).
+// components (see OpArgs): grid (G, classes).  range (or null, zero on entry): the largest
+// and the complement of the smallest |M| of each class as FP32 bit patterns.
 template <typename T>
-__global__ void __launch_bounds__(kThreads) k_voxel_fields(OpArgs<T> a, T* __restrict__ mfld, T* __restrict__ dfld) {
+__global__ void __launch_bounds__(kThreads) k_voxel_fields(OpArgs<T> a, T* __restrict__ mfld, T* __restrict__ dfld,
+                                                           unsigned* __restrict__ range) {
   const int cls = blockIdx.y;  // also the first component of the class
   const double g = (double)a.gpre[cls];
+  unsigned hi = 0u, lo = 0u;
   for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < a.fstride;
        v += (long long)gridDim.x * blockDim.x) {
     const T f = (T)a.scale[v];
@@ -1360,6 +1364,17 @@ __global__ void __launch_bounds__(kThreads) k_voxel_fields(OpArgs<T> a, T* __res
                        : (T)1 / (f * a.modtab[a.phase[v] * a.c + cls] - a.ref[cls]);
     mfld[cls * a.fstride + v] = m;
     if (dfld) dfld[cls * a.fstride + v] = (T)(1.0 / (fabs((double)m) + g));
+    const unsigned bits = __float_as_uint(fabsf((float)m));
+    hi = max(hi, bits);
+    lo = max(lo, ~bits);
+  }
+  if (range) {
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    lo = __reduce_max_sync(0xffffffffu, lo);
+    if ((threadIdx.x & 31) == 0) {
+      atomicMax(range + 2 * cls, hi);
+      atomicMax(range + 2 * cls + 1, lo);
+    }
   }
 }
 
@@ -1721,9 +1736,10 @@ void launch_d2f_begin(const OpArgs<float>& a, const double* r64, int src, float*
                             {k_d2f_begin<2, 0>, k_d2f_begin<2, 1>, k_d2f_begin<2, 2>}};
   k[src][a.pre]<<<g, kThreads, 0, s>>>(a, r64, r32, x32, st, partials, off2, tol, active);
 }
-template <typename T> void launch_voxel_fields(const OpArgs<T>& a, T* mfld, T* dfld, int B, cudaStream_t s) {
+template <typename T>
+void launch_voxel_fields(const OpArgs<T>& a, T* mfld, T* dfld, unsigned* range, int B, cudaStream_t s) {
   const int G = (int)std::max(1LL, std::min((B * a.V + kThreads - 1) / kThreads, 152LL * 8));
-  k_voxel_fields<T><<<dim3(G, a.physics != 0 ? 2 : a.c), kThreads, 0, s>>>(a, mfld, dfld);
+  k_voxel_fields<T><<<dim3(G, a.physics != 0 ? 2 : a.c), kThreads, 0, s>>>(a, mfld, dfld, range);
 }
 void launch_gamma_diag(const OpArgs<double>& a, double* partials, int nblk, double* out, cudaStream_t s) {
   k_gamma_diag<<<dim3(nblk, a.c), kThreads, 0, s>>>(a, partials);
@@ -1759,7 +1775,7 @@ void launch_scale_grad(const double* tau_all, const double* W, const unsigned ch
   template void launch_comp_sums<T>(const T*, int, long long, int, double*, int, double*, cudaStream_t);           \
   template void launch_gamma_table<T>(const OpArgs<T>&, int, int, int, const double*, const int*, const int*,      \
                                       cudaStream_t, const double*, const double*);                                 \
-  template void launch_voxel_fields<T>(const OpArgs<T>&, T*, T*, int, cudaStream_t);                               \
+  template void launch_voxel_fields<T>(const OpArgs<T>&, T*, T*, unsigned*, int, cudaStream_t);                    \
   template void launch_rotate_scalar<T>(const T*, T*, long long, int, int, const double*, int, cudaStream_t);
 
 LSH_INSTANTIATE(double)

@@ -471,6 +471,7 @@ struct lsh_handle {
   int *posx, *kofy, *kofz;
   int *kofy32, *kofz32;  // FP32 spectrum positions (natural order with the plane passes)
   double *sums, *Wdev, *tabd, *bbdev;
+  double gdiag[6] = {0, 0, 0, 0, 0, 0};  // diagonal of the Green operator in space (where D takes it)
   PrecBufs<double> pd;
   PrecBufs<float> pf;
   bool dfres = false;  // refinement residual in double-float (else native FP64)
@@ -1414,13 +1415,88 @@ lsh_status scan_microstructure(lsh_handle* h) {
   return LSH_OK;
 }
 
+// Whether D = 1 / (|M| + g) takes g = (a diagonal that stands for) the Green operator, or
+// g = 0 with an operator that is a projector up to A0 (truncated, finite differences; the
+// filtered one always takes its own diagonal).  lo, hi, mean: of |M| over the voxels; few:
+// the voxels take two values of it.  With g = 0 voxels of M far below the others' cost
+// iterations if they are rare and of many values; with g the count stayed at that of plain
+// CG or below it wherever it was tried.  Iterations of mixed solves to 1e-10, plain / g = 0 /
+// g, 64 x 64 conductivity, truncated (contrast; mean over the geometric mean of lo and hi):
+// random volume fractions (10; 1.9) 51 / 37 / 41, (100; 5.8) 69 / 102 / 55, (1000; 18) 72 /
+// 225 / 57; moduli evenly spread (1000; 0.3) 382 / 80 / 348, over their logarithm (100; 2.9)
+// 163 / 112 / 135, (10^4; 14) 960 / 930 / 798.  Two phases: stiff inclusions (10) 70 / 40 /
+// 47, (10^4) 2019 / 1297 / 1352, rare stiff voxels (10^6) 40 / 50 / 31; finite differences
+// (100) 87 / 56 / 60, (10^5) 101 / 153 / 72, (10^6) 74 / 305 / 53.
+bool full_diagonal(int green, double lo, double hi, double mean, bool few) {
+  if (green == LSH_GREEN_FILTERED) return true;
+  if (few) return !(hi <= (green == LSH_GREEN_TRUNCATED ? 1e5 : 4096.0) * lo);
+  return !(mean <= 5.0 * std::sqrt(hi * lo));
+}
+
+// The same for a problem with a phase map, every phase taken for as frequent as the others
+// (a fraction field: every value between its two ends).
+bool full_diagonal(const Derived& d) {
+  int active = 0;
+  for (int ph = 0; ph < d.nphase; ++ph) active += d.act[ph] ? 1 : 0;
+  bool full = d.green == LSH_GREEN_FILTERED;
+  for (int i = 0; i < d.c; ++i) {
+    double lo = 0.0, hi = 0.0, sum = 0.0;
+    for (int ph = 0; ph < d.nphase; ++ph) {
+      if (!d.act[ph]) continue;
+      const double m = std::fabs(d.m_in[(size_t)ph * d.c + i]);
+      lo = lo == 0.0 ? m : std::min(lo, m);
+      hi = std::max(hi, m);
+      sum += m;
+    }
+    if (active > 0) full = full || full_diagonal(d.green, lo, hi, sum / active, !d.has_scale && active <= 2);
+  }
+  return full;
+}
+
+// g of both precisions; graphs hold it in their kernels' arguments
+void set_precond_diag(lsh_handle* h, bool full) {
+  bool changed = false;
+  for (int i = 0; i < 6; ++i) {
+    const double g = full ? h->gdiag[i] : 0.0;
+    changed = changed || h->pd.a.gpre[i] != g;
+    h->pd.a.gpre[i] = g;
+    h->pf.a.gpre[i] = (float)g;
+  }
+  if (changed) h->drop_graphs();
+}
+
 // per-voxel M and D from the scale (fraction) field on the device
 lsh_status set_voxel_fields(lsh_handle* h) {
-  if (!h->d.has_scale) return LSH_OK;
-  launch_voxel_fields<double>(h->pd.a, const_cast<double*>(h->pd.a.mfld), const_cast<double*>(h->pd.a.dfld), h->d.B,
-                              h->stream);
-  if (h->d.precision == LSH_MIXED)
-    launch_voxel_fields<float>(h->pf.a, const_cast<float*>(h->pf.a.mfld), nullptr, h->d.B, h->stream);
+  const Derived& d = h->d;
+  if (!d.has_scale) return LSH_OK;
+  OpArgs<double>& a = h->pd.a;
+  double *mfld = const_cast<double*>(a.mfld), *dfld = const_cast<double*>(a.dfld);
+  // of a scale field lo, hi and the mean are known once its M are there
+  const bool open = !d.frac && d.green != LSH_GREEN_FILTERED;
+  const int classes = d.physics == LSH_ELASTIC_ISO ? 2 : d.c;
+  unsigned* range = open ? (unsigned*)h->Wdev : nullptr;
+  if (open) LSH_CK(cudaMemsetAsync(range, 0, sizeof(unsigned) * 2 * classes, h->stream));
+  launch_voxel_fields<double>(a, mfld, open ? nullptr : dfld, range, d.B, h->stream);
+  if (d.precision == LSH_MIXED)
+    launch_voxel_fields<float>(h->pf.a, const_cast<float*>(h->pf.a.mfld), nullptr, nullptr, d.B, h->stream);
+  if (open) {
+    launch_comp_sums<double>(mfld, classes, a.fstride, 1, h->partials, 152, h->sums, h->stream);
+    unsigned bits[6] = {0, 0, 0, 0, 0, 0};
+    double sum[3] = {0.0, 0.0, 0.0};
+    LSH_CK(cudaMemcpyAsync(bits, range, sizeof(unsigned) * 2 * classes, cudaMemcpyDeviceToHost, h->stream));
+    LSH_CK(cudaMemcpyAsync(sum, h->sums, sizeof(double) * classes, cudaMemcpyDeviceToHost, h->stream));
+    LSH_CK(cudaStreamSynchronize(h->stream));
+    bool full = false;
+    for (int k = 0; k < classes; ++k) {
+      const unsigned lo_bits = ~bits[2 * k + 1];
+      float hi, lo;
+      std::memcpy(&hi, &bits[2 * k], sizeof(hi));
+      std::memcpy(&lo, &lo_bits, sizeof(lo));
+      full = full || full_diagonal(d.green, lo, hi, std::fabs(sum[k]) / (double)a.fstride, false);
+    }
+    set_precond_diag(h, full);
+    launch_voxel_fields<double>(a, mfld, dfld, nullptr, d.B, h->stream);
+  }
   return last_launch();
 }
 
@@ -1632,32 +1708,36 @@ lsh_status lsh_setup(const lsh_problem* prob, void* workspace, size_t bytes, voi
     launch_gamma_table<float>(h->pf.a, d.dim, d.physics, d.green, d.ref_user, h->kofy32, h->kofz32, st,
                               d.rotated ? d.A0full : nullptr, d.rotated ? d.R : nullptr);
   if (h->pd.a.pre || (d.precision == LSH_MIXED && h->pf.a.pre)) {
-    // diagonal preconditioner 1 / (|M| + g): g = 0 where Gamma is a projector up to A0
-    // (truncated, finite differences), else the Green operator's diagonal in space
-    double g[6] = {0, 0, 0, 0, 0, 0};
+    // diagonal preconditioner 1 / (|M| + g), g = 0 or the Green operator's diagonal in space
+    const bool scaled = d.has_scale && !d.frac;  // decided with each scale field (set_voxel_fields)
+    const bool full = scaled ? d.green == LSH_GREEN_FILTERED : full_diagonal(d);
+    double* g = h->gdiag;
     if (d.green == LSH_GREEN_FILTERED) {
       launch_gamma_diag(h->pd.a, h->partials, 152, h->sums, st);
       SETUP_CK(cudaMemcpyAsync(g, h->sums, sizeof(double) * d.c, cudaMemcpyDeviceToHost, st));
       SETUP_CK(cudaStreamSynchronize(st));
+      if (d.has_scale && d.physics == LSH_ELASTIC_ISO) {
+        // the per-voxel fields hold one value for all deviatoric components
+        const double mean = (g[1] + g[2] + g[3] + g[4] + g[5]) / 5.0;
+        for (int i = 1; i < 6; ++i) g[i] = mean;
+      }
+    } else {
+      // A0^{-1} times the share of the components that the projector keeps.  Not its own
+      // diagonal, which on boxes of unequal lengths differs by component beyond A0: D would
+      // pull the projector's equal eigenvalues apart where M is small (20 x 24 x 28, random
+      // soft voxels of 10^-4, truncated: 490 iterations, 350 by plain CG).
+      for (int i = 0; i < d.c; ++i) g[i] = (d.physics == LSH_ELASTIC_ISO ? 0.5 : 1.0 / d.dim) / d.ref_in[i];
     }
-    if (d.has_scale && d.physics == LSH_ELASTIC_ISO) {
-      // the per-voxel fields hold one value for all deviatoric components
-      const double mean = (g[1] + g[2] + g[3] + g[4] + g[5]) / 5.0;
-      for (int i = 1; i < 6; ++i) g[i] = mean;
-    }
+    set_precond_diag(h, full);
     std::vector<double> dd(2 * 256 * 6, 1.0);  // D, then 1 / D
     std::vector<float> df(2 * 256 * 6, 1.0f);
     for (int ph = 0; ph < d.nphase; ++ph)
       for (int i = 0; i < d.c; ++i)
         if (d.act[ph] && !d.has_scale) {
-          dd[256 * 6 + ph * d.c + i] = std::fabs(d.m_in[ph * d.c + i]) + g[i];
+          dd[256 * 6 + ph * d.c + i] = std::fabs(d.m_in[ph * d.c + i]) + h->pd.a.gpre[i];
           dd[ph * d.c + i] = 1.0 / dd[256 * 6 + ph * d.c + i];
         }
     for (size_t i = 0; i < dd.size(); ++i) df[i] = (float)dd[i];
-    for (int i = 0; i < 6; ++i) {
-      h->pd.a.gpre[i] = g[i];
-      h->pf.a.gpre[i] = (float)g[i];
-    }
     SETUP_CK(cudaMemcpyAsync(const_cast<double*>(h->pd.a.dtab), dd.data(), sizeof(double) * dd.size(),
                              cudaMemcpyHostToDevice, st));
     if (d.precision == LSH_MIXED)
