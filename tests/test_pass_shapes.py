@@ -34,8 +34,9 @@ int main() {
 def shapes(tmp_path_factory):
     d = tmp_path_factory.mktemp("shapes")
     (d / "shapes.cu").write_text(PROGRAM)
-    subprocess.run([build._nvcc(), "-std=c++17", "-O0", "-I" + build.CSRC, "-I" + os.path.join(build.ROOT, "include"),
-                    "-o", str(d / "shapes"), str(d / "shapes.cu")], check=True, capture_output=True)
+    subprocess.run([build._nvcc(), *build.ARCH, "-std=c++17", "-O0", "-I" + build.CSRC,
+                    "-I" + os.path.join(build.ROOT, "include"), "-o", str(d / "shapes"), str(d / "shapes.cu")],
+                   check=True, capture_output=True)
     out = subprocess.run([str(d / "shapes")], check=True, capture_output=True, text=True).stdout
     return [tuple(int(v) for v in line.split()) for line in out.splitlines()]
 
