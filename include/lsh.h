@@ -132,7 +132,9 @@ typedef struct lsh_solve_opts {
                         later steps to half of what the least converged system of
                         the wave still needs: two refinement steps)                   */
   int max_outer;     /* LSH_MIXED: refinement steps (<= 0 selects 30)                    */
-  int check_every;   /* iterations between host convergence checks (<= 0 selects 8)     */
+  int check_every;   /* iterations between host convergence checks (<= 0 selects 8, on
+                        small problems more as the residual's decrease allows, at most
+                        as many as have run)                                           */
   int warm_start;    /* lsh_solve: tau holds the initial guess on entry                  */
   int no_graphs;     /* 0: each block of check_every CG iterations is captured once in a
                         CUDA graph (per handle, wave and precision) and replayed;

@@ -18,6 +18,7 @@
 #include <new>
 #include <thread>
 #include <type_traits>
+#include <utility>
 #include <vector>
 
 #include "df.cuh"
@@ -1049,25 +1050,35 @@ lsh_status cg_run(lsh_handle* h, PrecBufs<T>& P, const OpArgs<T>& a, int maxit, 
   // Chunks to enqueue before the states are read again.  Each reading leaves the device
   // idle for a round trip to the host (some 12 us, a third of an iteration of 32^3), and
   // iterations enqueued past convergence return at once.  With the default interval the
-  // residual's decrease so far says how many more the slowest system needs; 0.7 of them
-  // are enqueued in one go, because CG speeds up.  Beyond 2^23 elements an iteration is
-  // long against the round trip and the blocks of idle ones cost as much (90 x 100 x 84).
-  auto chunks_ahead = [&]() {
+  // residual's decrease, from the start or since the last reading if that was faster, says
+  // how many more the slowest system needs; 0.7 of them are enqueued in one go, because CG
+  // speeds up, and no more than have run: residuals that stand still at first and then drop
+  // (finite differences at contrast 10^-4, 80 iterations) would otherwise promise hundreds,
+  // and 256 x 256 of those in FP64 took 37 ms instead of 25.  Beyond 2^23 elements an
+  // iteration is long against the round trip and the blocks of idle ones cost as much
+  // (90 x 100 x 84).
+  std::vector<std::pair<int, double>> last(S, {0, 0.0});  // iterations and (r, r) at the reading before
+  auto chunks_ahead = [&](int run) {
     if (check_given || h->prof || (long long)S * a.c * a.V > (1ll << 23)) return 1;
     double most = 0.0;
     for (int s = 0; s < S; ++s) {
       const SolverState& t = out[s];
       if (t.done || t.iter < 1 || !(t.rr > 0.0) || !(t.bb > t.rr) || !(t.tol2 > 0.0)) continue;
-      most = std::max(most, t.iter * std::log(t.rr / t.tol2) / std::log(t.bb / t.rr));
+      const double left = std::log(t.rr / t.tol2);
+      double need = t.iter * left / std::log(t.bb / t.rr);
+      if (last[s].first > 0 && last[s].second > t.rr)
+        need = std::min(need, (t.iter - last[s].first) * left / std::log(last[s].second / t.rr));
+      most = std::max(most, need);
+      last[s] = {t.iter, t.rr};
     }
-    return (int)std::max(1.0, std::min(64.0, 0.7 * most / check_every));
+    return (int)std::max(1.0, std::min({64.0, 0.7 * most / check_every, (double)(run / check_every)}));
   };
   int it = 0;
   do {
     const int before = max_iter();
     long long live0 = 0;
     for (int k = 0; k < S; ++k) live0 += out[k].iter;
-    for (int ahead = chunks_ahead(); ahead > 0 && it < maxit; --ahead) {
+    for (int ahead = chunks_ahead(it); ahead > 0 && it < maxit; --ahead) {
       const int chunk = std::min(check_every, maxit - it);
       h->prof_now = h->prof && (h->prof_chunk++ % h->prof_every) == 0;
       if (graphs && chunk == check_every) {
