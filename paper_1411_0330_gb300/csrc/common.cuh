@@ -55,7 +55,9 @@ struct SolverState {
   unsigned int counter[4];  // last-block counters, reset by the last block
 };
 
-// the flag as the kernel ahead left it (not from a cache of invariant data)
+// The flag as the kernel ahead left it.  A kernel that may start before the one ahead has
+// ended (griddep_wait, chain_wait) reads the state through a volatile pointer: a load of
+// const __restrict__ data may come from a cache that such a kernel's start has not emptied.
 __device__ __forceinline__ bool is_done(const SolverState* st) {
   return *reinterpret_cast<const volatile int*>(&st->done) != 0;
 }

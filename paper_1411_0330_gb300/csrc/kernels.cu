@@ -118,9 +118,10 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) k_xfwd(OpArgs<T
   T alpha = 0, beta = 0;
   int k = 0;
   if (MODE == 1) {
-    k = st[s].iter;
-    alpha = (T)st[s].alpha;
-    beta = (T)st[s].beta;
+    const volatile SolverState* vst = st + s;  // as is_done
+    k = vst->iter;
+    alpha = (T)vst->alpha;
+    beta = (T)vst->beta;
   }
   const int nxv = nx / VEC;
   const FastDiv dxv(nxv), dxh(a.nxh);

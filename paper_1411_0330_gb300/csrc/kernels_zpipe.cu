@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(ZPipe<NC, N, FUSED>::THREADS, ZPipe<NC, N, FUS
         yp = (l - s * nqt) * TZ;
         kx0 = a.nx / 2;
       }
-      if (st == nullptr || !st[s].done) break;
+      if (st == nullptr || !is_done(st + s)) break;
     }
     tl_next = tl + gridDim.x;
     const bool live = tl < total;
