@@ -404,8 +404,7 @@ __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyinv(Op
   float2* PL = reinterpret_cast<float2*>(smem_raw);
   float2* tw = PL + N * RS;
   float* PR = reinterpret_cast<float*>(PL);
-  // this component's per-phase values after the plane (sized by the launch): M (or the
-  // modulus with a scale field), D, activity
+  // this component's per-phase values after the plane (sized by the launch): M, D, activity
   float* mloc = reinterpret_cast<float*>(tw + N);
   float* dloc = mloc + a.nphase;
   unsigned char* aloc = reinterpret_cast<unsigned char*>(dloc + a.nphase);
@@ -421,7 +420,7 @@ __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyinv(Op
     bulk_load_1d(PL + ky * RS, a.H + ((slab + ky) * a.nz + z) * a.hs, (uint32_t)(sizeof(float2) * RS), &bar);
   for (int u = threadIdx.x; u < N; u += TH) tw[u] = a.twx[u];
   for (int u = threadIdx.x; u < a.nphase; u += TH) {
-    mloc[u] = (a.scale && !a.frac) ? a.modtab[u * a.c + comp] : a.mtab[u * a.c + comp];
+    mloc[u] = a.mtab[u * a.c + comp];
     dloc[u] = MODE >= 5 && a.pre == 1 ? a.dtab[u * a.c + comp] : 1.f;
     aloc[u] = a.act[u];
   }
@@ -522,7 +521,7 @@ __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyinv(Op
   // two phases without a voxel field (the common case): both phases' M and
   // activity in registers, selected per voxel instead of read from the tables;
   // both active (A0 differs from both phases): no projection to apply
-  const bool two = MODE == 6 || (a.nphase <= 2 && !a.scale);
+  const bool two = MODE == 6 || (a.nphase <= 2 && !a.mfld);
   const float m0 = mloc[0], m1 = a.nphase > 1 ? mloc[1] : m0;
   const float d0 = dloc[0], d1 = a.nphase > 1 ? dloc[1] : d0;
   const float e0 = 1.f / d0, e1 = 1.f / d1;
@@ -537,6 +536,9 @@ __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyinv(Op
       const long long vox = pbase + (long long)row * N + xx;
       const float4 g4 = *reinterpret_cast<const float4*>(PR + 2 * RS * row + xx);
       const float xq[4] = {xc[b].x, xc[b].y, xc[b].z, xc[b].w};
+      float4 f4 = make_float4(0.f, 0.f, 0.f, 0.f);  // M of the voxels
+      if (MODE != 6 && a.mfld) f4 = *reinterpret_cast<const float4*>(a.mfld + field_class(a, comp) * a.fstride + vox);
+      const float field[4] = {f4.x, f4.y, f4.z, f4.w};
       const unsigned char ph[4] = {hc[b].x, hc[b].y, hc[b].z, hc[b].w};
       const float gv[4] = {g4.x, g4.y, g4.z, g4.w};
       float ov[4];
@@ -557,16 +559,12 @@ __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyinv(Op
             active = aloc[ph[u]] != 0;
             m = mloc[ph[u]];
             d = dloc[ph[u]];
-            if (a.scale) {
-              const float f = a.scale[vox + u];
-              if (a.frac) {
-                m = f * mloc[1] + (1.f - f) * mloc[0];  // Eq. (def_ah)
-              } else {
-                m = 1.f / (f * m - a.ref[comp]);
-              }
-              if (a.pre) d = 1.f / (fabsf(m) + a.gpre[comp]);
-            }
             e = 1.f / d;
+            if (a.mfld) {
+              m = field[u];
+              e = a.pre ? fabsf(m) + a.gpre[comp] : 1.f;
+              d = 1.f / e;
+            }
           }
           const float q = active ? fmaf(m, xq[u], gv[u]) : 0.f;
           z[u] = fmaf(-al, d * q, z[u]);
@@ -600,11 +598,7 @@ __global__ void __launch_bounds__(PlaneCfg<N>::TH, PlaneCfg<N>::MINB) k_xyinv(Op
           const int pp = ph[u];
           const bool active = aloc[pp] != 0;
           float m = mloc[pp];
-          if (a.scale) {
-            const float f = a.scale[vox + u];
-            m = a.frac ? f * mloc[1] + (1.f - f) * mloc[0]  // Eq. (def_ah)
-                       : 1.f / (f * m - a.ref[comp]);
-          }
+          if (a.mfld) m = field[u];
           ov[u] = active ? m * xq[u] + gv[u] : 0.f;
         }
       }

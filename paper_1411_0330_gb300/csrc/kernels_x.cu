@@ -133,11 +133,7 @@ __device__ __forceinline__ bool xinv_rows(const OpArgs<float>& a, const float* _
       const int p = ph[u];
       const bool active = aloc[p] != 0;
       float m = mloc[p * a.c + comp];
-      if (a.scale) {
-        const float f = a.scale[pbase + vox + u];
-        m = a.frac ? f * mloc[a.c + comp] + (1.f - f) * mloc[comp]  // Eq. (def_ah)
-                   : 1.f / (f * m - a.ref[comp]);
-      }
+      if (a.mfld) m = a.mfld[field_class(a, comp) * a.fstride + pbase + vox + u];
       if (MODE == 0) {
         ov[u] = active ? m * xq[u] + gv[u] : 0.f;
       } else if (MODE == 1) {
@@ -209,7 +205,7 @@ __global__ void __launch_bounds__(TH, (MODE == 5 ? 768 : 512) / TH) k_xinv_reg(O
   float *dloc = mloc + ntab, *eloc = dloc + ntab;  // MODE 5: D, 1 / D
   unsigned char* aloc = reinterpret_cast<unsigned char*>(MODE == 5 ? eloc + ntab : dloc);
   for (int u = threadIdx.x; u < N; u += blockDim.x) tw[u] = a.twx[u];
-  for (int u = threadIdx.x; u < ntab; u += blockDim.x) mloc[u] = (a.scale && !a.frac) ? a.modtab[u] : a.mtab[u];
+  for (int u = threadIdx.x; u < ntab; u += blockDim.x) mloc[u] = a.mtab[u];
   for (int u = threadIdx.x; u < a.nphase; u += blockDim.x) aloc[u] = a.act[u];
   if (MODE == 5)
     for (int u = threadIdx.x; u < ntab; u += blockDim.x) {
@@ -328,13 +324,7 @@ __global__ void __launch_bounds__(TH, (MODE == 5 ? 768 : 512) / TH) k_xinv_reg(O
         const int p = ph[u];
         const bool active = aloc[p] != 0;
         float m = mloc[p * a.c + comp];
-        if (MODE == 5 && a.mfld) {
-          m = a.mfld[field_class(a, comp) * a.fstride + pbase + vox + u];
-        } else if (a.scale) {
-          const float f = a.scale[pbase + vox + u];
-          m = a.frac ? f * mloc[a.c + comp] + (1.f - f) * mloc[comp]  // Eq. (def_ah)
-                     : 1.f / (f * m - a.ref[comp]);
-        }
+        if (a.mfld) m = a.mfld[field_class(a, comp) * a.fstride + pbase + vox + u];
         if constexpr (MODE == 5) {
           const int k = p * a.c + comp;
           const float e = a.mfld ? (a.pre ? fabsf(m) + a.gpre[comp] : 1.f) : eloc[k];
@@ -404,7 +394,7 @@ __global__ void __launch_bounds__(256, 2) k_xinv_regp(OpArgs<float> a, const flo
   const int ntab = a.nphase * a.c;
   unsigned char* aloc = reinterpret_cast<unsigned char*>(mloc + ntab);
   for (int u = threadIdx.x; u < N; u += blockDim.x) tw[u] = a.twx[u];
-  for (int u = threadIdx.x; u < ntab; u += blockDim.x) mloc[u] = (a.scale && !a.frac) ? a.modtab[u] : a.mtab[u];
+  for (int u = threadIdx.x; u < ntab; u += blockDim.x) mloc[u] = a.mtab[u];
   for (int u = threadIdx.x; u < a.nphase; u += blockDim.x) aloc[u] = a.act[u];
   const uint32_t bytes = (uint32_t)(sizeof(float2) * (size_t)XC::RY * a.hs);
   auto live = [&](long long rb) { return rb < nrb && (MODE != 1 || st[rb / bps].done == 0); };
