@@ -1437,10 +1437,12 @@ lsh_status scan_microstructure(lsh_handle* h) {
 // 225 / 57; moduli evenly spread (1000; 0.3) 382 / 80 / 348, over their logarithm (100; 2.9)
 // 163 / 112 / 135, (10^4; 14) 960 / 930 / 798.  Two phases: stiff inclusions (10) 70 / 40 /
 // 47, (10^4) 2019 / 1297 / 1352, rare stiff voxels (10^6) 40 / 50 / 31; finite differences
-// (100) 87 / 56 / 60, (10^5) 101 / 153 / 72, (10^6) 74 / 305 / 53.
+// (100) 87 / 56 / 60, (10^5) 101 / 153 / 72, (10^6) 74 / 305 / 53; elasticity at 32^3, spheres
+// (100) 305 / 146 / 168, (1000) 1159 / 603 / 649, random voxels 30 % stiff (100) 150 / 94 /
+// 88, 70 % soft (100; hi / lo 800) 136 / 136 / 84, (1000) 156 / 247 / 96.
 bool full_diagonal(int green, double lo, double hi, double mean, bool few) {
   if (green == LSH_GREEN_FILTERED) return true;
-  if (few) return !(hi <= (green == LSH_GREEN_TRUNCATED ? 1e5 : 4096.0) * lo);
+  if (few) return !(hi <= 512.0 * lo);
   return !(mean <= 5.0 * std::sqrt(hi * lo));
 }
 

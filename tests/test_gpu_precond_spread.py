@@ -6,6 +6,8 @@ whose inner solves start from nothing, worth up to half as many iterations again
 import numpy as np
 import pytest
 
+from helpers import k_mu
+
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 if torch.cuda.is_available():
@@ -81,3 +83,13 @@ def test_scale_fields_that_follow_one_another(precision, cluster, monkeypatch):
         want, fresh = lsh.Handle(ph, mods, scale=f, **kw).effective(tol=1e-9)
         assert np.array_equal(got, want)
         assert [i["iters"] for i in infos] == [i["iters"] for i in fresh]
+
+
+@pytest.mark.parametrize("share,contrast", [(0.7, 1e-2), (0.7, 1e-3), (0.3, 1e3)])
+@pytest.mark.parametrize("green", [0, 1])
+def test_elastic_voxels_of_two_kinds(share, contrast, green):
+    ph = (np.random.default_rng(2).random((16, 16, 16)) < share).astype(np.uint8)
+    mods = np.array([k_mu(1.0, 0.3), k_mu(contrast, 0.2)])
+    count = [most(lsh.Handle(torch.from_numpy(ph).cuda(), mods, physics=lsh.ELASTIC, green=green,
+                             precision=p).effective(tol=1e-10)[1]) for p in (lsh.FP64, lsh.MIXED)]
+    assert count[1] <= 1.2 * count[0] + 16, count
