@@ -1725,20 +1725,28 @@ lsh_status lsh_setup(const lsh_problem* prob, void* workspace, size_t bytes, voi
     const bool scaled = d.has_scale && !d.frac;  // decided with each scale field (set_voxel_fields)
     const bool full = scaled ? d.green == LSH_GREEN_FILTERED : full_diagonal(d);
     double* g = h->gdiag;
+    // Multiples of A0^{-1}: the operator is A0^{-1/2} (a projector, the filtered one a mean of
+    // projectors) A0^{-1/2}, and a g that differs by component beyond A0, as the operator's own
+    // diagonal does on boxes of unequal lengths, would pull its equal eigenvalues apart where M
+    // is small.  The multiple is the share of the components that the operator keeps, for the
+    // filtered one from its diagonal.  Conductivity, spheres, filtered, 8 x 64 x 64, mixed,
+    // plain / own diagonal / this: contrast 10 73 / 88 / 52, 10^-3 802 / 1569 / 573; truncated,
+    // 20 x 24 x 28, random soft voxels of 10^-4 350 / 490 / 281.  Elasticity keeps the filtered
+    // operator's own diagonal: it gains on every box tried.
     if (d.green == LSH_GREEN_FILTERED) {
       launch_gamma_diag(h->pd.a, h->partials, 152, h->sums, st);
       SETUP_CK(cudaMemcpyAsync(g, h->sums, sizeof(double) * d.c, cudaMemcpyDeviceToHost, st));
       SETUP_CK(cudaStreamSynchronize(st));
-      if (d.has_scale && d.physics == LSH_ELASTIC_ISO) {
+      if (d.physics == LSH_SCALAR) {
+        double share = 0.0;
+        for (int i = 0; i < d.c; ++i) share += g[i] * d.ref_in[i] / d.c;
+        for (int i = 0; i < d.c; ++i) g[i] = share / d.ref_in[i];
+      } else if (d.has_scale) {
         // the per-voxel fields hold one value for all deviatoric components
         const double mean = (g[1] + g[2] + g[3] + g[4] + g[5]) / 5.0;
         for (int i = 1; i < 6; ++i) g[i] = mean;
       }
     } else {
-      // A0^{-1} times the share of the components that the projector keeps.  Not its own
-      // diagonal, which on boxes of unequal lengths differs by component beyond A0: D would
-      // pull the projector's equal eigenvalues apart where M is small (20 x 24 x 28, random
-      // soft voxels of 10^-4, truncated: 490 iterations, 350 by plain CG).
       for (int i = 0; i < d.c; ++i) g[i] = (d.physics == LSH_ELASTIC_ISO ? 0.5 : 1.0 / d.dim) / d.ref_in[i];
     }
     set_precond_diag(h, full);

@@ -93,3 +93,24 @@ def test_elastic_voxels_of_two_kinds(share, contrast, green):
     count = [most(lsh.Handle(torch.from_numpy(ph).cuda(), mods, physics=lsh.ELASTIC, green=green,
                              precision=p).effective(tol=1e-10)[1]) for p in (lsh.FP64, lsh.MIXED)]
     assert count[1] <= 1.2 * count[0] + 16, count
+
+
+def spheres(shape, share):
+    rng, g = np.random.default_rng(3), np.zeros(shape, bool)
+    axes = np.meshgrid(*[np.arange(n) + 0.5 for n in shape], indexing="ij", sparse=True)
+    while g.mean() < share:
+        d2 = 0
+        for x, n in zip(axes, shape):
+            a = np.abs(x - rng.uniform(0, n))
+            d2 = d2 + np.minimum(a, n - a) ** 2
+        g |= d2 <= (min(shape) / 6) ** 2
+    return g.astype(np.uint8)
+
+
+@pytest.mark.parametrize("shape", [(8, 64, 64), (24, 20, 60), (16, 32, 64), (200, 30)])
+@pytest.mark.parametrize("contrast", [10.0, 1e-3])
+def test_filtered_operator_on_boxes_of_unequal_lengths(shape, contrast):
+    d = len(shape)
+    mods = np.array([np.eye(d), contrast * np.eye(d)])
+    count = phase_map_counts(spheres(shape, 0.3), mods, lsh.FILTERED)
+    assert count[1] <= 1.2 * count[0] + 16, count
