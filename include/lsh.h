@@ -309,8 +309,8 @@ lsh_status lsh_apply_noalloc(const lsh_problem *prob, const double *x, double *y
  * prologue), 1 y-forward, 2 z-forward + Gamma^h product + z-inverse,
  * 3 y-inverse, 4 x-inverse (with local term and (p, Kp)), 5 CG update.  The
  * plane passes with z variant 11, and the separate passes with inverse x variant
- * 0 and z variant 0 or 9, update the residual in the inverse pass: kind 4 then
- * covers that (with the scalars of the iteration) and kind 5 does not run. */
+ * 0, 1 or 3 and z variant 0 or 9, update the residual in the inverse pass: kind 4
+ * then covers that (with the scalars of the iteration) and kind 5 does not run. */
 typedef struct lsh_profile {
   long long launches;          /* kernels launched since the last reset            */
   long long timed_iters;       /* CG iterations covered by pass_ms                 */

@@ -74,7 +74,8 @@ template <typename T> struct OpArgs {
   // per-voxel local operator of handles with a scale or fraction field, formed once when
   // the field is set (a division per voxel instead of one per voxel, component, system
   // and pass): M, and D in FP64; [class][nbatch * V], class 0 / 1 the spherical /
-  // deviatoric components of elasticity, else the component.  Null: formed where used.
+  // deviatoric components of elasticity, else the component.  Null (no such field, or a call
+  // without a handle): formed where used.
   const T* mfld;
   const T* dfld;
   long long fstride;           // nbatch * V
@@ -122,8 +123,8 @@ template <typename T> struct OpArgs {
   double* dot; // FP32 z passes: each block's share of (p, Gamma p), zdot_blocks() of them per
                // system (null: not wanted)
   int pdl;     // the kernels of the fused plane iteration start before the one ahead has drained
-  int fuse;  // the CG update runs in the inverse pass: plane passes with z variant 11; other
-             // grids with the shared-memory inverse x pass and z variants 0 and 9
+  int fuse;  // the CG update runs in the inverse pass: plane passes with z variant 11; separate
+             // passes with inverse x variants 0, 1 and 3 and z variants 0 and 9
   int l2pf;  // plane passes, input planes requested into L2 at a block's start: bit 0 the
              // forward pass's x, r, p; bit 1 the inverse pass's p and phase planes
 };

@@ -32,7 +32,6 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
-#include <cstdint>
 #include <mutex>
 
 #include "internal.h"
