@@ -65,7 +65,7 @@ template <typename T> struct OpArgs {
   const T* mtab;               // per phase * c: diagonal of M (no scale field)
   const T* modtab;             // per phase * c: diagonal of A_phase (scale field)
   T ref[6];                    // diagonal of A0 (internal basis)
-  // diagonal preconditioner of the CG iterations, D = 1 / (|M_beta| + gpre): 0 none,
+  // diagonal preconditioner of the CG iterations, D = 1 / (|M_beta| + gpre).  pre: 0 none,
   // 1 per phase, 2 per voxel (scale or fraction field).  The residual buffer then
   // holds z = D r, so that p = z + beta p needs no phase map.
   int pre;
@@ -79,7 +79,7 @@ template <typename T> struct OpArgs {
   const T* mfld;
   const T* dfld;
   long long fstride;           // nbatch * V
-  T gpre[6];                   // share of the diagonal of the Green operator, per component
+  T gpre[6];                   // g per component: 0 or what stands for the Green operator's diagonal
   const T* loads;              // [S][6] macroscopic load per system (internal basis)
   // Green operator computed in the z pass instead of read from gtab (truncated
   // operator, FP32): physics, grid lengths, signed-frequency tables, constants

@@ -1051,7 +1051,7 @@ lsh_status cg_run(lsh_handle* h, PrecBufs<T>& P, const OpArgs<T>& a, int maxit, 
   // idle for a round trip to the host (some 12 us, a third of an iteration of 32^3), and
   // iterations enqueued past convergence return at once.  With the default interval the
   // residual's decrease, from the start or since the last reading if that was faster, says
-  // how many more the slowest system needs; 0.7 of them are enqueued in one go, because CG
+  // how many more the slowest system needs; 0.85 of them are enqueued in one go, because CG
   // speeds up, and no more than have run: residuals that stand still at first and then drop
   // (finite differences at contrast 10^-4, 80 iterations) would otherwise promise hundreds,
   // and 256 x 256 of those in FP64 took 37 ms instead of 25.  Beyond 2^23 elements an
@@ -1071,7 +1071,7 @@ lsh_status cg_run(lsh_handle* h, PrecBufs<T>& P, const OpArgs<T>& a, int maxit, 
       most = std::max(most, need);
       last[s] = {t.iter, t.rr};
     }
-    return (int)std::max(1.0, std::min({64.0, 0.7 * most / check_every, (double)(run / check_every)}));
+    return (int)std::max(1.0, std::min({64.0, 0.85 * most / check_every, (double)(run / check_every)}));
   };
   int it = 0;
   do {
