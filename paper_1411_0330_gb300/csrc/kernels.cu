@@ -1351,13 +1351,14 @@ __global__ void __launch_bounds__(kThreads) k_d2f_begin(OpArgs<float> a, const d
 
 // M (and D) of every voxel of a handle with a scale or fraction field, per class of
 // components (see OpArgs): grid (G, classes).  range (or null, zero on entry): the largest
-// and the complement of the smallest |M| of each class as FP32 bit patterns.
+// and the complement of the smallest |M| of each class as FP32 bit patterns, after them the
+// signs of M that occur (1: positive, 2: negative).
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_voxel_fields(OpArgs<T> a, T* __restrict__ mfld, T* __restrict__ dfld,
                                                            unsigned* __restrict__ range) {
   const int cls = blockIdx.y;  // also the first component of the class
   const double g = (double)a.gpre[cls];
-  unsigned hi = 0u, lo = 0u;
+  unsigned hi = 0u, lo = 0u, signs = 0u;
   for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < a.fstride;
        v += (long long)gridDim.x * blockDim.x) {
     const T f = (T)a.scale[v];
@@ -1368,13 +1369,16 @@ __global__ void __launch_bounds__(kThreads) k_voxel_fields(OpArgs<T> a, T* __res
     const unsigned bits = __float_as_uint(fabsf((float)m));
     hi = max(hi, bits);
     lo = max(lo, ~bits);
+    signs |= m > (T)0 ? 1u : (m < (T)0 ? 2u : 0u);
   }
   if (range) {
     hi = __reduce_max_sync(0xffffffffu, hi);
     lo = __reduce_max_sync(0xffffffffu, lo);
+    signs = __reduce_or_sync(0xffffffffu, signs);
     if ((threadIdx.x & 31) == 0) {
       atomicMax(range + 2 * cls, hi);
       atomicMax(range + 2 * cls + 1, lo);
+      atomicOr(range + 2 * gridDim.y, signs);
     }
   }
 }

@@ -462,6 +462,12 @@ struct lsh_handle {
   int* fault = nullptr;  // device word set by a kernel whose bounded wait ran out
   bool no_tma = false;
   bool no_cluster = false;  // kernel variants chosen by hand, or LSH_NO_CLUSTER=1
+  // M of one sign (of a scale field: of the present one).  CG asked for on an indefinite K
+  // runs without D, and in FP32 takes (p, K p) from the q that the update uses: summed from
+  // (p, Gamma p) and (p, M p) apart, which cancel there, alpha does not fit q and the
+  // residuals lose their orthogonality (32^3, contrast 100, mean reference, filtered: 2072
+  // iterations instead of 282).
+  bool definite = true;
   Layout lay;
   cudaStream_t stream;
   unsigned char* base;
@@ -749,6 +755,7 @@ template <typename T> OpArgs<T> wave_args(lsh_handle* h, const Wave& w) {
   a.TY = L.TY;
   a.TZ = L.TZ;
   a.pdl = 1;
+  if (!h->definite) a.pre = a.fuse = 0;
   return a;
 }
 
@@ -1033,7 +1040,7 @@ lsh_status cg_run_cluster(lsh_handle* h, PrecBufs<T>& P, const OpArgs<T>& a, int
 template <typename T>
 lsh_status cg_run(lsh_handle* h, PrecBufs<T>& P, const OpArgs<T>& a, int maxit, int check_every, bool check_given,
                   bool graphs, std::vector<SolverState>& out) {
-  if (P.cl_ok && !h->no_cluster) return cg_run_cluster<T>(h, P, a, maxit, check_every, out);
+  if (P.cl_ok && !h->no_cluster && (sizeof(T) == 8 || h->definite)) return cg_run_cluster<T>(h, P, a, maxit, check_every, out);
   const int S = a.S;
   out.assign(S, SolverState{});
   lsh_status stt;
@@ -1484,21 +1491,25 @@ lsh_status set_voxel_fields(lsh_handle* h) {
   if (!d.has_scale) return LSH_OK;
   OpArgs<double>& a = h->pd.a;
   double *mfld = const_cast<double*>(a.mfld), *dfld = const_cast<double*>(a.dfld);
-  // of a scale field lo, hi and the mean are known once its M are there
-  const bool open = !d.frac && d.green != LSH_GREEN_FILTERED;
+  // of a scale field the signs, lo, hi and the mean are known once its M are there; with the
+  // filtered operator D does not depend on them
+  const bool stats = !d.frac, open = stats && d.green != LSH_GREEN_FILTERED;
   const int classes = d.physics == LSH_ELASTIC_ISO ? 2 : d.c;
-  unsigned* range = open ? (unsigned*)h->Wdev : nullptr;
-  if (open) LSH_CK(cudaMemsetAsync(range, 0, sizeof(unsigned) * 2 * classes, h->stream));
+  unsigned* range = stats ? (unsigned*)h->Wdev : nullptr;
+  if (stats) LSH_CK(cudaMemsetAsync(range, 0, sizeof(unsigned) * (2 * classes + 1), h->stream));
   launch_voxel_fields<double>(a, mfld, open ? nullptr : dfld, range, d.B, h->stream);
   if (d.precision == LSH_MIXED)
     launch_voxel_fields<float>(h->pf.a, const_cast<float*>(h->pf.a.mfld), nullptr, nullptr, d.B, h->stream);
-  if (open) {
+  if (stats) {
     launch_comp_sums<double>(mfld, classes, a.fstride, 1, h->partials, 152, h->sums, h->stream);
-    unsigned bits[6] = {0, 0, 0, 0, 0, 0};
+    unsigned bits[7] = {0, 0, 0, 0, 0, 0, 0};
     double sum[3] = {0.0, 0.0, 0.0};
-    LSH_CK(cudaMemcpyAsync(bits, range, sizeof(unsigned) * 2 * classes, cudaMemcpyDeviceToHost, h->stream));
+    LSH_CK(cudaMemcpyAsync(bits, range, sizeof(unsigned) * (2 * classes + 1), cudaMemcpyDeviceToHost, h->stream));
     LSH_CK(cudaMemcpyAsync(sum, h->sums, sizeof(double) * classes, cudaMemcpyDeviceToHost, h->stream));
     LSH_CK(cudaStreamSynchronize(h->stream));
+    const bool definite = bits[2 * classes] != 3u;
+    if (definite != h->definite) h->drop_graphs();
+    h->definite = definite;
     bool full = false;
     for (int k = 0; k < classes; ++k) {
       const unsigned lo_bits = ~bits[2 * k + 1];
@@ -1508,7 +1519,7 @@ lsh_status set_voxel_fields(lsh_handle* h) {
       full = full || full_diagonal(d.green, lo, hi, std::fabs(sum[k]) / (double)a.fstride, false);
     }
     set_precond_diag(h, full);
-    launch_voxel_fields<double>(a, mfld, dfld, nullptr, d.B, h->stream);
+    if (open) launch_voxel_fields<double>(a, mfld, dfld, nullptr, d.B, h->stream);
   }
   return last_launch();
 }
@@ -1526,7 +1537,7 @@ lsh_status copy_microstructure(lsh_handle* h, const unsigned char* phase, const 
 
 // Separate passes: whether the inverse x pass can update z with these variants.
 int can_fuse(const lsh_handle* h, int x_variant, int z_variant) {
-  return h->d.precision == LSH_MIXED && x_variant != 2 && (z_variant == 0 || z_variant == 9) &&
+  return h->d.precision == LSH_MIXED && h->d.definite != 0 && x_variant != 2 && (z_variant == 0 || z_variant == 9) &&
                  (x_variant != 0 || make_cfg<float>(h->d, h->d.Smax).smem_x <= 200 * 1024)
              ? 1
              : 0;
@@ -1591,6 +1602,7 @@ lsh_status lsh_setup(const lsh_problem* prob, void* workspace, size_t bytes, voi
     delete h;
     return LSH_ERR_UNSUPPORTED_SIZE;
   }
+  h->definite = d.definite != 0;
   h->lay = make_layout(d);
   if (bytes < h->lay.total || ((uintptr_t)workspace % kAlign) != 0) { delete h; return LSH_ERR_WORKSPACE; }
   h->stream = (cudaStream_t)stream;
@@ -2164,7 +2176,8 @@ lsh_status lsh_autotune(lsh_handle* h, lsh_tune_report* rep) {
       b.plane = 1;
       b.tlay = 1;
       const int zc[7] = {0, 6, 8, 9, 7, 10, 11};
-      int bz = 0;  // the fastest of the variants that leave the update of r a kernel of its own
+      int bz = 0;  // the fastest of the variants that leave the update of r a kernel of its own (all
+                   // of them where K is indefinite)
       for (int k = 0; k < 7; ++k) {
         b.ztma = zc[k];
         r.zp_ms[k] = timeit([&]() {
@@ -2173,7 +2186,7 @@ lsh_status lsh_autotune(lsh_handle* h, lsh_tune_report* rep) {
           launch_zgamma<float>(b, P.L, nullptr, s);
           return true;
         });
-        if (zc[k] != 11 && r.zp_ms[k] > 0.f && (r.zp_ms[bz] < 0.f || r.zp_ms[k] < r.zp_ms[bz])) bz = k;
+        if ((zc[k] != 11 || d.definite == 0) && r.zp_ms[k] > 0.f && (r.zp_ms[bz] < 0.f || r.zp_ms[k] < r.zp_ms[bz])) bz = k;
       }
       b.ztma = zc[bz];
       const float f = timeit([&]() {
@@ -2185,7 +2198,7 @@ lsh_status lsh_autotune(lsh_handle* h, lsh_tune_report* rep) {
         return launch_xyinv(b, 1, P.p, P.q, P.st, h->partials, s);
       });
       float z = r.zp_ms[bz];
-      if (r.zp_ms[6] > 0.f) {
+      if (r.zp_ms[6] > 0.f && d.definite != 0) {
         // z variant 11 leaves (p, Gamma p), so that the inverse pass can update z
         b.ztma = 11;
         const float zf = timeit([&]() { return launch_zgamma_pipe(b, true, nullptr, s, h->partials); });
