@@ -103,10 +103,10 @@ __device__ __forceinline__ void line_stage_pair(double2* __restrict__ buf, int n
       y0 = a + c;
       y1 = fma(sg * (ao - co), wv.y, (a - c) * wv.x);
     }
-    // Both lanes of a pair have read before either writes.  The mask is the lanes that take
-    // this round, known from the indices: __activemask() would name whichever lanes happen to
-    // be together after the branches, and a partner may be missing from those.  One mask per
-    // warp, not one per pair, so that the barrier is a single instruction for all.
+    // Both lanes of a pair have read before either writes.  The mask is the lanes with an
+    // element left, known from the indices: __activemask() would name whichever lanes happen
+    // to be together after the branches, and a partner may be missing from those.  One mask
+    // per warp, not one per pair, so that the barrier is a single instruction for all.
     const int left = total - (w - (int)(threadIdx.x & 31));
     __syncwarp(left >= 32 ? 0xffffffffu : (1u << left) - 1u);
     f[i0 + im] = y0;
